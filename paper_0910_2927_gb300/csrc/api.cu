@@ -501,31 +501,27 @@ SGN_API int sgn_hw_apply(sgn_ctx* c, const void* in, void* out, int nrhs, int pr
     if (precision == SGN_PREC_FP64) {
         const double2* pi = reinterpret_cast<const double2*>(in);
         double2* po = reinterpret_cast<double2*>(out);
-        // staging (complex128 units): the packed copies of in and out, then the float-float
-        // (hi, lo) pairs of in and out (4 nn complex64 = 2 nn complex128)
-        const size_t need = (packed ? 0 : 2 * nn) + (ffa ? 2 * nn : 0);
-        double2* t = nullptr;
-        if (need) {
-            SGN_CHECK(dev_alloc(c, c->stage, need * sizeof(double2)));
-            t = as<double2>(c->stage);
-        }
-        if (!packed) {
-            SGN_CUDA(pack_fields<double2>(pi, t, c->vol, nrhs, c->work));
-            pi = t;
-            po = t + nn;
-        }
         if (ffa) {
+            // staging (complex128 units): the packed copies of in and out, then the float-float
+            // (hi, lo) pairs of in and out (4 nn complex64 = 2 nn complex128)
+            SGN_CHECK(dev_alloc(c, c->stage, ((packed ? 0 : 2 * nn) + 2 * nn) * sizeof(double2)));
+            double2* t = as<double2>(c->stage);
+            if (!packed) {
+                SGN_CUDA(pack_fields<double2>(pi, t, c->vol, nrhs, c->work));
+                pi = t;
+                po = t + nn;
+            }
             float2* f = reinterpret_cast<float2*>(t + (packed ? 0 : 2 * nn));
             float2 *ih = f, *il = f + nn, *oh = f + 2 * nn, *ol = f + 3 * nn;
             SGN_CUDA(split_ff(pi, ih, il, (int64_t)nn, c->work));
             SGN_CUDA(launch_hw_ff(oh, ol, ih, il, as<float4>(c->Uff), nrhs, stencil_params(c, adjoint), c->work));
             SGN_CUDA(join_ff(oh, ol, po, (int64_t)nn, c->work));
-        } else {
-            SGN_CHECK(tune_stencil(c, 0, nrhs, const_cast<double2*>(pi), po));
-            SGN_CUDA(apply_hw64(c, po, pi, nrhs, adjoint, nullptr, c->work));
+            if (!packed)
+                SGN_CUDA(unpack_fields<double2>(po, reinterpret_cast<double2*>(out), c->vol, nrhs, c->work));
+        } else {  // the FP64 stencil reads and writes either order
+            SGN_CUDA(launch_hw_f64(po, pi, as<double2>(c->U64), nrhs, stencil_params(c, adjoint), nullptr, c->work,
+                                   !packed));
         }
-        if (!packed)
-            SGN_CUDA(unpack_fields<double2>(po, reinterpret_cast<double2*>(out), c->vol, nrhs, c->work));
     } else {
         const float2* pi = reinterpret_cast<const float2*>(in);
         float2* po = reinterpret_cast<float2*>(out);
@@ -593,7 +589,6 @@ SGN_API int sgn_apply_direct(sgn_ctx* c, const double* b, double* x, int nrhs, i
     SGN_CHECK(dev_alloc(c, c->stage, 2 * nn * sizeof(double2)));
     double2* t = as<double2>(c->stage);
     SGN_CUDA(pack_fields<double2>(reinterpret_cast<const double2*>(b), t, c->vol, nrhs, c->work));
-    SGN_CHECK(tune_stencil(c, 0, nrhs, t, t + nn));
     int st = direct_projection(c, t, t + nn, nrhs, k, (flags & SGN_APPLY_ADJOINT) != 0, k_used);
     if (st == SGN_OK) SGN_CUDA(unpack_fields<double2>(t + nn, reinterpret_cast<double2*>(x), c->vol, nrhs, c->work));
     SGN_CHECK(ses.close());

@@ -150,12 +150,11 @@ cudaError_t apply_hw32(const sgn_ctx* c, float2* out, const float2* in, int ncol
 int solve(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int ncol, bool adjoint, bool no_a,
           sgn_report* rep,
           const std::vector<std::complex<double>>* cshift = nullptr);
-// Tuning key of the FP32 stencil for the context's link storage: 1 FP32, 2 BF16, 3 FP16 links
-// (0 is the FP64 stencil).
+// Tuning key of the FP32 stencil for the context's link storage: 1 FP32, 2 BF16, 3 FP16 links.
 inline int stencil_prec32(const sgn_ctx* c) {
     return c->link_storage == SGN_LINKS_BF16 ? 2 : c->link_storage == SGN_LINKS_FP16 ? 3 : 1;
 }
-// Pick the fastest stencil launch shape for (precision, ncol) by timing candidates
+// Pick the fastest FP32 stencil launch shape for (precision, ncol) by timing candidates
 // on the given buffers (ncol fields each); cached in the context.  Not during capture.
 int tune_stencil(sgn_ctx* c, int prec, int ncol, void* in, void* out);
 // Dot products <a_c, b_c> of ncol pairs of FP64 fields (host result, FP64 reductions).

@@ -99,8 +99,9 @@ cudaError_t pack_links(const double2* natural, double2* packed, int64_t vol, cud
 // ---------------------------------------------------------- kernel entry --
 // Stencil: out = H_W in for nrhs fields (packed layout).  Real = double or float; links in
 // double, float or bf16 (Link).  skip: per-field flags (non-zero: skip), may be null.
-// Launch shape: sx sites (x fastest) by rb threads per CTA, each thread nr
-// fields of its site (nr <= 3 FP32, 1 FP64); {0, 0, 1} picks the default.
+// The FP64 stencil (stencil_f64.cu) also takes both fields in natural order (nat).
+// Launch shape of the FP32 stencil: sx sites (x fastest) by rb threads per CTA, each thread nr
+// fields of its site (nr <= 3); {0, 0, 1} picks the default.
 // pipe = 1 selects the FP32 kernel that stages neighbour spinors through shared
 // memory with cp.async (a stage ahead of the computation; nr <= 2); pipe = 2 the
 // FP32 kernel with paired (FFMA2) arithmetic over two fields (nr = 2), pipe = 3 the
@@ -112,7 +113,7 @@ struct StencilShape {
     int pipe = 0;
 };
 cudaError_t launch_hw_f64(double2* out, const double2* in, const double2* U, int nrhs,
-                          const StencilParams& p, const int* skip, cudaStream_t st, StencilShape sh = {});
+                          const StencilParams& p, const int* skip, cudaStream_t st, bool nat = false);
 cudaError_t launch_hw_f32(float2* out, const float2* in, const float2* U, int nrhs,
                           const StencilParams& p, const int* skip, cudaStream_t st, StencilShape sh = {});
 cudaError_t launch_hw_f32_bf16links(float2* out, const float2* in, const __nv_bfloat162* U, int nrhs,

@@ -95,7 +95,7 @@ StencilShape shape_for(const sgn_ctx* c, int prec, int ncol) {
 cudaError_t apply_hw64(const sgn_ctx* c, double2* out, const double2* in, int ncol, bool adjoint, const int* skip,
                        cudaStream_t st) {
     return launch_hw_f64(out, in, reinterpret_cast<const double2*>(c->U64.p), ncol, stencil_params(c, adjoint), skip,
-                         st, shape_for(c, 0, ncol));
+                         st);
 }
 
 cudaError_t apply_hw32(const sgn_ctx* c, float2* out, const float2* in, int ncol, bool adjoint, const int* skip,
@@ -134,10 +134,9 @@ int tune_stencil(sgn_ctx* c, int prec, int ncol, void* in, void* out) {
     cudaStream_t st = c->work;
     const StencilParams p = stencil_params(c, false);
     std::vector<StencilShape> cands;
-    for (int pipe = 0; pipe <= (prec == 0 ? 0 : 3); ++pipe)
+    for (int pipe = 0; pipe <= 3; ++pipe)
         for (int nr : {1, 2, 3}) {
-            if (pipe == 4) continue;  // the colour-split kernel has its own shapes below
-            if (nr > ncol || (prec == 0 && nr > 1) || (pipe == 1 && nr > 2) || (pipe >= 2 && nr != 2)) continue;
+            if (nr > ncol || (pipe == 1 && nr > 2) || (pipe >= 2 && nr != 2)) continue;
             const int groups = (ncol + nr - 1) / nr;
             const int maxt = nr == 1 && !pipe ? 384 : 256;
             for (int rb : {1, 2, 3, 4, 6, 8, 12, 16}) {
@@ -146,15 +145,12 @@ int tune_stencil(sgn_ctx* c, int prec, int ncol, void* in, void* out) {
                     if (sx * rb <= maxt && sx * rb >= 64) cands.push_back({sx, rb, nr, pipe});
             }
         }
-    if (prec != 0)  // colour-split kernel: sg site groups of 10 sites x fw fields per CTA (<= 8 warps)
-        for (int fw : {1, 2, 3, 4, 6, 8})
-            for (int sg : {1, 2, 4, 8})
-                if (fw <= ncol && sg * fw <= 8 && sg * fw >= 2) cands.push_back({sg, fw, 1, 4});
+    // colour-split kernel: sg site groups of 10 sites x fw fields per CTA (<= 8 warps)
+    for (int fw : {1, 2, 3, 4, 6, 8})
+        for (int sg : {1, 2, 4, 8})
+            if (fw <= ncol && sg * fw <= 8 && sg * fw >= 2) cands.push_back({sg, fw, 1, 4});
     if (cands.empty()) cands.push_back({});
     auto run = [&](StencilShape sh) -> cudaError_t {
-        if (prec == 0)
-            return launch_hw_f64(reinterpret_cast<double2*>(out), reinterpret_cast<const double2*>(in),
-                                 reinterpret_cast<const double2*>(c->U64.p), ncol, p, nullptr, st, sh);
         if (prec == 2)
             return launch_hw_f32_bf16links(reinterpret_cast<float2*>(out), reinterpret_cast<const float2*>(in),
                                            reinterpret_cast<const __nv_bfloat162*>(c->U16.p), ncol, p, nullptr, st,
@@ -928,7 +924,6 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
     const int p32 = stencil_prec32(c);
     SGN_CHECK(tune_stencil(c, p32, ncol, E->V, E->t));
     SGN_CHECK(tune_stencil(c, p32, B, E1->V, E1->t));
-    SGN_CHECK(tune_stencil(c, 0, ncol, bt, t64));
 
     CycleArgs a;
     a.adjoint = adjoint;
@@ -1246,7 +1241,6 @@ int solve(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int ncol, 
     else
         SGN_CUDA(apply_hw64(c, reinterpret_cast<double2*>(E->V), rstart, ncol, adjoint, nullptr, st));
 
-    SGN_CHECK(tune_stencil(c, 0, ncol, E->V, E->t));
     CycleArgs a;
     a.adjoint = adjoint;
     a.L = Lb;
@@ -1347,7 +1341,6 @@ int solve_columns_gmres(sgn_ctx* c, const double2* rhs, int ncol, const std::vec
         SGN_CUDA(reduce(rd, m, ncol, RM_STORE, 0, E->S, nullptr, st));
         SGN_CUDA(maxpy_scale<double2>(RB, m, E->S.red, E->rstride, V0, n, V0, n, nullptr, n, ncol, nullptr, st));
     }
-    SGN_CHECK(tune_stencil(c, 0, ncol, E->V, E->t));
     CycleArgs a;
     a.adjoint = adjoint;
     a.L = Lb;

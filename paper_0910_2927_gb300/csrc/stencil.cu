@@ -1,5 +1,6 @@
-// Wilson kernel H_W(mu) = gamma5 D_W(mu) on nrhs fields (Sec. 1 of the paper;
-// D_W(mu) with e^{+mu} on forward and e^{-mu} on backward time hops).
+// Wilson kernel H_W(mu) = gamma5 D_W(mu) on nrhs fields in FP32 (Sec. 1 of the paper;
+// D_W(mu) with e^{+mu} on forward and e^{-mu} on backward time hops).  The FP64 stencil is in
+// stencil_f64.cu, the float-float one in stencil_ff.cu.
 //
 // One thread computes one site of one field.  A CTA covers SX consecutive
 // sites (x fastest) for RB fields, so the RB warps that share a site tile
@@ -51,38 +52,6 @@ __device__ __forceinline__ void cmac_conj(Cx<R>& acc, Cx<R> u, Cx<R> v) {
 template <class R>
 struct Field;
 template <>
-struct Field<double> {
-    using T = double2;
-    static __device__ __forceinline__ void load(const double2* __restrict__ f, int64_t site, int64_t vol2,
-                                                Cx<double> p[12]) {
-        const double2* s = f + 2 * site;
-#pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            const double2 a = __ldg(s + k * vol2);
-            const double2 b = __ldg(s + k * vol2 + 1);
-            p[2 * k] = {a.x, a.y};
-            p[2 * k + 1] = {b.x, b.y};
-        }
-    }
-    // CS: evict-first stores (see k_hw)
-    template <bool CS>
-    static __device__ __forceinline__ void store(double2* __restrict__ f, int64_t site, int64_t vol2,
-                                                 const Cx<double> p[12]) {
-        double2* s = f + 2 * site;
-#pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            const double2 a = make_double2(p[2 * k].x, p[2 * k].y), b = make_double2(p[2 * k + 1].x, p[2 * k + 1].y);
-            if constexpr (CS) {
-                __stcs(s + k * vol2, a);
-                __stcs(s + k * vol2 + 1, b);
-            } else {
-                s[k * vol2] = a;
-                s[k * vol2 + 1] = b;
-            }
-        }
-    }
-};
-template <>
 struct Field<float> {
     using T = float2;
     static __device__ __forceinline__ void load(const float2* __restrict__ f, int64_t site, int64_t vol2,
@@ -95,6 +64,7 @@ struct Field<float> {
             p[2 * k + 1] = {v.z, v.w};
         }
     }
+    // CS: evict-first stores (see k_hw)
     template <bool CS>
     static __device__ __forceinline__ void store(float2* __restrict__ f, int64_t site, int64_t vol2,
                                                  const Cx<float> p[12]) {
@@ -112,13 +82,6 @@ struct Field<float> {
 
 template <class R, class LinkT>
 struct Link;
-template <>
-struct Link<double, double2> {
-    static __device__ __forceinline__ Cx<double> ld(const double2* __restrict__ U, int64_t i) {
-        double2 v = __ldg(U + i);
-        return {v.x, v.y};
-    }
-};
 template <>
 struct Link<float, float2> {
     static __device__ __forceinline__ Cx<float> ld(const float2* __restrict__ U, int64_t i) {
@@ -246,19 +209,6 @@ __device__ __forceinline__ void hop(Cx<R> (&acc)[NR][12], const typename Field<R
     hop_links<R, LinkT, NU, S, NR>(acc, h0, h1, U, link_site, coef, vol);
 }
 
-template <class R>
-__device__ __forceinline__ R cf_of(const StencilParams& P, int nu) {
-    if constexpr (sizeof(R) == 4) return P.cf32[nu]; else return P.cf[nu];
-}
-template <class R>
-__device__ __forceinline__ R cb_of(const StencilParams& P, int nu) {
-    if constexpr (sizeof(R) == 4) return P.cb32[nu]; else return P.cb[nu];
-}
-template <class R>
-__device__ __forceinline__ R diag_of(const StencilParams& P) {
-    if constexpr (sizeof(R) == 4) return P.diag32; else return P.diag;
-}
-
 template <class R, class LinkT, int NU, int NR>
 __device__ __forceinline__ void both_hops(Cx<R> (&acc)[NR][12], const typename Field<R>::T* __restrict__ in,
                                           const bool (&act)[NR], const LinkT* __restrict__ U, int64_t site,
@@ -269,13 +219,13 @@ __device__ __forceinline__ void both_hops(Cx<R> (&acc)[NR][12], const typename F
     const int L = P.L[NU];
     // forward neighbour
     int64_t fw = site + stride;
-    R cf = cf_of<R>(P, NU);
+    R cf = P.cf32[NU];
     if (co[NU] == L - 1) {
         fw = site - (int64_t)(L - 1) * stride;
         if (P.ap[NU]) cf = -cf;
     }
     int64_t bw = site - stride;
-    R cb = cb_of<R>(P, NU);
+    R cb = P.cb32[NU];
     if (co[NU] == 0) {
         bw = site + (int64_t)(L - 1) * stride;
         if (P.ap[NU]) cb = -cb;
@@ -323,7 +273,7 @@ __global__ void __launch_bounds__(NR == 1 ? 384 : 256)
         co[3] = (int)q2;
     }
     Cx<R> acc[NR][12];
-    const R d = diag_of<R>(P);
+    const R d = P.diag32;
 #pragma unroll
     for (int i = 0; i < NR; ++i) {
         if (act[i]) {
@@ -1050,41 +1000,26 @@ template <class R, class LinkT>
 cudaError_t launch(typename Field<R>::T* out, const typename Field<R>::T* in, const LinkT* U, int nrhs,
                    const StencilParams& p, const int* skip, cudaStream_t st, StencilShape sh) {
     if (nrhs <= 0 || p.vol <= 0) return cudaSuccess;
-    if (sh.pipe == 4) {  // the colour-split FP32 kernel: sx site groups of 10 sites, rb fields per CTA
-        if constexpr (sizeof(R) == 4) {
-            if (sh.nr != 1) return cudaErrorInvalidValue;
-            return launch_cs<LinkT>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
-        } else {
-            return cudaErrorInvalidValue;
-        }
+    if (sh.pipe == 4) {  // the colour-split kernel: sx site groups of 10 sites, rb fields per CTA
+        if (sh.nr != 1) return cudaErrorInvalidValue;
+        return launch_cs<LinkT>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
     }
-    if (sh.pipe == 2 || sh.pipe == 3) {  // the paired FP32 kernel (3: capped at 128 registers)
-        if constexpr (sizeof(R) == 4) {
-            if (sh.sx % 32 != 0 || sh.rb < 1 || sh.sx * sh.rb > 256 || sh.nr != 2) return cudaErrorInvalidValue;
-            if (sh.pipe == 3) return launch_x2<LinkT, 2>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
-            return launch_x2<LinkT, 1>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
-        } else {
-            return cudaErrorInvalidValue;
-        }
+    if (sh.pipe == 2 || sh.pipe == 3) {  // the paired kernel (3: capped at 128 registers)
+        if (sh.sx % 32 != 0 || sh.rb < 1 || sh.sx * sh.rb > 256 || sh.nr != 2) return cudaErrorInvalidValue;
+        if (sh.pipe == 3) return launch_x2<LinkT, 2>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
+        return launch_x2<LinkT, 1>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
     }
-    if (sh.pipe) {  // the pipelined FP32 kernel: 1 or 2 fields per thread, up to 256 threads per CTA
-        if constexpr (sizeof(R) == 4) {
-            if (sh.sx % 32 != 0 || sh.rb < 1 || sh.sx * sh.rb > 256 || sh.nr < 1 || sh.nr > 2)
-                return cudaErrorInvalidValue;
-            if (sh.nr == 1) return launch_pipe<LinkT, 1>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
-            return launch_pipe<LinkT, 2>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
-        } else {
+    if (sh.pipe) {  // the pipelined kernel: 1 or 2 fields per thread, up to 256 threads per CTA
+        if (sh.sx % 32 != 0 || sh.rb < 1 || sh.sx * sh.rb > 256 || sh.nr < 1 || sh.nr > 2)
             return cudaErrorInvalidValue;
-        }
+        if (sh.nr == 1) return launch_pipe<LinkT, 1>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
+        return launch_pipe<LinkT, 2>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
     }
     if (sh.sx > 0 && sh.rb > 0) {  // a tuned shape: validate it against the kernel's launch bounds
-        const int maxnr = sizeof(R) == 8 ? 1 : 3;  // more fields per thread spill registers
-        if (sh.sx % 32 != 0 || sh.nr < 1 || sh.nr > maxnr || sh.sx * sh.rb > (sh.nr == 1 ? 384 : 256))
+        if (sh.sx % 32 != 0 || sh.nr < 1 || sh.nr > 3 || sh.sx * sh.rb > (sh.nr == 1 ? 384 : 256))
             return cudaErrorInvalidValue;
-        if constexpr (sizeof(R) == 4) {
-            if (sh.nr == 2) return launch_nr<R, LinkT, 2>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
-            if (sh.nr == 3) return launch_nr<R, LinkT, 3>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
-        }
+        if (sh.nr == 2) return launch_nr<R, LinkT, 2>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
+        if (sh.nr == 3) return launch_nr<R, LinkT, 3>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
         return launch_nr<R, LinkT, 1>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
     }
     // default: one field per thread, up to 12 fields of a site tile per CTA
@@ -1126,10 +1061,6 @@ cudaError_t pack_links(const double2* natural, double2* packed, int64_t vol, cud
     return cudaGetLastError();
 }
 
-cudaError_t launch_hw_f64(double2* out, const double2* in, const double2* U, int nrhs, const StencilParams& p,
-                          const int* skip, cudaStream_t st, StencilShape sh) {
-    return launch<double, double2>(out, in, U, nrhs, p, skip, st, sh);
-}
 cudaError_t launch_hw_f32(float2* out, const float2* in, const float2* U, int nrhs, const StencilParams& p,
                           const int* skip, cudaStream_t st, StencilShape sh) {
     return launch<float, float2>(out, in, U, nrhs, p, skip, st, sh);
