@@ -669,7 +669,7 @@ SGN_API int sgn_inner_products(sgn_ctx* c, const double* V, int J, const double*
     SGN_CHECK(enter(c));
     Session ses(c);
     const int64_t n = c->n;
-    const int nblk = reduce_blocks<double2>(n);
+    const int nblk = dot_blocks<double2>(n, nrhs);
     const int rs = (J + 8) & ~7;
     const size_t pbytes = (sizeof(double2) * (size_t)nrhs * rs * nblk + 255) & ~size_t(255);
     const size_t rbytes = (sizeof(double2) * (size_t)nrhs * rs + 255) & ~size_t(255);

@@ -10,7 +10,8 @@
 // (wave_blocks), and PKT follows from it.  Dot products: each thread forms its PKT pack products
 // (in FP32 for complex64 storage, i.e. chunks of 8 complex products), promotes
 // them to FP64 and the rest of the reduction -- warp shuffles, the CTA sum and
-// the per-column sum over CTAs -- is FP64 in a fixed order (no atomics).
+// the per-column sum over CTAs -- is FP64 in a fixed order (no atomics).  The FP64 inner products
+// are in gs_f64.cu.
 #include "blas.cuh"
 
 #include <cstdlib>
@@ -23,7 +24,7 @@ namespace {
 constexpr int NT = 256;
 constexpr int NWARP = NT / 32;
 constexpr int PK = 4;  // default packs per thread (reduce_blocks)
-constexpr int MAXSLOT = 136;  // >= 2 kmax + 3 (delayed CGS2), >= deflation size + 1, >= eigensolver block + 1
+constexpr int MAXSLOT = kMaxSlots;
 
 template <class T>
 struct Ops;
@@ -242,9 +243,11 @@ __device__ __forceinline__ void flush_partials(double2 (*sm)[NWARP], int nslot, 
 // ---------------------------------------------------------------- kernels --
 
 // partial[j] = sum_e conj(V_j[e]) w[e], j < J; slot J: ||w||^2 if with_norm.
-template <class T, int PKT>
-__global__ void __launch_bounds__(NT) k_mdot(Basis<T> V, int J, const T* __restrict__ w, int64_t wsr, int64_t npk,
+// FP32 storage (FP64: gs_f64.cu).
+template <int PKT>
+__global__ void __launch_bounds__(NT) k_mdot(Basis<float2> V, int J, const float2* __restrict__ w, int64_t wsr, int64_t npk,
                                              Reduce rd, int with_norm, const int* __restrict__ skip) {
+    using T = float2;
     using O = Ops<T>;
     const int col = blockIdx.y;
     if (skip && skip[col]) return;
@@ -261,38 +264,19 @@ __global__ void __launch_bounds__(NT) k_mdot(Basis<T> V, int J, const T* __restr
     const T* vb = V.base + col * V.sr;
     for (int j = 0; j < J; ++j) {
         const T* vj = vb + j * V.sj;
-        if constexpr (O::CPX == 2) {
-            float ax = 0.f, ay = 0.f;  // FP32 chunk of PKT packs (8 complex products)
+        float ax = 0.f, ay = 0.f;  // FP32 chunk of PKT packs (8 complex products)
 #pragma unroll
-            for (int p = 0; p < PKT; ++p) {
-                int64_t i = base + p * NT;
-                if (i < npk) O::dot_acc(ax, ay, O::ld_ro(vj, i), wv[p]);
-            }
-            warp_store_f(sm, j, ax, ay, lane, warp);
-        } else {
-            double2 acc = make_double2(0, 0);
-#pragma unroll
-            for (int p = 0; p < PKT; ++p) {
-                int64_t i = base + p * NT;
-                if (i < npk) acc = cadd(acc, O::dot(O::ld_ro(vj, i), wv[p]));
-            }
-            acc = warp_sum(acc);
-            if (lane == 0) sm[j][warp] = acc;
+        for (int p = 0; p < PKT; ++p) {
+            int64_t i = base + p * NT;
+            if (i < npk) O::dot_acc(ax, ay, O::ld_ro(vj, i), wv[p]);
         }
+        warp_store_f(sm, j, ax, ay, lane, warp);
     }
     if (with_norm) {
-        if constexpr (O::CPX == 2) {
-            float a = 0.f;
+        float a = 0.f;
 #pragma unroll
-            for (int p = 0; p < PKT; ++p) O::nrm2_acc(a, wv[p]);
-            warp_store_f(sm, J, a, 0.f, lane, warp);
-        } else {
-            double a = 0;
-#pragma unroll
-            for (int p = 0; p < PKT; ++p) a += O::nrm2(wv[p]);
-            double2 acc = warp_sum(make_double2(a, 0));
-            if (lane == 0) sm[J][warp] = acc;
-        }
+        for (int p = 0; p < PKT; ++p) O::nrm2_acc(a, wv[p]);
+        warp_store_f(sm, J, a, 0.f, lane, warp);
     }
     flush_partials(sm, J + (with_norm ? 1 : 0), rd, col);
 }
@@ -379,16 +363,16 @@ __global__ void __launch_bounds__(NT) k_maxpy_scale(Basis<T> V, int J, const dou
     const int col = blockIdx.y;
     if (skip && skip[col]) return;
     __shared__ typename O::C cs[MAXSLOT];
-    for (int j = threadIdx.x; j < J; j += NT) cs[j] = O::coef(coef[(int64_t)col * cstride + j]);
+    for (int j = threadIdx.x; j < J; j += blockDim.x) cs[j] = O::coef(coef[(int64_t)col * cstride + j]);
     __syncthreads();
     const T* wc = w + col * wsr;
     T* oc = out + col * osr;
     const double sc = scale ? scale[col] : 1.0;
-    const int64_t base = (int64_t)blockIdx.x * NT * PKT + threadIdx.x;
+    const int64_t base = (int64_t)blockIdx.x * blockDim.x * PKT + threadIdx.x;
     typename O::P wv[PKT];
 #pragma unroll
     for (int p = 0; p < PKT; ++p) {
-        int64_t i = base + p * NT;
+        int64_t i = base + p * (int)blockDim.x;
         wv[p] = i < npk ? O::ld(wc, i) : O::zero();
     }
     const T* vb = V.base + col * V.sr;
@@ -397,7 +381,7 @@ __global__ void __launch_bounds__(NT) k_maxpy_scale(Basis<T> V, int J, const dou
         const typename O::C c = cs[j];
 #pragma unroll
         for (int p = 0; p < PKT; ++p) {
-            int64_t i = base + p * NT;
+            int64_t i = base + p * (int)blockDim.x;
             if (i < npk) O::sub_cv(wv[p], c, O::ld_ro(vj, i));
         }
     }
@@ -405,13 +389,13 @@ __global__ void __launch_bounds__(NT) k_maxpy_scale(Basis<T> V, int J, const dou
         const float scf = (float)sc;
 #pragma unroll
         for (int p = 0; p < PKT; ++p) {
-            int64_t i = base + p * NT;
+            int64_t i = base + p * (int)blockDim.x;
             if (i < npk) O::st(oc, i, O::scalf(wv[p], scf));
         }
     } else {
 #pragma unroll
         for (int p = 0; p < PKT; ++p) {
-            int64_t i = base + p * NT;
+            int64_t i = base + p * (int)blockDim.x;
             if (i < npk) O::st(oc, i, O::scal(wv[p], sc));
         }
     }
@@ -427,11 +411,11 @@ __global__ void __launch_bounds__(NT) k_update_x(Basis<T> V, int J, const double
     if (skip && skip[col]) return;
     if (kk && kk[col] < J) J = kk[col];
     __shared__ double2 cs[MAXSLOT];
-    for (int j = threadIdx.x; j < J; j += NT) cs[j] = coef[(int64_t)col * cstride + j];
+    for (int j = threadIdx.x; j < J; j += blockDim.x) cs[j] = coef[(int64_t)col * cstride + j];
     __syncthreads();
     double2* xc = x + col * xsr;
     const T* vb = V.base + col * V.sr;
-    const int64_t base = (int64_t)blockIdx.x * NT * PKT + threadIdx.x;
+    const int64_t base = (int64_t)blockIdx.x * blockDim.x * PKT + threadIdx.x;
     double2 acc[PKT][O::CPX];
 #pragma unroll
     for (int p = 0; p < PKT; ++p)
@@ -445,7 +429,7 @@ __global__ void __launch_bounds__(NT) k_update_x(Basis<T> V, int J, const double
             const T* vj = vb + (j0 + g) * V.sj;
 #pragma unroll
             for (int p = 0; p < PKT; ++p) {
-                const int64_t i = base + p * NT;
+                const int64_t i = base + p * (int)blockDim.x;
                 q[g][p] = (j0 + g < J && i < npk) ? O::ld_ro(vj, i) : O::zero();
             }
         }
@@ -457,7 +441,7 @@ __global__ void __launch_bounds__(NT) k_update_x(Basis<T> V, int J, const double
     }
 #pragma unroll
     for (int p = 0; p < PKT; ++p) {
-        const int64_t i = base + p * NT;
+        const int64_t i = base + p * (int)blockDim.x;
         if (i >= npk) break;
 #pragma unroll
         for (int q = 0; q < O::CPX; ++q) {
@@ -489,12 +473,12 @@ __global__ void __launch_bounds__(NT) k_update_shifts(Basis<T> V, int J, const d
     const int ng = (s - g0) < SG ? (s - g0) : SG;
     extern __shared__ unsigned char smraw[];
     typename O::C* ys = reinterpret_cast<typename O::C*>(smraw);  // [ng][J]: this CTA's shifts
-    for (int t = threadIdx.x; t < ng * J; t += NT) {
+    for (int t = threadIdx.x; t < ng * J; t += blockDim.x) {
         int i = t / J, j = t % J;
         ys[t] = O::coef(y[((int64_t)col * s + g0 + i) * kmax + j]);
     }
     __syncthreads();
-    const int64_t i = tile * NT + threadIdx.x;
+    const int64_t i = tile * blockDim.x + threadIdx.x;
     if (i >= npk) return;
     const T* vb = V.base + col * V.sr;
     {
@@ -523,10 +507,12 @@ __global__ void __launch_bounds__(NT) k_update_shifts(Basis<T> V, int J, const d
 // once-orthogonalised candidate, z = A^2 u):  slots [0,J) s = Q^dag u,
 // [J,2J) t = Q^dag z, 2J: u^dag u, 2J+1: u^dag z, 2J+2: z^dag z.  With z = null
 // (the closing pass of a cycle) only s and u^dag u (slot J).
-template <class T, int PKT>
-__global__ void __launch_bounds__(NT) k_dcgs_dots(Basis<T> V, int J, const T* __restrict__ u,
-                                                  const T* __restrict__ z, int64_t wsr, int64_t npk, Reduce rd,
+// FP32 storage (FP64: gs_f64.cu).
+template <int PKT>
+__global__ void __launch_bounds__(NT) k_dcgs_dots(Basis<float2> V, int J, const float2* __restrict__ u,
+                                                  const float2* __restrict__ z, int64_t wsr, int64_t npk, Reduce rd,
                                                   const int* __restrict__ skip) {
+    using T = float2;
     using O = Ops<T>;
     const int col = blockIdx.y;
     if (skip && skip[col]) return;
@@ -542,199 +528,101 @@ __global__ void __launch_bounds__(NT) k_dcgs_dots(Basis<T> V, int J, const T* __
         zv[p] = (zc && i < npk) ? O::ld(zc, i) : O::zero();
     }
     const T* vb = V.base + col * V.sr;
-    if constexpr (O::CPX == 2) {
-        // FP32 storage: per-thread FP32 chunk partials are staged in shared memory
-        // for a tile of TL basis vectors; each (vector, component) slot is then summed
-        // over the whole CTA by one warp in double-float and written as this CTA's
-        // FP64 partial.  Four values per vector: Re/Im of q^dag u and of q^dag z.
-        constexpr int TL = 8;
-        __shared__ float st[TL * 4][NT + 8];  // rows padded: the segmented sums below are bank-conflict free
-        double* pd = reinterpret_cast<double*>(rd.partial);
-        auto put = [&](int slot, int comp, double v) {
-            pd[2 * (((int64_t)col * rd.stride + slot) * rd.nblk + blockIdx.x) + comp] = v;
-        };
-        const int nv = zc ? 4 : 2;
-        // loads of GB basis vectors are issued together: 8 independent 16-byte
-        // loads in flight per thread (4 with PKT = 4, whose registers hold 4 packs
-        // of u and z already)
-        constexpr int GB = PKT == 4 ? 1 : 8 / PKT;
-        for (int l0 = 0; l0 < J; l0 += TL) {
-            const int tl = (J - l0) < TL ? (J - l0) : TL;
+    // FP32 storage: per-thread FP32 chunk partials are staged in shared memory
+    // for a tile of TL basis vectors; each (vector, component) slot is then summed
+    // over the whole CTA by one warp in double-float and written as this CTA's
+    // FP64 partial.  Four values per vector: Re/Im of q^dag u and of q^dag z.
+    constexpr int TL = 8;
+    __shared__ float st[TL * 4][NT + 8];  // rows padded: the segmented sums below are bank-conflict free
+    double* pd = reinterpret_cast<double*>(rd.partial);
+    auto put = [&](int slot, int comp, double v) {
+        pd[2 * (((int64_t)col * rd.stride + slot) * rd.nblk + blockIdx.x) + comp] = v;
+    };
+    const int nv = zc ? 4 : 2;
+    // loads of GB basis vectors are issued together: 8 independent 16-byte
+    // loads in flight per thread (4 with PKT = 4, whose registers hold 4 packs
+    // of u and z already)
+    constexpr int GB = PKT == 4 ? 1 : 8 / PKT;
+    for (int l0 = 0; l0 < J; l0 += TL) {
+        const int tl = (J - l0) < TL ? (J - l0) : TL;
 #pragma unroll
-            for (int g0 = 0; g0 < TL; g0 += GB) {
-                if (g0 >= tl) break;
-                typename O::P q[GB][PKT];
+        for (int g0 = 0; g0 < TL; g0 += GB) {
+            if (g0 >= tl) break;
+            typename O::P q[GB][PKT];
 #pragma unroll
-                for (int g = 0; g < GB; ++g) {
-                    const T* vl = vb + (l0 + g0 + g) * V.sj;
+            for (int g = 0; g < GB; ++g) {
+                const T* vl = vb + (l0 + g0 + g) * V.sj;
+#pragma unroll
+                for (int p = 0; p < PKT; ++p) {
+                    const int64_t i = base + p * NT;
+                    q[g][p] = (g0 + g < tl && i < npk) ? O::ld_ro(vl, i) : O::zero();
+                }
+            }
+#pragma unroll
+            for (int g = 0; g < GB; ++g) {
+                if (g0 + g < tl) {
+                    float sx = 0.f, sy = 0.f, tx = 0.f, ty = 0.f;
 #pragma unroll
                     for (int p = 0; p < PKT; ++p) {
-                        const int64_t i = base + p * NT;
-                        q[g][p] = (g0 + g < tl && i < npk) ? O::ld_ro(vl, i) : O::zero();
+                        O::dot_acc(sx, sy, q[g][p], uv[p]);
+                        if (zc) O::dot_acc(tx, ty, q[g][p], zv[p]);
                     }
-                }
-#pragma unroll
-                for (int g = 0; g < GB; ++g) {
-                    if (g0 + g < tl) {
-                        float sx = 0.f, sy = 0.f, tx = 0.f, ty = 0.f;
-#pragma unroll
-                        for (int p = 0; p < PKT; ++p) {
-                            O::dot_acc(sx, sy, q[g][p], uv[p]);
-                            if (zc) O::dot_acc(tx, ty, q[g][p], zv[p]);
-                        }
-                        st[(g0 + g) * 4 + 0][threadIdx.x] = sx;
-                        st[(g0 + g) * 4 + 1][threadIdx.x] = sy;
-                        st[(g0 + g) * 4 + 2][threadIdx.x] = tx;
-                        st[(g0 + g) * 4 + 3][threadIdx.x] = ty;
-                    }
+                    st[(g0 + g) * 4 + 0][threadIdx.x] = sx;
+                    st[(g0 + g) * 4 + 1][threadIdx.x] = sy;
+                    st[(g0 + g) * 4 + 2][threadIdx.x] = tx;
+                    st[(g0 + g) * 4 + 3][threadIdx.x] = ty;
                 }
             }
-            __syncthreads();
-            {
-                // slot sl = tid / 8 (TL * 4 = 32 slots for 256 threads), summed by 8 lanes:
-                // lane seg adds values seg, seg + 8, ... in FP32, then a 3-level shuffle
-                // tree.  Every partial is a sum of at most a few hundred FP32 products
-                // (error ~ eps_32 times the sum of their moduli, the rounding the FP32
-                // products carry anyway); the sum over CTAs is FP64.
-                static_assert(TL * 4 * 8 == NT, "one 8-lane group per slot");
-                const int sl = threadIdx.x >> 3, seg = threadIdx.x & 7;
-                float a = 0.f;
-#pragma unroll
-                for (int k = 0; k < NT / 8; ++k) a += st[sl][k * 8 + seg];
-                a += __shfl_xor_sync(0xffffffffu, a, 1);
-                a += __shfl_xor_sync(0xffffffffu, a, 2);
-                a += __shfl_xor_sync(0xffffffffu, a, 4);
-                const int g = sl >> 2, v = sl & 3;
-                if (seg == 0 && g < tl && v < nv) put(v < 2 ? l0 + g : J + l0 + g, v & 1, (double)a);
-            }
-            __syncthreads();
         }
-        // norms and u^dag z
-        float a = 0.f, bx = 0.f, by = 0.f, gz = 0.f;
-#pragma unroll
-        for (int p = 0; p < PKT; ++p) {
-            O::nrm2_acc(a, uv[p]);
-            if (zc) {
-                O::dot_acc(bx, by, uv[p], zv[p]);
-                O::nrm2_acc(gz, zv[p]);
-            }
-        }
-        st[0][threadIdx.x] = a;
-        st[1][threadIdx.x] = bx;
-        st[2][threadIdx.x] = by;
-        st[3][threadIdx.x] = gz;
         __syncthreads();
-        const int bs = zc ? 2 * J : J;
-        if (warp < (zc ? 4 : 1)) {
-            const double r = cta_sum_df(st[warp], lane);
-            if (lane == 0) {
-                if (warp == 0) {
-                    put(bs, 0, r);
-                    put(bs, 1, 0.0);
-                } else if (warp == 1) {
-                    put(bs + 1, 0, r);
-                } else if (warp == 2) {
-                    put(bs + 1, 1, r);
-                } else {
-                    put(bs + 2, 0, r);
-                    put(bs + 2, 1, 0.0);
-                }
-            }
+        {
+            // slot sl = tid / 8 (TL * 4 = 32 slots for 256 threads), summed by 8 lanes:
+            // lane seg adds values seg, seg + 8, ... in FP32, then a 3-level shuffle
+            // tree.  Every partial is a sum of at most a few hundred FP32 products
+            // (error ~ eps_32 times the sum of their moduli, the rounding the FP32
+            // products carry anyway); the sum over CTAs is FP64.
+            static_assert(TL * 4 * 8 == NT, "one 8-lane group per slot");
+            const int sl = threadIdx.x >> 3, seg = threadIdx.x & 7;
+            float a = 0.f;
+#pragma unroll
+            for (int k = 0; k < NT / 8; ++k) a += st[sl][k * 8 + seg];
+            a += __shfl_xor_sync(0xffffffffu, a, 1);
+            a += __shfl_xor_sync(0xffffffffu, a, 2);
+            a += __shfl_xor_sync(0xffffffffu, a, 4);
+            const int g = sl >> 2, v = sl & 3;
+            if (seg == 0 && g < tl && v < nv) put(v < 2 ? l0 + g : J + l0 + g, v & 1, (double)a);
         }
-        return;
-    } else {
-        // FP64 storage: the same tiling with FP64 values; each (vector, component)
-        // slot is summed over the CTA by one warp in a fixed order (8 values per
-        // lane, then a shuffle tree), one warp-reduction per slot instead of one per
-        // warp and vector.
-        constexpr int TL = 4;
-        __shared__ double sd[TL * 4][NT];
-        double* pd = reinterpret_cast<double*>(rd.partial);
-        auto put = [&](int slot, int comp, double v) {
-            pd[2 * (((int64_t)col * rd.stride + slot) * rd.nblk + blockIdx.x) + comp] = v;
-        };
-        auto cta_sum = [&](const double* row) {
-            double a = 0;
-#pragma unroll
-            for (int k = 0; k < NT / 32; ++k) a += row[lane + 32 * k];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-            return a;
-        };
-        const int nv = zc ? 4 : 2;
-        constexpr int GB = PKT == 4 ? 1 : 4 / PKT;
-        for (int l0 = 0; l0 < J; l0 += TL) {
-            const int tl = (J - l0) < TL ? (J - l0) : TL;
-#pragma unroll
-            for (int g0 = 0; g0 < TL; g0 += GB) {
-                if (g0 >= tl) break;
-                typename O::P q[GB][PKT];
-#pragma unroll
-                for (int g = 0; g < GB; ++g) {
-                    const T* vl = vb + (l0 + g0 + g) * V.sj;
-#pragma unroll
-                    for (int p = 0; p < PKT; ++p) {
-                        const int64_t i = base + p * NT;
-                        q[g][p] = (g0 + g < tl && i < npk) ? O::ld_ro(vl, i) : O::zero();
-                    }
-                }
-#pragma unroll
-                for (int g = 0; g < GB; ++g) {
-                    if (g0 + g < tl) {
-                        double2 as = make_double2(0, 0), at = make_double2(0, 0);
-#pragma unroll
-                        for (int p = 0; p < PKT; ++p) {
-                            as = cadd(as, O::dot(q[g][p], uv[p]));
-                            if (zc) at = cadd(at, O::dot(q[g][p], zv[p]));
-                        }
-                        sd[(g0 + g) * 4 + 0][threadIdx.x] = as.x;
-                        sd[(g0 + g) * 4 + 1][threadIdx.x] = as.y;
-                        sd[(g0 + g) * 4 + 2][threadIdx.x] = at.x;
-                        sd[(g0 + g) * 4 + 3][threadIdx.x] = at.y;
-                    }
-                }
-            }
-            __syncthreads();
-            for (int sl = warp; sl < tl * 4; sl += NWARP) {
-                const int g = sl >> 2, v = sl & 3;
-                if (v >= nv) continue;
-                const double r = cta_sum(sd[sl]);
-                if (lane == 0) put(v < 2 ? l0 + g : J + l0 + g, v & 1, r);
-            }
-            __syncthreads();
-        }
-        // norms and u^dag z
-        double a = 0, bx = 0, by = 0, gz = 0;
-#pragma unroll
-        for (int p = 0; p < PKT; ++p) {
-            a += O::nrm2(uv[p]);
-            if (zc) {
-                const double2 d = O::dot(uv[p], zv[p]);
-                bx += d.x;
-                by += d.y;
-                gz += O::nrm2(zv[p]);
-            }
-        }
-        sd[0][threadIdx.x] = a;
-        sd[1][threadIdx.x] = bx;
-        sd[2][threadIdx.x] = by;
-        sd[3][threadIdx.x] = gz;
         __syncthreads();
-        const int bs = zc ? 2 * J : J;
-        if (warp < (zc ? 4 : 1)) {
-            const double r = cta_sum(sd[warp]);
-            if (lane == 0) {
-                if (warp == 0) {
-                    put(bs, 0, r);
-                    put(bs, 1, 0.0);
-                } else if (warp == 1) {
-                    put(bs + 1, 0, r);
-                } else if (warp == 2) {
-                    put(bs + 1, 1, r);
-                } else {
-                    put(bs + 2, 0, r);
-                    put(bs + 2, 1, 0.0);
-                }
+    }
+    // norms and u^dag z
+    float a = 0.f, bx = 0.f, by = 0.f, gz = 0.f;
+#pragma unroll
+    for (int p = 0; p < PKT; ++p) {
+        O::nrm2_acc(a, uv[p]);
+        if (zc) {
+            O::dot_acc(bx, by, uv[p], zv[p]);
+            O::nrm2_acc(gz, zv[p]);
+        }
+    }
+    st[0][threadIdx.x] = a;
+    st[1][threadIdx.x] = bx;
+    st[2][threadIdx.x] = by;
+    st[3][threadIdx.x] = gz;
+    __syncthreads();
+    const int bs = zc ? 2 * J : J;
+    if (warp < (zc ? 4 : 1)) {
+        const double r = cta_sum_df(st[warp], lane);
+        if (lane == 0) {
+            if (warp == 0) {
+                put(bs, 0, r);
+                put(bs, 1, 0.0);
+            } else if (warp == 1) {
+                put(bs + 1, 0, r);
+            } else if (warp == 2) {
+                put(bs + 1, 1, r);
+            } else {
+                put(bs + 2, 0, r);
+                put(bs + 2, 1, 0.0);
             }
         }
     }
@@ -743,17 +631,19 @@ __global__ void __launch_bounds__(NT) k_dcgs_dots(Basis<T> V, int J, const T* __
 // Delayed CGS2, update of step j:  q_j = (u - Q s) / rho  (written over u), and
 // the next candidate  u_{j+1} = z / rho - Q c - d q_j  (when next != null).
 // Coefficients per column: [0,J) s, [J,2J) c, 2J: (1/rho, 0), 2J+1: d.
-template <class T, int PKT>
-__global__ void __launch_bounds__(NT) k_dcgs_update(Basis<T> V, int J, const double2* __restrict__ coef,
-                                                    int cstride, T* u, const T* __restrict__ z, T* next,
+// FP32 storage (FP64: gs_f64.cu).
+template <int PKT>
+__global__ void __launch_bounds__(NT) k_dcgs_update(Basis<float2> V, int J, const double2* __restrict__ coef,
+                                                    int cstride, float2* u, const float2* __restrict__ z, float2* next,
                                                     int64_t wsr, int64_t npk, const int* __restrict__ skip) {
+    using T = float2;
     using O = Ops<T>;
     const int col = blockIdx.y;
     if (skip && skip[col]) return;
     __shared__ typename O::C cs[MAXSLOT], cc[MAXSLOT];
     __shared__ double ex[2][2];
     const double2* cf = coef + (int64_t)col * cstride;
-    for (int l = threadIdx.x; l < J; l += NT) {
+    for (int l = threadIdx.x; l < J; l += blockDim.x) {
         cs[l] = O::coef(cf[l]);
         cc[l] = O::coef(cf[J + l]);
     }
@@ -763,14 +653,13 @@ __global__ void __launch_bounds__(NT) k_dcgs_update(Basis<T> V, int J, const dou
         ex[1][1] = cf[2 * J + 1].y;
     }
     __syncthreads();
-    const double inv_rho = ex[0][0];
-    const float inv_rho_f = (float)inv_rho;
+    const float inv_rho_f = (float)ex[0][0];
     const typename O::C dd = O::coef(make_double2(ex[1][0], ex[1][1]));
     T* uc = u + col * wsr;
     const T* zc = next ? z + col * wsr : nullptr;
     T* nc = next ? next + col * wsr : nullptr;
     const T* vb = V.base + col * V.sr;
-    const int64_t base = (int64_t)blockIdx.x * NT * PKT + threadIdx.x;
+    const int64_t base = (int64_t)blockIdx.x * blockDim.x * PKT + threadIdx.x;
     // Q s and Q c with the basis loop outside: the loads of UNR basis vectors
     // (PKT packs each) are independent and in flight together
     typename O::P qs[PKT], qc[PKT];
@@ -787,7 +676,7 @@ __global__ void __launch_bounds__(NT) k_dcgs_update(Basis<T> V, int J, const dou
             const T* vl = vb + (l0 + g) * V.sj;
 #pragma unroll
             for (int p = 0; p < PKT; ++p) {
-                const int64_t i = base + p * NT;
+                const int64_t i = base + p * (int)blockDim.x;
                 q[g][p] = (l0 + g < J && i < npk) ? O::ld_ro(vl, i) : O::zero();
             }
         }
@@ -803,33 +692,18 @@ __global__ void __launch_bounds__(NT) k_dcgs_update(Basis<T> V, int J, const dou
             }
         }
     }
-    typename O::C one;
-    if constexpr (O::CPX == 1) {
-        one = make_double2(1.0, 0.0);
-    } else {
-        one = make_float2(1.0f, 0.0f);
-    }
+    const typename O::C one = make_float2(1.0f, 0.0f);
 #pragma unroll
     for (int p = 0; p < PKT; ++p) {
-        const int64_t i = base + p * NT;
+        const int64_t i = base + p * (int)blockDim.x;
         if (i >= npk) break;
         typename O::P uv = O::ld(uc, i);
         // q_j = (u - qs) / rho
         O::sub_cv(uv, one, qs[p]);
-        typename O::P qj;
-        if constexpr (O::CPX == 2) {
-            qj = O::scalf(uv, inv_rho_f);
-        } else {
-            qj = O::scal(uv, inv_rho);
-        }
+        const typename O::P qj = O::scalf(uv, inv_rho_f);
         O::st(uc, i, qj);
         if (nc) {
-            typename O::P nv;
-            if constexpr (O::CPX == 2) {
-                nv = O::scalf(O::ld(zc, i), inv_rho_f);
-            } else {
-                nv = O::scal(O::ld(zc, i), inv_rho);
-            }
+            typename O::P nv = O::scalf(O::ld(zc, i), inv_rho_f);
             O::sub_cv(nv, one, qc[p]);
             O::sub_cv(nv, dd, qj);
             O::st(nc, i, nv);
@@ -1311,6 +1185,26 @@ int wave_blocks(int64_t n, int ncol) {
     return best;
 }
 
+namespace {
+// CTAs per column, threads per CTA and packs per thread of the update kernels (one thread's
+// elements, all basis vectors).  FP32: whole waves of 256 threads.  FP64: those kernels are bound
+// by the two FP64 lanes of an SM, so what counts is that every SM gets the same number of warps:
+// one element per thread in CTAs of two warps, or of one while that leaves SMs without a CTA.
+struct Split {
+    int nb, threads, pkt;
+};
+template <class T>
+Split split_for(int64_t n, int ncol) {
+    if constexpr (Ops<T>::CPX == 1) {
+        const int threads = n * ncol < 64 * kFewWarps ? 32 : 64;
+        return {(int)((n + threads - 1) / threads), threads, 1};
+    } else {
+        const int nb = wave_blocks<T>(n, ncol);
+        return {nb, NT, pk_for(n / Ops<T>::CPX, nb)};
+    }
+}
+}  // namespace
+
 // Instantiate the kernel call for PKT = 1, 2 or 4.
 #define SGN_PK_SWITCH(PKV, ...)               \
     switch (PKV) {                            \
@@ -1333,13 +1227,13 @@ int wave_blocks(int64_t n, int ncol) {
             return cudaErrorInvalidValue;     \
     }
 
-template <class T>
-cudaError_t mdot(Basis<T> V, int J, const T* w, int64_t wsr, int64_t n, int ncol, const Reduce& rd, int with_norm,
-                 const int* skip, cudaStream_t st) {
+template <>
+cudaError_t mdot<float2>(Basis<float2> V, int J, const float2* w, int64_t wsr, int64_t n, int ncol, const Reduce& rd,
+                         int with_norm, const int* skip, cudaStream_t st) {
     if (J + 1 > MAXSLOT) return cudaErrorInvalidValue;
-    int64_t npk = n / Ops<T>::CPX;
+    int64_t npk = n / Ops<float2>::CPX;
     dim3 grid(rd.nblk, ncol);
-    SGN_PK_SWITCH(pk_for(npk, rd.nblk), k_mdot<T, PKT_><<<grid, NT, 0, st>>>(V, J, w, wsr, npk, rd, with_norm, skip))
+    SGN_PK_SWITCH(pk_for(npk, rd.nblk), k_mdot<PKT_><<<grid, NT, 0, st>>>(V, J, w, wsr, npk, rd, with_norm, skip))
     count_launch();
     return cudaGetLastError();
 }
@@ -1373,9 +1267,8 @@ cudaError_t maxpy_scale(Basis<T> V, int J, const double2* coef, int cstride, con
                         int64_t osr, const double* scale, int64_t n, int ncol, const int* skip, cudaStream_t st) {
     if (J > MAXSLOT) return cudaErrorInvalidValue;
     int64_t npk = n / Ops<T>::CPX;
-    const int nb = wave_blocks<T>(n, ncol);
-    dim3 grid(nb, ncol);
-    SGN_PK_SWITCH(pk_for(npk, nb), k_maxpy_scale<T, PKT_><<<grid, NT, 0, st>>>(V, J, coef, cstride, w, wsr, out, osr,
+    const Split sp = split_for<T>(n, ncol);
+    SGN_PK_SWITCH(sp.pkt, k_maxpy_scale<T, PKT_><<<dim3(sp.nb, ncol), sp.threads, 0, st>>>(V, J, coef, cstride, w, wsr, out, osr,
                                                                               scale, npk, skip))
     count_launch();
     return cudaGetLastError();
@@ -1386,10 +1279,9 @@ cudaError_t update_x(Basis<T> V, int J, const double2* coef, int cstride, double
                      int ncol, const int* skip, const int* kk, cudaStream_t st) {
     if (J > MAXSLOT) return cudaErrorInvalidValue;
     int64_t npk = n / Ops<T>::CPX;
-    const int nb = wave_blocks<T>(n, ncol);
-    dim3 grid(nb, ncol);
-    SGN_PK_SWITCH(pk_for(npk, nb),
-                  k_update_x<T, PKT_><<<grid, NT, 0, st>>>(V, J, coef, cstride, x, xsr, npk, skip, kk))
+    const Split sp = split_for<T>(n, ncol);
+    SGN_PK_SWITCH(sp.pkt,
+                  k_update_x<T, PKT_><<<dim3(sp.nb, ncol), sp.threads, 0, st>>>(V, J, coef, cstride, x, xsr, npk, skip, kk))
     count_launch();
     return cudaGetLastError();
 }
@@ -1407,58 +1299,49 @@ cudaError_t update_shifts(Basis<T> V, int J, const double2* y, int s, int kmax, 
     const int sg = (forced == 20 && s <= 20) || forced == 10 || forced == 8 || forced == 4 || forced == 1 ? forced : 2;
     size_t smem = sizeof(typename Ops<T>::C) * (size_t)(s < sg ? s : sg) * (size_t)J;
     if (smem > 48 * 1024) return cudaErrorInvalidValue;
-    const int64_t tiles = (npk + NT - 1) / NT;
+    const int threads = split_for<T>(n, ncol).threads;
+    const int64_t tiles = (npk + threads - 1) / threads;
     const int64_t nblk = tiles * ((s + sg - 1) / sg);
     if (nblk > 0x7fffffff) return cudaErrorInvalidValue;
     dim3 grid((unsigned)nblk, ncol);
     if (sg == 20)
-        k_update_shifts<T, 20><<<grid, NT, smem, st>>>(V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
+        k_update_shifts<T, 20><<<grid, threads, smem, st>>>(V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
     else if (sg == 10)
-        k_update_shifts<T, 10><<<grid, NT, smem, st>>>(V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
+        k_update_shifts<T, 10><<<grid, threads, smem, st>>>(V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
     else if (sg == 8)
-        k_update_shifts<T, 8><<<grid, NT, smem, st>>>(V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
+        k_update_shifts<T, 8><<<grid, threads, smem, st>>>(V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
     else if (sg == 4)
-        k_update_shifts<T, 4><<<grid, NT, smem, st>>>(V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
+        k_update_shifts<T, 4><<<grid, threads, smem, st>>>(V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
     else if (sg == 1)
-        k_update_shifts<T, 1><<<grid, NT, smem, st>>>(V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
+        k_update_shifts<T, 1><<<grid, threads, smem, st>>>(V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
     else
-        k_update_shifts<T, 2><<<grid, NT, smem, st>>>(V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
+        k_update_shifts<T, 2><<<grid, threads, smem, st>>>(V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
     count_launch();
     return cudaGetLastError();
 }
 
-template <class T>
-cudaError_t dcgs_dots(Basis<T> V, int J, const T* u, const T* z, int64_t wsr, int64_t n, int ncol, const Reduce& rd,
-                      const int* skip, cudaStream_t st) {
+template <>
+cudaError_t dcgs_dots<float2>(Basis<float2> V, int J, const float2* u, const float2* z, int64_t wsr, int64_t n,
+                              int ncol, const Reduce& rd, const int* skip, cudaStream_t st) {
     if (2 * J + 3 > MAXSLOT) return cudaErrorInvalidValue;
-    int64_t npk = n / Ops<T>::CPX;
+    int64_t npk = n / Ops<float2>::CPX;
     dim3 grid(rd.nblk, ncol);
-    SGN_PK_SWITCH(pk_for(npk, rd.nblk), k_dcgs_dots<T, PKT_><<<grid, NT, 0, st>>>(V, J, u, z, wsr, npk, rd, skip))
+    SGN_PK_SWITCH(pk_for(npk, rd.nblk), k_dcgs_dots<PKT_><<<grid, NT, 0, st>>>(V, J, u, z, wsr, npk, rd, skip))
     count_launch();
     return cudaGetLastError();
 }
 
-template <class T>
-cudaError_t dcgs_update(Basis<T> V, int J, const double2* coef, int cstride, T* u, const T* z, T* next, int64_t wsr,
-                        int64_t n, int ncol, const int* skip, cudaStream_t st) {
+template <>
+cudaError_t dcgs_update<float2>(Basis<float2> V, int J, const double2* coef, int cstride, float2* u, const float2* z,
+                                float2* next, int64_t wsr, int64_t n, int ncol, const int* skip, cudaStream_t st) {
     if (J > MAXSLOT) return cudaErrorInvalidValue;
-    int64_t npk = n / Ops<T>::CPX;
-    const int nb = wave_blocks<T>(n, ncol);
-    dim3 grid(nb, ncol);
-    SGN_PK_SWITCH(pk_for(npk, nb), k_dcgs_update<T, PKT_><<<grid, NT, 0, st>>>(V, J, coef, cstride, u, z, next, wsr,
-                                                                              npk, skip))
+    int64_t npk = n / Ops<float2>::CPX;
+    const Split sp = split_for<float2>(n, ncol);
+    SGN_PK_SWITCH(sp.pkt, k_dcgs_update<PKT_><<<dim3(sp.nb, ncol), sp.threads, 0, st>>>(V, J, coef, cstride, u, z, next,
+                                                                                       wsr, npk, skip))
     count_launch();
     return cudaGetLastError();
 }
-
-template cudaError_t dcgs_dots<double2>(Basis<double2>, int, const double2*, const double2*, int64_t, int64_t, int,
-                                        const Reduce&, const int*, cudaStream_t);
-template cudaError_t dcgs_dots<float2>(Basis<float2>, int, const float2*, const float2*, int64_t, int64_t, int,
-                                       const Reduce&, const int*, cudaStream_t);
-template cudaError_t dcgs_update<double2>(Basis<double2>, int, const double2*, int, double2*, const double2*,
-                                          double2*, int64_t, int64_t, int, const int*, cudaStream_t);
-template cudaError_t dcgs_update<float2>(Basis<float2>, int, const double2*, int, float2*, const float2*, float2*,
-                                         int64_t, int64_t, int, const int*, cudaStream_t);
 
 cudaError_t gamma5_axpy(double2* y, const double2* a, const double2* s, double beta, int64_t vol, int nfield,
                         cudaStream_t st) {
@@ -1538,8 +1421,6 @@ cudaError_t links_f64_to_f16(const double2* in, __half2* out, int64_t count, cud
 #define SGN_INST(T)                                                                                              \
     template int reduce_blocks<T>(int64_t);                                                                      \
     template int wave_blocks<T>(int64_t, int);                                                                   \
-    template cudaError_t mdot<T>(Basis<T>, int, const T*, int64_t, int64_t, int, const Reduce&, int, const int*, \
-                                 cudaStream_t);                                                                  \
     template cudaError_t maxpy_mdot<T>(Basis<T>, int, const double2*, int, T*, int64_t, int64_t, int,           \
                                        const Reduce&, const int*, cudaStream_t);                                 \
     template cudaError_t maxpy_scale<T>(Basis<T>, int, const double2*, int, const T*, int64_t, T*, int64_t,     \

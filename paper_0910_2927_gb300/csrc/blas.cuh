@@ -40,6 +40,9 @@ struct DevState {
     double bd_tol;     // breakdown threshold relative to norm0
 };
 
+// Slots of one reduction: >= 2 kmax + 3 (delayed CGS2), >= deflation size + 1, >= eigensolver block + 1.
+constexpr int kMaxSlots = 136;
+
 enum ReduceMode {
     RM_STORE = 0,        // red[col][j] = sum_j
     RM_H1 = 1,           // h1[col][j] = sum_j (j < J), norm0 = sqrt(sum_J)
@@ -54,6 +57,12 @@ enum ReduceMode {
 template <class T>
 cudaError_t mdot(Basis<T> V, int J, const T* w, int64_t wsr, int64_t n, int ncol, const Reduce& rd,
                  int with_norm, const int* skip, cudaStream_t st);
+template <>
+cudaError_t mdot<double2>(Basis<double2> V, int J, const double2* w, int64_t wsr, int64_t n, int ncol,
+                          const Reduce& rd, int with_norm, const int* skip, cudaStream_t st);
+template <>
+cudaError_t mdot<float2>(Basis<float2> V, int J, const float2* w, int64_t wsr, int64_t n, int ncol,
+                         const Reduce& rd, int with_norm, const int* skip, cudaStream_t st);
 cudaError_t reduce(const Reduce& rd, int nslot, int ncol, int mode, int colidx, const DevState& S,
                    const double2* lambda, cudaStream_t st);
 template <class T>
@@ -73,9 +82,22 @@ cudaError_t update_shifts(Basis<T> V, int J, const double2* y, int s, int kmax, 
 template <class T>
 cudaError_t dcgs_dots(Basis<T> V, int J, const T* u, const T* z, int64_t wsr, int64_t n, int ncol, const Reduce& rd,
                       const int* skip, cudaStream_t st);
+template <>
+cudaError_t dcgs_dots<double2>(Basis<double2> V, int J, const double2* u, const double2* z, int64_t wsr, int64_t n,
+                               int ncol, const Reduce& rd, const int* skip, cudaStream_t st);
+template <>
+cudaError_t dcgs_dots<float2>(Basis<float2> V, int J, const float2* u, const float2* z, int64_t wsr, int64_t n,
+                              int ncol, const Reduce& rd, const int* skip, cudaStream_t st);
 template <class T>
 cudaError_t dcgs_update(Basis<T> V, int J, const double2* coef, int cstride, T* u, const T* z, T* next, int64_t wsr,
                         int64_t n, int ncol, const int* skip, cudaStream_t st);
+template <>
+cudaError_t dcgs_update<double2>(Basis<double2> V, int J, const double2* coef, int cstride, double2* u,
+                                 const double2* z, double2* next, int64_t wsr, int64_t n, int ncol, const int* skip,
+                                 cudaStream_t st);
+template <>
+cudaError_t dcgs_update<float2>(Basis<float2> V, int J, const double2* coef, int cstride, float2* u, const float2* z,
+                                float2* next, int64_t wsr, int64_t n, int ncol, const int* skip, cudaStream_t st);
 
 // out = a x + b y + c z over `count` complex elements (z may be null).
 template <class T>
@@ -126,6 +148,14 @@ cudaError_t tsmm_nn(const TV* V, int64_t sv, int J, const double2* C, int cstrid
 // Number of blocks per column used by the reductions for n complex elements.
 template <class T>
 int reduce_blocks(int64_t n);
+// CTAs per column of the FP64 inner products of ncol columns (gs_f64.cu), at most ceil(n / 128).
+// mdot and dcgs_dots on double2 take any Reduce::nblk >= 1.
+template <class T>
+int dot_blocks(int64_t n, int ncol);
+template <>
+int dot_blocks<double2>(int64_t n, int ncol);
+// Two warps on each of 152 SMs: fewer warps than this leave FP64 pipes idle.
+constexpr int64_t kFewWarps = 304;
 // CTAs per column for a grid of ncol columns that fills whole waves (1, 2 or 4
 // packs per thread); a Reduce built with it serves every kernel of the file.
 template <class T>

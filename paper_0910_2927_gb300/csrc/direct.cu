@@ -228,7 +228,7 @@ int direct_projection(sgn_ctx* c, const double2* b, double2* x, int ncol, int k,
     const int m = c->m;
     const size_t field = (size_t)n * sizeof(double2);
     const int rs = GS_BLOCK + 8;
-    const int nblk = reduce_blocks<double2>(n);
+    const int nblk = dot_blocks<double2>(n, ncol);
     const size_t oV = 0, ow = oV + align256(field * (size_t)(k + 1) * ncol);
     const size_t op = ow + align256(field * ncol);
     const size_t ored = op + align256(sizeof(double2) * (size_t)ncol * rs * nblk);

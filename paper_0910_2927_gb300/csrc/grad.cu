@@ -55,7 +55,7 @@ struct Small {
         c = c_;
         rs = ((nx + 1) + 7) & ~7;
         ncap = ncols;
-        const int nblk = reduce_blocks<double2>(c->n);
+        const int nblk = dot_blocks<double2>(c->n, ncols);
         const size_t pb = align256(sizeof(double2) * (size_t)ncols * rs * nblk);
         const size_t rb = align256(sizeof(double2) * (size_t)ncols * rs);
         const size_t fb = align256(sizeof(int) * 2 * (size_t)ncols);

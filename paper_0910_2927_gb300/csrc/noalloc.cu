@@ -6,6 +6,7 @@
 // device array instead of memory from an allocator.
 #include "blas.cuh"
 
+#include <algorithm>
 #include <mutex>
 
 namespace sgn {
@@ -58,14 +59,16 @@ SGN_API int sgn_inner_products_noalloc(const double* V, int J, const double* w, 
         set_error("sgn_inner_products_noalloc: need 1 <= J <= 64, nrhs >= 1, even n >= 2, non-NULL pointers");
         return SGN_ERR_ARG;
     }
-    const int nblk = reduce_blocks<double2>((int64_t)n);
-    const size_t need = sizeof(double2) * (size_t)nrhs * J * nblk;
+    const size_t per_block = sizeof(double2) * (size_t)nrhs * J;
+    const size_t need = per_block * reduce_blocks<double2>((int64_t)n);
     if (need > kStaticScratchBytes || (size_t)nrhs * 2 * sizeof(int) > kFlagBytes) {
         set_error("sgn_inner_products_noalloc: nrhs * J * ceil(n / 1024) * 16 bytes = " + std::to_string(need) +
                   " exceeds the fixed scratch of " + std::to_string(kStaticScratchBytes) +
                   " bytes (or nrhs > 512); use sgn_inner_products");
         return SGN_ERR_ARG;
     }
+    // at least ceil(n / 1024) CTAs per column fit (checked above); as many as the kernel likes, if they fit
+    const int nblk = (int)std::min<size_t>(dot_blocks<double2>((int64_t)n, nrhs), kStaticScratchBytes / per_block);
     void* base = nullptr;
     SGN_CHECK(scratch_address(&base));
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);

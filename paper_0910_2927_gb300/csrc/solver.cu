@@ -462,7 +462,9 @@ int get_engine(sgn_ctx* c, int ncol, int k, int s, int prec, Engine** out) {
     E->m = c->m;
     E->n = c->n;
     const size_t esz = prec == SGN_PREC_FP64 ? sizeof(double2) : sizeof(float2);
-    E->nblk = prec == SGN_PREC_FP64 ? wave_blocks<double2>(c->n, ncol) : wave_blocks<float2>(c->n, ncol);
+    E->nblk = prec != SGN_PREC_FP64 ? wave_blocks<float2>(c->n, ncol)
+              : use_cgs2()          ? wave_blocks<double2>(c->n, ncol)
+                                    : dot_blocks<double2>(c->n, ncol);
     int rs = std::max(2 * k + 4, c->m + 1);
     E->rstride = (rs + 7) & ~7;
     const size_t nc = (size_t)ncol;
@@ -846,7 +848,7 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
 
     // io: xs (s ncol) | r0, bt, xP, t, u (ncol each) | d (B) | omega table | FP64 partials
     const size_t field = (size_t)n * sizeof(double2);
-    const int nblk64 = reduce_blocks<double2>(n);
+    const int nblk64 = dot_blocks<double2>(n, ncol);
     const int rs64 = ((std::max(m, s) + 2) + 7) & ~7;
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -1363,7 +1365,7 @@ int solve_columns_gmres(sgn_ctx* c, const double2* rhs, int ncol, const std::vec
 int field_dots(sgn_ctx* c, const double2* a, const double2* b, int ncol, std::vector<std::complex<double>>& out) {
     cudaStream_t st = c->work;
     const int64_t n = c->n;
-    const int nblk = reduce_blocks<double2>(n);
+    const int nblk = dot_blocks<double2>(n, ncol);
     const int rs = 8;
     DevBuf buf;
     const size_t pbytes = align256(sizeof(double2) * (size_t)ncol * rs * nblk);
