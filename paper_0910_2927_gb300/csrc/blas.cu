@@ -631,15 +631,22 @@ __global__ void __launch_bounds__(NT) k_dcgs_dots(Basis<float2> V, int J, const 
 // Delayed CGS2, update of step j:  q_j = (u - Q s) / rho  (written over u), and
 // the next candidate  u_{j+1} = z / rho - Q c - d q_j  (when next != null).
 // Coefficients per column: [0,J) s, [J,2J) c, 2J: (1/rho, 0), 2J+1: d.
-// FP32 storage (FP64: gs_f64.cu).
+// FP32 storage (FP64: gs_f64.cu).  Four CTAs per SM (64 registers): as the compiler sizes it with the
+// Hessenberg column in the kernel, PKT = 4 takes 107 registers and ran 87 instead of 74 us.
 template <int PKT>
-__global__ void __launch_bounds__(NT) k_dcgs_update(Basis<float2> V, int J, const double2* __restrict__ coef,
+__global__ void __launch_bounds__(NT, 4) k_dcgs_update(Basis<float2> V, int J, const double2* __restrict__ coef,
                                                     int cstride, float2* u, const float2* __restrict__ z, float2* next,
-                                                    int64_t wsr, int64_t npk, const int* __restrict__ skip) {
+                                                    int64_t wsr, int64_t npk, double2* H, int km,
+                                                    const int* __restrict__ skip) {
     using T = float2;
     using O = Ops<T>;
     const int col = blockIdx.y;
     if (skip && skip[col]) return;
+    if (H && blockIdx.x == 0) {  // one CTA per column forms the Hessenberg column beside the update
+        hess_column(H + (int64_t)col * (km + 1) * km, coef + (int64_t)col * cstride, J, km);
+        return;
+    }
+    const int tile = H ? blockIdx.x - 1 : blockIdx.x;
     __shared__ typename O::C cs[MAXSLOT], cc[MAXSLOT];
     __shared__ double ex[2][2];
     const double2* cf = coef + (int64_t)col * cstride;
@@ -659,7 +666,7 @@ __global__ void __launch_bounds__(NT) k_dcgs_update(Basis<float2> V, int J, cons
     const T* zc = next ? z + col * wsr : nullptr;
     T* nc = next ? next + col * wsr : nullptr;
     const T* vb = V.base + col * V.sr;
-    const int64_t base = (int64_t)blockIdx.x * blockDim.x * PKT + threadIdx.x;
+    const int64_t base = (int64_t)tile * blockDim.x * PKT + threadIdx.x;
     // Q s and Q c with the basis loop outside: the loads of UNR basis vectors
     // (PKT packs each) are independent and in flight together
     typename O::P qs[PKT], qc[PKT];
@@ -711,23 +718,48 @@ __global__ void __launch_bounds__(NT) k_dcgs_update(Basis<float2> V, int J, cons
     }
 }
 
-// Second stage of every reduction plus the scalar bookkeeping that consumes it.
+// ---- second stage of the reductions ------------------------------------------
+// A latency chain of one to a few CTAs per column, in FP64 instructions of 64 cycles each: sums with
+// eight lanes per slot and the Hessenberg column formed beside the update took a step's reduction
+// from 12.6 to 6 us (4^4 FP64, 6^4 mixed), 15.3 to 7.6 (7x6x9x8 x 3 FP64), 18 to 12 (10^4 x 12 mixed).
+// LPS lanes per slot (8 slots of 8 lanes would fill a warp's FP64 instructions; one slot per warp
+// where there are few): FP64 additions over the CTAs' partial sums in a fixed order.  Valid in
+// every lane of the slot's group.
+template <int LPS>
+__device__ __forceinline__ double2 slot_sum(const Reduce& rd, int col, int slot, bool act) {
+    const int seg = threadIdx.x % LPS;
+    double2 a = make_double2(0, 0);
+    if (act) {
+        const double2* p = rd.partial + ((int64_t)col * rd.stride + slot) * rd.nblk;
+#pragma unroll 8
+        for (int b = seg; b < rd.nblk; b += LPS) a = cadd(a, p[b]);
+    }
+#pragma unroll
+    for (int o = LPS / 2; o > 0; o >>= 1) {
+        a.x += __shfl_xor_sync(0xffffffffu, a.x, o);
+        a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
+    }
+    return a;
+}
+
+// RM_STORE and RM_SIGNED: every slot on its own.  Grid (column, NT / LPS slots).
+template <int LPS>
+__global__ void __launch_bounds__(NT) k_reduce_store(Reduce rd, int nslot, int mode, DevState S,
+                                                     const double2* __restrict__ lambda) {
+    const int col = blockIdx.x;
+    if (S.skip[col]) return;
+    const int j = (blockIdx.y * NT + threadIdx.x) / LPS;
+    double2 a = slot_sum<LPS>(rd, col, j, j < nslot);
+    if (j >= nslot || threadIdx.x % LPS) return;
+    if (mode == RM_SIGNED && !(lambda[j].x > 0)) a = make_double2(-a.x, -a.y);
+    S.red[(int64_t)col * S.rstride + j] = a;
+}
+
 // The scalar work of a reduction once the slot sums of column col are known
 // (sums: shared memory, nslot entries).  Called by every thread of one CTA.
-__device__ void reduce_tail(const double2* sums, int col, int nslot, int mode, int colidx, const DevState& S,
-                            const double2* __restrict__ lambda) {
-    __shared__ double2 gsh[MAXSLOT];
+__device__ void reduce_tail(const double2* sums, int col, int nslot, int mode, int colidx, const DevState& S) {
     const int64_t cr = (int64_t)col * S.rstride;
     switch (mode) {
-        case RM_STORE:
-            for (int j = threadIdx.x; j < nslot; j += NT) S.red[cr + j] = sums[j];
-            break;
-        case RM_SIGNED:
-            for (int j = threadIdx.x; j < nslot; j += NT) {
-                double sg = lambda[j].x > 0 ? 1.0 : -1.0;
-                S.red[cr + j] = make_double2(sg * sums[j].x, sg * sums[j].y);
-            }
-            break;
         case RM_H1:
             for (int j = threadIdx.x; j < nslot - 1; j += NT) S.h1[cr + j] = sums[j];
             if (threadIdx.x == 0) S.norm0[col] = sqrt(sums[nslot - 1].x);
@@ -758,125 +790,87 @@ __device__ void reduce_tail(const double2* sums, int col, int nslot, int mode, i
         }
         case RM_DCGS:
         case RM_DCGS_FINAL: {
-            // Delayed CGS2 bookkeeping of step j = colidx (see k_dcgs_dots for the slots).
+            // Delayed CGS2 bookkeeping of step j = colidx (see k_dcgs_dots for the slots).  Only
+            // what the update of the step waits for is done here: rho, the coefficients s, c = t / rho
+            // and d = (u^dag z - s^dag t) / rho^2, and s added to column j - 1 of H.  The tentative
+            // column j, which takes j^2 / 2 products, is formed beside the update (hess_column).
+            // FP64 instructions take 64 cycles each here, so the three sums over l share one
+            // reduction, and rho and ||z|| one rsqrt (lanes 0 and 1).
             const int j = colidx;
             const bool fin = mode == RM_DCGS_FINAL;
-            const int64_t hb = (int64_t)col * (S.kmax + 1) * S.kmax;
             const int km = S.kmax;
-            double2* H = S.H + hb;
-            const double2 alpha = sums[fin ? j : 2 * j];
-            __shared__ double rho_sh;
+            double2* H = S.H + (int64_t)col * (km + 1) * km;
+            __shared__ double ir_sh;
             __shared__ int broke_sh;
-            __shared__ double2 st_sh;
             const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
             if (warp == 0) {
-                // s2 = sum_l |s_l|^2 and st = sum_l conj(s_l) t_l, l < j: lanes over l, fixed-order tree
-                double2 s2v = make_double2(0, 0), st = make_double2(0, 0);
+                // sum_l |s_l|^2 and sum_l conj(s_l) t_l, l < j
+                double a[4] = {0.0, 0.0, 0.0, 0.0};
                 for (int l = lane; l < j; l += 32) {
-                    s2v.x += cabs2(sums[l]);
-                    if (!fin) st = cadd(st, cconjmul(sums[l], sums[j + l]));
-                }
-                s2v = warp_sum(s2v);
-                st = warp_sum(st);
-                if (lane == 0) {
-                    st_sh = st;
-                    const double s2 = s2v.x;
-                    double r2 = alpha.x - s2;
-                    double rho = r2 > 0 ? sqrt(r2) : 0.0;
-                    int broke = 0;
-                    if (j == 0) {
-                        S.beta[col] = rho;
-                        broke = !(rho > 0);
-                    } else {
-                        broke = !(rho > S.bd_tol * S.norm0[col]);
-                        H[(int64_t)j * km + (j - 1)] = make_double2(rho, 0);
+                    const double2 sl = sums[l];
+                    a[0] = fma(sl.x, sl.x, a[0]);
+                    a[0] = fma(sl.y, sl.y, a[0]);
+                    if (!fin) {
+                        const double2 t = sums[j + l];
+                        a[1] = fma(sl.x, t.x, a[1]);
+                        a[1] = fma(sl.y, t.y, a[1]);
+                        a[2] = fma(sl.x, t.y, a[2]);
+                        a[2] = fma(-sl.y, t.x, a[2]);
                     }
-                    if (!isfinite(r2)) {
+                }
+                const double mine = reduce_few<4>(a, lane);  // lane l: sum l mod 4
+                const double stx = __shfl_sync(0xffffffffu, mine, 1), sty = __shfl_sync(0xffffffffu, mine, 2);
+                const double v = lane == 0 ? sums[fin ? j : 2 * j].x - mine : fin ? 0.0 : sums[2 * j + 2].x;
+                const double rs = v > 0 ? rsqrt(v) : 0.0;
+                const double root = v > 0 ? v * rs : 0.0;  // lane 0: rho, lane 1: ||z||
+                const double nz = __shfl_sync(0xffffffffu, root, 1);
+                if (lane == 0) {
+                    int broke = j == 0 ? !(root > 0) : !(root > S.bd_tol * S.norm0[col]);
+                    if (j == 0)
+                        S.beta[col] = root;
+                    else
+                        H[(int64_t)j * km + (j - 1)] = make_double2(root, 0);
+                    if (!isfinite(v)) {
                         atomicOr(S.err, 2);
                         broke = 1;
                     }
-                    rho_sh = rho;
+                    // closing pass: q_k = (u - Q s) / rho; an invariant Krylov space (rho ~ 0) leaves
+                    // q_k = 0, so the restart norm is 0 and the column converges
+                    const double ir = broke ? 0.0 : rs;
+                    S.red[cr + 2 * j] = make_double2(ir, 0);
+                    if (!fin) {
+                        if (broke) {  // the Krylov space is invariant: FOM on its j columns is exact
+                            S.kk[col] = j;
+                            S.skip[col] = 1;
+                        } else {
+                            const double2 b = sums[2 * j + 1];
+                            S.red[cr + 2 * j + 1] = make_double2((b.x - stx) * ir * ir, (b.y - sty) * ir * ir);
+                            S.norm0[col] = nz * ir;  // ~ ||A^2 q_j|| for the next breakdown test
+                        }
+                    }
+                    ir_sh = ir;
                     broke_sh = broke;
                 }
+            } else if (threadIdx.x - 32 < j) {  // column j - 1: H[0:j, j-1] += s (j <= 64 < NT - 32)
+                const int l = threadIdx.x - 32;
+                double2* h = H + (int64_t)l * km + (j - 1);
+                *h = cadd(*h, sums[l]);
+                S.red[cr + l] = sums[l];
             }
             __syncthreads();
-            // correct column j-1: H[0:j, j-1] += s
-            for (int l = threadIdx.x; l < j; l += NT) {
-                double2 h = H[(int64_t)l * km + (j - 1)];
-                H[(int64_t)l * km + (j - 1)] = cadd(h, sums[l]);
-            }
-            __syncthreads();
-            const double rho = rho_sh;
-            const int64_t cr = (int64_t)col * S.rstride;
-            if (fin) {
-                // closing pass: q_k = (u - Q s) / rho; an invariant Krylov space (rho ~ 0)
-                // leaves q_k = 0, so the restart norm is 0 and the column converges
-                for (int l = threadIdx.x; l < j; l += NT) S.red[cr + l] = sums[l];
-                if (threadIdx.x == 0) S.red[cr + 2 * j] = make_double2(broke_sh ? 0.0 : 1.0 / rho, 0);
-                break;
-            }
-            if (broke_sh) {  // the Krylov space is invariant: FOM on its j columns is exact
-                if (threadIdx.x == 0) {
-                    S.kk[col] = j;
-                    S.skip[col] = 1;
-                }
-                break;
-            }
-            for (int l = threadIdx.x; l < j; l += NT) S.red[cr + l] = sums[l];  // s
-            // g = Hbar s, Hbar = H[0:j+1, 0:j]: warp w takes rows w, w + 8, ...; lanes split the
-            // row (l = lane, lane + 32); every H load of the warp is issued before the sums
-            if (j <= 64) {
-                constexpr int RPW = (65 + NWARP - 1) / NWARP;
-                double2 hv[RPW][2];
-#pragma unroll
-                for (int r = 0; r < RPW; ++r)
-#pragma unroll
-                    for (int q = 0; q < 2; ++q) {
-                        const int i = warp + r * NWARP, l = lane + 32 * q;
-                        hv[r][q] = (i <= j && l < j && l >= i - 1) ? H[(int64_t)i * km + l] : make_double2(0, 0);
-                    }
-                const double2 s0 = lane < j ? sums[lane] : make_double2(0, 0);
-                const double2 s1 = lane + 32 < j ? sums[lane + 32] : make_double2(0, 0);
-#pragma unroll
-                for (int r = 0; r < RPW; ++r) {
-                    const int i = warp + r * NWARP;
-                    if (i > j) break;  // uniform over the warp
-                    const double2 g = warp_sum(cadd(cmul(hv[r][0], s0), cmul(hv[r][1], s1)));
-                    if (lane == 0) gsh[i] = g;
-                }
-            } else {
-                for (int i = threadIdx.x; i <= j; i += NT) {
-                    double2 g = make_double2(0, 0);
-                    for (int l = (i > 0 ? i - 1 : 0); l < j; ++l) g = cadd(g, cmul(H[(int64_t)i * km + l], sums[l]));
-                    gsh[i] = g;
-                }
-            }
-            __syncthreads();
-            const double ir = 1.0 / rho;
-            for (int i = threadIdx.x; i < j; i += NT) {
-                double2 t = sums[j + i];
-                double2 hp = make_double2((t.x - gsh[i].x) * ir, (t.y - gsh[i].y) * ir);
-                H[(int64_t)i * km + j] = hp;                                             // tentative column j
-                S.red[cr + j + i] = make_double2(gsh[i].x * ir + hp.x, gsh[i].y * ir + hp.y);  // c
-            }
-            if (threadIdx.x == 0) {
-                const double2 st = st_sh;
-                double2 beta = sums[2 * j + 1];
-                double2 hjj = make_double2(((beta.x - st.x) * ir - gsh[j].x) * ir, ((beta.y - st.y) * ir - gsh[j].y) * ir);
-                H[(int64_t)j * km + j] = hjj;
-                S.red[cr + 2 * j] = make_double2(ir, 0);
-                S.red[cr + 2 * j + 1] = make_double2(gsh[j].x * ir + hjj.x, gsh[j].y * ir + hjj.y);  // d
-                S.norm0[col] = sqrt(sums[2 * j + 2].x) * ir;  // ~ ||A^2 q_j|| for the next breakdown test
-            }
+            if (fin || broke_sh) break;
+            const double ir = ir_sh;
+            for (int l = threadIdx.x; l < j; l += NT)
+                S.red[cr + j + l] = make_double2(sums[j + l].x * ir, sums[j + l].y * ir);
             break;
         }
-        case RM_BETA_FIRST:
+        case RM_BETA_FIRST: {
+            const double beta = sqrt(sums[0].x);
+            for (int i = threadIdx.x; i < S.s; i += NT) S.rho[(int64_t)col * S.s + i] = make_double2(1, 0);
             if (threadIdx.x == 0) {
-                double beta = sqrt(sums[0].x);
                 S.beta[col] = beta;
                 S.bnorm[col] = beta;
                 S.kk[col] = S.kmax;
-                for (int i = 0; i < S.s; ++i) S.rho[(int64_t)col * S.s + i] = make_double2(1, 0);
                 if (!isfinite(beta)) atomicOr(S.err, 2);
                 if (beta > 0 && isfinite(beta)) {
                     S.scale[col] = 1.0 / beta;
@@ -891,8 +885,21 @@ __device__ void reduce_tail(const double2* sums, int col, int nslot, int mode, i
                 }
             }
             break;
+        }
         case RM_BETA_RESTART:
-            if (threadIdx.x == 0) {
+            if (threadIdx.x < 32) {
+                // max_i |rho_i|^2, lanes over the shifts
+                double m = 0;
+                for (int i = threadIdx.x; i < S.s; i += 32) {
+                    const double a = cabs2(S.rho[(int64_t)col * S.s + i]);
+                    m = a > m ? a : m;
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    const double a = __shfl_xor_sync(0xffffffffu, m, o);
+                    m = a > m ? a : m;
+                }
+                if (threadIdx.x != 0) break;
                 if (S.kk[col] < S.kmax) {  // invariant subspace met: FOM is exact
                     S.resest[col] = 0;
                     S.done[col] = 1;
@@ -900,13 +907,8 @@ __device__ void reduce_tail(const double2* sums, int col, int nslot, int mode, i
                     S.scale[col] = 0;
                     break;
                 }
-                double beta = sqrt(sums[0].x);
-                double rmax = 0;
-                for (int i = 0; i < S.s; ++i) {
-                    double2 r = S.rho[(int64_t)col * S.s + i];
-                    double a = sqrt(cabs2(r)) * beta / S.bnorm[col];
-                    rmax = a > rmax ? a : rmax;
-                }
+                const double beta = sqrt(sums[0].x);
+                const double rmax = sqrt(m) * beta / S.bnorm[col];
                 S.beta[col] = beta;
                 S.resest[col] = rmax;
                 if (!isfinite(rmax)) {
@@ -925,61 +927,42 @@ __device__ void reduce_tail(const double2* sums, int col, int nslot, int mode, i
     }
 }
 
-__global__ void __launch_bounds__(NT) k_reduce(Reduce rd, int nslot, int mode, int colidx, DevState S,
-                                               const double2* __restrict__ lambda) {
+// Slot sums, then the column's scalar work.  CTA (col, g) sums slots g * NT / LPS ...; with more
+// than one CTA per column the sums go to S.sums and the last CTA to arrive loads them all and does
+// the scalar work (the sums are the same whatever the arrival order).
+template <int LPS>
+__global__ void __launch_bounds__(NT) k_reduce(Reduce rd, int nslot, int mode, int colidx, DevState S) {
     const int col = blockIdx.x;
     // RM_BETA_FIRST starts a solve; RM_BETA_RESTART must still see columns that
     // broke down in this cycle; every other mode is column work proper.
     if (mode == RM_BETA_RESTART && S.done[col]) return;
     if (mode != RM_BETA_FIRST && mode != RM_BETA_RESTART && S.skip[col]) return;
     __shared__ double2 sums[MAXSLOT];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int j = warp; j < nslot; j += NWARP) {
-        const double2* p = rd.partial + ((int64_t)col * rd.stride + j) * rd.nblk;
-        double2 a = make_double2(0, 0);
-        // unrolled so that the loads of up to 8 partials per lane are in flight together
-        // (the sum order, b = lane, lane + 32, ..., is fixed either way)
-#pragma unroll 8
-        for (int b = lane; b < rd.nblk; b += 32) a = cadd(a, p[b]);
-        a = warp_sum(a);
-        if (lane == 0) sums[j] = a;
-    }
-    __syncthreads();
-    reduce_tail(sums, col, nslot, mode, colidx, S, lambda);
-}
-
-// Split form: CTA (col, g) sums slots g * NWARP .. g * NWARP + NWARP - 1 (one warp each,
-// the same fixed order as k_reduce) into S.sums; the last CTA of the column to
-// arrive loads all sums and does the scalar work.  Results are identical to
-// k_reduce's whatever the arrival order.
-__global__ void __launch_bounds__(NT) k_reduce_split(Reduce rd, int nslot, int mode, int colidx, DevState S,
-                                                     const double2* __restrict__ lambda) {
-    const int col = blockIdx.x;
-    if (mode == RM_BETA_RESTART && S.done[col]) return;
-    if (mode != RM_BETA_FIRST && mode != RM_BETA_RESTART && S.skip[col]) return;
-    __shared__ double2 sums[MAXSLOT];
     __shared__ int last;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t cr = (int64_t)col * S.rstride;
-    const int j = blockIdx.y * NWARP + warp;
-    if (j < nslot) {
-        const double2* p = rd.partial + ((int64_t)col * rd.stride + j) * rd.nblk;
-        double2 a = make_double2(0, 0);
-#pragma unroll 8
-        for (int b = lane; b < rd.nblk; b += 32) a = cadd(a, p[b]);
-        a = warp_sum(a);
-        if (lane == 0) S.sums[cr + j] = a;
+    const bool split = gridDim.y > 1;
+    for (int j0 = blockIdx.y * (NT / LPS); j0 < nslot; j0 += gridDim.y * (NT / LPS)) {
+        const int j = j0 + threadIdx.x / LPS;
+        const double2 a = slot_sum<LPS>(rd, col, j, j < nslot);
+        if (j < nslot && threadIdx.x % LPS == 0) {
+            if (split)
+                S.sums[cr + j] = a;
+            else
+                sums[j] = a;
+        }
     }
-    __threadfence();  // this CTA's sums are visible device-wide before it is counted
+    if (split) __threadfence();  // this CTA's sums are visible device-wide before it is counted
     __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(&S.rcount[col], 1) == (int)gridDim.y - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    for (int i = threadIdx.x; i < nslot; i += NT) sums[i] = __ldcg(S.sums + cr + i);  // from L2, not a stale L1
-    if (threadIdx.x == 0) S.rcount[col] = 0;  // ready for the next launch
-    __syncthreads();
-    reduce_tail(sums, col, nslot, mode, colidx, S, lambda);
+    if (split) {
+        if (threadIdx.x == 0) last = atomicAdd(&S.rcount[col], 1) == (int)gridDim.y - 1;
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        for (int i = threadIdx.x; i < nslot; i += NT) sums[i] = __ldcg(S.sums + cr + i);  // from L2, not a stale L1
+        if (threadIdx.x == 0) S.rcount[col] = 0;  // ready for the next launch
+        __syncthreads();
+    }
+    reduce_tail(sums, col, nslot, mode, colidx, S);
 }
 
 // out = a x + b y + c z on whole blocks (real coefficients; z may be null).
@@ -1241,11 +1224,20 @@ cudaError_t mdot<float2>(Basis<float2> V, int J, const float2* w, int64_t wsr, i
 cudaError_t reduce(const Reduce& rd, int nslot, int ncol, int mode, int colidx, const DevState& S,
                    const double2* lambda, cudaStream_t st) {
     if (nslot > MAXSLOT) return cudaErrorInvalidValue;
-    const int groups = (nslot + NWARP - 1) / NWARP;
-    if (S.sums && S.rcount && groups > 1)
-        k_reduce_split<<<dim3(ncol, groups), NT, 0, st>>>(rd, nslot, mode, colidx, S, lambda);
-    else
-        k_reduce<<<ncol, NT, 0, st>>>(rd, nslot, mode, colidx, S, lambda);
+    const bool few = nslot <= NWARP;
+    const int groups = few ? 1 : (nslot + NT / 8 - 1) / (NT / 8);
+    if (mode == RM_STORE || mode == RM_SIGNED) {
+        if (few)
+            k_reduce_store<32><<<dim3(ncol, groups), NT, 0, st>>>(rd, nslot, mode, S, lambda);
+        else
+            k_reduce_store<8><<<dim3(ncol, groups), NT, 0, st>>>(rd, nslot, mode, S, lambda);
+    } else {
+        const dim3 grid(ncol, S.sums && S.rcount ? groups : 1);
+        if (few)
+            k_reduce<32><<<grid, NT, 0, st>>>(rd, nslot, mode, colidx, S);
+        else
+            k_reduce<8><<<grid, NT, 0, st>>>(rd, nslot, mode, colidx, S);
+    }
     count_launch();
     return cudaGetLastError();
 }
@@ -1333,12 +1325,14 @@ cudaError_t dcgs_dots<float2>(Basis<float2> V, int J, const float2* u, const flo
 
 template <>
 cudaError_t dcgs_update<float2>(Basis<float2> V, int J, const double2* coef, int cstride, float2* u, const float2* z,
-                                float2* next, int64_t wsr, int64_t n, int ncol, const int* skip, cudaStream_t st) {
-    if (J > MAXSLOT) return cudaErrorInvalidValue;
+                                float2* next, int64_t wsr, int64_t n, int ncol, double2* H, int km, const int* skip,
+                                cudaStream_t st) {
+    if (2 * J + 2 > MAXSLOT) return cudaErrorInvalidValue;
     int64_t npk = n / Ops<float2>::CPX;
     const Split sp = split_for<float2>(n, ncol);
-    SGN_PK_SWITCH(sp.pkt, k_dcgs_update<PKT_><<<dim3(sp.nb, ncol), sp.threads, 0, st>>>(V, J, coef, cstride, u, z, next,
-                                                                                       wsr, npk, skip))
+    const dim3 grid(sp.nb + (H ? 1 : 0), ncol);
+    SGN_PK_SWITCH(sp.pkt, k_dcgs_update<PKT_><<<grid, sp.threads, 0, st>>>(V, J, coef, cstride, u, z, next, wsr, npk, H,
+                                                                          km, skip))
     count_launch();
     return cudaGetLastError();
 }

@@ -40,6 +40,65 @@ struct DevState {
     double bd_tol;     // breakdown threshold relative to norm0
 };
 
+#ifdef __CUDACC__
+// Sum over the lanes of N = 2^k <= 32 values per lane; lane l ends with the sum of value l mod N.
+template <int N>
+__device__ __forceinline__ double reduce_scatter(const double (&a)[N], int lane) {
+    if constexpr (N == 1) {
+        return a[0];
+    } else {
+        constexpr int H = N / 2;
+        const bool up = lane & H;
+        double h[H];
+#pragma unroll
+        for (int i = 0; i < H; ++i) {
+            const double keep = up ? a[H + i] : a[i], send = up ? a[i] : a[H + i];
+            h[i] = keep + __shfl_xor_sync(0xffffffffu, send, H);
+        }
+        return reduce_scatter<H>(h, lane);
+    }
+}
+// The same for N < 32: the lanes beyond N are added first.
+template <int N>
+__device__ __forceinline__ double reduce_few(double (&a)[N], int lane) {
+#pragma unroll
+    for (int o = 16; o >= N; o >>= 1)
+#pragma unroll
+        for (int i = 0; i < N; ++i) a[i] += __shfl_xor_sync(0xffffffffu, a[i], o);
+    return reduce_scatter<N>(a, lane);
+}
+
+// Tentative column j of the Hessenberg matrix in a delayed-CGS2 step, by one CTA:
+//   H[i][j] = c_i - g_i / rho (i < j),  H[j][j] = d - g_j / rho,  g = H[0:j+1, 0:j] s,
+// with the step's coefficients s = red[0, j), c = red[j, 2j), 1 / rho = red[2j], d = red[2j + 1].
+// Four lanes per row.
+__device__ __forceinline__ void hess_column(double2* __restrict__ H, const double2* __restrict__ red, int j, int km) {
+    const int q = threadIdx.x & 3;
+    const double ir = red[2 * j].x;
+    for (int i0 = 0; i0 <= j; i0 += blockDim.x / 4) {
+        const int i = i0 + threadIdx.x / 4;
+        double gx = 0.0, gy = 0.0;
+        if (i <= j)
+            for (int l = (i > 0 ? i - 1 : 0) + q; l < j; l += 4) {
+                const double2 h = H[(int64_t)i * km + l], s = red[l];
+                gx = fma(h.x, s.x, gx);
+                gx = fma(-h.y, s.y, gx);
+                gy = fma(h.x, s.y, gy);
+                gy = fma(h.y, s.x, gy);
+            }
+#pragma unroll
+        for (int o = 1; o <= 2; o <<= 1) {
+            gx += __shfl_xor_sync(0xffffffffu, gx, o);
+            gy += __shfl_xor_sync(0xffffffffu, gy, o);
+        }
+        if (i <= j && q == 0) {
+            const double2 c = red[i < j ? j + i : 2 * j + 1];
+            H[(int64_t)i * km + j] = make_double2(fma(-gx, ir, c.x), fma(-gy, ir, c.y));
+        }
+    }
+}
+#endif
+
 // Slots of one reduction: >= 2 kmax + 3 (delayed CGS2), >= deflation size + 1, >= eigensolver block + 1.
 constexpr int kMaxSlots = 136;
 
@@ -50,7 +109,7 @@ enum ReduceMode {
     RM_BETA_FIRST = 3,   // bnorm = beta = sqrt(sum_0), rho = 1, scale = 1/beta
     RM_BETA_RESTART = 4, // beta = sqrt(sum_0), residual estimate, convergence, scale = 1/beta
     RM_SIGNED = 5,       // red[col][j] = sign(Re lambda_j) * sum_j (x_P coefficients)
-    RM_DCGS = 6,         // delayed CGS2 step j: rho, column j-1 correction, tentative column j, update coefficients
+    RM_DCGS = 6,         // delayed CGS2 step j: rho, column j-1 correction, update coefficients
     RM_DCGS_FINAL = 7    // delayed CGS2 closing pass of a cycle (no new candidate)
 };
 
@@ -78,7 +137,9 @@ template <class T>
 cudaError_t update_shifts(Basis<T> V, int J, const double2* y, int s, int kmax, double2* xs, int64_t xs_shift,
                           int64_t xs_col, int64_t n, int ncol, const int* skip, const int* kk, cudaStream_t st);
 
-// Delayed CGS2 (one fused reduction and one fused update per Arnoldi step).
+// Delayed CGS2 (one fused reduction and one fused update per Arnoldi step).  dcgs_update with
+// H (the columns' Hessenberg matrices, row stride km; null: not) also forms column J of H from the
+// step's coefficients (hess_column).
 template <class T>
 cudaError_t dcgs_dots(Basis<T> V, int J, const T* u, const T* z, int64_t wsr, int64_t n, int ncol, const Reduce& rd,
                       const int* skip, cudaStream_t st);
@@ -90,14 +151,15 @@ cudaError_t dcgs_dots<float2>(Basis<float2> V, int J, const float2* u, const flo
                               int ncol, const Reduce& rd, const int* skip, cudaStream_t st);
 template <class T>
 cudaError_t dcgs_update(Basis<T> V, int J, const double2* coef, int cstride, T* u, const T* z, T* next, int64_t wsr,
-                        int64_t n, int ncol, const int* skip, cudaStream_t st);
+                        int64_t n, int ncol, double2* H, int km, const int* skip, cudaStream_t st);
 template <>
 cudaError_t dcgs_update<double2>(Basis<double2> V, int J, const double2* coef, int cstride, double2* u,
-                                 const double2* z, double2* next, int64_t wsr, int64_t n, int ncol, const int* skip,
-                                 cudaStream_t st);
+                                 const double2* z, double2* next, int64_t wsr, int64_t n, int ncol, double2* H, int km,
+                                 const int* skip, cudaStream_t st);
 template <>
 cudaError_t dcgs_update<float2>(Basis<float2> V, int J, const double2* coef, int cstride, float2* u, const float2* z,
-                                float2* next, int64_t wsr, int64_t n, int ncol, const int* skip, cudaStream_t st);
+                                float2* next, int64_t wsr, int64_t n, int ncol, double2* H, int km, const int* skip,
+                                cudaStream_t st);
 
 // out = a x + b y + c z over `count` complex elements (z may be null).
 template <class T>

@@ -13,9 +13,9 @@
 // instructions: small lattices are split over CTAs by elements and by groups of basis vectors.
 //
 // Measured, us per launch averaged over the steps of a solve, before (one butterfly per sum, CTAs
-// of 256 elements) and now.  Two-field products: 4^4 x 1 column 24.6 -> 7.0, 6^4 x 1 32.0 -> 16.6, 7x6x9x8 x 3 85.6 -> 44.4.
-// 30 x 12 products on 16^4 (one field): 4472 -> 2055 (floor 1810: 8 flops per product at the FP64
-// rate).  Update: 4^4 x 1 10.8 -> 3.9, 6^4 x 1 13.4 -> 8.0.
+// of 256 elements) and now.  Two-field products: 4^4 x 1 column 24.6 -> 7.0, 6^4 x 1 32.0 -> 16.6,
+// 7x6x9x8 x 3 85.6 -> 42.5.  30 x 12 products on 16^4 (one field): 4472 -> 2055 (floor 1810: 8 flops
+// per product at the FP64 rate).  Update: 4^4 x 1 10.8 -> 3.9, 6^4 x 1 13.4 -> 8.0.
 #include "blas.cuh"
 
 #include <algorithm>
@@ -26,33 +26,6 @@ namespace {
 
 constexpr int MAXW = 4;             // warps per CTA: one per sub-partition
 constexpr int64_t PIPES = 4 * 152;  // sub-partitions of the chip
-
-// Sum over the lanes of N = 2^k <= 32 values per lane; lane l ends with the sum of value l mod N.
-template <int N>
-__device__ __forceinline__ double reduce_scatter(const double (&a)[N], int lane) {
-    if constexpr (N == 1) {
-        return a[0];
-    } else {
-        constexpr int H = N / 2;
-        const bool up = lane & H;
-        double h[H];
-#pragma unroll
-        for (int i = 0; i < H; ++i) {
-            const double keep = up ? a[H + i] : a[i], send = up ? a[i] : a[H + i];
-            h[i] = keep + __shfl_xor_sync(0xffffffffu, send, H);
-        }
-        return reduce_scatter<H>(h, lane);
-    }
-}
-// The same for N < 32: the lanes beyond N are added first.
-template <int N>
-__device__ __forceinline__ double reduce_few(double (&a)[N], int lane) {
-#pragma unroll
-    for (int o = 16; o >= N; o >>= 1)
-#pragma unroll
-        for (int i = 0; i < N; ++i) a[i] += __shfl_xor_sync(0xffffffffu, a[i], o);
-    return reduce_scatter<N>(a, lane);
-}
 
 __device__ __forceinline__ void dot_acc(double& re, double& im, double2 v, double2 w) {  // += conj(v) w
     re = fma(v.x, w.x, re);
@@ -194,11 +167,15 @@ cudaError_t launch(Basis<double2> V, int J, const double2* u, const double2* z, 
 template <int S>
 __global__ void __launch_bounds__(S == 1 ? 64 : 32 * S)
     k_dcgs_update_f64(Basis<double2> V, int J, const double2* __restrict__ coef, int cstride, double2* u,
-                      const double2* __restrict__ z, double2* next, int64_t wsr, int64_t n,
+                      const double2* __restrict__ z, double2* next, int64_t wsr, int64_t n, double2* H, int km,
                       const int* __restrict__ skip) {
     const int col = blockIdx.y;
     if (skip && skip[col]) return;
-    const int64_t tile = blockIdx.x;
+    if (H && blockIdx.x == 0) {  // one CTA per column forms the Hessenberg column beside the update
+        hess_column(H + (int64_t)col * (km + 1) * km, coef + (int64_t)col * cstride, J, km);
+        return;
+    }
+    const int64_t tile = H ? blockIdx.x - 1 : blockIdx.x;
     __shared__ double2 cf[kMaxSlots];
     for (int l = threadIdx.x; l < 2 * J + 2; l += blockDim.x) cf[l] = coef[(int64_t)col * cstride + l];
     __syncthreads();
@@ -304,18 +281,18 @@ cudaError_t dcgs_dots<double2>(Basis<double2> V, int J, const double2* u, const 
 
 template <>
 cudaError_t dcgs_update<double2>(Basis<double2> V, int J, const double2* coef, int cstride, double2* u,
-                                 const double2* z, double2* next, int64_t wsr, int64_t n, int ncol, const int* skip,
-                                 cudaStream_t st) {
+                                 const double2* z, double2* next, int64_t wsr, int64_t n, int ncol, double2* H, int km,
+                                 const int* skip, cudaStream_t st) {
     if (2 * J + 2 > kMaxSlots) return cudaErrorInvalidValue;
     // four warps per 32 elements where that shortens the busiest sub-partition's work (the extra
     // sums cost about an eighth)
     const int64_t warps = (n + 31) / 32 * ncol;
     const bool split = J > 4 && 9 * ((4 * warps + PIPES - 1) / PIPES) < 32 * ((warps + PIPES - 1) / PIPES);
-    const dim3 grid((unsigned)((split ? (n + 31) / 32 : (n + 63) / 64)), ncol);
+    const dim3 grid((unsigned)((split ? (n + 31) / 32 : (n + 63) / 64) + (H ? 1 : 0)), ncol);
     if (split)
-        k_dcgs_update_f64<4><<<grid, 128, 0, st>>>(V, J, coef, cstride, u, z, next, wsr, n, skip);
+        k_dcgs_update_f64<4><<<grid, 128, 0, st>>>(V, J, coef, cstride, u, z, next, wsr, n, H, km, skip);
     else
-        k_dcgs_update_f64<1><<<grid, 64, 0, st>>>(V, J, coef, cstride, u, z, next, wsr, n, skip);
+        k_dcgs_update_f64<1><<<grid, 64, 0, st>>>(V, J, coef, cstride, u, z, next, wsr, n, H, km, skip);
     count_launch();
     return cudaGetLastError();
 }

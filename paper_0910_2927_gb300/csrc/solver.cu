@@ -343,7 +343,8 @@ cudaError_t cycle_dcgs(const sgn_ctx* c, Engine& E, const CycleArgs& a, cudaStre
         CU(reduce(rd, 2 * j + 3, ncol, RM_DCGS, j, S, nullptr, st));
         CU(tm.end());
         CU(tm.begin(2, (j + 4) * fb));
-        CU(dcgs_update<T>(VB, j, S.red, S.rstride, V + j * sj, w, V + (j + 1) * sj, sr, n, ncol, S.skip, st));
+        CU(dcgs_update<T>(VB, j, S.red, S.rstride, V + j * sj, w, V + (j + 1) * sj, sr, n, ncol, S.H, S.kmax,
+                          S.skip, st));
         CU(tm.end());
     }
     // closing pass: second projection of v_k
@@ -354,7 +355,8 @@ cudaError_t cycle_dcgs(const sgn_ctx* c, Engine& E, const CycleArgs& a, cudaStre
     CU(reduce(rd, k + 1, ncol, RM_DCGS_FINAL, k, S, nullptr, st));
     CU(tm.end());
     CU(tm.begin(2, (k + 2) * fb));
-    CU(dcgs_update<T>(VB, k, S.red, S.rstride, V + k * sj, nullptr, nullptr, sr, n, ncol, S.skip, st));
+    CU(dcgs_update<T>(VB, k, S.red, S.rstride, V + k * sj, nullptr, nullptr, sr, n, ncol, nullptr, 0,
+                      S.skip, st));
     CU(tm.end());
     if (a.gmres) {
         CU(shifted_lsq(S, ncol, st));
