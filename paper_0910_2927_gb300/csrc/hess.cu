@@ -2,10 +2,6 @@
 //   y_i = beta rho_i (H_k - sigma_i I)^{-1} e_1          (one warp per column and shift)
 //   rho_i <- -h_{k+1,k} e_k^T y_i                        (collinearity factor, eq. (3.1))
 //   c = sum_i omega_i y_i                                (the combination of eq. (2.3))
-// The shifted Hessenberg systems are solved by Gaussian elimination with
-// partial pivoting: on a Hessenberg matrix the pivot of column r is chosen
-// between the running row r and the untouched row r+1 (larger modulus, the
-// running row on ties), and each lane of the warp owns two matrix columns.
 #include "blas.cuh"
 
 namespace sgn {
@@ -13,122 +9,144 @@ namespace {
 
 constexpr int KMAX = 64;
 
-__device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
-    double d = b.x * b.x + b.y * b.y;
-    return make_double2((a.x * b.x + a.y * b.y) / d, (a.y * b.x - a.x * b.y) / d);
+// a / b, b scaled by a power of two so that |b|^2 neither overflows nor underflows
+__device__ __forceinline__ double2 cdiv_scaled(double2 a, double2 b) {
+    const int e = max((__double2hiint(b.x) >> 20) & 0x7ff, (__double2hiint(b.y) >> 20) & 0x7ff);
+    const double f = e == 0 ? 0x1p1000 : e >= 2046 ? 0x1p-1020 : __hiloint2double((2046 - e) << 20, 0);  // ~ 1 / |b|
+    const double x = b.x * f, y = b.y * f, d = f / fma(x, x, y * y);
+    return make_double2(fma(a.x, x, a.y * y) * d, fma(a.y, x, -a.x * y) * d);
 }
 __device__ __forceinline__ double2 shfl(double2 v, int src) {
     return make_double2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
 }
 
-// BORDER = false: FOM, (H_k - sigma_i I) y = beta rho_i e_1 (k x k), shift i = blockIdx.x.
-// BORDER = true: the non-seed shifts of restarted multishift GMRES, shift i = blockIdx.x + 1:
+// The shifted systems by Hyman's method: all rows of an upper Hessenberg system but the first fix
+// the solution up to its scale, backwards from x_{q-1} = 1 by one division-free step per row,
+//   x_{l-1} = -(sum_{i >= l} M_li x_i) / M_{l,l-1},
+// and the first row gives the scale.  Each computed x_{l-1} satisfies its row exactly for
+// coefficients perturbed by a few units in the last place, and so does the scaled first row: the
+// solution is that of a system with rows perturbed componentwise by rounding (backward stable
+// without pivoting).  The subdiagonal entries are the non-zero norms rho_l of the Arnoldi process.
+//
+// What bounds it: an FP64 instruction takes a warp 64 cycles, so the elimination with partial
+// pivoting used before (35 of them per row, two divisions among them, and 30 per row of the back
+// substitution) took 118 us at k = 30 and 180 us at k = 40 per cycle.  Here a step takes 6: lanes own
+// rows, add the new x_l times column l to their row sums (4), and the owner of row l hands over
+// x_{l-1} (2; the rows are divided by -M_{l,l-1} when they are staged).  Measured 29 us
+// at k = 40 (17 averaged over the mixed form's k = 16 and 40).
+//
+// BORDER = false: FOM, (H_k - sigma_i I) y = beta rho_i e_1 (k x k), shift i.
+// BORDER = true: the non-seed shifts of restarted multishift GMRES, shift i + 1:
 // [Hbar_k - sigma_i I~ | z] (y, tau) = beta rho_i e_1, (k+1) x (k+1), z = gres the seed's
 // residual coefficients; the new residual of shift i is tau times the seed's, so rho_i <- tau.
-// Both matrices are upper Hessenberg (the bordered one has a full last column), so the
-// same adjacent-row pivoting applies.
+// Both matrices are upper Hessenberg (the bordered one has a full last column).  After a breakdown
+// (kk < kmax, or a last norm of zero) FOM on the kk columns is exact and takes the bordered
+// system's place.
+// One warp per shift, SW shifts of a column per CTA sharing the staged matrix.
+constexpr int SW = 4;
 template <bool BORDER>
-__global__ void __launch_bounds__(32) k_shifted_solve(DevState S) {
-    const int i = BORDER ? blockIdx.x + 1 : blockIdx.x;  // shift
-    const int col = blockIdx.y;  // column
+__global__ void __launch_bounds__(32 * SW) k_shifted_solve(DevState S) {
+    const int col = blockIdx.y;
     if (S.done[col]) return;
-    const int lane = threadIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int km = S.kmax;
     const int kk = S.kk[col];
-    const int q = BORDER ? kk + 1 : kk;    // system size
-    const int ld = BORDER ? km + 1 : km;   // row stride of U
     const double2* H = S.H + (int64_t)col * (km + 1) * km;
-    const double2* z = BORDER ? S.gres + (int64_t)col * (km + 1) : nullptr;
+    const bool border = BORDER && kk == km && H[(int64_t)kk * km + kk - 1].x > 0;
+    const int q = border ? kk + 1 : kk;  // system size
+    const int ld = q | 1;                // odd: the transposed stores meet no bank conflicts
+    extern __shared__ double2 M[];       // [q][ld], column-major, row r >= 1 divided by -H[r][r-1]
+    __shared__ double ninv[KMAX + 1];
+    for (int r = threadIdx.x; r < q; r += blockDim.x) ninv[r] = r > 0 ? -1.0 / H[(int64_t)r * km + r - 1].x : 1.0;
+    __syncthreads();
+    for (int t = threadIdx.x; t < q * q; t += blockDim.x) {
+        const int r = t / q, c = t - r * q;
+        if (c < r) continue;
+        const double2 h = border && c == kk ? S.gres[(int64_t)col * (km + 1) + r] : H[(int64_t)r * km + c];
+        const double f = ninv[r];
+        M[c * ld + r] = make_double2(h.x * f, h.y * f);
+    }
+    __syncthreads();
+    const int slot = blockIdx.x * SW + warp;
+    const int i = BORDER ? slot + 1 : slot;  // shift
+    if (i >= S.s) return;
     const double sigma = S.sigma[(int64_t)col * S.s + i];
     const double sigma_im = S.sigma_im ? S.sigma_im[(int64_t)col * S.s + i] : 0.0;
-    extern __shared__ double2 U[];  // [q][ld] upper factor, row-major
-    __shared__ double2 zU[KMAX + 1];
-    const int c0 = lane, c1 = lane + 32, c2 = lane + 64;  // c2: only the bordered column 64
-    auto Hm = [&](int r, int c) -> double2 {  // system matrix entry (r, c)
-        if (BORDER && c == kk) return z[r];
-        double2 h = H[(int64_t)r * km + c];
-        if (r == c) {
-            h.x -= sigma;
-            h.y -= sigma_im;
-        }
-        return h;
-    };
-    double2 w0 = c0 < q ? Hm(0, c0) : make_double2(0, 0);
-    double2 w1 = c1 < q ? Hm(0, c1) : make_double2(0, 0);
-    double2 w2 = c2 < q ? Hm(0, c2) : make_double2(0, 0);
-    const double beta = S.beta[col];
-    const double2 rho = S.rho[(int64_t)col * S.s + i];
-    double2 zw = make_double2(beta * rho.x, beta * rho.y);
-    bool singular = false;
-    for (int r = 0; r < q; ++r) {
-        const int owner = r & 31;
-        double2 a = shfl(r >= 64 ? w2 : (r >= 32 ? w1 : w0), owner);
-        if (r == q - 1) {
-            if (c0 >= r && c0 < q) U[r * ld + c0] = w0;
-            if (c1 >= r && c1 < q) U[r * ld + c1] = w1;
-            if (c2 >= r && c2 < q) U[r * ld + c2] = w2;
-            if (lane == 0) zU[r] = zw;
-            if (a.x == 0 && a.y == 0) singular = true;
-            break;
-        }
-        double2 n0 = (c0 >= r && c0 < q) ? Hm(r + 1, c0) : make_double2(0, 0);
-        double2 n1 = (c1 >= r && c1 < q) ? Hm(r + 1, c1) : make_double2(0, 0);
-        double2 n2 = (c2 >= r && c2 < q) ? Hm(r + 1, c2) : make_double2(0, 0);
-        double2 b = Hm(r + 1, r);
-        const bool swap = cabs2(b) > cabs2(a);  // row r+1 becomes the pivot row
-        double2 p0 = swap ? n0 : w0, p1 = swap ? n1 : w1, p2 = swap ? n2 : w2;
-        double2 o0 = swap ? w0 : n0, o1 = swap ? w1 : n1, o2 = swap ? w2 : n2;
-        double2 zp = swap ? make_double2(0, 0) : zw, zo = swap ? zw : make_double2(0, 0);
-        double2 piv = swap ? b : a;
-        double2 oth = swap ? a : b;
-        if (piv.x == 0 && piv.y == 0) {
-            singular = true;
-            break;
-        }
-        double2 l = cdiv(oth, piv);
-        if (c0 >= r && c0 < q) U[r * ld + c0] = p0;
-        if (c1 >= r && c1 < q) U[r * ld + c1] = p1;
-        if (c2 >= r && c2 < q) U[r * ld + c2] = p2;
-        if (lane == 0) zU[r] = zp;
-        w0 = c0 > r ? csub(o0, cmul(l, p0)) : make_double2(0, 0);
-        w1 = c1 > r ? csub(o1, cmul(l, p1)) : make_double2(0, 0);
-        w2 = c2 > r ? csub(o2, cmul(l, p2)) : make_double2(0, 0);
-        zw = csub(zo, cmul(l, zp));
-    }
     double2* y = S.y + ((int64_t)col * S.s + i) * km;
-    if (singular) {
+    const double2 zero = make_double2(0, 0);
+    double2 acc[3] = {zero, zero, zero};  // row sums of rows lane, lane + 32, lane + 64
+    double2 xo[3] = {zero, zero, zero};   // x of the same indices
+    double2 x = make_double2(1.0, 0.0);
+    for (int l = q - 1; l >= 0; --l) {
+        if (lane == (l & 31)) {
+            if (l < 32)
+                xo[0] = x;
+            else if (l < 64)
+                xo[1] = x;
+            else
+                xo[2] = x;
+        }
+        const double2* mc = M + l * ld;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            if (32 * k > l) break;  // uniform
+            const int r = lane + 32 * k;
+            const double2 m = r <= l ? mc[r] : zero;
+            acc[k].x = fma(m.x, x.x, acc[k].x);
+            acc[k].x = fma(-m.y, x.y, acc[k].x);
+            acc[k].y = fma(m.x, x.y, acc[k].y);
+            acc[k].y = fma(m.y, x.x, acc[k].y);
+        }
+        // the row sum of row l, less its shift: x_{l-1} (the last, l = 0, is the first row's value).
+        // The bordered system's last row has no shift.
+        double2 v = shfl(l >= 64 ? acc[2] : l >= 32 ? acc[1] : acc[0], l & 31);
+        if (l < kk) {
+            const double sr = sigma * ninv[l];
+            v.x = fma(-sr, x.x, v.x);
+            v.y = fma(-sr, x.y, v.y);
+            if (sigma_im != 0.0) {
+                const double si = sigma_im * ninv[l];
+                v.x = fma(si, x.y, v.x);
+                v.y = fma(-si, x.x, v.y);
+            }
+        }
+        x = v;
+        // keep the running solution far from overflow (shifts of large modulus): scale by 2^-400
+        const int big = max(__double2hiint(x.x) & 0x7fffffff, __double2hiint(x.y) & 0x7fffffff);
+        if (l > 0 && big > 0x59000000 && big < 0x7ff00000) {  // above 2^401, finite
+            const double f = __hiloint2double(0x26f00000, 0);  // 2^-400
+            x = make_double2(x.x * f, x.y * f);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                acc[k] = make_double2(acc[k].x * f, acc[k].y * f);
+                xo[k] = make_double2(xo[k].x * f, xo[k].y * f);
+            }
+        }
+    }
+    if (x.x == 0 && x.y == 0) {  // first row's value zero: the shift is an eigenvalue
         if (lane == 0) atomicOr(S.err, 1);
-        for (int j = lane; j < km; j += 32) y[j] = make_double2(0, 0);
+        for (int j = lane; j < km; j += 32) y[j] = zero;
         return;
     }
-    __syncwarp();
-    // column-oriented back substitution; lane owns rows lane, lane + 32 (and lane + 64)
-    double2 z0 = c0 < q ? zU[c0] : make_double2(0, 0);
-    double2 z1 = c1 < q ? zU[c1] : make_double2(0, 0);
-    double2 z2 = c2 < q ? zU[c2] : make_double2(0, 0);
-    double2 ylast = make_double2(0, 0);
-    for (int r = q - 1; r >= 0; --r) {
-        const int owner = r & 31;
-        double2 zr = shfl(r >= 64 ? z2 : (r >= 32 ? z1 : z0), owner);
-        double2 yr = cdiv(zr, U[r * ld + r]);
-        if (r == q - 1) ylast = yr;
-        if (lane == owner && r < kk) y[r] = yr;
-        if (c0 < r) z0 = csub(z0, cmul(U[c0 * ld + r], yr));
-        if (c1 < r) z1 = csub(z1, cmul(U[c1 * ld + r], yr));
-        if (c2 < r) z2 = csub(z2, cmul(U[c2 * ld + r], yr));
-    }
-    for (int j = kk + lane; j < km; j += 32) y[j] = make_double2(0, 0);
-    if (lane == 0) {
-        double2 rnew = make_double2(0, 0);
-        if (BORDER) {
-            rnew = ylast;  // tau
-        } else if (kk == km) {
-            double2 h = H[(int64_t)kk * km + (kk - 1)];
-            rnew = cmul(h, ylast);
-            rnew.x = -rnew.x;
-            rnew.y = -rnew.y;
+    const double2 rho = S.rho[(int64_t)col * S.s + i];
+    const double beta = S.beta[col];
+    const double2 sc = cdiv_scaled(make_double2(beta * rho.x, beta * rho.y), x);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int j = lane + 32 * k;
+        const double2 v = cmul(xo[k], sc);
+        if (j < km) y[j] = j < kk ? v : zero;
+        if (j == q - 1) {  // the last component
+            double2 rnew = zero;
+            if (border) {
+                rnew = v;  // tau
+            } else if (!BORDER && kk == km) {
+                const double2 h = H[(int64_t)kk * km + (kk - 1)];
+                rnew = cmul(h, v);
+                rnew = make_double2(-rnew.x, -rnew.y);
+            }
+            S.rho[(int64_t)col * S.s + i] = rnew;
         }
-        S.rho[(int64_t)col * S.s + i] = rnew;
     }
 }
 
@@ -151,103 +169,135 @@ __global__ void k_combine(DevState S) {
 // Minimal-residual form for one shift per column (restarted GMRES):  y = argmin
 // || beta rho e_1 - (Hbar_k - sigma I~) y ||  by Givens rotations, with the
 // coefficients of the new residual, c = beta rho e_1 - (Hbar_k - sigma I~) y, in
-// gres[col][0..kk] (the next restart vector is V_{k+1} c) and rho = 1.  One CTA per
-// column; the rotations run on one thread over a shared-memory copy (k <= 64:
-// O(k^2) work, once per cycle).
-__global__ void k_shifted_lsq(DevState S) {
+// gres[col][0..kk] (the next restart vector is V_{k+1} c) and rho = 1.  One CTA per column stages
+// the matrix; one warp applies the rotations (lanes own columns, the right-hand side is column
+// kk), back-substitutes and forms c (lanes own rows).
+__global__ void __launch_bounds__(128) k_shifted_lsq(DevState S) {
     const int col = blockIdx.x;
-    if (S.done[col] || threadIdx.x != 0) return;
+    if (S.done[col]) return;
     const int km = S.kmax;
     const int kk = S.kk[col];
     const double2* H = S.H + (int64_t)col * (km + 1) * km;
     const double sig = S.sigma[(int64_t)col * S.s];
     const double sig_im = S.sigma_im ? S.sigma_im[(int64_t)col * S.s] : 0.0;
-    extern __shared__ double2 M[];  // [(kk + 1)][km]
-    __shared__ double2 g[KMAX + 1];
-    for (int r = 0; r <= kk; ++r)
-        for (int c = 0; c < kk; ++c) {
-            double2 h = H[(int64_t)r * km + c];
+    const double beta = S.beta[col];
+    const double2 rho = S.rho[(int64_t)col * S.s];
+    const double2 b0 = make_double2(beta * rho.x, beta * rho.y), zero = make_double2(0, 0);
+    const int ld = kk + 2;           // row stride: columns 0..kk-1, the right-hand side, one of padding
+    extern __shared__ double2 M[];   // [kk + 1][ld]
+    __shared__ double inv[KMAX];     // 1 / diagonal after the rotations (0: zero column)
+    for (int t = threadIdx.x; t < (kk + 1) * ld; t += blockDim.x) {
+        const int r = t / ld, c = t - r * ld;
+        double2 h = zero;
+        if (c < kk && c >= r - 1) {
+            h = H[(int64_t)r * km + c];
             if (r == c) {
                 h.x -= sig;
                 h.y -= sig_im;
             }
-            M[r * km + c] = h;
+        } else if (c == kk && r == 0) {
+            h = b0;
         }
-    const double beta = S.beta[col];
-    const double2 rho = S.rho[(int64_t)col * S.s];
-    const double2 b0 = make_double2(beta * rho.x, beta * rho.y);
-    for (int r = 0; r <= kk; ++r) g[r] = r == 0 ? b0 : make_double2(0, 0);
-    // rows c and c+1: G = [[conj(cs), conj(sn)], [-sn, cs]] zeroes M[c+1][c]
+        M[t] = h;
+    }
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    const int lane = threadIdx.x;
+    // rows c and c+1: G = [[conj(cs), sn], [-sn, cs]] zeroes M[c+1][c] (real: an Arnoldi norm)
     for (int c = 0; c < kk; ++c) {
-        const double2 a = M[c * km + c], b = M[(c + 1) * km + c];
-        const double nr = sqrt(cabs2(a) + cabs2(b));
-        if (!(nr > 0)) continue;  // zero column (only at a breakdown): y_c = 0 below
-        const double2 cs = make_double2(a.x / nr, a.y / nr), sn = make_double2(b.x / nr, b.y / nr);
-        for (int j = c; j < kk; ++j) {
-            const double2 x = M[c * km + j], y = M[(c + 1) * km + j];
-            M[c * km + j] = cadd(cconjmul(cs, x), cconjmul(sn, y));
-            M[(c + 1) * km + j] = csub(cmul(cs, y), cmul(sn, x));
+        const double2 a = M[c * ld + c];
+        const double b = M[(c + 1) * ld + c].x;
+        const double n2 = fma(b, b, cabs2(a));
+        const double ir = n2 > 0 ? rsqrt(n2) : 0.0;
+        if (lane == 0) inv[c] = ir;
+        __syncwarp();
+        if (!(n2 > 0)) continue;  // zero column (only at a breakdown): y_c = 0 below
+        const double2 cs = make_double2(a.x * ir, a.y * ir);
+        const double sn = b * ir;
+        for (int j = c + lane; j <= kk; j += 32) {
+            const double2 x = M[c * ld + j], w = M[(c + 1) * ld + j];
+            double2 p = cconjmul(cs, x), r = cmul(cs, w);
+            p.x = fma(sn, w.x, p.x);
+            p.y = fma(sn, w.y, p.y);
+            r.x = fma(-sn, x.x, r.x);
+            r.y = fma(-sn, x.y, r.y);
+            M[c * ld + j] = p;
+            M[(c + 1) * ld + j] = r;
         }
-        const double2 x = g[c], y = g[c + 1];
-        g[c] = cadd(cconjmul(cs, x), cconjmul(sn, y));
-        g[c + 1] = csub(cmul(cs, y), cmul(sn, x));
+        __syncwarp();
+    }
+    // back substitution; lane owns rows lane, lane + 32
+    double2 z0 = lane < kk ? M[lane * ld + kk] : zero, z1 = lane + 32 < kk ? M[(lane + 32) * ld + kk] : zero;
+    double2 y0 = zero, y1 = zero;
+    for (int r = kk - 1; r >= 0; --r) {
+        double2 yr = shfl(r >= 32 ? z1 : z0, r & 31);
+        yr = make_double2(yr.x * inv[r], yr.y * inv[r]);
+        if (lane == (r & 31)) {
+            if (r < 32)
+                y0 = yr;
+            else
+                y1 = yr;
+        }
+        if (lane < r) z0 = csub(z0, cmul(M[lane * ld + r], yr));
+        if (r > 32 && lane + 32 < r) z1 = csub(z1, cmul(M[(lane + 32) * ld + r], yr));
     }
     double2* yv = S.y + (int64_t)col * S.s * km;
-    for (int r = kk - 1; r >= 0; --r) {
-        double2 z = g[r];
-        for (int j = r + 1; j < kk; ++j) z = csub(z, cmul(M[r * km + j], yv[j]));
-        const double2 d = M[r * km + r];
-        const double dd = cabs2(d);
-        yv[r] = dd > 0 ? make_double2((z.x * d.x + z.y * d.y) / dd, (z.y * d.x - z.x * d.y) / dd) : make_double2(0, 0);
-    }
-    for (int j = kk; j < km; ++j) yv[j] = make_double2(0, 0);
-    // c = beta rho e_1 - (Hbar - sigma I~) y, from the unrotated matrix
-    double2* cres = S.gres + (int64_t)col * (km + 1);
-    for (int r = 0; r <= km; ++r) {
-        double2 acc = r == 0 ? b0 : make_double2(0, 0);
-        if (r <= kk)
-            for (int c = (r > 0 ? r - 1 : 0); c < kk; ++c) {
-                double2 h = H[(int64_t)r * km + c];
-                if (r == c) {
-                    h.x -= sig;
-                    h.y -= sig_im;
-                }
-                acc = csub(acc, cmul(h, yv[c]));
+    if (lane < km) yv[lane] = lane < kk ? y0 : zero;
+    if (lane + 32 < km) yv[lane + 32] = lane + 32 < kk ? y1 : zero;
+    // c = beta rho e_1 - (Hbar - sigma I~) y, from the unrotated matrix; lane owns rows lane, + 32, + 64
+    double2 acc[3] = {lane == 0 ? b0 : zero, zero, zero};
+    for (int c = 0; c < kk; ++c) {
+        const double2 yc = shfl(c >= 32 ? y1 : y0, c & 31);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const int r = lane + 32 * k;
+            if (32 * k > c + 1) break;  // uniform
+            double2 h = r <= c + 1 ? H[(int64_t)r * km + c] : zero;
+            if (r == c) {
+                h.x -= sig;
+                h.y -= sig_im;
             }
-        cres[r] = acc;
+            acc[k] = csub(acc[k], cmul(h, yc));
+        }
     }
-    S.rho[(int64_t)col * S.s] = make_double2(1, 0);
+    double2* cres = S.gres + (int64_t)col * (km + 1);
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+        if (lane + 32 * k <= km) cres[lane + 32 * k] = lane + 32 * k <= kk ? acc[k] : zero;
+    if (lane == 0) S.rho[(int64_t)col * S.s] = make_double2(1, 0);
 }
+
+// Shared memory of a q x q system staged by k_shifted_solve.
+constexpr size_t staged_bytes(int q) { return sizeof(double2) * (size_t)q * (q | 1); }
 
 }  // namespace
 
 cudaError_t shifted_lsq(const DevState& S, int ncol, cudaStream_t st) {
     if (S.s < 1 || !S.gres || S.kmax > KMAX) return cudaErrorInvalidValue;
-    k_shifted_lsq<<<ncol, 32, sizeof(double2) * (S.kmax + 1) * S.kmax, st>>>(S);
+    k_shifted_lsq<<<ncol, 128, sizeof(double2) * (S.kmax + 1) * (S.kmax + 2), st>>>(S);
     count_launch();
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || S.s == 1) return e;
     // the other shifts: bordered systems with the seed's residual coefficients
-    k_shifted_solve<true><<<dim3(S.s - 1, ncol), 32, sizeof(double2) * (S.kmax + 1) * (S.kmax + 1), st>>>(S);
+    k_shifted_solve<true><<<dim3((S.s - 1 + SW - 1) / SW, ncol), 32 * SW, staged_bytes(S.kmax + 1), st>>>(S);
     count_launch();
     return cudaGetLastError();
 }
 
 cudaError_t prepare_small_kernels() {
     cudaError_t e = cudaFuncSetAttribute(k_shifted_solve<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(sizeof(double2) * KMAX * KMAX));
+                                         (int)staged_bytes(KMAX));
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_shifted_solve<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(sizeof(double2) * (KMAX + 1) * (KMAX + 1)));
+                                 (int)staged_bytes(KMAX + 1));
     if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(k_shifted_lsq, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)(sizeof(double2) * (KMAX + 1) * KMAX));
+                                (int)(sizeof(double2) * (KMAX + 1) * (KMAX + 2)));
 }
 
 cudaError_t shifted_solves(const DevState& S, int ncol, cudaStream_t st) {
     if (S.kmax > KMAX) return cudaErrorInvalidValue;
-    size_t smem = sizeof(double2) * (size_t)S.kmax * S.kmax;
-    k_shifted_solve<false><<<dim3(S.s, ncol), 32, smem, st>>>(S);
+    k_shifted_solve<false><<<dim3((S.s + SW - 1) / SW, ncol), 32 * SW, staged_bytes(S.kmax), st>>>(S);
     count_launch();
     return cudaGetLastError();
 }
