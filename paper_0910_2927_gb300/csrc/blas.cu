@@ -631,10 +631,9 @@ __global__ void __launch_bounds__(NT) k_dcgs_dots(Basis<float2> V, int J, const 
 // Delayed CGS2, update of step j:  q_j = (u - Q s) / rho  (written over u), and
 // the next candidate  u_{j+1} = z / rho - Q c - d q_j  (when next != null).
 // Coefficients per column: [0,J) s, [J,2J) c, 2J: (1/rho, 0), 2J+1: d.
-// FP32 storage (FP64: gs_f64.cu).  Four CTAs per SM (64 registers): as the compiler sizes it with the
-// Hessenberg column in the kernel, PKT = 4 takes 107 registers and ran 87 instead of 74 us.
+// FP32 storage (FP64: gs_f64.cu).
 template <int PKT>
-__global__ void __launch_bounds__(NT, 4) k_dcgs_update(Basis<float2> V, int J, const double2* __restrict__ coef,
+__global__ void __launch_bounds__(NT) k_dcgs_update(Basis<float2> V, int J, const double2* __restrict__ coef,
                                                     int cstride, float2* u, const float2* __restrict__ z, float2* next,
                                                     int64_t wsr, int64_t npk, double2* H, int km,
                                                     const int* __restrict__ skip) {
@@ -650,7 +649,7 @@ __global__ void __launch_bounds__(NT, 4) k_dcgs_update(Basis<float2> V, int J, c
     __shared__ typename O::C cs[MAXSLOT], cc[MAXSLOT];
     __shared__ double ex[2][2];
     const double2* cf = coef + (int64_t)col * cstride;
-    for (int l = threadIdx.x; l < J; l += blockDim.x) {
+    for (int l = threadIdx.x; l < J; l += NT) {
         cs[l] = O::coef(cf[l]);
         cc[l] = O::coef(cf[J + l]);
     }
@@ -666,7 +665,7 @@ __global__ void __launch_bounds__(NT, 4) k_dcgs_update(Basis<float2> V, int J, c
     const T* zc = next ? z + col * wsr : nullptr;
     T* nc = next ? next + col * wsr : nullptr;
     const T* vb = V.base + col * V.sr;
-    const int64_t base = (int64_t)tile * blockDim.x * PKT + threadIdx.x;
+    const int64_t base = (int64_t)tile * NT * PKT + threadIdx.x;
     // Q s and Q c with the basis loop outside: the loads of UNR basis vectors
     // (PKT packs each) are independent and in flight together
     typename O::P qs[PKT], qc[PKT];
@@ -683,7 +682,7 @@ __global__ void __launch_bounds__(NT, 4) k_dcgs_update(Basis<float2> V, int J, c
             const T* vl = vb + (l0 + g) * V.sj;
 #pragma unroll
             for (int p = 0; p < PKT; ++p) {
-                const int64_t i = base + p * (int)blockDim.x;
+                const int64_t i = base + p * NT;
                 q[g][p] = (l0 + g < J && i < npk) ? O::ld_ro(vl, i) : O::zero();
             }
         }
@@ -702,7 +701,7 @@ __global__ void __launch_bounds__(NT, 4) k_dcgs_update(Basis<float2> V, int J, c
     const typename O::C one = make_float2(1.0f, 0.0f);
 #pragma unroll
     for (int p = 0; p < PKT; ++p) {
-        const int64_t i = base + p * (int)blockDim.x;
+        const int64_t i = base + p * NT;
         if (i >= npk) break;
         typename O::P uv = O::ld(uc, i);
         // q_j = (u - qs) / rho

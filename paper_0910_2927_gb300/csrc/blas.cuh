@@ -71,8 +71,9 @@ __device__ __forceinline__ double reduce_few(double (&a)[N], int lane) {
 // Tentative column j of the Hessenberg matrix in a delayed-CGS2 step, by one CTA:
 //   H[i][j] = c_i - g_i / rho (i < j),  H[j][j] = d - g_j / rho,  g = H[0:j+1, 0:j] s,
 // with the step's coefficients s = red[0, j), c = red[j, 2j), 1 / rho = red[2j], d = red[2j + 1].
-// Four lanes per row.
-__device__ __forceinline__ void hess_column(double2* __restrict__ H, const double2* __restrict__ red, int j, int km) {
+// Four lanes per row.  Not inlined: in the FP32 update it would take that kernel from 80 to 107
+// registers, a third of its resident warps (74 -> 87 us on 120 columns of 10^4).
+__device__ __noinline__ static void hess_column(double2* __restrict__ H, const double2* __restrict__ red, int j, int km) {
     const int q = threadIdx.x & 3;
     const double ir = red[2 * j].x;
     for (int i0 = 0; i0 <= j; i0 += blockDim.x / 4) {
