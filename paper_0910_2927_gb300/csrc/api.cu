@@ -201,7 +201,7 @@ SGN_API int sgn_load_gauge(sgn_ctx* c, const double* links, int on_device) {
     SGN_CUDA(convert_f64_to_f32(as<double2>(c->U64), as<float2>(c->U32), (int64_t)count, c->work));
     SGN_CUDA(links_f64_to_bf16(as<double2>(c->U64), as<__nv_bfloat162>(c->U16), (int64_t)count, c->work));
     SGN_CUDA(links_f64_to_f16(as<double2>(c->U64), as<__half2>(c->UH), (int64_t)count, c->work));
-    SGN_CUDA(links_ff(as<double2>(c->U64), as<float2>(c->U32), as<float4>(c->Uff), (int64_t)count, c->work));
+    SGN_CUDA(split_ff(as<double2>(c->U64), as<float4>(c->Uff), (int64_t)count, c->work));
     SGN_CUDA(cudaStreamSynchronize(c->work));
     SGN_CHECK(ses.close());
     c->have_gauge = true;
@@ -501,24 +501,12 @@ SGN_API int sgn_hw_apply(sgn_ctx* c, const void* in, void* out, int nrhs, int pr
     if (precision == SGN_PREC_FP64) {
         const double2* pi = reinterpret_cast<const double2*>(in);
         double2* po = reinterpret_cast<double2*>(out);
-        if (ffa) {
-            // staging (complex128 units): the packed copies of in and out, then the float-float
-            // (hi, lo) pairs of in and out (4 nn complex64 = 2 nn complex128)
-            SGN_CHECK(dev_alloc(c, c->stage, ((packed ? 0 : 2 * nn) + 2 * nn) * sizeof(double2)));
-            double2* t = as<double2>(c->stage);
-            if (!packed) {
-                SGN_CUDA(pack_fields<double2>(pi, t, c->vol, nrhs, c->work));
-                pi = t;
-                po = t + nn;
-            }
-            float2* f = reinterpret_cast<float2*>(t + (packed ? 0 : 2 * nn));
-            float2 *ih = f, *il = f + nn, *oh = f + 2 * nn, *ol = f + 3 * nn;
-            SGN_CUDA(split_ff(pi, ih, il, (int64_t)nn, c->work));
-            SGN_CUDA(launch_hw_ff(oh, ol, ih, il, as<float4>(c->Uff), nrhs, stencil_params(c, adjoint), c->work));
-            SGN_CUDA(join_ff(oh, ol, po, (int64_t)nn, c->work));
-            if (!packed)
-                SGN_CUDA(unpack_fields<double2>(po, reinterpret_cast<double2*>(out), c->vol, nrhs, c->work));
-        } else {  // the FP64 stencil reads and writes either order
+        if (ffa) {  // the float-float copy of the input; both stencils read and write either order
+            SGN_CHECK(dev_alloc(c, c->stage, nn * sizeof(float4)));
+            SGN_CUDA(split_ff(pi, as<float4>(c->stage), (int64_t)nn, c->work));
+            SGN_CUDA(hw_ff_doubles(po, as<float4>(c->stage), as<float4>(c->Uff), nrhs, stencil_params(c, adjoint),
+                                   !packed, c->work));
+        } else {
             SGN_CUDA(launch_hw_f64(po, pi, as<double2>(c->U64), nrhs, stencil_params(c, adjoint), nullptr, c->work,
                                    !packed));
         }

@@ -13,6 +13,7 @@
 // the per-column sum over CTAs -- is FP64 in a fixed order (no atomics).  The FP64 inner products
 // are in gs_f64.cu.
 #include "blas.cuh"
+#include "cvt.cuh"
 
 #include <cstdlib>
 
@@ -145,18 +146,19 @@ struct Ops<float2> {
     }
     static __device__ __forceinline__ void add_to(double2* x, int64_t pk, P v) {
         double2 a = x[2 * pk], b = x[2 * pk + 1];
-        x[2 * pk] = make_double2(a.x + v.x, a.y + v.y);
-        x[2 * pk + 1] = make_double2(b.x + v.z, b.y + v.w);
+        x[2 * pk] = make_double2(a.x + f2d(v.x), a.y + f2d(v.y));
+        x[2 * pk + 1] = make_double2(b.x + f2d(v.z), b.y + f2d(v.w));
     }
     static __device__ __forceinline__ void add_cv_f64(double2 acc[2], double2 c, P v) {
-        acc[0].x = fma(c.x, (double)v.x, acc[0].x);
-        acc[0].x = fma(-c.y, (double)v.y, acc[0].x);
-        acc[0].y = fma(c.x, (double)v.y, acc[0].y);
-        acc[0].y = fma(c.y, (double)v.x, acc[0].y);
-        acc[1].x = fma(c.x, (double)v.z, acc[1].x);
-        acc[1].x = fma(-c.y, (double)v.w, acc[1].x);
-        acc[1].y = fma(c.x, (double)v.w, acc[1].y);
-        acc[1].y = fma(c.y, (double)v.z, acc[1].y);
+        const double x = f2d(v.x), y = f2d(v.y), z = f2d(v.z), w = f2d(v.w);
+        acc[0].x = fma(c.x, x, acc[0].x);
+        acc[0].x = fma(-c.y, y, acc[0].x);
+        acc[0].y = fma(c.x, y, acc[0].y);
+        acc[0].y = fma(c.y, x, acc[0].y);
+        acc[1].x = fma(c.x, z, acc[1].x);
+        acc[1].x = fma(-c.y, w, acc[1].x);
+        acc[1].y = fma(c.x, w, acc[1].y);
+        acc[1].y = fma(c.y, z, acc[1].y);
     }
 };
 
@@ -1053,19 +1055,19 @@ __global__ void k_random_fill(T* out, int64_t count, uint64_t seed) {
 __global__ void k_f64_to_f32(const double2* __restrict__ in, float2* __restrict__ out, int64_t count) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
         double2 v = in[i];
-        out[i] = make_float2((float)v.x, (float)v.y);
+        out[i] = make_float2(d2f(v.x), d2f(v.y));
     }
 }
 __global__ void k_f32_to_f64(const float2* __restrict__ in, double2* __restrict__ out, int64_t count) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
         float2 v = in[i];
-        out[i] = make_double2(v.x, v.y);
+        out[i] = make_double2(f2d(v.x), f2d(v.y));
     }
 }
 __global__ void k_f64_to_bf16(const double2* __restrict__ in, __nv_bfloat162* __restrict__ out, int64_t count) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
         double2 v = in[i];
-        out[i] = __floats2bfloat162_rn((float)v.x, (float)v.y);
+        out[i] = __floats2bfloat162_rn(d2f(v.x), d2f(v.y));
     }
 }
 // FP16 links: SU(3) entries have modulus <= 1, inside FP16's normal range (one rounding
@@ -1074,7 +1076,7 @@ __global__ void k_f64_to_bf16(const double2* __restrict__ in, __nv_bfloat162* __
 __global__ void k_f64_to_f16(const double2* __restrict__ in, __half2* __restrict__ out, int64_t count) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
         double2 v = in[i];
-        out[i] = __floats2half2_rn((float)v.x, (float)v.y);
+        out[i] = __floats2half2_rn(d2f(v.x), d2f(v.y));
     }
 }
 

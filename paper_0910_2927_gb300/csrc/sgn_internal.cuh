@@ -121,17 +121,17 @@ cudaError_t launch_hw_f32_bf16links(float2* out, const float2* in, const __nv_bf
                                     StencilShape sh = {});
 cudaError_t launch_hw_f32_f16links(float2* out, const float2* in, const __half2* U, int nrhs,
                                    const StencilParams& p, const int* skip, cudaStream_t st, StencilShape sh = {});
-// Float-float stencil (stencil_ff.cu): fields as (hi, lo) pairs of packed FP32 fields, links as
-// one float4 (U32, fl(U - U32)) per packed entry; about 1e-13 of the FP64 result.
-cudaError_t launch_hw_ff(float2* oh, float2* ol, const float2* ih, const float2* il, const float4* Uf, int nrhs,
-                         const StencilParams& p, cudaStream_t st);
-// FP64 <-> (hi, lo) conversions of count complex entries, the FP64 true residual
-// r = b - (yh + yl) + sigma x, and the float-float links (U32, fl(U - U32)).
-cudaError_t split_ff(const double2* in, float2* hi, float2* lo, int64_t count, cudaStream_t st);
-cudaError_t join_ff(const float2* hi, const float2* lo, double2* out, int64_t count, cudaStream_t st);
-cudaError_t residual_ff(double2* r, const double2* b, const float2* yh, const float2* yl, double sigma,
-                        const double2* x, int64_t count, cudaStream_t st);
-cudaError_t links_ff(const double2* U, const float2* U32, float4* out, int64_t count, cudaStream_t st);
+// Float-float stencil (stencil_ff.cu): fields and links as a float4 (Re hi, Im hi, Re lo, Im lo) per
+// complex number, in the place the complex128 number has (packed, or natural with nat); about
+// 1e-13 of the FP64 result.  The result as float-float, as complex128, or as the true residuals
+// r_f = b_c - H in_f + sigma_i x_f of fields f = i ncol + c (sigma: device, one per shift).
+cudaError_t hw_ff(float4* out, const float4* in, const float4* Uf, int nrhs, const StencilParams& p, cudaStream_t st);
+cudaError_t hw_ff_doubles(double2* out, const float4* in, const float4* Uf, int nrhs, const StencilParams& p, bool nat,
+                          cudaStream_t st);
+cudaError_t hw_ff_residual(double2* r, const float4* in, const float4* Uf, int nrhs, const StencilParams& p,
+                           const double2* b, int ncol, const double2* x, const double* sigma, cudaStream_t st);
+// complex128 -> float-float, elementwise (fields and links)
+cudaError_t split_ff(const double2* in, float4* out, int64_t count, cudaStream_t st);
 
 // ------------------------------------------------------------ vector ops --
 // A "basis" is J fields per column: element e of vector j of column r lives at

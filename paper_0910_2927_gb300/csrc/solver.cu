@@ -848,7 +848,7 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
     Engine* E1 = nullptr;
     SGN_CHECK(get_engine(c, B, k1, 1, SGN_PREC_MIXED, &E1));
 
-    // io: xs (s ncol) | r0, bt, xP, t, u (ncol each) | d (B) | omega table | FP64 partials
+    // io: xs (s ncol) | r0, bt, xP (ncol each) | float-float x, A x | d (B) | omega table | FP64 partials
     const size_t field = (size_t)n * sizeof(double2);
     const int nblk64 = dot_blocks<double2>(n, ncol);
     const int rs64 = ((std::max(m, s) + 2) + 7) & ~7;
@@ -860,11 +860,13 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
     };
     size_t o_xs = take(field * ncol * s);
     size_t o_r0 = take(field * ncol), o_bt = take(field * ncol), o_xp = take(field * ncol);
-    size_t o_t = take(field * ncol), o_u = take(field * ncol);
+    // float-float copies of x_i and A x_i: of as many shifts as it takes to fill the chip
+    const int fsh = (int)std::min<int64_t>(s, std::max<int64_t>(1, (int64_t)131072 / (c->vol * ncol)));
+    size_t o_t = take(field * ncol * fsh), o_u = take(field * ncol * fsh);
     size_t o_d = take(field * B);
     size_t o_rs = take(field * ncol * s);
     const int ncmax = std::max({ncol, B, s * ncol});
-    size_t o_om = take(sizeof(double2) * ncol * rs64);
+    size_t o_om = take(sizeof(double2) * ncol * rs64), o_sig = take(sizeof(double) * s);
     size_t o_red = take(sizeof(double2) * ncmax * rs64);
     size_t o_part = take(sizeof(double2) * (size_t)ncmax * rs64 * nblk64);
     size_t o_flags = take(sizeof(int) * 2 * ncmax);
@@ -875,8 +877,9 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
     double2* r0 = reinterpret_cast<double2*>(io + o_r0);
     double2* bt = reinterpret_cast<double2*>(io + o_bt);
     double2* xP = reinterpret_cast<double2*>(io + o_xp);
-    double2* t64 = reinterpret_cast<double2*>(io + o_t);
-    double2* u64 = reinterpret_cast<double2*>(io + o_u);
+    float4* xf = reinterpret_cast<float4*>(io + o_t);
+    float4* tf = reinterpret_cast<float4*>(io + o_u);
+    double* sig_dev = reinterpret_cast<double*>(io + o_sig);
     double2* d = reinterpret_cast<double2*>(io + o_d);
     double2* rsd = reinterpret_cast<double2*>(io + o_rs);  // true residuals r_i, [i][col][n]
     double2* omtab = reinterpret_cast<double2*>(io + o_om);
@@ -900,6 +903,7 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
             omh[(size_t)col * rs64 + i] = make_double2(c->omega[i], 0);
         }
     SGN_CHECK(fill_shift_tables(c, *E, sig_cols.data(), om_cols.data()));
+    SGN_CUDA(cudaMemcpyAsync(sig_dev, c->sigma.data(), sizeof(double) * s, cudaMemcpyHostToDevice, st));
     SGN_CUDA(cudaMemcpyAsync(omtab, omh.data(), sizeof(double2) * omh.size(), cudaMemcpyHostToDevice, st));
 
     const double2* Lb = reinterpret_cast<const double2*>(adjoint ? c->R64.p : c->L64.p);
@@ -992,23 +996,17 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
         // r_i -= (A^2 - sigma_i) d_i with x_i += d_i), where FP32 products of the small d_i are
         // exact to ~1e-7 ||r_i||.
         // Round 0 forms A^2 x_i in float-float arithmetic on the FP32 units (stencil_ff.cu; ~1e-13
-        // of the FP64 stencil, which GB300 runs at 1/64 of the FP32 rate); the (hi, lo) pairs of
-        // x_i and A x_i live in the space of t64 and u64 (4 ncol complex64 fields = 2 ncol
-        // complex128 fields).
+        // of the FP64 stencil, which GB300 runs at 1/64 of the FP32 rate), fsh shifts at a time.
         if (round == 0) {
             const size_t nf = (size_t)ncol * n;
-            float2* xh = reinterpret_cast<float2*>(t64);
-            float2* xl = xh + nf;
-            float2* th = reinterpret_cast<float2*>(u64);
-            float2* tl = th + nf;
             const StencilParams pf = stencil_params(c, adjoint);
             const float4* Uf = reinterpret_cast<const float4*>(c->Uff.p);
-            for (int i = 0; i < s; ++i) {
-                double2* xi = xs + (size_t)i * nf;
-                SGN_CUDA(split_ff(xi, xh, xl, (int64_t)nf, st));
-                SGN_CUDA(launch_hw_ff(th, tl, xh, xl, Uf, ncol, pf, st));
-                SGN_CUDA(launch_hw_ff(xh, xl, th, tl, Uf, ncol, pf, st));
-                SGN_CUDA(residual_ff(rsd + (size_t)i * nf, bt, xh, xl, c->sigma[i], xi, (int64_t)nf, st));
+            for (int i = 0; i < s; i += fsh) {
+                const int g = std::min(fsh, s - i), nc = g * ncol;
+                const double2* xi = xs + (size_t)i * nf;
+                SGN_CUDA(split_ff(xi, xf, (int64_t)(g * nf), st));
+                SGN_CUDA(hw_ff(tf, xf, Uf, nc, pf, st));
+                SGN_CUDA(hw_ff_residual(rsd + (size_t)i * nf, tf, Uf, nc, pf, bt, ncol, xi, sig_dev + i, st));
             }
         }
         SGN_CUDA(mdot<double2>(Basis<double2>{rsd, 0, n}, 0, rsd, n, n, nall, rd64, 1, nullptr, st));

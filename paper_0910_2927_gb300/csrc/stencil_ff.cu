@@ -7,9 +7,17 @@
 // Use: the mixed form's true residuals r_i = b~ - (A^2 - sigma_i) x_i need A^2 x_i to far better
 // than FP32 (they decide convergence at 1e-8 ||b~||), and GB300 executes FP64 at 1/64 of its FP32
 // rate: the FP64 stencil is bound by the FP64 pipe.  The float-float stencil reaches ~1e-13 of the
-// FP64 result with FP32 instructions only.  Fields enter and leave as (hi, lo) pairs of packed FP32
-// fields (the FP32 layout of stencil.cu); the links as float4 (U32, fl(U - U32)) per entry.  Same hop structure as stencil.cu: rank-2 spin projection, gamma5 folded into
-// the store, one thread per site and field, CTA = SX sites x RB fields of one site tile.
+// FP64 result with FP32 instructions only.
+//
+// Layout: a float4 (Re hi, Im hi, Re lo, Im lo) per complex number, in the place the complex128
+// number has in the natural or the packed order, so that conversion is elementwise; links too.
+// Eight lanes per site and field, one per hop, as in stencil_f64.cu (see there for the hop-dependent
+// selects): about 1,500 instructions per lane.  One thread per site (11,000) needed 128 registers
+// for its accumulators and waited for loads most of the time (FMA pipe 32 % busy).  Measured per
+// launch: 16^4 x 4 fields 201 -> 179 us, 10^4 x 12 85 -> 76; 6^4 x 1 27.5 us per shift, now 20 us for
+// twenty shifts together.  The conversions were bound by FP64 conversion instructions (cvt.cuh): split
+// 47 -> 31 us on 16^4 x 4; the join (36 us) and the residual assembly are part of the stencil.
+#include "cvt.cuh"
 #include "sgn_internal.cuh"
 
 namespace sgn {
@@ -51,9 +59,6 @@ __device__ __forceinline__ ff ff_mul(ff a, ff b) {
     e = __fmaf_rn(a.lo, b.hi, e);
     return fast_two_sum(p, e);
 }
-// scaling by a float whose product is exact (a power of two: the hop coefficient -1/2 of the
-// space directions)
-__device__ __forceinline__ ff ff_scale2(ff a, float s) { return {a.hi * s, a.lo * s}; }
 
 // Compensated dot-product accumulator: value s + c.  add(a, b) adds a * b: the product's
 // rounding error (TwoProd) and the sum's (TwoSum) go into c.
@@ -75,70 +80,109 @@ struct ffc {
     ff re, im;
 };
 __device__ __forceinline__ ffc cadd(ffc a, ffc b) { return {ff_add_u(a.re, b.re), ff_add_u(a.im, b.im)}; }
-__device__ __forceinline__ ffc csub(ffc a, ffc b) { return {ff_add_u(a.re, ff_neg(b.re)), ff_add_u(a.im, ff_neg(b.im))}; }
-__device__ __forceinline__ ffc mul_i(ffc a) { return {ff_neg(a.im), a.re}; }   // i a
-__device__ __forceinline__ ffc mul_mi(ffc a) { return {a.im, ff_neg(a.re)}; }  // -i a
+// x with its sign flipped where mask is 0x80000000 (0: unchanged)
+__device__ __forceinline__ float flip(float x, unsigned mask) { return __uint_as_float(__float_as_uint(x) ^ mask); }
+__device__ __forceinline__ ff flip(ff a, unsigned mask) { return {flip(a.hi, mask), flip(a.lo, mask)}; }
+// c v (imag = false) or c i v (imag = true), c = +-1 given by its sign mask
+__device__ __forceinline__ ffc phase(ffc v, bool imag, unsigned c) {
+    const ff a = imag ? v.im : v.re, b = imag ? v.re : v.im;
+    return {flip(a, imag ? c ^ 0x80000000u : c), flip(b, c)};
+}
+__device__ __forceinline__ ffc ld(const float4* __restrict__ p) {
+    const float4 v = __ldg(p);
+    return {{v.x, v.z}, {v.y, v.w}};
+}
+__device__ __forceinline__ ff shfl_xor(ff a, int o) {
+    return {__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
+}
+__device__ __forceinline__ ff sel(bool c, ff a, ff b) { return {c ? a.hi : b.hi, c ? a.lo : b.lo}; }
 
-// 12 spin-colour entries of one site from the (hi, lo) packed fields: plane p holds entries
-// 2p, 2p + 1 at float2 offset p * 2 vol + 2 site.
-__device__ __forceinline__ void load_site(const float2* __restrict__ fh, const float2* __restrict__ fl, int64_t site,
-                                          int64_t vol2, ffc (&p)[12]) {
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        const float4 h = __ldg(reinterpret_cast<const float4*>(fh + k * vol2 + 2 * site));
-        const float4 l = __ldg(reinterpret_cast<const float4*>(fl + k * vol2 + 2 * site));
-        p[2 * k] = {{h.x, l.x}, {h.y, l.y}};
-        p[2 * k + 1] = {{h.z, l.z}, {h.w, l.w}};
-    }
+// Offset of entry k of a site: natural order, or plane k/2 of the packed order.
+template <bool NAT>
+__device__ __forceinline__ int64_t entry(int64_t site, int k, int64_t vol) {
+    return NAT ? site * 12 + k : (int64_t)(k >> 1) * 2 * vol + 2 * site + (k & 1);
 }
 
-// Spin projection h = psi_up + S B psi_dn (B = -i sigma_{x,y,z}, or 1 for t; see stencil.cu).
-template <int NU, int S>
-__device__ __forceinline__ void project(const ffc (&p)[12], ffc (&h0)[3], ffc (&h1)[3]) {
+constexpr int kMaxThreads = 128;
+
+// What becomes of H psi.
+enum FfOut {
+    FF_PAIRS,    // float-float field
+    FF_DOUBLES,  // complex128 field
+    FF_RESIDUAL  // r_f = b_c - H psi_f + sigma_i x_f (complex128) for field f = i ncol + c
+};
+struct FfResidual {
+    const double2 *b, *x;
+    const double* sigma;  // device, one per shift
+    int ncol;
+};
+
+// CTA b: site tile b / nrhs (blockDim.x / 8 sites) of field b % nrhs.
+template <bool NAT, FfOut OUT>
+__global__ void __launch_bounds__(kMaxThreads, 4)
+    k_hw_ff(void* __restrict__ out, const float4* __restrict__ in, const float4* __restrict__ Uf, int nrhs,
+            StencilParams P, FfResidual R) {
+    const int64_t tile = blockIdx.x / (unsigned)nrhs;
+    const int rhs = (int)(blockIdx.x - tile * nrhs);
+    const int64_t s0 = tile * (blockDim.x >> 3) + (threadIdx.x >> 3);
+    const bool act = s0 < P.vol;
+    const int64_t site = act ? s0 : P.vol - 1;  // idle lanes take part in the shuffles
+    const int l = threadIdx.x & 7, nu = l >> 1;
+    const bool fwd = !(l & 1);
+    const float4* f = in + rhs * P.stride_rhs;
+
+    int co, L;
+    int64_t stride;
+    {
+        const uint32_t q0 = P.div[0].div((uint32_t)site);
+        const uint32_t q1 = P.div[1].div(q0);
+        const uint32_t q2 = P.div[2].div(q1);
+        const int c0 = (int)((uint32_t)site - q0 * (uint32_t)P.L[0]), c1 = (int)(q0 - q1 * (uint32_t)P.L[1]),
+                  c2 = (int)(q1 - q2 * (uint32_t)P.L[2]), c3 = (int)q2;
+        co = nu < 2 ? (nu == 0 ? c0 : c1) : (nu == 2 ? c2 : c3);
+        L = nu < 2 ? (nu == 0 ? P.L[0] : P.L[1]) : (nu == 2 ? P.L[2] : P.L[3]);
+        const int64_t s1 = P.L[0], s2 = s1 * P.L[1], s3 = s2 * P.L[2];
+        stride = nu < 2 ? (nu == 0 ? 1 : s1) : (nu == 2 ? s2 : s3);
+    }
+    const bool wrap = fwd ? co == L - 1 : co == 0;
+    const int64_t nb = fwd ? (wrap ? site - (int64_t)(L - 1) * stride : site + stride)
+                           : (wrap ? site + (int64_t)(L - 1) * stride : site - stride);
+    const int apf = nu < 2 ? (nu == 0 ? P.ap[0] : P.ap[1]) : (nu == 2 ? P.ap[2] : P.ap[3]);
+
+    const unsigned NEG = 0x80000000u;
+    const unsigned bs = wrap && apf ? NEG : 0u;  // sign of a hop across an antiperiodic boundary
+    const bool imag = !(nu & 1);
+    const int ka = nu < 2 ? 9 : 6, kb = nu < 2 ? 6 : 9;
+    // spin projection h = psi_up + S B psi_dn, S = -1 forward, +1 backward
+    const unsigned sS = fwd ? NEG : 0u;
+    const unsigned c0 = nu == 3 ? sS : sS ^ NEG;  // factors of the paired spins: -S, -S, -S, S (times i for nu even)
+    const unsigned c1 = nu == 0 ? sS ^ NEG : sS;  // -S, S, S, S
+    ffc h0[3], h1[3], u[9];
+    const float4* lb = Uf + (int64_t)nu * 9 * P.vol + (fwd ? site : nb);
+    const int ra = fwd ? 3 : 1, rb = fwd ? 1 : 3;
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) u[3 * a + b] = ld(lb + (int64_t)(ra * a + rb * b) * P.vol);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const ffc p0 = p[c], p1 = p[3 + c], p2 = p[6 + c], p3 = p[9 + c];
-        if constexpr (NU == 0) {  // (-i p3, -i p2)
-            h0[c] = S > 0 ? cadd(p0, mul_mi(p3)) : csub(p0, mul_mi(p3));
-            h1[c] = S > 0 ? cadd(p1, mul_mi(p2)) : csub(p1, mul_mi(p2));
-        } else if constexpr (NU == 1) {  // (-p3, p2)
-            h0[c] = S > 0 ? csub(p0, p3) : cadd(p0, p3);
-            h1[c] = S > 0 ? cadd(p1, p2) : csub(p1, p2);
-        } else if constexpr (NU == 2) {  // (-i p2, i p3)
-            h0[c] = S > 0 ? cadd(p0, mul_mi(p2)) : csub(p0, mul_mi(p2));
-            h1[c] = S > 0 ? cadd(p1, mul_i(p3)) : csub(p1, mul_i(p3));
-        } else {  // (p2, p3)
-            h0[c] = S > 0 ? cadd(p0, p2) : csub(p0, p2);
-            h1[c] = S > 0 ? cadd(p1, p3) : csub(p1, p3);
-        }
+        const ffc p0 = ld(f + entry<NAT>(nb, c, P.vol)), p1 = ld(f + entry<NAT>(nb, 3 + c, P.vol));
+        const ffc qa = ld(f + entry<NAT>(nb, ka + c, P.vol)), qb = ld(f + entry<NAT>(nb, kb + c, P.vol));
+        h0[c] = cadd(p0, phase(qa, imag, c0));
+        h1[c] = cadd(p1, phase(qb, imag, c1));
     }
-}
-
-// acc += coef (1 + S gamma_NU) W psi(nb), W = U_NU(site) (S = -1) or U_NU(nb)^dag (S = +1).
-// coef: -1/2 (times -1 across an antiperiodic boundary) in the space directions, applied
-// exactly; -1/2 e^{+-mu} in time, a float-float product.
-template <int NU, int S>
-__device__ __forceinline__ void hop(ffc (&acc)[12], const float2* __restrict__ fh, const float2* __restrict__ fl,
-                                    const float4* __restrict__ Uf, int64_t link_site,
-                                    int64_t nb, ff coef, int64_t vol) {
-    ffc h0[3], h1[3];
-    {
-        ffc p[12];
-        load_site(fh, fl, nb, 2 * vol, p);
-        project<NU, S>(p, h0, h1);
-    }
-    const int64_t lb = (int64_t)NU * 9 * vol + link_site;
+    const unsigned cj = fwd ? 0u : NEG;
+    const ff tc = fwd ? ff{P.cf32[3], P.cf_lo[3]} : ff{P.cb32[3], P.cb_lo[3]};
+    const float sc = fwd ? (nu == 0 ? P.cf32[0] : nu == 1 ? P.cf32[1] : P.cf32[2])
+                         : (nu == 0 ? P.cb32[0] : nu == 1 ? P.cb32[1] : P.cb32[2]);  // -1/2: exact
+    ff v[24];  // the hop's contribution: spins 0, 1 from g0, g1, spins 2, 3 by reconstruction
+    const unsigned c3 = (nu == 1 || nu == 2) ? sS ^ NEG : sS;  // spin 3: S, -S, -S, S (times i for nu even)
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         Dot g0r, g0i, g1r, g1i;
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
-            const int64_t e = lb + (int64_t)(S < 0 ? a * 3 + b : b * 3 + a) * vol;
-            const float4 u = __ldg(Uf + e);  // (Re hi, Im hi, Re lo, Im lo)
-            const ff ur = {u.x, u.z};
-            // U h (forward) or conj(U) h (backward, the dagger's transpose is in the index)
-            const ff ui = S < 0 ? ff{u.y, u.w} : ff{-u.y, -u.w};
-            const ff nui = ff_neg(ui);
+            const ff ur = u[3 * a + b].re, ui = flip(u[3 * a + b].im, cj), nui = flip(ui, NEG);
             g0r.add(ur, h0[b].re);
             g0r.add(nui, h0[b].im);
             g0i.add(ur, h0[b].im);
@@ -148,148 +192,80 @@ __device__ __forceinline__ void hop(ffc (&acc)[12], const float2* __restrict__ f
             g1i.add(ur, h1[b].im);
             g1i.add(ui, h1[b].re);
         }
-        ffc g0 = {g0r.value(), g0i.value()}, g1 = {g1r.value(), g1i.value()};
-        if (NU == 3 || coef.lo != 0.f) {  // the space directions' -1/2 is exact: lo = 0
-            g0 = {ff_mul(g0.re, coef), ff_mul(g0.im, coef)};
-            g1 = {ff_mul(g1.re, coef), ff_mul(g1.im, coef)};
+        ff g[4] = {g0r.value(), g0i.value(), g1r.value(), g1i.value()};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            g[k] = nu == 3 ? ff_mul(g[k], tc) : ff{g[k].hi * sc, g[k].lo * sc};
+            g[k] = flip(g[k], bs);
+        }
+        const ffc g0 = {g[0], g[1]}, g1 = {g[2], g[3]};
+        const ffc e2 = {sel(nu < 2, g1.re, g0.re), sel(nu < 2, g1.im, g0.im)},
+                  e3 = {sel(nu < 2, g0.re, g1.re), sel(nu < 2, g0.im, g1.im)};
+        const ffc l2 = phase(e2, imag, sS), l3 = phase(e3, imag, c3);
+        v[2 * a] = g0.re;
+        v[2 * a + 1] = g0.im;
+        v[6 + 2 * a] = g1.re;
+        v[6 + 2 * a + 1] = g1.im;
+        v[12 + 2 * a] = l2.re;
+        v[12 + 2 * a + 1] = l2.im;
+        v[18 + 2 * a] = l3.re;
+        v[18 + 2 * a + 1] = l3.im;
+    }
+    // sum over the eight hops: at each level a lane keeps one half of its numbers and adds the
+    // partner's same half; lane l ends with numbers 3 l .. 3 l + 2
+    ff w[12], x[6], y[3];
+#pragma unroll
+    for (int i = 0; i < 12; ++i) {
+        const bool up = l & 4;
+        w[i] = ff_add_u(sel(up, v[12 + i], v[i]), shfl_xor(sel(up, v[i], v[12 + i]), 4));
+    }
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        const bool up = l & 2;
+        x[i] = ff_add_u(sel(up, w[6 + i], w[i]), shfl_xor(sel(up, w[i], w[6 + i]), 2));
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const bool up = l & 1;
+        y[i] = ff_add_u(sel(up, x[3 + i], x[i]), shfl_xor(sel(up, x[i], x[3 + i]), 1));
+    }
+    if (!act) return;
+    const unsigned g5 = l & 4 ? NEG : 0u;  // gamma5 = diag(1, 1, -1, -1): numbers 12.. are spins 2, 3
+    const float* own = reinterpret_cast<const float*>(f);
+    const ff d = {P.diag32, P.diag_lo};
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int r = 3 * l + i, im = r & 1;
+        const int64_t e = entry<NAT>(site, r >> 1, P.vol);
+        const ff psi = {__ldg(own + 4 * e + im), __ldg(own + 4 * e + 2 + im)};
+        ff z = ff_add_u(ff_mul(psi, d), y[i]);
+        z = flip(two_sum(z.hi, z.lo), g5);
+        const int64_t o = rhs * P.stride_rhs + e;
+        if constexpr (OUT == FF_PAIRS) {
+            float* q = reinterpret_cast<float*>(out) + 4 * o;
+            q[im] = z.hi;
+            q[2 + im] = z.lo;
         } else {
-            g0 = {ff_scale2(g0.re, coef.hi), ff_scale2(g0.im, coef.hi)};
-            g1 = {ff_scale2(g1.re, coef.hi), ff_scale2(g1.im, coef.hi)};
-        }
-        acc[a] = cadd(acc[a], g0);
-        acc[3 + a] = cadd(acc[3 + a], g1);
-        // lower spins: S B^dag g
-        if constexpr (NU == 0) {  // B^dag g = (i g1, i g0)
-            acc[6 + a] = S > 0 ? cadd(acc[6 + a], mul_i(g1)) : csub(acc[6 + a], mul_i(g1));
-            acc[9 + a] = S > 0 ? cadd(acc[9 + a], mul_i(g0)) : csub(acc[9 + a], mul_i(g0));
-        } else if constexpr (NU == 1) {  // (g1, -g0)
-            acc[6 + a] = S > 0 ? cadd(acc[6 + a], g1) : csub(acc[6 + a], g1);
-            acc[9 + a] = S > 0 ? csub(acc[9 + a], g0) : cadd(acc[9 + a], g0);
-        } else if constexpr (NU == 2) {  // (i g0, -i g1)
-            acc[6 + a] = S > 0 ? cadd(acc[6 + a], mul_i(g0)) : csub(acc[6 + a], mul_i(g0));
-            acc[9 + a] = S > 0 ? cadd(acc[9 + a], mul_mi(g1)) : csub(acc[9 + a], mul_mi(g1));
-        } else {  // (g0, g1)
-            acc[6 + a] = S > 0 ? cadd(acc[6 + a], g0) : csub(acc[6 + a], g0);
-            acc[9 + a] = S > 0 ? cadd(acc[9 + a], g1) : csub(acc[9 + a], g1);
+            const double zd = f2d(z.hi) + f2d(z.lo);
+            double* q = reinterpret_cast<double*>(out) + 2 * o + im;
+            if constexpr (OUT == FF_DOUBLES) {
+                *q = zd;
+            } else {
+                const int sh = rhs / R.ncol, col = rhs - sh * R.ncol;
+                const double bv = __ldg(reinterpret_cast<const double*>(R.b + col * P.stride_rhs + e) + im);
+                const double xv = __ldg(reinterpret_cast<const double*>(R.x + o) + im);
+                *q = fma(__ldg(R.sigma + sh), xv, bv - zd);
+            }
         }
     }
 }
 
-__device__ __forceinline__ ff coef_ff(float hi, float lo, bool flip) { return flip ? ff{-hi, -lo} : ff{hi, lo}; }
-
-template <int NU>
-__device__ __forceinline__ void both_hops(ffc (&acc)[12], const float2* __restrict__ fh, const float2* __restrict__ fl,
-                                          const float4* __restrict__ Uf, int64_t site,
-                                          const int co[4], const StencilParams& P) {
-    int64_t stride = 1;
-#pragma unroll
-    for (int d = 0; d < NU; ++d) stride *= P.L[d];
-    const int L = P.L[NU];
-    int64_t fw = site + stride;
-    bool ffl = false;
-    if (co[NU] == L - 1) {
-        fw = site - (int64_t)(L - 1) * stride;
-        ffl = P.ap[NU];
-    }
-    int64_t bw = site - stride;
-    bool bfl = false;
-    if (co[NU] == 0) {
-        bw = site + (int64_t)(L - 1) * stride;
-        bfl = P.ap[NU];
-    }
-    hop<NU, -1>(acc, fh, fl, Uf, site, fw, coef_ff(P.cf32[NU], P.cf_lo[NU], ffl), P.vol);
-    hop<NU, +1>(acc, fh, fl, Uf, bw, bw, coef_ff(P.cb32[NU], P.cb_lo[NU], bfl), P.vol);
-}
-
-// Thread (x, y) of CTA b: site (b / ngrp) * SX + x, field (b % ngrp) * RB + y.  Capped at 128
-// registers (four CTAs of 128 threads per SM; as the compiler sizes it, 144 registers and three
-// CTAs ran 20 % slower at 10^4 despite a few spilled values).
-__global__ void __launch_bounds__(128, 4)
-    k_hw_ff(float2* __restrict__ oh, float2* __restrict__ ol, const float2* __restrict__ ih,
-            const float2* __restrict__ il, const float4* __restrict__ Uf, int nrhs,
-            StencilParams P, int ngrp) {
-    const int64_t tile = blockIdx.x / (unsigned)ngrp;
-    const int grp = (int)(blockIdx.x - tile * ngrp);
-    const int64_t site = tile * blockDim.x + threadIdx.x;
-    const int rhs = grp * blockDim.y + threadIdx.y;
-    if (site >= P.vol || rhs >= nrhs) return;
-    const float2* fh = ih + rhs * P.stride_rhs;
-    const float2* fl = il + rhs * P.stride_rhs;
-    int co[4];
-    {
-        const uint32_t s0 = (uint32_t)site;
-        const uint32_t q0 = P.div[0].div(s0);
-        co[0] = (int)(s0 - q0 * (uint32_t)P.L[0]);
-        const uint32_t q1 = P.div[1].div(q0);
-        co[1] = (int)(q0 - q1 * (uint32_t)P.L[1]);
-        const uint32_t q2 = P.div[2].div(q1);
-        co[2] = (int)(q1 - q2 * (uint32_t)P.L[2]);
-        co[3] = (int)q2;
-    }
-    ffc acc[12];
-    {
-        load_site(fh, fl, site, 2 * P.vol, acc);
-        const ff d = {P.diag32, P.diag_lo};
-#pragma unroll
-        for (int k = 0; k < 12; ++k) acc[k] = {ff_mul(acc[k].re, d), ff_mul(acc[k].im, d)};
-    }
-    both_hops<0>(acc, fh, fl, Uf, site, co, P);
-    both_hops<1>(acc, fh, fl, Uf, site, co, P);
-    both_hops<2>(acc, fh, fl, Uf, site, co, P);
-    both_hops<3>(acc, fh, fl, Uf, site, co, P);
-    float2* gh = oh + rhs * P.stride_rhs;
-    float2* gl = ol + rhs * P.stride_rhs;
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        const float g = k < 3 ? 1.f : -1.f;  // gamma5 = diag(1, 1, -1, -1): planes 3..5 hold spins 2, 3
-        const ff ar = two_sum(acc[2 * k].re.hi, acc[2 * k].re.lo), ai = two_sum(acc[2 * k].im.hi, acc[2 * k].im.lo);
-        const ff br = two_sum(acc[2 * k + 1].re.hi, acc[2 * k + 1].re.lo),
-                 bi = two_sum(acc[2 * k + 1].im.hi, acc[2 * k + 1].im.lo);
-        const ffc a = {ar, ai}, b = {br, bi};
-        *reinterpret_cast<float4*>(gh + k * 2 * P.vol + 2 * site) =
-            make_float4(g * a.re.hi, g * a.im.hi, g * b.re.hi, g * b.im.hi);
-        *reinterpret_cast<float4*>(gl + k * 2 * P.vol + 2 * site) =
-            make_float4(g * a.re.lo, g * a.im.lo, g * b.re.lo, g * b.im.lo);
-    }
-}
-
-// hi = fl(v), lo = fl(v - hi): v = hi + lo to about 2^-48 relative.
-__global__ void k_split_ff(const double2* __restrict__ in, float2* __restrict__ hi, float2* __restrict__ lo,
-                           int64_t count) {
+// complex128 -> float-float, elementwise
+__global__ void k_split_ff(const double2* __restrict__ in, float4* __restrict__ out, int64_t count) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
         const double2 v = in[i];
-        const float hx = (float)v.x, hy = (float)v.y;
-        hi[i] = make_float2(hx, hy);
-        lo[i] = make_float2((float)(v.x - (double)hx), (float)(v.y - (double)hy));
-    }
-}
-// out = hi + lo in FP64
-__global__ void k_join_ff(const float2* __restrict__ hi, const float2* __restrict__ lo, double2* __restrict__ out,
-                          int64_t count) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
-        const float2 h = hi[i], l = lo[i];
-        out[i] = make_double2((double)h.x + (double)l.x, (double)h.y + (double)l.y);
-    }
-}
-// r = b - (yh + yl) + sigma x, FP64 (the true residual of (A^2 - sigma) x = b with y = A^2 x)
-__global__ void k_residual_ff(double2* __restrict__ r, const double2* __restrict__ b, const float2* __restrict__ yh,
-                              const float2* __restrict__ yl, double sigma, const double2* __restrict__ x,
-                              int64_t count) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
-        const float2 h = yh[i], l = yl[i];
-        const double2 bv = b[i], xv = x[i];
-        r[i] = make_double2(bv.x - ((double)h.x + (double)l.x) + sigma * xv.x,
-                            bv.y - ((double)h.y + (double)l.y) + sigma * xv.y);
-    }
-}
-// links as float-float pairs, one 16-byte load per entry: (Re hi, Im hi, Re lo, Im lo) with
-// hi = U32 and lo = fl(U - U32)
-__global__ void k_links_ff(const double2* __restrict__ U, const float2* __restrict__ U32, float4* __restrict__ out,
-                           int64_t count) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
-        const double2 u = U[i];
-        const float2 h = U32[i];
-        out[i] = make_float4(h.x, h.y, (float)(u.x - (double)h.x), (float)(u.y - (double)h.y));
+        const float2 re = d2ff(v.x), im = d2ff(v.y);
+        out[i] = make_float4(re.x, im.x, re.y, im.y);
     }
 }
 
@@ -298,44 +274,39 @@ unsigned grid_of(int64_t count) {
     return (unsigned)(b < 152 * 16 ? (b > 0 ? b : 1) : 152 * 16);
 }
 
+template <FfOut OUT>
+cudaError_t launch_ff(void* out, const float4* in, const float4* Uf, int nrhs, const StencilParams& p, bool nat,
+                      const FfResidual& r, cudaStream_t st) {
+    if (nrhs <= 0 || p.vol <= 0) return cudaSuccess;
+    // one-warp CTAs (4 sites) while they fit in a few per SM, as in stencil_f64.cu
+    const int threads = p.vol * nrhs < 4 * 16 * 152 ? 32 : kMaxThreads, sites = threads / 8;
+    const int64_t blocks = (p.vol + sites - 1) / sites * nrhs;
+    if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+    if (nat)
+        k_hw_ff<true, OUT><<<(unsigned)blocks, threads, 0, st>>>(out, in, Uf, nrhs, p, r);
+    else
+        k_hw_ff<false, OUT><<<(unsigned)blocks, threads, 0, st>>>(out, in, Uf, nrhs, p, r);
+    count_launch();
+    return cudaGetLastError();
+}
+
 }  // namespace
 
-cudaError_t launch_hw_ff(float2* oh, float2* ol, const float2* ih, const float2* il, const float4* Uf, int nrhs,
-                         const StencilParams& p, cudaStream_t st) {
-    if (nrhs <= 0 || p.vol <= 0) return cudaSuccess;
-    // 64 sites x 2 fields per CTA (128 x 1 for one field); the fields of a site tile in
-    // consecutive CTAs share links in L2
-    const int rb = nrhs >= 2 ? 2 : 1, sx = 128 / rb;
-    const int ngrp = (nrhs + rb - 1) / rb;
-    const int64_t tiles = (p.vol + sx - 1) / sx;
-    if (tiles * ngrp > 0x7fffffffLL) return cudaErrorInvalidValue;
-    k_hw_ff<<<(unsigned)(tiles * ngrp), dim3(sx, rb), 0, st>>>(oh, ol, ih, il, Uf, nrhs, p, ngrp);
-    count_launch();
-    return cudaGetLastError();
+cudaError_t hw_ff(float4* out, const float4* in, const float4* Uf, int nrhs, const StencilParams& p, cudaStream_t st) {
+    return launch_ff<FF_PAIRS>(out, in, Uf, nrhs, p, false, {}, st);
+}
+cudaError_t hw_ff_doubles(double2* out, const float4* in, const float4* Uf, int nrhs, const StencilParams& p, bool nat,
+                          cudaStream_t st) {
+    return launch_ff<FF_DOUBLES>(out, in, Uf, nrhs, p, nat, {}, st);
+}
+cudaError_t hw_ff_residual(double2* r, const float4* in, const float4* Uf, int nrhs, const StencilParams& p,
+                           const double2* b, int ncol, const double2* x, const double* sigma, cudaStream_t st) {
+    return launch_ff<FF_RESIDUAL>(r, in, Uf, nrhs, p, false, {b, x, sigma, ncol}, st);
 }
 
-cudaError_t split_ff(const double2* in, float2* hi, float2* lo, int64_t count, cudaStream_t st) {
+cudaError_t split_ff(const double2* in, float4* out, int64_t count, cudaStream_t st) {
     if (count <= 0) return cudaSuccess;
-    k_split_ff<<<grid_of(count), 256, 0, st>>>(in, hi, lo, count);
-    count_launch();
-    return cudaGetLastError();
-}
-cudaError_t join_ff(const float2* hi, const float2* lo, double2* out, int64_t count, cudaStream_t st) {
-    if (count <= 0) return cudaSuccess;
-    k_join_ff<<<grid_of(count), 256, 0, st>>>(hi, lo, out, count);
-    count_launch();
-    return cudaGetLastError();
-}
-cudaError_t residual_ff(double2* r, const double2* b, const float2* yh, const float2* yl, double sigma,
-                        const double2* x, int64_t count, cudaStream_t st) {
-    if (count <= 0) return cudaSuccess;
-    k_residual_ff<<<grid_of(count), 256, 0, st>>>(r, b, yh, yl, sigma, x, count);
-    count_launch();
-    return cudaGetLastError();
-}
-cudaError_t links_ff(const double2* U, const float2* U32, float4* out, int64_t count, cudaStream_t st) {
-    if (count <= 0) return cudaSuccess;
-    k_links_ff<<<grid_of(count), 256, 0, st>>>(U, U32, out, count);
+    k_split_ff<<<grid_of(count), 256, 0, st>>>(in, out, count);
     count_launch();
     return cudaGetLastError();
 }

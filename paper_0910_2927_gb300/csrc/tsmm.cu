@@ -11,6 +11,7 @@
 // corrections of size ~1e-6 ||b~|| in refinement, where an FP32 relative error
 // is far below every tolerance; the FP64 form does not use these kernels.
 #include "blas.cuh"
+#include "cvt.cuh"
 
 namespace sgn {
 namespace {
@@ -23,7 +24,7 @@ constexpr int TN_JMAX = 64;
 __device__ __forceinline__ float2 ld_f2(const float2* p) { return __ldg(p); }
 __device__ __forceinline__ float2 ld_f2(const double2* p) {
     const double2 v = __ldg(p);
-    return make_float2((float)v.x, (float)v.y);
+    return make_float2(d2f(v.x), d2f(v.y));
 }
 
 // partial[((col * rstride + j) * nblk + b)] = sum over this CTA's rows of conj(V_j) W_col,
@@ -125,7 +126,7 @@ __global__ void __launch_bounds__(TN_THREADS)
         if (col < N) {
             double2* p = W + col * sw + row;
             const double2 a = *p;
-            *p = make_double2(a.x + alpha * (double)acc[q].x, a.y + alpha * (double)acc[q].y);
+            *p = make_double2(fma(alpha, f2d(acc[q].x), a.x), fma(alpha, f2d(acc[q].y), a.y));
         }
     }
 }
