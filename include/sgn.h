@@ -250,10 +250,9 @@ SGN_API int sgn_apply_shifts(sgn_ctx* ctx, const double* b, double* x, double* x
  * SGN_HW_ADJOINT) for nrhs fields.  precision SGN_PREC_FP64: complex128 fields;
  * SGN_PREC_MIXED: complex64 fields with the FP32 (or BF16, see
  * sgn_set_precision) links.  Device pointers; in and out must not overlap.
- * With SGN_HW_PACKED the stencil runs on the caller's packed fields directly (no
- * staging, one kernel); the FP64 stencil does so for natural-order fields too.  Other
- * natural-order fields are packed into a staging buffer, the stencil runs on the
- * packed copy and the result is unpacked.
+ * The stencils run on the caller's fields directly in either order (FP32 natural-order
+ * fields that are not 16-byte aligned go through packed copies; the float-float stencil
+ * makes a float-float copy of its input).
  * SGN_HW_FLOAT_FLOAT (SGN_PREC_FP64 only): complex128 in and out, the stencil in
  * float-float arithmetic (each real a sum of two floats, error-free transforms)
  * on the FP32 units, within about 1e-13 of the FP64 stencil; the mixed form

@@ -513,16 +513,18 @@ SGN_API int sgn_hw_apply(sgn_ctx* c, const void* in, void* out, int nrhs, int pr
     } else {
         const float2* pi = reinterpret_cast<const float2*>(in);
         float2* po = reinterpret_cast<float2*>(out);
-        if (!packed) {
+        const bool aligned = ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
+        const bool nat = !packed && aligned;  // else natural-order fields go through packed copies
+        if (!packed && !nat) {
             SGN_CHECK(dev_alloc(c, c->stage, 2 * nn * sizeof(float2)));
             float2* t = as<float2>(c->stage);
             SGN_CUDA(pack_fields<float2>(pi, t, c->vol, nrhs, c->work));
             pi = t;
             po = t + nn;
         }
-        SGN_CHECK(tune_stencil(c, stencil_prec32(c), nrhs, const_cast<float2*>(pi), po));
-        SGN_CUDA(apply_hw32(c, po, pi, nrhs, adjoint, nullptr, c->work));
-        if (!packed)
+        SGN_CHECK(tune_stencil(c, stencil_prec32(c), nrhs, const_cast<float2*>(pi), po, nat));
+        SGN_CUDA(apply_hw32(c, po, pi, nrhs, adjoint, nullptr, c->work, false, nat));
+        if (!packed && !nat)
             SGN_CUDA(unpack_fields<float2>(po, reinterpret_cast<float2*>(out), c->vol, nrhs, c->work));
     }
     SGN_CHECK(ses.close());

@@ -144,8 +144,7 @@ void fill_fp32_coefficients(StencilParams& p);
 cudaError_t apply_hw64(const sgn_ctx* c, double2* out, const double2* in, int ncol, bool adjoint, const int* skip,
                        cudaStream_t st);
 cudaError_t apply_hw32(const sgn_ctx* c, float2* out, const float2* in, int ncol, bool adjoint, const int* skip,
-                       cudaStream_t st,
-                       bool fp32_links = false);
+                       cudaStream_t st, bool fp32_links = false, bool nat = false);
 
 int solve(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int ncol, bool adjoint, bool no_a,
           sgn_report* rep,
@@ -155,8 +154,9 @@ inline int stencil_prec32(const sgn_ctx* c) {
     return c->link_storage == SGN_LINKS_BF16 ? 2 : c->link_storage == SGN_LINKS_FP16 ? 3 : 1;
 }
 // Pick the fastest FP32 stencil launch shape for (precision, ncol) by timing candidates
-// on the given buffers (ncol fields each); cached in the context.  Not during capture.
-int tune_stencil(sgn_ctx* c, int prec, int ncol, void* in, void* out);
+// on the given buffers (ncol fields each, packed or, with nat, natural); cached in the context,
+// one shape for both orders, so that they give the same bits.  Not during capture.
+int tune_stencil(sgn_ctx* c, int prec, int ncol, void* in, void* out, bool nat = false);
 // Dot products <a_c, b_c> of ncol pairs of FP64 fields (host result, FP64 reductions).
 int field_dots(sgn_ctx* c, const double2* a, const double2* b, int ncol, std::vector<std::complex<double>>& out);
 // overlap operator D_ov = 1 + gamma5 F(A) (overlap.cu), packed fields

@@ -99,7 +99,7 @@ cudaError_t pack_links(const double2* natural, double2* packed, int64_t vol, cud
 // ---------------------------------------------------------- kernel entry --
 // Stencil: out = H_W in for nrhs fields (packed layout).  Real = double or float; links in
 // double, float or bf16 (Link).  skip: per-field flags (non-zero: skip), may be null.
-// The FP64 stencil (stencil_f64.cu) also takes both fields in natural order (nat).
+// With nat, in and out are in natural order (FP32: 16-byte aligned).
 // Launch shape of the FP32 stencil: sx sites (x fastest) by rb threads per CTA, each thread nr
 // fields of its site (nr <= 3); {0, 0, 1} picks the default.
 // pipe = 1 selects the FP32 kernel that stages neighbour spinors through shared
@@ -115,12 +115,12 @@ struct StencilShape {
 cudaError_t launch_hw_f64(double2* out, const double2* in, const double2* U, int nrhs,
                           const StencilParams& p, const int* skip, cudaStream_t st, bool nat = false);
 cudaError_t launch_hw_f32(float2* out, const float2* in, const float2* U, int nrhs,
-                          const StencilParams& p, const int* skip, cudaStream_t st, StencilShape sh = {});
+                          const StencilParams& p, const int* skip, cudaStream_t st, StencilShape sh = {}, bool nat = false);
 cudaError_t launch_hw_f32_bf16links(float2* out, const float2* in, const __nv_bfloat162* U, int nrhs,
                                     const StencilParams& p, const int* skip, cudaStream_t st,
-                                    StencilShape sh = {});
+                                    StencilShape sh = {}, bool nat = false);
 cudaError_t launch_hw_f32_f16links(float2* out, const float2* in, const __half2* U, int nrhs,
-                                   const StencilParams& p, const int* skip, cudaStream_t st, StencilShape sh = {});
+                                   const StencilParams& p, const int* skip, cudaStream_t st, StencilShape sh = {}, bool nat = false);
 // Float-float stencil (stencil_ff.cu): fields and links as a float4 (Re hi, Im hi, Re lo, Im lo) per
 // complex number, in the place the complex128 number has (packed, or natural with nat); about
 // 1e-13 of the FP64 result.  The result as float-float, as complex128, or as the true residuals

@@ -54,28 +54,31 @@ struct Field;
 template <>
 struct Field<float> {
     using T = float2;
+    // NAT: natural order, entries 0..11 of a site contiguous (96 bytes)
+    template <bool NAT>
     static __device__ __forceinline__ void load(const float2* __restrict__ f, int64_t site, int64_t vol2,
                                                 Cx<float> p[12]) {
-        const float2* s = f + 2 * site;
+        const float2* s = f + (NAT ? 12 : 2) * site;
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-            const float4 v = __ldg(reinterpret_cast<const float4*>(s + k * vol2));
+            const float4 v = __ldg(reinterpret_cast<const float4*>(s + (NAT ? 2 * k : k * vol2)));
             p[2 * k] = {v.x, v.y};
             p[2 * k + 1] = {v.z, v.w};
         }
     }
     // CS: evict-first stores (see k_hw)
-    template <bool CS>
+    template <bool CS, bool NAT>
     static __device__ __forceinline__ void store(float2* __restrict__ f, int64_t site, int64_t vol2,
                                                  const Cx<float> p[12]) {
-        float2* s = f + 2 * site;
+        float2* s = f + (NAT ? 12 : 2) * site;
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
             const float4 v = make_float4(p[2 * k].x, p[2 * k].y, p[2 * k + 1].x, p[2 * k + 1].y);
+            float4* o = reinterpret_cast<float4*>(s + (NAT ? 2 * k : k * vol2));
             if constexpr (CS)
-                __stcs(reinterpret_cast<float4*>(s + k * vol2), v);
+                __stcs(o, v);
             else
-                *reinterpret_cast<float4*>(s + k * vol2) = v;
+                *o = v;
         }
     }
 };
@@ -190,7 +193,7 @@ __device__ __forceinline__ void hop_links(Cx<R> (&acc)[NR][12], const Cx<R> (&h0
 }
 
 
-template <class R, class LinkT, int NU, int S, int NR>
+template <class R, class LinkT, int NU, int S, int NR, bool NAT>
 __device__ __forceinline__ void hop(Cx<R> (&acc)[NR][12], const typename Field<R>::T* __restrict__ in,
                                     int64_t stride_rhs, const bool (&act)[NR], const LinkT* __restrict__ U,
                                     int64_t link_site, int64_t nb, R coef, int64_t vol) {
@@ -199,7 +202,7 @@ __device__ __forceinline__ void hop(Cx<R> (&acc)[NR][12], const typename Field<R
     for (int i = 0; i < NR; ++i) {
         Cx<R> p[12];
         if (act[i]) {
-            Field<R>::load(in + i * stride_rhs, nb, 2 * vol, p);
+            Field<R>::template load<NAT>(in + i * stride_rhs, nb, 2 * vol, p);
         } else {
 #pragma unroll
             for (int k = 0; k < 12; ++k) p[k] = {R(0), R(0)};
@@ -209,7 +212,7 @@ __device__ __forceinline__ void hop(Cx<R> (&acc)[NR][12], const typename Field<R
     hop_links<R, LinkT, NU, S, NR>(acc, h0, h1, U, link_site, coef, vol);
 }
 
-template <class R, class LinkT, int NU, int NR>
+template <class R, class LinkT, int NU, int NR, bool NAT>
 __device__ __forceinline__ void both_hops(Cx<R> (&acc)[NR][12], const typename Field<R>::T* __restrict__ in,
                                           const bool (&act)[NR], const LinkT* __restrict__ U, int64_t site,
                                           const int co[4], const StencilParams& P) {
@@ -230,8 +233,8 @@ __device__ __forceinline__ void both_hops(Cx<R> (&acc)[NR][12], const typename F
         bw = site + (int64_t)(L - 1) * stride;
         if (P.ap[NU]) cb = -cb;
     }
-    hop<R, LinkT, NU, -1, NR>(acc, in, P.stride_rhs, act, U, site, fw, cf, P.vol);
-    hop<R, LinkT, NU, +1, NR>(acc, in, P.stride_rhs, act, U, bw, bw, cb, P.vol);
+    hop<R, LinkT, NU, -1, NR, NAT>(acc, in, P.stride_rhs, act, U, site, fw, cf, P.vol);
+    hop<R, LinkT, NU, +1, NR, NAT>(acc, in, P.stride_rhs, act, U, bw, bw, cb, P.vol);
 }
 
 // CTA b of the 1D grid covers site tile b / ngrp and field group b % ngrp: the
@@ -242,7 +245,7 @@ __device__ __forceinline__ void both_hops(Cx<R> (&acc)[NR][12], const typename F
 // CS: evict-first stores, for field sets far larger than L2, where a spinor is
 // last read as the neighbour of a site one time slice away and the streaming
 // result would otherwise push it out of L2 first.
-template <class R, class LinkT, int NR, bool CS>
+template <class R, class LinkT, int NR, bool CS, bool NAT>
 __global__ void __launch_bounds__(NR == 1 ? 384 : 256)
     k_hw(typename Field<R>::T* __restrict__ out, const typename Field<R>::T* __restrict__ in,
          const LinkT* __restrict__ U, int nrhs, StencilParams P, const int* __restrict__ skip, int ngrp) {
@@ -277,7 +280,7 @@ __global__ void __launch_bounds__(NR == 1 ? 384 : 256)
 #pragma unroll
     for (int i = 0; i < NR; ++i) {
         if (act[i]) {
-            Field<R>::load(fin + i * P.stride_rhs, site, 2 * P.vol, acc[i]);
+            Field<R>::template load<NAT>(fin + i * P.stride_rhs, site, 2 * P.vol, acc[i]);
         } else {
 #pragma unroll
             for (int k = 0; k < 12; ++k) acc[i][k] = {R(0), R(0)};
@@ -285,17 +288,17 @@ __global__ void __launch_bounds__(NR == 1 ? 384 : 256)
 #pragma unroll
         for (int k = 0; k < 12; ++k) acc[i][k] = scale(acc[i][k], d);
     }
-    both_hops<R, LinkT, 0, NR>(acc, fin, act, U, site, co, P);
-    both_hops<R, LinkT, 1, NR>(acc, fin, act, U, site, co, P);
-    both_hops<R, LinkT, 2, NR>(acc, fin, act, U, site, co, P);
-    both_hops<R, LinkT, 3, NR>(acc, fin, act, U, site, co, P);
+    both_hops<R, LinkT, 0, NR, NAT>(acc, fin, act, U, site, co, P);
+    both_hops<R, LinkT, 1, NR, NAT>(acc, fin, act, U, site, co, P);
+    both_hops<R, LinkT, 2, NR, NAT>(acc, fin, act, U, site, co, P);
+    both_hops<R, LinkT, 3, NR, NAT>(acc, fin, act, U, site, co, P);
 #pragma unroll
     for (int i = 0; i < NR; ++i) {
         if (!act[i]) continue;
         // gamma5 = diag(1, 1, -1, -1)
 #pragma unroll
         for (int k = 6; k < 12; ++k) acc[i][k] = {-acc[i][k].x, -acc[i][k].y};
-        Field<R>::template store<CS>(out + (rhs0 + i) * P.stride_rhs, site, 2 * P.vol, acc[i]);
+        Field<R>::template store<CS, NAT>(out + (rhs0 + i) * P.stride_rhs, site, 2 * P.vol, acc[i]);
     }
 }
 
@@ -310,7 +313,7 @@ __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b
 __device__ __forceinline__ float2 f2s(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
-template <class LinkT, int NU, int S>
+template <class LinkT, int NU, int S, bool NAT>
 __device__ __forceinline__ void hop_x2(float2 (&ar)[12], float2 (&ai)[12], const float2* __restrict__ in,
                                        int64_t stride_rhs, const bool (&act)[2], const LinkT* __restrict__ U,
                                        int64_t link_site, int64_t nb, float coef, int64_t vol) {
@@ -318,13 +321,13 @@ __device__ __forceinline__ void hop_x2(float2 (&ar)[12], float2 (&ai)[12], const
     {
         Cx<float> pa[12], pb[12], ha0[3], ha1[3], hb0[3], hb1[3];
         if (act[0]) {
-            Field<float>::load(in, nb, 2 * vol, pa);
+            Field<float>::load<NAT>(in, nb, 2 * vol, pa);
         } else {
 #pragma unroll
             for (int k = 0; k < 12; ++k) pa[k] = {0.f, 0.f};
         }
         if (act[1]) {
-            Field<float>::load(in + stride_rhs, nb, 2 * vol, pb);
+            Field<float>::load<NAT>(in + stride_rhs, nb, 2 * vol, pb);
         } else {
 #pragma unroll
             for (int k = 0; k < 12; ++k) pb[k] = {0.f, 0.f};
@@ -404,7 +407,7 @@ __device__ __forceinline__ void hop_x2(float2 (&ar)[12], float2 (&ai)[12], const
     }
 }
 
-template <class LinkT, int NU>
+template <class LinkT, int NU, bool NAT>
 __device__ __forceinline__ void both_hops_x2(float2 (&ar)[12], float2 (&ai)[12], const float2* __restrict__ in,
                                              const bool (&act)[2], const LinkT* __restrict__ U, int64_t site,
                                              const int co[4], const StencilParams& P) {
@@ -424,12 +427,12 @@ __device__ __forceinline__ void both_hops_x2(float2 (&ar)[12], float2 (&ai)[12],
         bw = site + (int64_t)(L - 1) * stride;
         if (P.ap[NU]) cb = -cb;
     }
-    hop_x2<LinkT, NU, -1>(ar, ai, in, P.stride_rhs, act, U, site, fw, cf, P.vol);
-    hop_x2<LinkT, NU, +1>(ar, ai, in, P.stride_rhs, act, U, bw, bw, cb, P.vol);
+    hop_x2<LinkT, NU, -1, NAT>(ar, ai, in, P.stride_rhs, act, U, site, fw, cf, P.vol);
+    hop_x2<LinkT, NU, +1, NAT>(ar, ai, in, P.stride_rhs, act, U, bw, bw, cb, P.vol);
 }
 
 // One site, fields rhs0 and rhs0 + 1.
-template <class LinkT, bool CS>
+template <class LinkT, bool CS, bool NAT>
 __device__ __forceinline__ void x2_site(float2* __restrict__ out, const float2* __restrict__ in,
                                         const LinkT* __restrict__ U, int nrhs, const StencilParams& P,
                                         const int* __restrict__ skip, int64_t site, int rhs0) {
@@ -454,13 +457,13 @@ __device__ __forceinline__ void x2_site(float2* __restrict__ out, const float2* 
     {
         Cx<float> pa[12], pb[12];
         if (act[0]) {
-            Field<float>::load(fin, site, 2 * P.vol, pa);
+            Field<float>::load<NAT>(fin, site, 2 * P.vol, pa);
         } else {
 #pragma unroll
             for (int k = 0; k < 12; ++k) pa[k] = {0.f, 0.f};
         }
         if (act[1]) {
-            Field<float>::load(fin + P.stride_rhs, site, 2 * P.vol, pb);
+            Field<float>::load<NAT>(fin + P.stride_rhs, site, 2 * P.vol, pb);
         } else {
 #pragma unroll
             for (int k = 0; k < 12; ++k) pb[k] = {0.f, 0.f};
@@ -472,10 +475,10 @@ __device__ __forceinline__ void x2_site(float2* __restrict__ out, const float2* 
             ai[k] = f2(d * pa[k].y, d * pb[k].y);
         }
     }
-    both_hops_x2<LinkT, 0>(ar, ai, fin, act, U, site, co, P);
-    both_hops_x2<LinkT, 1>(ar, ai, fin, act, U, site, co, P);
-    both_hops_x2<LinkT, 2>(ar, ai, fin, act, U, site, co, P);
-    both_hops_x2<LinkT, 3>(ar, ai, fin, act, U, site, co, P);
+    both_hops_x2<LinkT, 0, NAT>(ar, ai, fin, act, U, site, co, P);
+    both_hops_x2<LinkT, 1, NAT>(ar, ai, fin, act, U, site, co, P);
+    both_hops_x2<LinkT, 2, NAT>(ar, ai, fin, act, U, site, co, P);
+    both_hops_x2<LinkT, 3, NAT>(ar, ai, fin, act, U, site, co, P);
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
         if (!act[i]) continue;
@@ -485,34 +488,34 @@ __device__ __forceinline__ void x2_site(float2* __restrict__ out, const float2* 
             const float g5 = k < 6 ? 1.f : -1.f;  // gamma5 = diag(1, 1, -1, -1)
             o[k] = {g5 * (i ? ar[k].y : ar[k].x), g5 * (i ? ai[k].y : ai[k].x)};
         }
-        Field<float>::template store<CS>(out + (rhs0 + i) * P.stride_rhs, site, 2 * P.vol, o);
+        Field<float>::template store<CS, NAT>(out + (rhs0 + i) * P.stride_rhs, site, 2 * P.vol, o);
     }
 }
 
 // Grid and thread layout as k_hw with NR = 2.
-template <class LinkT, bool CS>
+template <class LinkT, bool CS, bool NAT>
 __device__ __forceinline__ void hw_x2_body(float2* __restrict__ out, const float2* __restrict__ in,
                                            const LinkT* __restrict__ U, int nrhs, const StencilParams& P,
                                            const int* __restrict__ skip, int ngrp) {
     const int64_t tile = blockIdx.x / (unsigned)ngrp;
     const int grp = (int)(blockIdx.x - tile * ngrp);
-    x2_site<LinkT, CS>(out, in, U, nrhs, P, skip, tile * blockDim.x + threadIdx.x,
+    x2_site<LinkT, CS, NAT>(out, in, U, nrhs, P, skip, tile * blockDim.x + threadIdx.x,
                        (grp * blockDim.y + threadIdx.y) * 2);
 }
 
 // The kernel as the compiler sizes it (144 registers: 12 warps per SM), and capped at 128
 // registers (16 warps per SM, a few values spilled to local memory).
-template <class LinkT, bool CS>
+template <class LinkT, bool CS, bool NAT>
 __global__ void __launch_bounds__(256)
     k_hw_x2(float2* __restrict__ out, const float2* __restrict__ in, const LinkT* __restrict__ U, int nrhs,
             StencilParams P, const int* __restrict__ skip, int ngrp) {
-    hw_x2_body<LinkT, CS>(out, in, U, nrhs, P, skip, ngrp);
+    hw_x2_body<LinkT, CS, NAT>(out, in, U, nrhs, P, skip, ngrp);
 }
-template <class LinkT, bool CS>
+template <class LinkT, bool CS, bool NAT>
 __global__ void __launch_bounds__(256, 2)
     k_hw_x2_r128(float2* __restrict__ out, const float2* __restrict__ in, const LinkT* __restrict__ U, int nrhs,
                  StencilParams P, const int* __restrict__ skip, int ngrp) {
-    hw_x2_body<LinkT, CS>(out, in, U, nrhs, P, skip, ngrp);
+    hw_x2_body<LinkT, CS, NAT>(out, in, U, nrhs, P, skip, ngrp);
 }
 
 // ---- pipelined FP32 form ------------------------------------------------------
@@ -530,7 +533,7 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-template <int NR>
+template <int NR, bool NAT>
 struct PipeCtx {
     float4* sbuf;
     int nthr, tid;
@@ -545,9 +548,9 @@ struct PipeCtx {
 #pragma unroll
         for (int i = 0; i < NR; ++i) {
             if (!act[i]) continue;
-            const float2* src = in + i * stride_rhs + 2 * (int64_t)nb;
+            const float2* src = in + i * stride_rhs + (NAT ? 12 : 2) * (int64_t)nb;
 #pragma unroll
-            for (int k = 0; k < 6; ++k) cp_async16(slot(buf, i, k), src + k * vol2);
+            for (int k = 0; k < 6; ++k) cp_async16(slot(buf, i, k), src + (NAT ? 2 * k : k * vol2));
         }
     }
     __device__ __forceinline__ void read(int buf, int i, Cx<float> (&p)[12]) const {
@@ -603,8 +606,8 @@ __device__ __forceinline__ int stage_site(int site, const int (&co)[4], const St
 // Stage ST (1..8) = hop NU = (ST - 1) / 2, forward (S = -1) for odd ST; its data sit in
 // buffer ST % 2.  Before computing it, the next stage's copy is issued into the other
 // buffer, which the previous stage finished reading.
-template <class LinkT, int NR, int ST>
-__device__ __forceinline__ void pipe_stage(Cx<float> (&acc)[NR][12], const PipeCtx<NR>& pc,
+template <class LinkT, int NR, int ST, bool NAT>
+__device__ __forceinline__ void pipe_stage(Cx<float> (&acc)[NR][12], const PipeCtx<NR, NAT>& pc,
                                            const LinkT* __restrict__ U, int site, const int (&co)[4],
                                            const StencilParams& P) {
     constexpr int NU = (ST - 1) / 2;
@@ -630,7 +633,7 @@ __device__ __forceinline__ void pipe_stage(Cx<float> (&acc)[NR][12], const PipeC
     hop_links<float, LinkT, NU, S, NR>(acc, h0, h1, U, (ST % 2) ? site : nb, coef, P.vol);
 }
 
-template <class LinkT, int NR, bool CS>
+template <class LinkT, int NR, bool CS, bool NAT>
 __global__ void __launch_bounds__(256)
     k_hw_pipe(float2* __restrict__ out, const float2* __restrict__ in, const LinkT* __restrict__ U, int nrhs,
               StencilParams P, const int* __restrict__ skip, int ngrp) {
@@ -640,7 +643,7 @@ __global__ void __launch_bounds__(256)
     const int64_t site = tile * blockDim.x + threadIdx.x;
     const int rhs0 = (grp * blockDim.y + threadIdx.y) * NR;
     if (site >= P.vol || rhs0 >= nrhs) return;  // no barrier below: early exit is safe
-    PipeCtx<NR> pc;
+    PipeCtx<NR, NAT> pc;
     pc.sbuf = sbuf;
     pc.nthr = blockDim.x * blockDim.y;
     pc.tid = threadIdx.y * blockDim.x + threadIdx.x;
@@ -695,7 +698,7 @@ __global__ void __launch_bounds__(256)
         if (!pc.act[i]) continue;
 #pragma unroll
         for (int k = 6; k < 12; ++k) acc[i][k] = {-acc[i][k].x, -acc[i][k].y};
-        Field<float>::template store<CS>(out + (rhs0 + i) * P.stride_rhs, site, 2 * P.vol, acc[i]);
+        Field<float>::template store<CS, NAT>(out + (rhs0 + i) * P.stride_rhs, site, 2 * P.vol, acc[i]);
     }
 }
 
@@ -726,16 +729,22 @@ __device__ __forceinline__ void cmac_cs(Cx<float>& acc, Cx<float> u, Cx<float> v
     if constexpr (CONJ) cmac_conj(acc, u, v); else cmac(acc, u, v);
 }
 
-template <class LinkT, int NU, int S>
+// Offset of entry k = 3 spin + colour of a site.
+template <bool NAT>
+__device__ __forceinline__ int64_t entry_cs(int64_t site, int k, int64_t vol2) {
+    return NAT ? 12 * site + k : (int64_t)(k >> 1) * vol2 + 2 * site + (k & 1);
+}
+
+template <class LinkT, int NU, int S, bool NAT>
 __device__ __forceinline__ void hop_cs(Cx<float> (&acc)[4], const float2* __restrict__ fin, int64_t vol2,
                                        bool act, const LinkT* __restrict__ U, int64_t link_site, int64_t nb,
                                        float coef, int64_t vol, int a, int a1, int a2, int src1, int src2) {
-    // spins 0..3 of colour a at the neighbour: entry k = 3 s + a at (k/2) vol2 + 2 nb + k % 2
+    // spins 0..3 of colour a at the neighbour
     Cx<float> p[4];
 #pragma unroll
     for (int sp = 0; sp < 4; ++sp) {
         const int k = 3 * sp + a;
-        p[sp] = act ? ldc(fin + (int64_t)(k >> 1) * vol2 + 2 * nb + (k & 1)) : Cx<float>{0.f, 0.f};
+        p[sp] = act ? ldc(fin + entry_cs<NAT>(nb, k, vol2)) : Cx<float>{0.f, 0.f};
     }
     // this colour of the projected half-spinor h = psi_up + S B psi_dn
     const float sg = float(S);
@@ -789,7 +798,7 @@ __device__ __forceinline__ void hop_cs(Cx<float> (&acc)[4], const float2* __rest
     }
 }
 
-template <class LinkT, int NU>
+template <class LinkT, int NU, bool NAT>
 __device__ __forceinline__ void both_hops_cs(Cx<float> (&acc)[4], const float2* __restrict__ fin, bool act,
                                              const LinkT* __restrict__ U, int64_t site, const int co[4],
                                              const StencilParams& P, int a, int a1, int a2, int src1, int src2) {
@@ -809,11 +818,11 @@ __device__ __forceinline__ void both_hops_cs(Cx<float> (&acc)[4], const float2* 
         bw = site + (int64_t)(L - 1) * stride;
         if (P.ap[NU]) cb = -cb;
     }
-    hop_cs<LinkT, NU, -1>(acc, fin, 2 * P.vol, act, U, site, fw, cf, P.vol, a, a1, a2, src1, src2);
-    hop_cs<LinkT, NU, +1>(acc, fin, 2 * P.vol, act, U, bw, bw, cb, P.vol, a, a1, a2, src1, src2);
+    hop_cs<LinkT, NU, -1, NAT>(acc, fin, 2 * P.vol, act, U, site, fw, cf, P.vol, a, a1, a2, src1, src2);
+    hop_cs<LinkT, NU, +1, NAT>(acc, fin, 2 * P.vol, act, U, bw, bw, cb, P.vol, a, a1, a2, src1, src2);
 }
 
-template <class LinkT, bool CS>
+template <class LinkT, bool CS, bool NAT>
 __global__ void __launch_bounds__(256, 4)
     k_hw_cs(float2* __restrict__ out, const float2* __restrict__ in, const LinkT* __restrict__ U, int nrhs,
             StencilParams P, const int* __restrict__ skip, int ngrp, int fw) {
@@ -852,12 +861,12 @@ __global__ void __launch_bounds__(256, 4)
 #pragma unroll
     for (int sp = 0; sp < 4; ++sp) {
         const int k = 3 * sp + a;
-        acc[sp] = act ? scale(ldc(fin + (int64_t)(k >> 1) * vol2 + 2 * site + (k & 1)), d) : Cx<float>{0.f, 0.f};
+        acc[sp] = act ? scale(ldc(fin + entry_cs<NAT>(site, k, vol2)), d) : Cx<float>{0.f, 0.f};
     }
-    both_hops_cs<LinkT, 0>(acc, fin, act, U, site, co, P, a, a1, a2, src1, src2);
-    both_hops_cs<LinkT, 1>(acc, fin, act, U, site, co, P, a, a1, a2, src1, src2);
-    both_hops_cs<LinkT, 2>(acc, fin, act, U, site, co, P, a, a1, a2, src1, src2);
-    both_hops_cs<LinkT, 3>(acc, fin, act, U, site, co, P, a, a1, a2, src1, src2);
+    both_hops_cs<LinkT, 0, NAT>(acc, fin, act, U, site, co, P, a, a1, a2, src1, src2);
+    both_hops_cs<LinkT, 1, NAT>(acc, fin, act, U, site, co, P, a, a1, a2, src1, src2);
+    both_hops_cs<LinkT, 2, NAT>(acc, fin, act, U, site, co, P, a, a1, a2, src1, src2);
+    both_hops_cs<LinkT, 3, NAT>(acc, fin, act, U, site, co, P, a, a1, a2, src1, src2);
     if (!act) return;
     float2* fo = out + (int64_t)field * P.stride_rhs;
 #pragma unroll
@@ -865,7 +874,7 @@ __global__ void __launch_bounds__(256, 4)
         const int k = 3 * sp + a;
         const float g5 = sp < 2 ? 1.f : -1.f;  // gamma5 = diag(1, 1, -1, -1)
         const float2 v = make_float2(g5 * acc[sp].x, g5 * acc[sp].y);
-        float2* dst = fo + (int64_t)(k >> 1) * vol2 + 2 * site + (k & 1);
+        float2* dst = fo + entry_cs<NAT>(site, k, vol2);
         if constexpr (CS) __stcs(dst, v); else *dst = v;
     }
 }
@@ -904,7 +913,7 @@ __global__ void k_pack_links(const double2* __restrict__ in, double2* __restrict
     for (int e = 0; e < 36; ++e) out[e * vol + site] = in[site * 36 + e];
 }
 
-template <class R, class LinkT, int NR>
+template <class R, class LinkT, int NR, bool NAT>
 cudaError_t launch_nr(typename Field<R>::T* out, const typename Field<R>::T* in, const LinkT* U, int nrhs,
                       const StencilParams& p, const int* skip, cudaStream_t st, int sx, int rb) {
     const int groups = (nrhs + NR - 1) / NR;
@@ -914,14 +923,14 @@ cudaError_t launch_nr(typename Field<R>::T* out, const typename Field<R>::T* in,
     dim3 block(sx, rb);
     const bool cs = (double)nrhs * (double)p.vol * 12.0 * sizeof(typename Field<R>::T) > 256.0 * (1 << 20);
     if (cs)
-        k_hw<R, LinkT, NR, true><<<(unsigned)(tiles * ngrp), block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp);
+        k_hw<R, LinkT, NR, true, NAT><<<(unsigned)(tiles * ngrp), block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp);
     else
-        k_hw<R, LinkT, NR, false><<<(unsigned)(tiles * ngrp), block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp);
+        k_hw<R, LinkT, NR, false, NAT><<<(unsigned)(tiles * ngrp), block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp);
     count_launch();
     return cudaGetLastError();
 }
 
-template <class LinkT, int NR>
+template <class LinkT, int NR, bool NAT>
 cudaError_t launch_pipe(float2* out, const float2* in, const LinkT* U, int nrhs, const StencilParams& p,
                         const int* skip, cudaStream_t st, int sx, int rb) {
     const int groups = (nrhs + NR - 1) / NR;
@@ -938,22 +947,22 @@ cudaError_t launch_pipe(float2* out, const float2* in, const LinkT* U, int nrhs,
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     const int maxs = 2 * 2 * 6 * (int)sizeof(float4) * 256;
     if (!opted[cs][dev]) {
-        e = cs ? cudaFuncSetAttribute(k_hw_pipe<LinkT, NR, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs)
-               : cudaFuncSetAttribute(k_hw_pipe<LinkT, NR, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs);
+        e = cs ? cudaFuncSetAttribute(k_hw_pipe<LinkT, NR, true, NAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs)
+               : cudaFuncSetAttribute(k_hw_pipe<LinkT, NR, false, NAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs);
         if (e != cudaSuccess) return e;
         opted[cs][dev] = true;
     }
     dim3 block(sx, rb);
     if (cs)
-        k_hw_pipe<LinkT, NR, true><<<(unsigned)(tiles * ngrp), block, smem, st>>>(out, in, U, nrhs, p, skip, ngrp);
+        k_hw_pipe<LinkT, NR, true, NAT><<<(unsigned)(tiles * ngrp), block, smem, st>>>(out, in, U, nrhs, p, skip, ngrp);
     else
-        k_hw_pipe<LinkT, NR, false><<<(unsigned)(tiles * ngrp), block, smem, st>>>(out, in, U, nrhs, p, skip, ngrp);
+        k_hw_pipe<LinkT, NR, false, NAT><<<(unsigned)(tiles * ngrp), block, smem, st>>>(out, in, U, nrhs, p, skip, ngrp);
     count_launch();
     return cudaGetLastError();
 }
 
 // Colour-split kernel: CTA = 32 lanes x (sg site groups x fw fields) warps.
-template <class LinkT>
+template <class LinkT, bool NAT>
 cudaError_t launch_cs(float2* out, const float2* in, const LinkT* U, int nrhs, const StencilParams& p, const int* skip,
                       cudaStream_t st, int sg, int fw) {
     if (sg < 1 || fw < 1 || sg * fw > 8) return cudaErrorInvalidValue;
@@ -965,14 +974,14 @@ cudaError_t launch_cs(float2* out, const float2* in, const LinkT* U, int nrhs, c
     const bool cs = (double)nrhs * (double)p.vol * 12.0 * sizeof(float2) > 256.0 * (1 << 20);
     const unsigned grid = (unsigned)(tiles * ngrp);
     if (cs)
-        k_hw_cs<LinkT, true><<<grid, block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp, fw);
+        k_hw_cs<LinkT, true, NAT><<<grid, block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp, fw);
     else
-        k_hw_cs<LinkT, false><<<grid, block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp, fw);
+        k_hw_cs<LinkT, false, NAT><<<grid, block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp, fw);
     count_launch();
     return cudaGetLastError();
 }
 
-template <class LinkT, int MINB>
+template <class LinkT, int MINB, bool NAT>
 cudaError_t launch_x2(float2* out, const float2* in, const LinkT* U, int nrhs, const StencilParams& p,
                       const int* skip, cudaStream_t st, int sx, int rb) {
     const int groups = (nrhs + 1) / 2;
@@ -984,50 +993,50 @@ cudaError_t launch_x2(float2* out, const float2* in, const LinkT* U, int nrhs, c
     const unsigned grid = (unsigned)(tiles * ngrp);
     if (MINB == 2) {
         if (cs)
-            k_hw_x2_r128<LinkT, true><<<grid, block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp);
+            k_hw_x2_r128<LinkT, true, NAT><<<grid, block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp);
         else
-            k_hw_x2_r128<LinkT, false><<<grid, block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp);
+            k_hw_x2_r128<LinkT, false, NAT><<<grid, block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp);
     } else if (cs) {
-        k_hw_x2<LinkT, true><<<grid, block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp);
+        k_hw_x2<LinkT, true, NAT><<<grid, block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp);
     } else {
-        k_hw_x2<LinkT, false><<<grid, block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp);
+        k_hw_x2<LinkT, false, NAT><<<grid, block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp);
     }
     count_launch();
     return cudaGetLastError();
 }
 
-template <class R, class LinkT>
+template <class R, class LinkT, bool NAT>
 cudaError_t launch(typename Field<R>::T* out, const typename Field<R>::T* in, const LinkT* U, int nrhs,
                    const StencilParams& p, const int* skip, cudaStream_t st, StencilShape sh) {
     if (nrhs <= 0 || p.vol <= 0) return cudaSuccess;
     if (sh.pipe == 4) {  // the colour-split kernel: sx site groups of 10 sites, rb fields per CTA
         if (sh.nr != 1) return cudaErrorInvalidValue;
-        return launch_cs<LinkT>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
+        return launch_cs<LinkT, NAT>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
     }
     if (sh.pipe == 2 || sh.pipe == 3) {  // the paired kernel (3: capped at 128 registers)
         if (sh.sx % 32 != 0 || sh.rb < 1 || sh.sx * sh.rb > 256 || sh.nr != 2) return cudaErrorInvalidValue;
-        if (sh.pipe == 3) return launch_x2<LinkT, 2>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
-        return launch_x2<LinkT, 1>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
+        if (sh.pipe == 3) return launch_x2<LinkT, 2, NAT>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
+        return launch_x2<LinkT, 1, NAT>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
     }
     if (sh.pipe) {  // the pipelined kernel: 1 or 2 fields per thread, up to 256 threads per CTA
         if (sh.sx % 32 != 0 || sh.rb < 1 || sh.sx * sh.rb > 256 || sh.nr < 1 || sh.nr > 2)
             return cudaErrorInvalidValue;
-        if (sh.nr == 1) return launch_pipe<LinkT, 1>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
-        return launch_pipe<LinkT, 2>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
+        if (sh.nr == 1) return launch_pipe<LinkT, 1, NAT>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
+        return launch_pipe<LinkT, 2, NAT>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
     }
     if (sh.sx > 0 && sh.rb > 0) {  // a tuned shape: validate it against the kernel's launch bounds
         if (sh.sx % 32 != 0 || sh.nr < 1 || sh.nr > 3 || sh.sx * sh.rb > (sh.nr == 1 ? 384 : 256))
             return cudaErrorInvalidValue;
-        if (sh.nr == 2) return launch_nr<R, LinkT, 2>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
-        if (sh.nr == 3) return launch_nr<R, LinkT, 3>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
-        return launch_nr<R, LinkT, 1>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
+        if (sh.nr == 2) return launch_nr<R, LinkT, 2, NAT>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
+        if (sh.nr == 3) return launch_nr<R, LinkT, 3, NAT>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
+        return launch_nr<R, LinkT, 1, NAT>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
     }
     // default: one field per thread, up to 12 fields of a site tile per CTA
     int rb = nrhs <= 12 ? nrhs : 8;
     int sx = 256 / rb;
     sx = sx < 32 ? 32 : (sx / 32) * 32;
     if (sx * rb > 384) sx = 32;
-    return launch_nr<R, LinkT, 1>(out, in, U, nrhs, p, skip, st, sx, rb);
+    return launch_nr<R, LinkT, 1, NAT>(out, in, U, nrhs, p, skip, st, sx, rb);
 }
 
 }  // namespace
@@ -1062,16 +1071,22 @@ cudaError_t pack_links(const double2* natural, double2* packed, int64_t vol, cud
 }
 
 cudaError_t launch_hw_f32(float2* out, const float2* in, const float2* U, int nrhs, const StencilParams& p,
-                          const int* skip, cudaStream_t st, StencilShape sh) {
-    return launch<float, float2>(out, in, U, nrhs, p, skip, st, sh);
+                          const int* skip, cudaStream_t st, StencilShape sh,
+                          bool nat) {
+    if (nat) return launch<float, float2, true>(out, in, U, nrhs, p, skip, st, sh);
+    return launch<float, float2, false>(out, in, U, nrhs, p, skip, st, sh);
 }
 cudaError_t launch_hw_f32_bf16links(float2* out, const float2* in, const __nv_bfloat162* U, int nrhs,
-                                    const StencilParams& p, const int* skip, cudaStream_t st, StencilShape sh) {
-    return launch<float, __nv_bfloat162>(out, in, U, nrhs, p, skip, st, sh);
+                                    const StencilParams& p, const int* skip, cudaStream_t st, StencilShape sh,
+                          bool nat) {
+    if (nat) return launch<float, __nv_bfloat162, true>(out, in, U, nrhs, p, skip, st, sh);
+    return launch<float, __nv_bfloat162, false>(out, in, U, nrhs, p, skip, st, sh);
 }
 cudaError_t launch_hw_f32_f16links(float2* out, const float2* in, const __half2* U, int nrhs,
-                                   const StencilParams& p, const int* skip, cudaStream_t st, StencilShape sh) {
-    return launch<float, __half2>(out, in, U, nrhs, p, skip, st, sh);
+                                   const StencilParams& p, const int* skip, cudaStream_t st, StencilShape sh,
+                          bool nat) {
+    if (nat) return launch<float, __half2, true>(out, in, U, nrhs, p, skip, st, sh);
+    return launch<float, __half2, false>(out, in, U, nrhs, p, skip, st, sh);
 }
 
 }  // namespace sgn
