@@ -100,7 +100,7 @@ typedef struct {
     int cycles;           /* restart cycles of the multishift phase (max over columns) */
     int matvecs;          /* applications of H_W per column (max over columns) */
     int refine_rounds;    /* mixed form: refinement rounds */
-    int refine_cycles;    /* mixed form: restart cycles spent in refinement */
+    int refine_cycles;    /* mixed form: restart cycles and BiCGStab iterations spent in refinement */
     int breakdown;        /* 1 if some Arnoldi cycle met an invariant subspace */
     double res_est;       /* max over columns and shifts of |rho_i| ||r|| / ||b~|| */
     double err_est;       /* mixed form: estimated relative error of x after refinement */
@@ -183,11 +183,13 @@ SGN_API int sgn_set_formulation(sgn_ctx* ctx, int form);
  * makes sgn_apply return SGN_ERR_STATE.  Errors: SGN_ERR_ARG. */
 SGN_API int sgn_set_method(sgn_ctx* ctx, int method);
 
-/* Mixed form only (no counterpart in the paper, which works in FP64): the
- * restart length of the FP32 correction solves that bring each shifted
- * system's true FP64 residual below the tolerance (0: min(k, 16)), and how many
- * shifted systems one correction batch solves side by side (0: up to 10 nrhs,
- * bounded by memory).  Errors: SGN_ERR_ARG (k_refine > 64, max_batch > 4096). */
+/* Mixed form only (no counterpart in the paper, which works in FP64): the FP32
+ * correction solves that bring each shifted system's true FP64 residual below the
+ * tolerance.  k_refine = 0 (default): BiCGStab, and restarted FOM(min(k, 16)) for the
+ * systems it fails on; k_refine > 0: restarted FOM of that restart length.  max_batch:
+ * how many shifted systems one correction batch solves side by side (0: up to 10 nrhs,
+ * on small lattices all, bounded by memory).  Errors: SGN_ERR_ARG (k_refine > 64,
+ * max_batch > 4096). */
 SGN_API int sgn_set_refinement(sgn_ctx* ctx, int k_refine, int max_batch);
 
 /* LR deflation data of Sec. 4 (eq. (4.1)): m right eigenvectors R and left

@@ -1080,23 +1080,6 @@ __global__ void k_f64_to_f16(const double2* __restrict__ in, __half2* __restrict
     }
 }
 
-// r_j += sigma_j d_j - w_j for nb systems: r_j at r + roff[j] (complex128), w_j = A^2 d_j
-// in FP32 and d_j in FP64, both at j * n.
-__global__ void k_correct_residuals(double2* __restrict__ r, const long long* __restrict__ roff,
-                                    const double* __restrict__ sig, const float2* __restrict__ w,
-                                    const double2* __restrict__ d, int64_t n) {
-    const int j = blockIdx.y;
-    double2* rj = r + roff[j];
-    const double s = sig[j];
-    const float2* wj = w + (int64_t)j * n;
-    const double2* dj = d + (int64_t)j * n;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-        const double2 rv = rj[e], dv = dj[e];
-        const float2 wv = wj[e];
-        rj[e] = make_double2(rv.x - (double)wv.x + s * dv.x, rv.y - (double)wv.y + s * dv.y);
-    }
-}
-
 // y_f = a_f + beta gamma5 s_f for nfield packed complex128 fields of vol sites: gamma5 =
 // diag(1, 1, -1, -1) in spin negates spins 2 and 3, i.e. planes 3..5 of the packed
 // field, its second half.
@@ -1343,16 +1326,6 @@ cudaError_t gamma5_axpy(double2* y, const double2* a, const double2* s, double b
     const int64_t total = (int64_t)nfield * 12 * vol;
     if (total <= 0) return cudaSuccess;
     k_gamma5_axpy<<<grid_for(total), NT, 0, st>>>(y, a, s, beta, 6 * vol, total);
-    count_launch();
-    return cudaGetLastError();
-}
-
-cudaError_t correct_residuals(double2* r, const long long* roff, const double* sig, const float2* w,
-                              const double2* d, int64_t n, int nb, cudaStream_t st) {
-    if (nb < 1) return cudaSuccess;
-    if (nb > 65535) return cudaErrorInvalidValue;
-    unsigned gx = (unsigned)std::min<int64_t>((n + NT - 1) / NT, 1024);
-    k_correct_residuals<<<dim3(gx, nb), NT, 0, st>>>(r, roff, sig, w, d, n);
     count_launch();
     return cudaGetLastError();
 }

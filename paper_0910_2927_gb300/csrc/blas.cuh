@@ -192,10 +192,33 @@ cudaError_t combine_shifts(const DevState& S, int ncol, cudaStream_t st);
 cudaError_t gamma5_axpy(double2* y, const double2* a, const double2* s, double beta, int64_t vol, int nfield,
                         cudaStream_t st);
 
-// Refinement residual update r_j += sigma_j d_j - w_j (w_j = A^2 d_j in FP32) for nb
-// systems: r_j at r + roff[j], w_j and d_j at j * n.
-cudaError_t correct_residuals(double2* r, const long long* roff, const double* sig, const float2* w,
-                              const double2* d, int64_t n, int nb, cudaStream_t st);
+// BiCGStab correction solves of the refinement (bicgstab.cu): FP32 fields of ncol columns back to
+// back, FP64 scalars per column.
+enum BiStatus { BI_RUN = 0, BI_DONE = 1, BI_IDLE = 2, BI_FAILED = 3 };
+struct BiState {
+    float2 *r, *rt, *p, *w, *s, *t, *d;  // residual, shadow residual, direction, A^2 p, half step, A^2 s, solution
+    double2 *rho, *alpha, *omega, *beta;
+    double *lim, *rn0;    // ||r||^2 to reach, and of the start
+    const double* tol;    // relative residual to reach
+    const double* sigma;
+    int* done;            // BiStatus (non-zero: skip)
+    int* count;           // arrival counters of the sums
+    float* partial;
+    int64_t npk;          // packs of two complex numbers per column
+    int nblk, pkt;        // CTAs per column, packs per thread
+};
+void bi_shape(BiState& S, int64_t n, int ncol);
+size_t bi_partial_bytes(const BiState& S, int ncol);
+cudaError_t bi_init(const BiState& S, int ncol, const double2* src, const long long* off, int nb, cudaStream_t st);
+cudaError_t bi_v(const BiState& S, int ncol, cudaStream_t st);
+cudaError_t bi_s(const BiState& S, int ncol, cudaStream_t st);
+cudaError_t bi_t(const BiState& S, int ncol, cudaStream_t st);
+cudaError_t bi_x(const BiState& S, int ncol, cudaStream_t st);
+
+// x_j += d_j and r_j += sigma_j d_j - w_j (w_j = A^2 d_j) for nb systems: x_j, r_j at off[j], d_j
+// and w_j (FP32) at j n; with done, only systems marked BI_DONE.
+cudaError_t apply_corrections(double2* x, double2* r, const long long* off, const double* sig, const int* done,
+                              const float2* w, const float2* d, int64_t n, int nb, cudaStream_t st);
 
 // Tall-skinny products of a basis V (J <= 64 fields, stride sv) with N columns W
 // (complex128, stride sw): tsmm_tn writes the partials of V^dag W into rd (then

@@ -65,6 +65,21 @@ struct Engine {
     std::vector<std::pair<int, double>> tmarks;
 };
 
+// Workspace and captured iterations of the refinement's BiCGStab corrections for ncol columns.
+struct BiCg {
+    int ncol = 0;
+    DevBuf arena;
+    BiState S{};
+    double *tol = nullptr, *sigma = nullptr;
+    long long* off = nullptr;  // [ncol] offset of each system's x and r
+    int *err = nullptr, *cyc = nullptr;
+    int* h_done = nullptr;  // pinned: done[ncol], err, cyc
+    cudaGraphExec_t one = nullptr, loop = nullptr;
+    uint64_t one_key = 0, loop_key = 0;
+    long long kernels = 0;
+    bool loop_unavailable = false;
+};
+
 }  // namespace sgn
 
 struct sgn_ctx {
@@ -98,8 +113,8 @@ struct sgn_ctx {
     int link_storage = SGN_LINKS_FP32;
     int form = SGN_FORM_A2;  // Krylov space of the partial fractions (sgn_formulation)
     int method = SGN_METHOD_FOM;  // multishift FOM-LR or GMRES-LR (sgn_method)
-    int k_refine = 0;    // restart length of the mixed form's correction solves (0: min(k, 16))
-    int refine_batch = 0;  // shifted systems per correction batch (0: min(s nrhs, 4 nrhs), memory-bounded)
+    int k_refine = 0;    // restart length of FOM correction solves (0: BiCGStab, FOM(min(k, 16)) behind it)
+    int refine_batch = 0;  // shifted systems per correction batch (0: see solve_mixed)
 
     // deflation (R, L as n x m column blocks)
     int m = 0;
@@ -117,6 +132,8 @@ struct sgn_ctx {
 
     // engines keyed by configuration
     std::map<uint64_t, std::unique_ptr<sgn::Engine>> engines;
+    std::map<int, std::unique_ptr<sgn::BiCg>> bicg;  // by columns
+    sgn::DevBuf fom_d;  // FP64 corrections of the refinement's FOM solves
     // engine of the last FP64-form multishift solve (sgn_get_hessenberg reads its H_k)
     sgn::Engine* last_fp64 = nullptr;
     // scratch fields for apply (b copy, x accumulators, FP64 temporaries)

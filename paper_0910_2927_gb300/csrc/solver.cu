@@ -244,6 +244,22 @@ struct CycleArgs {
     bool op_a = false;        // Krylov space of A itself (the split form), else of A^2
 };
 
+// The operator as captured launches hold it: links and their storage, coefficients, boundary.
+uint64_t operator_key(const sgn_ctx* c) {
+    uint64_t h = 1469598103934665603ULL;
+    auto mixd = [&](double d) {
+        uint64_t u;
+        std::memcpy(&u, &d, 8);
+        h = mix(h, u);
+    };
+    for (const DevBuf* b : {&c->U64, &c->U32, &c->U16, &c->UH}) h = mix(h, (uint64_t)(uintptr_t)b->p);
+    h = mix(h, c->link_storage);
+    mixd(c->mu);
+    mixd(c->mass);
+    for (int d = 0; d < 4; ++d) h = mix(h, c->ap[d]);
+    return h;
+}
+
 uint64_t cycle_key(const sgn_ctx* c, const Engine& E, const CycleArgs& a) {
     uint64_t h = 1469598103934665603ULL;
     auto mixd = [&](double d) {
@@ -263,17 +279,9 @@ uint64_t cycle_key(const sgn_ctx* c, const Engine& E, const CycleArgs& a) {
     h = mix(h, a.xs_col);
     h = mix(h, a.gmres);
     h = mix(h, a.op_a);
-    h = mix(h, (uint64_t)(uintptr_t)c->U64.p);
-    h = mix(h, (uint64_t)(uintptr_t)c->U32.p);
-    h = mix(h, (uint64_t)(uintptr_t)c->U16.p);
-    h = mix(h, (uint64_t)(uintptr_t)c->UH.p);
-    h = mix(h, c->link_storage);
-    mixd(c->mu);
-    mixd(c->mass);
-    for (int d = 0; d < 4; ++d) h = mix(h, c->ap[d]);
     mixd(E.S.tol);
     h = mix(h, c->timing);
-    return h;
+    return mix(h, operator_key(c));
 }
 
 // Event pair around one launch of a timed kernel class (only while capturing a
@@ -581,6 +589,15 @@ void release_engines(sgn_ctx* c) {
         if (E.h_kk) cudaFreeHost(E.h_kk);
     }
     c->engines.clear();
+    for (auto& kv : c->bicg) {
+        BiCg& G = *kv.second;
+        if (G.one) cudaGraphExecDestroy(G.one);
+        if (G.loop) cudaGraphExecDestroy(G.loop);
+        dev_free(c, G.arena);
+        if (G.h_done) cudaFreeHost(G.h_done);
+    }
+    c->bicg.clear();
+    dev_free(c, c->fom_d);
     c->last_fp64 = nullptr;
 }
 
@@ -601,6 +618,82 @@ __global__ void k_loop_decide(cudaGraphConditionalHandle h, const int* __restric
         const bool stop = all || *err != 0 || cnum >= max_cycles;
         cudaGraphSetConditional(h, stop ? 0u : 1u);
     }
+}
+
+bool no_graph() {
+    static const bool v = [] {
+        const char* s = getenv("SGN_NO_GRAPH");
+        return s && s[0] == '1';
+    }();
+    return v;
+}
+bool host_loop() {
+    static const bool v = [] {
+        const char* s = getenv("SGN_HOST_LOOP");
+        return s && s[0] == '1';
+    }();
+    return v;
+}
+
+// The launches of body() on st as an executable graph; *kernels: how many there are.
+template <class F>
+cudaError_t capture_body(cudaStream_t st, F body, cudaGraphExec_t* out, long long* kernels) {
+    cudaGraph_t g = nullptr;
+    cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return e;
+    const long long before = g_launches;
+    const cudaError_t ce = body();
+    const cudaError_t ee = cudaStreamEndCapture(st, &g);
+    *kernels = g_launches - before;
+    g_launches = before;  // capturing launches nothing
+    e = ce != cudaSuccess ? ce : ee;
+    if (e == cudaSuccess) e = cudaGraphInstantiate(out, g, 0);
+    if (g) cudaGraphDestroy(g);
+    if (e != cudaSuccess) *out = nullptr;
+    return e;
+}
+
+// The same launches as the body of a device-side loop: a conditional WHILE node that repeats body()
+// and k_loop_decide until all ncol done flags or the error word are set, or max_cycles bodies ran.
+template <class F>
+cudaError_t capture_loop(cudaStream_t st, F body, const int* done, int ncol, const int* err, int* cyc, int max_cycles,
+                         cudaGraphExec_t* out) {
+    cudaGraph_t g = nullptr;
+    cudaGraphConditionalHandle h = 0;
+    cudaGraphNode_t node = nullptr;
+    cudaGraphNodeParams cp{};
+    cudaError_t e = cudaGraphCreate(&g, 0);
+    if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault);
+    if (e == cudaSuccess) {
+        cp.type = cudaGraphNodeTypeConditional;
+        cp.conditional.handle = h;
+        cp.conditional.type = cudaGraphCondTypeWhile;
+        cp.conditional.size = 1;
+        e = cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &cp);
+    }
+    if (e == cudaSuccess)
+        e = cudaStreamBeginCaptureToGraph(st, cp.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                          cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+        const long long before = g_launches;
+        cudaError_t ce = body();
+        if (ce == cudaSuccess) {
+            k_loop_decide<<<1, 32, 0, st>>>(h, done, ncol, err, cyc, max_cycles);
+            ce = cudaGetLastError();
+        }
+        g_launches = before;
+        cudaGraph_t cap = nullptr;
+        const cudaError_t ee = cudaStreamEndCapture(st, &cap);
+        e = ce != cudaSuccess ? ce : ee;
+    }
+    if (e == cudaSuccess) e = cudaGraphInstantiate(out, g, 0);
+    if (g) cudaGraphDestroy(g);
+    if (e != cudaSuccess) {
+        *out = nullptr;
+        cudaGetLastError();  // clear the refusal; the host loop takes over
+        if (debug_log()) fprintf(stderr, "[sgn] device-side loop unavailable: %s\n", cudaGetErrorString(e));
+    }
+    return e;
 }
 
 struct RunResult {
@@ -637,30 +730,14 @@ int run_engine(sgn_ctx* c, Engine& E, const CycleArgs& a, double tol, int max_cy
         cudaGraphExecDestroy(E.graph);
         E.graph = nullptr;
     }
-    static const bool no_graph = [] {
-        const char* s = getenv("SGN_NO_GRAPH");
-        return s && s[0] == '1';
-    }();
-    if (!E.graph && !no_graph) {
-        cudaGraph_t g = nullptr;
+    auto body = [&] {
         E.tmarks.clear();
-        SGN_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-        const long long before = g_launches;
-        cudaError_t ce = cycle<T>(c, E, a, st);
-        cudaError_t ee = cudaStreamEndCapture(st, &g);
-        E.graph_kernels = g_launches - before;
-        g_launches = before;  // capturing launches nothing
-        if (ce != cudaSuccess || ee != cudaSuccess) {
-            if (g) cudaGraphDestroy(g);
-            set_error(std::string("capturing the restart cycle failed: ") +
-                      cudaGetErrorString(ce != cudaSuccess ? ce : ee));
-            return SGN_ERR_CUDA;
-        }
-        cudaError_t ie = cudaGraphInstantiate(&E.graph, g, 0);
-        cudaGraphDestroy(g);
-        if (ie != cudaSuccess) {
-            E.graph = nullptr;
-            set_error(std::string("cudaGraphInstantiate: ") + cudaGetErrorString(ie));
+        return cycle<T>(c, E, a, st);
+    };
+    if (!E.graph && !no_graph()) {
+        const cudaError_t e = capture_body(st, body, &E.graph, &E.graph_kernels);
+        if (e != cudaSuccess) {
+            set_error(std::string("capturing the restart cycle failed: ") + cudaGetErrorString(e));
             return SGN_ERR_CUDA;
         }
         E.graph_key = key;
@@ -671,57 +748,16 @@ int run_engine(sgn_ctx* c, Engine& E, const CycleArgs& a, double tol, int max_cy
     // converged (no host round trip per cycle).  Not with per-kernel timing (event nodes
     // are not allowed inside a conditional body) or the per-cycle debug log; if the runtime
     // refuses the conditional node, the host loop below runs instead.
-    static const bool no_loop = [] {
-        const char* s = getenv("SGN_HOST_LOOP");
-        return s && s[0] == '1';
-    }();
-    if (E.graph && !c->timing && !debug_log() && !no_loop && !E.loop_unavailable) {
+    if (E.graph && !c->timing && !debug_log() && !host_loop() && !E.loop_unavailable) {
         const uint64_t lkey = mix(key, (uint64_t)max_cycles);
         if (E.loop && E.loop_key != lkey) {
             cudaGraphExecDestroy(E.loop);
             E.loop = nullptr;
         }
         if (!E.loop) {
-            cudaGraph_t g = nullptr;
-            cudaGraphConditionalHandle h = 0;
-            cudaGraphNode_t node = nullptr;
-            cudaGraphNodeParams cp{};
-            cudaError_t e = cudaGraphCreate(&g, 0);
-            if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault);
-            if (e == cudaSuccess) {
-                cp.type = cudaGraphNodeTypeConditional;
-                cp.conditional.handle = h;
-                cp.conditional.type = cudaGraphCondTypeWhile;
-                cp.conditional.size = 1;
-                e = cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &cp);
-            }
-            if (e == cudaSuccess) {
-                cudaGraph_t body = cp.conditional.phGraph_out[0];
-                e = cudaStreamBeginCaptureToGraph(st, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
-                if (e == cudaSuccess) {
-                    const long long before = g_launches;
-                    E.tmarks.clear();
-                    cudaError_t ce = cycle<T>(c, E, a, st);
-                    if (ce == cudaSuccess) {
-                        k_loop_decide<<<1, 32, 0, st>>>(h, E.S.done, ncol, E.S.err, E.cyc_dev, max_cycles);
-                        ce = cudaGetLastError();
-                    }
-                    g_launches = before;
-                    cudaGraph_t cap = nullptr;
-                    cudaError_t ee = cudaStreamEndCapture(st, &cap);
-                    e = ce != cudaSuccess ? ce : ee;
-                }
-            }
-            if (e == cudaSuccess) e = cudaGraphInstantiate(&E.loop, g, 0);
-            if (g) cudaGraphDestroy(g);
-            if (e != cudaSuccess) {
-                E.loop = nullptr;
-                E.loop_unavailable = true;
-                cudaGetLastError();  // clear the refusal; the host loop takes over
-                if (debug_log()) fprintf(stderr, "[sgn] device restart loop unavailable: %s\n", cudaGetErrorString(e));
-            } else {
-                E.loop_key = lkey;
-            }
+            E.loop_unavailable =
+                capture_loop(st, body, E.S.done, ncol, E.S.err, E.cyc_dev, max_cycles, &E.loop) != cudaSuccess;
+            E.loop_key = lkey;
         }
         if (E.loop) {
             SGN_CUDA(cudaMemsetAsync(E.cyc_dev, 0, sizeof(int), st));
@@ -754,8 +790,7 @@ int run_engine(sgn_ctx* c, Engine& E, const CycleArgs& a, double tol, int max_cy
             SGN_CUDA(cudaGraphLaunch(E.graph, st));
             count_launch(E.graph_kernels);
         } else {
-            E.tmarks.clear();
-            SGN_CUDA(cycle<T>(c, E, a, st));
+            SGN_CUDA(body());
         }
         SGN_CUDA(cudaMemcpyAsync(E.h_done, E.S.done, ncol * sizeof(int), cudaMemcpyDeviceToHost, st));
         SGN_CUDA(cudaMemcpyAsync(E.h_err, E.S.err, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -836,10 +871,128 @@ namespace {
 // FP64.  Phase 2 (iterative refinement, not part of the paper): the true
 // residual r_i = b~ - (A^2 - sigma_i) x_i of every shifted system is formed in
 // FP64; systems whose relative residual exceeds the tolerance get a correction
-// d_i from restarted FOM on (A^2 - sigma_i) d = (I - P) r_i, again FP32 basis
-// with FP64 scalars, batched one system per column; x_i += d_i.  Rounds repeat
+// d_i of (A^2 - sigma_i) d = (I - P) r_i, again FP32 fields with FP64 scalars, batched one
+// system per column, by BiCGStab (bicgstab.cu), or by restarted FOM where that fails or a
+// restart length was set (sgn_set_refinement); x_i += d_i.  Rounds repeat
 // until every true residual meets the tolerance that stops the FP64 form.
 constexpr size_t kRefineBudgetBytes = size_t(48) << 30;
+constexpr int kBiCap = 400;    // iterations of a BiCGStab solve
+constexpr int kBiUnroll = 2;   // iterations per body of its device loop
+constexpr double kBiFloor = 3e-6;  // relative residual a BiCGStab solve aims at, at best (FP32 fields)
+
+int get_bicg(sgn_ctx* c, int ncol, BiCg** out) {
+    auto it = c->bicg.find(ncol);
+    if (it != c->bicg.end()) {
+        *out = it->second.get();
+        return SGN_OK;
+    }
+    auto G = std::make_unique<BiCg>();
+    G->ncol = ncol;
+    BiState& S = G->S;
+    bi_shape(S, c->n, ncol);
+    const size_t nc = (size_t)ncol, field = align256(nc * c->n * sizeof(float2));
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        const size_t o = off;
+        off += align256(bytes);
+        return o;
+    };
+    size_t of[7], oc[4], od[4], oi[2];
+    for (size_t& o : of) o = take(field);
+    for (size_t& o : oc) o = take(nc * sizeof(double2));
+    for (size_t& o : od) o = take(nc * sizeof(double));
+    const size_t ooff = take(nc * sizeof(long long));
+    for (size_t& o : oi) o = take(nc * sizeof(int));
+    const size_t oe = take(2 * sizeof(int)), op = take(bi_partial_bytes(S, ncol));
+    SGN_CHECK(dev_alloc(c, G->arena, off));
+    char* b = reinterpret_cast<char*>(G->arena.p);
+    float2** fields[7] = {&S.r, &S.rt, &S.p, &S.w, &S.s, &S.t, &S.d};
+    for (int i = 0; i < 7; ++i) *fields[i] = reinterpret_cast<float2*>(b + of[i]);
+    double2** coefs[4] = {&S.rho, &S.alpha, &S.omega, &S.beta};
+    for (int i = 0; i < 4; ++i) *coefs[i] = reinterpret_cast<double2*>(b + oc[i]);
+    S.lim = reinterpret_cast<double*>(b + od[0]);
+    S.rn0 = reinterpret_cast<double*>(b + od[1]);
+    S.tol = G->tol = reinterpret_cast<double*>(b + od[2]);
+    S.sigma = G->sigma = reinterpret_cast<double*>(b + od[3]);
+    G->off = reinterpret_cast<long long*>(b + ooff);
+    S.done = reinterpret_cast<int*>(b + oi[0]);
+    S.count = reinterpret_cast<int*>(b + oi[1]);
+    G->err = reinterpret_cast<int*>(b + oe);
+    G->cyc = G->err + 1;
+    S.partial = reinterpret_cast<float*>(b + op);
+    // zero the whole arena once so no kernel ever reads uninitialised memory
+    SGN_CUDA(cudaMemsetAsync(G->arena.p, 0, off, c->work));
+    SGN_CUDA(cudaHostAlloc(&G->h_done, (nc + 1) * sizeof(int), cudaHostAllocDefault));
+    *out = G.get();
+    c->bicg[ncol] = std::move(G);
+    return SGN_OK;
+}
+
+// Iterate until every column is done or failed, or kBiCap iterations; h_done holds the columns'
+// status after it, *iters the iterations run.
+int run_bicg(sgn_ctx* c, BiCg& G, bool adjoint, int max_iters, int* iters) {
+    cudaStream_t st = c->work;
+    const BiState& S = G.S;
+    const int nc = G.ncol, cap = std::max(1, max_iters / kBiUnroll);
+    auto body = [&]() -> cudaError_t {
+        for (int u = 0; u < kBiUnroll; ++u) {
+            // FP32 links always: solved on 16-bit ones, a correction gains little on the true residual
+            // and leaves its error in the smooth modes (10^4 at tol 1e-10: three rounds on FP16 links,
+            // six on BF16 ones)
+            CU(apply_hw32(c, S.t, S.p, nc, adjoint, S.done, st, true));
+            CU(apply_hw32(c, S.w, S.t, nc, adjoint, S.done, st, true));
+            CU(bi_v(S, nc, st));
+            CU(bi_s(S, nc, st));
+            CU(apply_hw32(c, S.r, S.s, nc, adjoint, S.done, st, true));  // r is free until k_bi_x writes it
+            CU(apply_hw32(c, S.t, S.r, nc, adjoint, S.done, st, true));
+            CU(bi_t(S, nc, st));
+            CU(bi_x(S, nc, st));
+        }
+        return cudaSuccess;
+    };
+    const uint64_t key = mix(operator_key(c), adjoint), lkey = mix(key, cap);
+    const bool dev = !c->timing && !debug_log() && !host_loop() && !no_graph() && !G.loop_unavailable;
+    int ran = 0;
+    SGN_CUDA(cudaMemsetAsync(G.err, 0, 2 * sizeof(int), st));
+    if (dev && (!G.loop || G.loop_key != lkey)) {
+        if (G.loop) cudaGraphExecDestroy(G.loop);
+        G.loop = nullptr;
+        const long long before = g_launches;
+        const cudaError_t e = capture_loop(st, body, S.done, nc, G.err, G.cyc, cap, &G.loop);
+        g_launches = before;
+        G.loop_unavailable = e != cudaSuccess;
+        G.loop_key = lkey;
+    }
+    if (dev && G.loop) {
+        SGN_CUDA(cudaGraphLaunch(G.loop, st));
+        SGN_CUDA(cudaMemcpyAsync(G.h_done, S.done, nc * sizeof(int), cudaMemcpyDeviceToHost, st));
+        SGN_CUDA(cudaMemcpyAsync(G.h_done + nc, G.cyc, sizeof(int), cudaMemcpyDeviceToHost, st));
+        SGN_CUDA(cudaStreamSynchronize(st));
+        ran = G.h_done[nc];
+        count_launch((8LL * kBiUnroll + 1) * ran);
+    } else {
+        if (!no_graph() && (!G.one || G.one_key != key)) {
+            if (G.one) cudaGraphExecDestroy(G.one);
+            SGN_CUDA(capture_body(st, body, &G.one, &G.kernels));
+            G.one_key = key;
+        }
+        bool all = false;
+        for (; ran < cap && !all; ++ran) {
+            if (no_graph()) {
+                SGN_CUDA(body());
+            } else {
+                SGN_CUDA(cudaGraphLaunch(G.one, st));
+                count_launch(G.kernels);
+            }
+            SGN_CUDA(cudaMemcpyAsync(G.h_done, S.done, nc * sizeof(int), cudaMemcpyDeviceToHost, st));
+            SGN_CUDA(cudaStreamSynchronize(st));
+            all = true;
+            for (int i = 0; i < nc; ++i) all = all && G.h_done[i] != BI_RUN;
+        }
+    }
+    *iters = ran * kBiUnroll;
+    return SGN_OK;
+}
 
 int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int ncol, bool adjoint, bool no_a,
                 sgn_report* rep) {
@@ -850,18 +1003,28 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
     const int m = c->m;
     Engine* E = nullptr;
     SGN_CHECK(get_engine(c, ncol, k, s, SGN_PREC_MIXED, &E));
-    // refinement batch: one shifted system per column, bounded by memory.  The
-    // corrections only have to gain a factor tol / (FP32 floor ~1e-6) and most of
-    // them converge in a few steps, so they restart sooner than the multishift
-    // phase: a cycle of the engine always runs all its k_refine steps.
+    // Refinement batches: one shifted system per column, bounded by memory.  BiCGStab: all systems
+    // together while they are few (small lattices are bound by launches), else 10 ncol, so that the
+    // quickly converging half (shifts far from the spectrum) does not idle along with the slow one.
+    const int nall = s * ncol;  // every (shift, column) pair as one column of [i][col][n]
+    const bool shortrec = c->k_refine == 0;
     const int k1 = c->k_refine > 0 ? c->k_refine : std::min(k, 16);
-    const size_t per_col = (size_t)(k1 + 4) * n * sizeof(float2) + (size_t)n * sizeof(double2);
-    size_t bmax = c->refine_batch > 0 ? (size_t)c->refine_batch : (size_t)10 * ncol;
-    int B = (int)std::min<size_t>({(size_t)s * ncol, bmax, std::max<size_t>(1, kRefineBudgetBytes / per_col)});
+    auto batch = [&](size_t fields_per_col) {
+        const size_t per_col = fields_per_col * n * sizeof(float2);
+        const size_t bmax = c->refine_batch > 0                               ? (size_t)c->refine_batch
+                            : shortrec && (size_t)nall * n <= (size_t)4 << 20 ? (size_t)nall
+                                                                              : (size_t)10 * ncol;
+        return (int)std::min<size_t>({(size_t)nall, bmax, std::max<size_t>(1, kRefineBudgetBytes / per_col)});
+    };
+    // FOM corrections restart sooner than the multishift phase: they only have to gain a factor
+    // tol / (FP32 floor ~1e-6), and a cycle of the engine always runs all its k1 steps
+    const int B = batch(k1 + 6);  // columns of a FOM batch
     Engine* E1 = nullptr;
-    SGN_CHECK(get_engine(c, B, k1, 1, SGN_PREC_MIXED, &E1));
+    if (!shortrec) SGN_CHECK(get_engine(c, B, k1, 1, SGN_PREC_MIXED, &E1));
+    BiCg* G = nullptr;
+    if (shortrec) SGN_CHECK(get_bicg(c, batch(7), &G));
 
-    // io: xs (s ncol) | r0, bt, xP (ncol each) | float-float x, A x | d (B) | omega table | FP64 partials
+    // io: xs (s ncol) | r0, bt, xP (ncol each) | float-float x, A x | rs (s ncol) | omega table | FP64 partials
     const size_t field = (size_t)n * sizeof(double2);
     const int nblk64 = dot_blocks<double2>(n, ncol);
     const int rs64 = ((std::max(m, s) + 2) + 7) & ~7;
@@ -876,9 +1039,8 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
     // float-float copies of x_i and A x_i: of as many shifts as it takes to fill the chip
     const int fsh = (int)std::min<int64_t>(s, std::max<int64_t>(1, (int64_t)131072 / (c->vol * ncol)));
     size_t o_t = take(field * ncol * fsh), o_u = take(field * ncol * fsh);
-    size_t o_d = take(field * B);
     size_t o_rs = take(field * ncol * s);
-    const int ncmax = std::max({ncol, B, s * ncol});
+    const int ncmax = std::max({ncol, B, nall});
     size_t o_om = take(sizeof(double2) * ncol * rs64), o_sig = take(sizeof(double) * s);
     size_t o_red = take(sizeof(double2) * ncmax * rs64);
     size_t o_part = take(sizeof(double2) * (size_t)ncmax * rs64 * nblk64);
@@ -893,7 +1055,6 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
     float4* xf = reinterpret_cast<float4*>(io + o_t);
     float4* tf = reinterpret_cast<float4*>(io + o_u);
     double* sig_dev = reinterpret_cast<double*>(io + o_sig);
-    double2* d = reinterpret_cast<double2*>(io + o_d);
     double2* rsd = reinterpret_cast<double2*>(io + o_rs);  // true residuals r_i, [i][col][n]
     double2* omtab = reinterpret_cast<double2*>(io + o_om);
     long long* roff_dev = reinterpret_cast<long long*>(io + o_roff);
@@ -944,7 +1105,8 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
     SGN_CUDA(convert_f64_to_f32(bt, reinterpret_cast<float2*>(E->V), (int64_t)ncol * n, st));
     const int p32 = stencil_prec32(c);
     SGN_CHECK(tune_stencil(c, p32, ncol, E->V, E->t));
-    SGN_CHECK(tune_stencil(c, p32, B, E1->V, E1->t));
+    if (shortrec) SGN_CHECK(tune_stencil(c, 1, G->ncol, G->S.p, G->S.t));
+    if (!shortrec) SGN_CHECK(tune_stencil(c, p32, B, E1->V, E1->t));
 
     CycleArgs a;
     a.adjoint = adjoint;
@@ -977,40 +1139,158 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
         for (int col = 0; col < ncol; ++col) bnorm[col] = std::sqrt(h[(size_t)col * rs64].x);
     }
 
-    CycleArgs a1;
-    a1.adjoint = adjoint;
-    a1.L = Lb32;
-    a1.R = Rb32;
-    a1.m = m;
-    a1.project = c->project;
-    a1.xs = d;
-    a1.xs_shift = (int64_t)B * n;
-    a1.xs_col = n;
+    const double rtol = c->tol;
+    const int max_rounds = 8;
+    std::vector<double2> hall((size_t)nall * rs64);
+    // a system to correct: its position in [i][col] order and its relative true residual
+    struct System {
+        int at;
+        double rel;
+    };
+
     // Correction solves by restarted FOM (Galerkin, like the multishift phase); a batch whose
     // FOM does not converge within kFomCap cycles, or meets a non-finite value, is solved again
     // from the same residuals with minimal-residual (GMRES) restarts.  Restarted FOM on a single
     // strongly non-normal shifted system can diverge (at mu = 1 its residual grew without bound
-    // over 1,800 cycles); GMRES cannot.  GMRES corrections leave residuals along unrelated
+    // over 1,800 cycles); GMRES cannot.  GMRES corrections leave their residuals along unrelated
     // directions, whose errors add up less favourably: the retry aims at a third of the target
     // (on the 10^4 workload at tol 1e-8, GMRES corrections gave a relative error of x of 1.4e-8
     // at the target and 4.7e-9 at a third of it; FOM corrections 2.9e-9 at the target).
     constexpr int kFomCap = 300;
-    const double rtol = c->tol;
-    const int max_rounds = 8;
-    std::vector<double> sig1(B), om1(B, 1.0);
-    const int nall = s * ncol;  // every (shift, column) pair as one column of [i][col][n]
-    std::vector<double2> hall((size_t)nall * rs64);
-    std::vector<long long> roff(B);
-    std::vector<double> rsig(B);
+    auto fom_corrections = [&](const std::vector<System>& todo) -> int {
+        if (!E1) {
+            SGN_CHECK(get_engine(c, B, k1, 1, SGN_PREC_MIXED, &E1));
+            SGN_CHECK(tune_stencil(c, p32, B, E1->V, E1->t));
+        }
+        SGN_CHECK(dev_alloc(c, c->fom_d, field * B));
+        double2* d = as<double2>(c->fom_d);
+        CycleArgs a1;
+        a1.adjoint = adjoint;
+        a1.L = Lb32;
+        a1.R = Rb32;
+        a1.m = m;
+        a1.project = c->project;
+        a1.xs = d;
+        a1.xs_shift = (int64_t)B * n;
+        a1.xs_col = n;
+        std::vector<double> sig1(B), om1(B, 1.0), rsig(B);
+        std::vector<long long> roff(B);
+        for (size_t t0 = 0; t0 < todo.size(); t0 += B) {
+            const int nb = (int)std::min<size_t>(B, todo.size() - t0);
+            float2* V0 = reinterpret_cast<float2*>(E1->V);
+            for (int j = 0; j < B; ++j) sig1[j] = j < nb ? c->sigma[todo[t0 + j].at / ncol] : c->sigma[0];
+            SGN_CHECK(fill_shift_tables(c, *E1, sig1.data(), om1.data()));
+            // the correction needs to reduce the worst residual of the batch to a third
+            // of the tolerance, not further (FP32 bases reach about 1e-6 at best)
+            double brel = 0;
+            for (int j = 0; j < nb; ++j) brel = std::max(brel, todo[t0 + j].rel);
+            int st1 = SGN_OK;
+            RunResult r1;
+            for (int attempt = 0; attempt < 2; ++attempt) {
+                a1.gmres = attempt == 1;
+                SGN_CUDA(cudaMemsetAsync(V0, 0, sizeof(float2) * (size_t)B * n, st));
+                for (int j = 0; j < nb; ++j)
+                    SGN_CUDA(convert_f64_to_f32(rsd + (size_t)todo[t0 + j].at * n, V0 + (size_t)j * n, n, st));
+                SGN_CUDA(cudaMemsetAsync(d, 0, field * B, st));
+                const double inner = std::min(0.1, std::max(1e-5, rtol / ((a1.gmres ? 9.0 : 3.0) * brel)));
+                st1 = run_engine<float2>(c, *E1, a1, inner, a1.gmres ? c->max_cycles : std::min(c->max_cycles, kFomCap),
+                                         &r1);
+                if (debug_log())
+                    fprintf(stderr,
+                            "[sgn mixed]   batch at %zu (%d systems, %s): inner tol %.1e status %d cycles %d "
+                            "resmax %.3e\n",
+                            t0, nb, a1.gmres ? "GMRES" : "FOM", inner, st1, r1.cycles, r1.resmax);
+                ref_cycles += r1.cycles;
+                const bool fom_failed = !a1.gmres && (st1 == SGN_ERR_NONFINITE || st1 == SGN_ERR_BREAKDOWN ||
+                                                      (st1 == SGN_OK && !r1.converged));
+                if (!fom_failed) break;
+                SGN_CUDA(cudaMemsetAsync(E1->S.err, 0, sizeof(int), st));
+            }
+            if (st1 != SGN_OK) return st1;
+            // x_i += d_i, r_i -= (A^2 - sigma_i) d_i: A^2 d in FP32 on the engine's fields.  FP32 links
+            // even when the solves run on 16-bit ones: the carried residual must see the true
+            // operator, not the one the corrections were solved with
+            float2 *d32 = reinterpret_cast<float2*>(E1->w), *t32 = reinterpret_cast<float2*>(E1->t);
+            SGN_CUDA(convert_f64_to_f32(d, d32, (int64_t)nb * n, st));
+            SGN_CUDA(apply_hw32(c, t32, d32, nb, adjoint, nullptr, st, true));
+            SGN_CUDA(apply_hw32(c, V0, t32, nb, adjoint, nullptr, st, true));
+            for (int j = 0; j < nb; ++j) {
+                roff[j] = (long long)todo[t0 + j].at * n;
+                rsig[j] = c->sigma[todo[t0 + j].at / ncol];
+            }
+            SGN_CUDA(cudaMemcpyAsync(roff_dev, roff.data(), sizeof(long long) * nb, cudaMemcpyHostToDevice, st));
+            SGN_CUDA(cudaMemcpyAsync(rsig_dev, rsig.data(), sizeof(double) * nb, cudaMemcpyHostToDevice, st));
+            SGN_CUDA(apply_corrections(xs, rsd, roff_dev, rsig_dev, nullptr, V0, d32, n, nb, st));
+        }
+        return SGN_OK;
+    };
+
+    // A system once corrected is done below rtol * accept, six times its correction's aim: the first
+    // correction of a solution from 16-bit links may leave it anywhere below rtol.
+    std::vector<double> accept(nall, 1.0);
+    // Correction solves by BiCGStab, each system to its own residual; the systems it gave up on are
+    // left as they were and returned in `failed`.  What a residual r_i leaves in x is about
+    // omega_i r_i / (spectrum - sigma_i), largest for the smallest shifts, which are also the slow
+    // ones: the systems aim at tol / margin_i, margin_i from 36 for the largest omega / |sigma| down
+    // with its fourth root (at a margin of 9 for all, the error of x on the 10^4 workload was 2.3
+    // times that of FOM corrections).
+    std::vector<double> margin(s);
+    {
+        double wmax = 0;
+        for (int i = 0; i < s; ++i) {
+            margin[i] = std::abs(c->omega[i]) / std::max(std::abs(c->sigma[i]), 1e-300);
+            if (std::isfinite(margin[i])) wmax = std::max(wmax, margin[i]);
+        }
+        for (double& w : margin)
+            w = wmax > 0 && std::isfinite(w) ? std::max(4.0, 36.0 * std::sqrt(std::sqrt(w / wmax))) : 36.0;
+    }
+    auto bicg_corrections = [&](const std::vector<System>& todo, std::vector<System>& failed) -> int {
+        const int nc = G->ncol;
+        std::vector<double> sg(nc, -1.0), tl(nc, 1.0);
+        std::vector<long long> off_h(nc, 0);
+        for (size_t t0 = 0; t0 < todo.size(); t0 += nc) {
+            const int nb = (int)std::min<size_t>(nc, todo.size() - t0);
+            for (int j = 0; j < nb; ++j) {
+                const System& y = todo[t0 + j];
+                sg[j] = c->sigma[y.at / ncol];
+                tl[j] = std::min(0.1, std::max(kBiFloor, rtol / (margin[y.at / ncol] * y.rel)));
+                off_h[j] = (long long)y.at * n;
+            }
+            SGN_CUDA(cudaMemcpyAsync(G->sigma, sg.data(), sizeof(double) * nc, cudaMemcpyHostToDevice, st));
+            SGN_CUDA(cudaMemcpyAsync(G->tol, tl.data(), sizeof(double) * nc, cudaMemcpyHostToDevice, st));
+            SGN_CUDA(cudaMemcpyAsync(G->off, off_h.data(), sizeof(long long) * nc, cudaMemcpyHostToDevice, st));
+            SGN_CUDA(bi_init(G->S, nc, rsd, G->off, nb, st));
+            int iters = 0;
+            // as many applications of A^2 as FOM's cycle cap allows
+            const int cap = (int)std::min<long long>(kBiCap, std::max<long long>(2, (long long)c->max_cycles * k1 / 2));
+            SGN_CHECK(run_bicg(c, *G, adjoint, cap, &iters));
+            ref_cycles += iters;
+            for (int j = 0; j < nb; ++j)
+                if (G->h_done[j] != BI_DONE)
+                    failed.push_back(todo[t0 + j]);
+                else
+                    accept[todo[t0 + j].at] = std::min(1.0, 6.0 / margin[todo[t0 + j].at / ncol]);
+            if (debug_log())
+                fprintf(stderr, "[sgn mixed]   batch at %zu (%d systems): %d iterations, %zu failed so far\n", t0, nb,
+                        iters, failed.size());
+            const BiState& S = G->S;
+            SGN_CUDA(apply_hw32(c, S.t, S.d, nc, adjoint, nullptr, st, true));
+            SGN_CUDA(apply_hw32(c, S.w, S.t, nc, adjoint, nullptr, st, true));
+            SGN_CUDA(apply_corrections(xs, rsd, G->off, G->sigma, S.done, S.w, S.d, n, nb, st));
+            SGN_CUDA(cudaStreamSynchronize(st));  // the host tables are filled again
+        }
+        return SGN_OK;
+    };
     for (int round = 0; round <= max_rounds; ++round) {
         // true residuals r_i = b~ - (A^2 - sigma_i) x_i of every shifted system: from
         // scratch in refinement round 0, assembled in FP64; later rounds carry them along with
         // the corrections (r_i -= R c_i with x_i += R (Lambda^2 - sigma_i)^{-1} c_i,
         // r_i -= (A^2 - sigma_i) d_i with x_i += d_i), where FP32 products of the small d_i are
-        // exact to ~1e-7 ||r_i||.
-        // Round 0 forms A^2 x_i in float-float arithmetic on the FP32 units (stencil_ff.cu; ~1e-13
+        // exact to ~1e-6 ||r_i||: from scratch again where that is not far below the tolerance
+        // (solutions from 16-bit links, whose first residuals are about 1e-3).
+        // From scratch means A^2 x_i in float-float arithmetic on the FP32 units (stencil_ff.cu; ~1e-13
         // of the FP64 stencil, which GB300 runs at 1/64 of the FP32 rate), fsh shifts at a time.
-        if (round == 0) {
+        if (round == 0 || 1e-6 * worst > 0.02 * rtol) {
             const size_t nf = (size_t)ncol * n;
             const StencilParams pf = stencil_params(c, adjoint);
             const float4* Uf = reinterpret_cast<const float4*>(c->Uff.p);
@@ -1026,8 +1306,7 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
         SGN_CUDA(reduce(rd64, 1, nall, RM_STORE, 0, S64, nullptr, st));
         SGN_CUDA(cudaMemcpyAsync(hall.data(), S64.red, sizeof(double2) * hall.size(), cudaMemcpyDeviceToHost, st));
         SGN_CUDA(cudaStreamSynchronize(st));
-        std::vector<std::pair<int, int>> todo;  // (shift, column)
-        std::vector<double> todo_rel;           // its relative true residual
+        std::vector<System> todo;
         worst = 0;
         for (int i = 0; i < s; ++i)
             for (int col = 0; col < ncol; ++col) {
@@ -1038,10 +1317,7 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
                     return SGN_ERR_NONFINITE;
                 }
                 worst = std::max(worst, rel);
-                if (rel > rtol) {
-                    todo.emplace_back(i, col);
-                    todo_rel.push_back(rel);
-                }
+                if (rel > rtol * accept[i * ncol + col]) todo.push_back({i * ncol + col, rel});
             }
         if (debug_log())
             fprintf(stderr, "[sgn mixed] round %d: worst true residual %.3e, %zu of %d systems above tol\n", round,
@@ -1070,64 +1346,12 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
             SGN_CUDA(tsmm_nn<float2>(Rb32, n, m, S64.red, rs64, xs, n, nall, n, 1.0, st));
             SGN_CUDA(cudaStreamSynchronize(st));
         }
-        // correction solves, B systems at a time, one system per column
-        for (size_t t0 = 0; t0 < todo.size(); t0 += B) {
-            const int nb = (int)std::min<size_t>(B, todo.size() - t0);
-            float2* V0 = reinterpret_cast<float2*>(E1->V);
-            for (int j = 0; j < B; ++j) sig1[j] = j < nb ? c->sigma[todo[t0 + j].first] : c->sigma[0];
-            SGN_CHECK(fill_shift_tables(c, *E1, sig1.data(), om1.data()));
-            // the correction needs to reduce the worst residual of the batch to a third
-            // of the tolerance, not further (FP32 bases reach about 1e-6 at best)
-            double brel = 0;
-            for (int j = 0; j < nb; ++j) brel = std::max(brel, todo_rel[t0 + j]);
-            int st1 = SGN_OK;
-            RunResult r1;
-            for (int attempt = 0; attempt < 2; ++attempt) {
-                a1.gmres = attempt == 1;
-                SGN_CUDA(cudaMemsetAsync(V0, 0, sizeof(float2) * (size_t)B * n, st));
-                for (int j = 0; j < nb; ++j) {
-                    const int i = todo[t0 + j].first, col = todo[t0 + j].second;
-                    SGN_CUDA(convert_f64_to_f32(rsd + ((size_t)i * ncol + col) * n, V0 + (size_t)j * n, n, st));
-                }
-                SGN_CUDA(cudaMemsetAsync(d, 0, field * B, st));
-                const double inner = std::min(0.1, std::max(1e-5, rtol / ((a1.gmres ? 9.0 : 3.0) * brel)));
-                st1 = run_engine<float2>(c, *E1, a1, inner, a1.gmres ? c->max_cycles : std::min(c->max_cycles, kFomCap),
-                                         &r1);
-                if (debug_log())
-                    fprintf(stderr,
-                            "[sgn mixed]   batch at %zu (%d systems, %s): inner tol %.1e status %d cycles %d "
-                            "resmax %.3e\n",
-                            t0, nb, a1.gmres ? "GMRES" : "FOM", inner, st1, r1.cycles, r1.resmax);
-                ref_cycles += r1.cycles;
-                const bool fom_failed = !a1.gmres && (st1 == SGN_ERR_NONFINITE || st1 == SGN_ERR_BREAKDOWN ||
-                                                      (st1 == SGN_OK && !r1.converged));
-                if (!fom_failed) break;
-                SGN_CUDA(cudaMemsetAsync(E1->S.err, 0, sizeof(int), st));
-            }
-            if (st1 != SGN_OK) return st1;
-            // r_i -= (A^2 - sigma_i) d_i:  A^2 d in FP32 on the engine's scratch fields
-            {
-                float2* w32 = reinterpret_cast<float2*>(E1->w);
-                float2* t32 = reinterpret_cast<float2*>(E1->t);
-                SGN_CUDA(convert_f64_to_f32(d, w32, (int64_t)nb * n, st));
-                // FP32 links even when the solves run on BF16 ones: the carried residual
-                // must see the true operator, not the one the corrections were solved with
-                SGN_CUDA(apply_hw32(c, t32, w32, nb, adjoint, nullptr, st, true));
-                SGN_CUDA(apply_hw32(c, w32, t32, nb, adjoint, nullptr, st, true));
-                for (int j = 0; j < nb; ++j) {
-                    roff[j] = (long long)((size_t)todo[t0 + j].first * ncol + todo[t0 + j].second) * n;
-                    rsig[j] = c->sigma[todo[t0 + j].first];
-                }
-                SGN_CUDA(cudaMemcpyAsync(roff_dev, roff.data(), sizeof(long long) * nb, cudaMemcpyHostToDevice, st));
-                SGN_CUDA(cudaMemcpyAsync(rsig_dev, rsig.data(), sizeof(double) * nb, cudaMemcpyHostToDevice, st));
-                SGN_CUDA(correct_residuals(rsd, roff_dev, rsig_dev, w32, d, n, nb, st));
-            }
-            for (int j = 0; j < nb; ++j) {
-                const int i = todo[t0 + j].first, col = todo[t0 + j].second;
-                double2* xi = xs + ((size_t)i * ncol + col) * n;
-                SGN_CUDA(axpby3<double2>(xi, 1.0, xi, 1.0, d + (size_t)j * n, 0.0, nullptr, n, st));
-            }
-        }
+        std::vector<System> rest;
+        if (shortrec)
+            SGN_CHECK(bicg_corrections(todo, rest));
+        else
+            rest = todo;
+        if (!rest.empty()) SGN_CHECK(fom_corrections(rest));
     }
     // x = x_P + sum_i omega_i x_i
     SGN_CUDA(cudaMemcpyAsync(x, xP, field * ncol, cudaMemcpyDeviceToDevice, st));
