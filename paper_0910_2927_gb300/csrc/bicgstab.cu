@@ -128,6 +128,7 @@ __global__ void __launch_bounds__(NT) k_bi_init(const double2* __restrict__ src,
 // alpha = rho / <rt, v>, v = w - sigma p
 template <int PKT>
 __global__ void __launch_bounds__(NT) k_bi_v(BiState S) {
+    pdl_begin();
     const int col = blockIdx.y;
     if (S.done[col]) return;
     const int64_t c = (int64_t)col * 2 * S.npk, base = (int64_t)blockIdx.x * NT * PKT + threadIdx.x;
@@ -158,6 +159,7 @@ __global__ void __launch_bounds__(NT) k_bi_v(BiState S) {
 // s = r - alpha v
 template <int PKT>
 __global__ void __launch_bounds__(NT) k_bi_s(BiState S) {
+    pdl_begin();
     const int col = blockIdx.y;
     if (S.done[col]) return;
     const int64_t c = (int64_t)col * 2 * S.npk, base = (int64_t)blockIdx.x * NT * PKT + threadIdx.x;
@@ -181,6 +183,7 @@ __global__ void __launch_bounds__(NT) k_bi_s(BiState S) {
 // q = t - sigma s: omega = <q, s> / <q, q>, rho' = <rt, s> - omega <rt, q>, beta = rho' alpha / (rho omega)
 template <int PKT>
 __global__ void __launch_bounds__(NT) k_bi_t(BiState S) {
+    pdl_begin();
     const int col = blockIdx.y;
     if (S.done[col]) return;
     const int64_t c = (int64_t)col * 2 * S.npk, base = (int64_t)blockIdx.x * NT * PKT + threadIdx.x;
@@ -222,6 +225,7 @@ __global__ void __launch_bounds__(NT) k_bi_t(BiState S) {
 // d += alpha p + omega s, r = s - omega q, p = r + beta (p - omega v); convergence test on ||r||
 template <int PKT>
 __global__ void __launch_bounds__(NT) k_bi_x(BiState S) {
+    pdl_begin();
     const int col = blockIdx.y;
     if (S.done[col]) return;
     const int64_t c = (int64_t)col * 2 * S.npk, base = (int64_t)blockIdx.x * NT * PKT + threadIdx.x;
@@ -290,9 +294,9 @@ template <class K1, class K2, class K4>
 cudaError_t launch(const BiState& S, int ncol, cudaStream_t st, K1 k1, K2 k2, K4 k4) {
     const dim3 grid(S.nblk, ncol);
     switch (S.pkt) {
-        case 1: k1<<<grid, NT, 0, st>>>(S); break;
-        case 2: k2<<<grid, NT, 0, st>>>(S); break;
-        case 4: k4<<<grid, NT, 0, st>>>(S); break;
+        case 1: launch_pdl(k1, grid, NT, 0, st, S); break;
+        case 2: launch_pdl(k2, grid, NT, 0, st, S); break;
+        case 4: launch_pdl(k4, grid, NT, 0, st, S); break;
         default: return cudaErrorInvalidValue;
     }
     count_launch();

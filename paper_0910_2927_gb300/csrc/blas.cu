@@ -249,6 +249,7 @@ __device__ __forceinline__ void flush_partials(double2 (*sm)[NWARP], int nslot, 
 template <int PKT>
 __global__ void __launch_bounds__(NT) k_mdot(Basis<float2> V, int J, const float2* __restrict__ w, int64_t wsr, int64_t npk,
                                              Reduce rd, int with_norm, const int* __restrict__ skip) {
+    pdl_begin();
     using T = float2;
     using O = Ops<T>;
     const int col = blockIdx.y;
@@ -361,6 +362,7 @@ __global__ void __launch_bounds__(NT) k_maxpy_scale(Basis<T> V, int J, const dou
                                                     const T* w, int64_t wsr, T* out, int64_t osr,
                                                     const double* __restrict__ scale, int64_t npk,
                                                     const int* __restrict__ skip) {
+    pdl_begin();
     using O = Ops<T>;
     const int col = blockIdx.y;
     if (skip && skip[col]) return;
@@ -408,6 +410,7 @@ template <class T, int PKT>
 __global__ void __launch_bounds__(NT) k_update_x(Basis<T> V, int J, const double2* __restrict__ coef, int cstride,
                                                  double2* __restrict__ x, int64_t xsr, int64_t npk,
                                                  const int* __restrict__ skip, const int* __restrict__ kk) {
+    pdl_begin();
     using O = Ops<T>;
     const int col = blockIdx.y;
     if (skip && skip[col]) return;
@@ -465,6 +468,7 @@ __global__ void __launch_bounds__(NT) k_update_shifts(Basis<T> V, int J, const d
                                                       int kmax, double2* __restrict__ xs, int64_t xs_shift,
                                                       int64_t xs_col, int64_t npk, const int* __restrict__ skip,
                                                       const int* __restrict__ kk) {
+    pdl_begin();
     using O = Ops<T>;
     const int col = blockIdx.y;
     if (skip && skip[col]) return;
@@ -514,6 +518,7 @@ template <int PKT>
 __global__ void __launch_bounds__(NT) k_dcgs_dots(Basis<float2> V, int J, const float2* __restrict__ u,
                                                   const float2* __restrict__ z, int64_t wsr, int64_t npk, Reduce rd,
                                                   const int* __restrict__ skip) {
+    pdl_begin();
     using T = float2;
     using O = Ops<T>;
     const int col = blockIdx.y;
@@ -639,6 +644,7 @@ __global__ void __launch_bounds__(NT) k_dcgs_update(Basis<float2> V, int J, cons
                                                     int cstride, float2* u, const float2* __restrict__ z, float2* next,
                                                     int64_t wsr, int64_t npk, double2* H, int km,
                                                     const int* __restrict__ skip) {
+    pdl_begin();
     using T = float2;
     using O = Ops<T>;
     const int col = blockIdx.y;
@@ -747,6 +753,7 @@ __device__ __forceinline__ double2 slot_sum(const Reduce& rd, int col, int slot,
 template <int LPS>
 __global__ void __launch_bounds__(NT) k_reduce_store(Reduce rd, int nslot, int mode, DevState S,
                                                      const double2* __restrict__ lambda) {
+    pdl_begin();
     const int col = blockIdx.x;
     if (S.skip[col]) return;
     const int j = (blockIdx.y * NT + threadIdx.x) / LPS;
@@ -933,6 +940,7 @@ __device__ void reduce_tail(const double2* sums, int col, int nslot, int mode, i
 // the scalar work (the sums are the same whatever the arrival order).
 template <int LPS>
 __global__ void __launch_bounds__(NT) k_reduce(Reduce rd, int nslot, int mode, int colidx, DevState S) {
+    pdl_begin();
     const int col = blockIdx.x;
     // RM_BETA_FIRST starts a solve; RM_BETA_RESTART must still see columns that
     // broke down in this cycle; every other mode is column work proper.
@@ -1200,7 +1208,7 @@ cudaError_t mdot<float2>(Basis<float2> V, int J, const float2* w, int64_t wsr, i
     if (J + 1 > MAXSLOT) return cudaErrorInvalidValue;
     int64_t npk = n / Ops<float2>::CPX;
     dim3 grid(rd.nblk, ncol);
-    SGN_PK_SWITCH(pk_for(npk, rd.nblk), k_mdot<PKT_><<<grid, NT, 0, st>>>(V, J, w, wsr, npk, rd, with_norm, skip))
+    SGN_PK_SWITCH(pk_for(npk, rd.nblk), launch_pdl(k_mdot<PKT_>, grid, NT, 0, st, V, J, w, wsr, npk, rd, with_norm, skip))
     count_launch();
     return cudaGetLastError();
 }
@@ -1212,15 +1220,15 @@ cudaError_t reduce(const Reduce& rd, int nslot, int ncol, int mode, int colidx, 
     const int groups = few ? 1 : (nslot + NT / 8 - 1) / (NT / 8);
     if (mode == RM_STORE || mode == RM_SIGNED) {
         if (few)
-            k_reduce_store<32><<<dim3(ncol, groups), NT, 0, st>>>(rd, nslot, mode, S, lambda);
+            launch_pdl(k_reduce_store<32>, dim3(ncol, groups), NT, 0, st, rd, nslot, mode, S, lambda);
         else
-            k_reduce_store<8><<<dim3(ncol, groups), NT, 0, st>>>(rd, nslot, mode, S, lambda);
+            launch_pdl(k_reduce_store<8>, dim3(ncol, groups), NT, 0, st, rd, nslot, mode, S, lambda);
     } else {
         const dim3 grid(ncol, S.sums && S.rcount ? groups : 1);
         if (few)
-            k_reduce<32><<<grid, NT, 0, st>>>(rd, nslot, mode, colidx, S);
+            launch_pdl(k_reduce<32>, grid, NT, 0, st, rd, nslot, mode, colidx, S);
         else
-            k_reduce<8><<<grid, NT, 0, st>>>(rd, nslot, mode, colidx, S);
+            launch_pdl(k_reduce<8>, grid, NT, 0, st, rd, nslot, mode, colidx, S);
     }
     count_launch();
     return cudaGetLastError();
@@ -1244,7 +1252,7 @@ cudaError_t maxpy_scale(Basis<T> V, int J, const double2* coef, int cstride, con
     if (J > MAXSLOT) return cudaErrorInvalidValue;
     int64_t npk = n / Ops<T>::CPX;
     const Split sp = split_for<T>(n, ncol);
-    SGN_PK_SWITCH(sp.pkt, k_maxpy_scale<T, PKT_><<<dim3(sp.nb, ncol), sp.threads, 0, st>>>(V, J, coef, cstride, w, wsr, out, osr,
+    SGN_PK_SWITCH(sp.pkt, launch_pdl(k_maxpy_scale<T, PKT_>, dim3(sp.nb, ncol), sp.threads, 0, st, V, J, coef, cstride, w, wsr, out, osr,
                                                                               scale, npk, skip))
     count_launch();
     return cudaGetLastError();
@@ -1257,7 +1265,7 @@ cudaError_t update_x(Basis<T> V, int J, const double2* coef, int cstride, double
     int64_t npk = n / Ops<T>::CPX;
     const Split sp = split_for<T>(n, ncol);
     SGN_PK_SWITCH(sp.pkt,
-                  k_update_x<T, PKT_><<<dim3(sp.nb, ncol), sp.threads, 0, st>>>(V, J, coef, cstride, x, xsr, npk, skip, kk))
+                  launch_pdl(k_update_x<T, PKT_>, dim3(sp.nb, ncol), sp.threads, 0, st, V, J, coef, cstride, x, xsr, npk, skip, kk))
     count_launch();
     return cudaGetLastError();
 }
@@ -1281,17 +1289,17 @@ cudaError_t update_shifts(Basis<T> V, int J, const double2* y, int s, int kmax, 
     if (nblk > 0x7fffffff) return cudaErrorInvalidValue;
     dim3 grid((unsigned)nblk, ncol);
     if (sg == 20)
-        k_update_shifts<T, 20><<<grid, threads, smem, st>>>(V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
+        launch_pdl(k_update_shifts<T, 20>, grid, threads, smem, st, V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
     else if (sg == 10)
-        k_update_shifts<T, 10><<<grid, threads, smem, st>>>(V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
+        launch_pdl(k_update_shifts<T, 10>, grid, threads, smem, st, V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
     else if (sg == 8)
-        k_update_shifts<T, 8><<<grid, threads, smem, st>>>(V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
+        launch_pdl(k_update_shifts<T, 8>, grid, threads, smem, st, V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
     else if (sg == 4)
-        k_update_shifts<T, 4><<<grid, threads, smem, st>>>(V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
+        launch_pdl(k_update_shifts<T, 4>, grid, threads, smem, st, V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
     else if (sg == 1)
-        k_update_shifts<T, 1><<<grid, threads, smem, st>>>(V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
+        launch_pdl(k_update_shifts<T, 1>, grid, threads, smem, st, V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
     else
-        k_update_shifts<T, 2><<<grid, threads, smem, st>>>(V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
+        launch_pdl(k_update_shifts<T, 2>, grid, threads, smem, st, V, J, y, s, kmax, xs, xs_shift, xs_col, npk, skip, kk);
     count_launch();
     return cudaGetLastError();
 }
@@ -1302,7 +1310,7 @@ cudaError_t dcgs_dots<float2>(Basis<float2> V, int J, const float2* u, const flo
     if (2 * J + 3 > MAXSLOT) return cudaErrorInvalidValue;
     int64_t npk = n / Ops<float2>::CPX;
     dim3 grid(rd.nblk, ncol);
-    SGN_PK_SWITCH(pk_for(npk, rd.nblk), k_dcgs_dots<PKT_><<<grid, NT, 0, st>>>(V, J, u, z, wsr, npk, rd, skip))
+    SGN_PK_SWITCH(pk_for(npk, rd.nblk), launch_pdl(k_dcgs_dots<PKT_>, grid, NT, 0, st, V, J, u, z, wsr, npk, rd, skip))
     count_launch();
     return cudaGetLastError();
 }
@@ -1315,7 +1323,7 @@ cudaError_t dcgs_update<float2>(Basis<float2> V, int J, const double2* coef, int
     int64_t npk = n / Ops<float2>::CPX;
     const Split sp = split_for<float2>(n, ncol);
     const dim3 grid(sp.nb + (H ? 1 : 0), ncol);
-    SGN_PK_SWITCH(sp.pkt, k_dcgs_update<PKT_><<<grid, sp.threads, 0, st>>>(V, J, coef, cstride, u, z, next, wsr, npk, H,
+    SGN_PK_SWITCH(sp.pkt, launch_pdl(k_dcgs_update<PKT_>, grid, sp.threads, 0, st, V, J, coef, cstride, u, z, next, wsr, npk, H,
                                                                           km, skip))
     count_launch();
     return cudaGetLastError();

@@ -42,6 +42,7 @@ template <int NF, int E>
 __global__ void __launch_bounds__(32 * MAXW, 3)
     k_dots_f64(Basis<double2> V, int J, const double2* __restrict__ u, const double2* __restrict__ z, int64_t wsr,
                int64_t n, int64_t per, Reduce rd, int norm, const int* __restrict__ skip) {
+    pdl_begin();
     constexpr int VG = 16 / NF;
     const int col = blockIdx.y;
     if (skip && skip[col]) return;
@@ -153,11 +154,11 @@ cudaError_t launch(Basis<double2> V, int J, const double2* u, const double2* z, 
     const int groups = std::max(1, (J * NF + 15) / 16);
     const dim3 grid(rd.nblk, ncol, rounds(warps, groups).first);
     if (per <= 128)
-        k_dots_f64<NF, 1><<<grid, threads, 0, st>>>(V, J, u, z, wsr, n, per, rd, norm, skip);
+        launch_pdl(k_dots_f64<NF, 1>, grid, threads, 0, st, V, J, u, z, wsr, n, per, rd, norm, skip);
     else if (per <= 256)
-        k_dots_f64<NF, 2><<<grid, threads, 0, st>>>(V, J, u, z, wsr, n, per, rd, norm, skip);
+        launch_pdl(k_dots_f64<NF, 2>, grid, threads, 0, st, V, J, u, z, wsr, n, per, rd, norm, skip);
     else
-        k_dots_f64<NF, 4><<<grid, threads, 0, st>>>(V, J, u, z, wsr, n, per, rd, norm, skip);
+        launch_pdl(k_dots_f64<NF, 4>, grid, threads, 0, st, V, J, u, z, wsr, n, per, rd, norm, skip);
     count_launch();
     return cudaGetLastError();
 }
@@ -169,6 +170,7 @@ __global__ void __launch_bounds__(S == 1 ? 64 : 32 * S)
     k_dcgs_update_f64(Basis<double2> V, int J, const double2* __restrict__ coef, int cstride, double2* u,
                       const double2* __restrict__ z, double2* next, int64_t wsr, int64_t n, double2* H, int km,
                       const int* __restrict__ skip) {
+    pdl_begin();
     const int col = blockIdx.y;
     if (skip && skip[col]) return;
     if (H && blockIdx.x == 0) {  // one CTA per column forms the Hessenberg column beside the update
@@ -290,9 +292,9 @@ cudaError_t dcgs_update<double2>(Basis<double2> V, int J, const double2* coef, i
     const bool split = J > 4 && 9 * ((4 * warps + PIPES - 1) / PIPES) < 32 * ((warps + PIPES - 1) / PIPES);
     const dim3 grid((unsigned)((split ? (n + 31) / 32 : (n + 63) / 64) + (H ? 1 : 0)), ncol);
     if (split)
-        k_dcgs_update_f64<4><<<grid, 128, 0, st>>>(V, J, coef, cstride, u, z, next, wsr, n, H, km, skip);
+        launch_pdl(k_dcgs_update_f64<4>, grid, 128, 0, st, V, J, coef, cstride, u, z, next, wsr, n, H, km, skip);
     else
-        k_dcgs_update_f64<1><<<grid, 64, 0, st>>>(V, J, coef, cstride, u, z, next, wsr, n, H, km, skip);
+        launch_pdl(k_dcgs_update_f64<1>, grid, 64, 0, st, V, J, coef, cstride, u, z, next, wsr, n, H, km, skip);
     count_launch();
     return cudaGetLastError();
 }

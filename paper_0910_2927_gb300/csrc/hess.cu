@@ -46,6 +46,7 @@ __device__ __forceinline__ double2 shfl(double2 v, int src) {
 constexpr int SW = 4;
 template <bool BORDER>
 __global__ void __launch_bounds__(32 * SW) k_shifted_solve(DevState S) {
+    pdl_begin();
     const int col = blockIdx.y;
     if (S.done[col]) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -151,6 +152,7 @@ __global__ void __launch_bounds__(32 * SW) k_shifted_solve(DevState S) {
 }
 
 __global__ void k_combine(DevState S) {
+    pdl_begin();
     const int col = blockIdx.x;
     if (S.done[col]) return;
     const int km = S.kmax;
@@ -173,6 +175,7 @@ __global__ void k_combine(DevState S) {
 // the matrix; one warp applies the rotations (lanes own columns, the right-hand side is column
 // kk), back-substitutes and forms c (lanes own rows).
 __global__ void __launch_bounds__(128) k_shifted_lsq(DevState S) {
+    pdl_begin();
     const int col = blockIdx.x;
     if (S.done[col]) return;
     const int km = S.kmax;
@@ -274,12 +277,12 @@ constexpr size_t staged_bytes(int q) { return sizeof(double2) * (size_t)q * (q |
 
 cudaError_t shifted_lsq(const DevState& S, int ncol, cudaStream_t st) {
     if (S.s < 1 || !S.gres || S.kmax > KMAX) return cudaErrorInvalidValue;
-    k_shifted_lsq<<<ncol, 128, sizeof(double2) * (S.kmax + 1) * (S.kmax + 2), st>>>(S);
+    launch_pdl(k_shifted_lsq, ncol, 128, sizeof(double2) * (S.kmax + 1) * (S.kmax + 2), st, S);
     count_launch();
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || S.s == 1) return e;
     // the other shifts: bordered systems with the seed's residual coefficients
-    k_shifted_solve<true><<<dim3((S.s - 1 + SW - 1) / SW, ncol), 32 * SW, staged_bytes(S.kmax + 1), st>>>(S);
+    launch_pdl(k_shifted_solve<true>, dim3((S.s - 1 + SW - 1) / SW, ncol), 32 * SW, staged_bytes(S.kmax + 1), st, S);
     count_launch();
     return cudaGetLastError();
 }
@@ -297,13 +300,13 @@ cudaError_t prepare_small_kernels() {
 
 cudaError_t shifted_solves(const DevState& S, int ncol, cudaStream_t st) {
     if (S.kmax > KMAX) return cudaErrorInvalidValue;
-    k_shifted_solve<false><<<dim3((S.s + SW - 1) / SW, ncol), 32 * SW, staged_bytes(S.kmax), st>>>(S);
+    launch_pdl(k_shifted_solve<false>, dim3((S.s + SW - 1) / SW, ncol), 32 * SW, staged_bytes(S.kmax), st, S);
     count_launch();
     return cudaGetLastError();
 }
 
 cudaError_t combine_shifts(const DevState& S, int ncol, cudaStream_t st) {
-    k_combine<<<ncol, 64, 0, st>>>(S);
+    launch_pdl(k_combine, ncol, 64, 0, st, S);
     count_launch();
     return cudaGetLastError();
 }

@@ -249,6 +249,7 @@ template <class R, class LinkT, int NR, bool CS, bool NAT>
 __global__ void __launch_bounds__(NR == 1 ? 384 : 256)
     k_hw(typename Field<R>::T* __restrict__ out, const typename Field<R>::T* __restrict__ in,
          const LinkT* __restrict__ U, int nrhs, StencilParams P, const int* __restrict__ skip, int ngrp) {
+    pdl_begin();
     const int64_t tile = blockIdx.x / (unsigned)ngrp;
     const int grp = (int)(blockIdx.x - tile * ngrp);
     const int64_t site = tile * blockDim.x + threadIdx.x;
@@ -509,12 +510,14 @@ template <class LinkT, bool CS, bool NAT>
 __global__ void __launch_bounds__(256)
     k_hw_x2(float2* __restrict__ out, const float2* __restrict__ in, const LinkT* __restrict__ U, int nrhs,
             StencilParams P, const int* __restrict__ skip, int ngrp) {
+    pdl_begin();
     hw_x2_body<LinkT, CS, NAT>(out, in, U, nrhs, P, skip, ngrp);
 }
 template <class LinkT, bool CS, bool NAT>
 __global__ void __launch_bounds__(256, 2)
     k_hw_x2_r128(float2* __restrict__ out, const float2* __restrict__ in, const LinkT* __restrict__ U, int nrhs,
                  StencilParams P, const int* __restrict__ skip, int ngrp) {
+    pdl_begin();
     hw_x2_body<LinkT, CS, NAT>(out, in, U, nrhs, P, skip, ngrp);
 }
 
@@ -637,6 +640,7 @@ template <class LinkT, int NR, bool CS, bool NAT>
 __global__ void __launch_bounds__(256)
     k_hw_pipe(float2* __restrict__ out, const float2* __restrict__ in, const LinkT* __restrict__ U, int nrhs,
               StencilParams P, const int* __restrict__ skip, int ngrp) {
+    pdl_begin();
     extern __shared__ float4 sbuf[];
     const int64_t tile = blockIdx.x / (unsigned)ngrp;
     const int grp = (int)(blockIdx.x - tile * ngrp);
@@ -826,6 +830,7 @@ template <class LinkT, bool CS, bool NAT>
 __global__ void __launch_bounds__(256, 4)
     k_hw_cs(float2* __restrict__ out, const float2* __restrict__ in, const LinkT* __restrict__ U, int nrhs,
             StencilParams P, const int* __restrict__ skip, int ngrp, int fw) {
+    pdl_begin();
     const int warp = threadIdx.y, lane = threadIdx.x;
     const int64_t tile = blockIdx.x / (unsigned)ngrp;
     const int grp = (int)(blockIdx.x - tile * ngrp);
@@ -923,9 +928,9 @@ cudaError_t launch_nr(typename Field<R>::T* out, const typename Field<R>::T* in,
     dim3 block(sx, rb);
     const bool cs = (double)nrhs * (double)p.vol * 12.0 * sizeof(typename Field<R>::T) > 256.0 * (1 << 20);
     if (cs)
-        k_hw<R, LinkT, NR, true, NAT><<<(unsigned)(tiles * ngrp), block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp);
+        launch_pdl(k_hw<R, LinkT, NR, true, NAT>, (unsigned)(tiles * ngrp), block, 0, st, out, in, U, nrhs, p, skip, ngrp);
     else
-        k_hw<R, LinkT, NR, false, NAT><<<(unsigned)(tiles * ngrp), block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp);
+        launch_pdl(k_hw<R, LinkT, NR, false, NAT>, (unsigned)(tiles * ngrp), block, 0, st, out, in, U, nrhs, p, skip, ngrp);
     count_launch();
     return cudaGetLastError();
 }
@@ -954,9 +959,9 @@ cudaError_t launch_pipe(float2* out, const float2* in, const LinkT* U, int nrhs,
     }
     dim3 block(sx, rb);
     if (cs)
-        k_hw_pipe<LinkT, NR, true, NAT><<<(unsigned)(tiles * ngrp), block, smem, st>>>(out, in, U, nrhs, p, skip, ngrp);
+        launch_pdl(k_hw_pipe<LinkT, NR, true, NAT>, (unsigned)(tiles * ngrp), block, smem, st, out, in, U, nrhs, p, skip, ngrp);
     else
-        k_hw_pipe<LinkT, NR, false, NAT><<<(unsigned)(tiles * ngrp), block, smem, st>>>(out, in, U, nrhs, p, skip, ngrp);
+        launch_pdl(k_hw_pipe<LinkT, NR, false, NAT>, (unsigned)(tiles * ngrp), block, smem, st, out, in, U, nrhs, p, skip, ngrp);
     count_launch();
     return cudaGetLastError();
 }
@@ -974,9 +979,9 @@ cudaError_t launch_cs(float2* out, const float2* in, const LinkT* U, int nrhs, c
     const bool cs = (double)nrhs * (double)p.vol * 12.0 * sizeof(float2) > 256.0 * (1 << 20);
     const unsigned grid = (unsigned)(tiles * ngrp);
     if (cs)
-        k_hw_cs<LinkT, true, NAT><<<grid, block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp, fw);
+        launch_pdl(k_hw_cs<LinkT, true, NAT>, grid, block, 0, st, out, in, U, nrhs, p, skip, ngrp, fw);
     else
-        k_hw_cs<LinkT, false, NAT><<<grid, block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp, fw);
+        launch_pdl(k_hw_cs<LinkT, false, NAT>, grid, block, 0, st, out, in, U, nrhs, p, skip, ngrp, fw);
     count_launch();
     return cudaGetLastError();
 }
@@ -993,13 +998,13 @@ cudaError_t launch_x2(float2* out, const float2* in, const LinkT* U, int nrhs, c
     const unsigned grid = (unsigned)(tiles * ngrp);
     if (MINB == 2) {
         if (cs)
-            k_hw_x2_r128<LinkT, true, NAT><<<grid, block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp);
+            launch_pdl(k_hw_x2_r128<LinkT, true, NAT>, grid, block, 0, st, out, in, U, nrhs, p, skip, ngrp);
         else
-            k_hw_x2_r128<LinkT, false, NAT><<<grid, block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp);
+            launch_pdl(k_hw_x2_r128<LinkT, false, NAT>, grid, block, 0, st, out, in, U, nrhs, p, skip, ngrp);
     } else if (cs) {
-        k_hw_x2<LinkT, true, NAT><<<grid, block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp);
+        launch_pdl(k_hw_x2<LinkT, true, NAT>, grid, block, 0, st, out, in, U, nrhs, p, skip, ngrp);
     } else {
-        k_hw_x2<LinkT, false, NAT><<<grid, block, 0, st>>>(out, in, U, nrhs, p, skip, ngrp);
+        launch_pdl(k_hw_x2<LinkT, false, NAT>, grid, block, 0, st, out, in, U, nrhs, p, skip, ngrp);
     }
     count_launch();
     return cudaGetLastError();

@@ -55,6 +55,7 @@ template <bool NAT, bool RATIO>
 __global__ void __launch_bounds__(kMaxThreads, 4)
     k_hw_hops(double2* __restrict__ out, const double2* __restrict__ in, const double2* __restrict__ U, int nrhs,
               StencilParams P, HopRatios Q, const int* __restrict__ skip) {
+    pdl_begin();
     const int64_t tile = blockIdx.x / (unsigned)nrhs;
     const int rhs = (int)(blockIdx.x - tile * nrhs);
     if (skip && skip[rhs]) return;
@@ -223,13 +224,13 @@ cudaError_t launch_hw_f64(double2* out, const double2* in, const double2* U, int
     for (double r : {q.t[0], q.t[1], q.ti[0], q.ti[1], q.bf, q.fb}) ratio = ratio && r > 1e-100 && r < 1e100;
     const unsigned grid = (unsigned)blocks;
     if (nat && ratio)
-        k_hw_hops<true, true><<<grid, threads, 0, st>>>(out, in, U, nrhs, p, q, skip);
+        launch_pdl(k_hw_hops<true, true>, grid, threads, 0, st, out, in, U, nrhs, p, q, skip);
     else if (nat)
-        k_hw_hops<true, false><<<grid, threads, 0, st>>>(out, in, U, nrhs, p, q, skip);
+        launch_pdl(k_hw_hops<true, false>, grid, threads, 0, st, out, in, U, nrhs, p, q, skip);
     else if (ratio)
-        k_hw_hops<false, true><<<grid, threads, 0, st>>>(out, in, U, nrhs, p, q, skip);
+        launch_pdl(k_hw_hops<false, true>, grid, threads, 0, st, out, in, U, nrhs, p, q, skip);
     else
-        k_hw_hops<false, false><<<grid, threads, 0, st>>>(out, in, U, nrhs, p, q, skip);
+        launch_pdl(k_hw_hops<false, false>, grid, threads, 0, st, out, in, U, nrhs, p, q, skip);
     count_launch();
     return cudaGetLastError();
 }

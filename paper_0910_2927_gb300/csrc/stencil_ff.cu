@@ -122,6 +122,7 @@ template <bool NAT, FfOut OUT>
 __global__ void __launch_bounds__(kMaxThreads, 4)
     k_hw_ff(void* __restrict__ out, const float4* __restrict__ in, const float4* __restrict__ Uf, int nrhs,
             StencilParams P, FfResidual R) {
+    pdl_begin();
     const int64_t tile = blockIdx.x / (unsigned)nrhs;
     const int rhs = (int)(blockIdx.x - tile * nrhs);
     const int64_t s0 = tile * (blockDim.x >> 3) + (threadIdx.x >> 3);
@@ -262,6 +263,7 @@ __global__ void __launch_bounds__(kMaxThreads, 4)
 
 // complex128 -> float-float, elementwise
 __global__ void k_split_ff(const double2* __restrict__ in, float4* __restrict__ out, int64_t count) {
+    pdl_begin();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
         const double2 v = in[i];
         const float2 re = d2ff(v.x), im = d2ff(v.y);
@@ -283,9 +285,9 @@ cudaError_t launch_ff(void* out, const float4* in, const float4* Uf, int nrhs, c
     const int64_t blocks = (p.vol + sites - 1) / sites * nrhs;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
     if (nat)
-        k_hw_ff<true, OUT><<<(unsigned)blocks, threads, 0, st>>>(out, in, Uf, nrhs, p, r);
+        launch_pdl(k_hw_ff<true, OUT>, (unsigned)blocks, threads, 0, st, out, in, Uf, nrhs, p, r);
     else
-        k_hw_ff<false, OUT><<<(unsigned)blocks, threads, 0, st>>>(out, in, Uf, nrhs, p, r);
+        launch_pdl(k_hw_ff<false, OUT>, (unsigned)blocks, threads, 0, st, out, in, Uf, nrhs, p, r);
     count_launch();
     return cudaGetLastError();
 }
@@ -306,7 +308,7 @@ cudaError_t hw_ff_residual(double2* r, const float4* in, const float4* Uf, int n
 
 cudaError_t split_ff(const double2* in, float4* out, int64_t count, cudaStream_t st) {
     if (count <= 0) return cudaSuccess;
-    k_split_ff<<<grid_of(count), 256, 0, st>>>(in, out, count);
+    launch_pdl(k_split_ff, grid_of(count), 256, 0, st, in, out, count);
     count_launch();
     return cudaGetLastError();
 }
