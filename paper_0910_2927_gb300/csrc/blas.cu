@@ -35,7 +35,7 @@ struct Ops<double2> {
     using P = double2;
     using C = double2;  // coefficient type used in the arithmetic
     static constexpr int CPX = 1;
-    static __device__ __forceinline__ P ld_ro(const double2* b, int64_t pk) { return __ldg(b + pk); }
+    static __device__ __forceinline__ P ld_ro(const double2* b, int64_t pk) { return b[pk]; }
     static __device__ __forceinline__ P ld(const double2* b, int64_t pk) { return b[pk]; }
     static __device__ __forceinline__ void st(double2* b, int64_t pk, P v) { b[pk] = v; }
     static __device__ __forceinline__ P zero() { return make_double2(0, 0); }
@@ -77,9 +77,7 @@ struct Ops<float2> {
     using P = float4;
     using C = float2;
     static constexpr int CPX = 2;
-    static __device__ __forceinline__ P ld_ro(const float2* b, int64_t pk) {
-        return __ldg(reinterpret_cast<const float4*>(b) + pk);
-    }
+    static __device__ __forceinline__ P ld_ro(const float2* b, int64_t pk) { return reinterpret_cast<const float4*>(b)[pk]; }
     static __device__ __forceinline__ P ld(const float2* b, int64_t pk) { return reinterpret_cast<const float4*>(b)[pk]; }
     static __device__ __forceinline__ void st(float2* b, int64_t pk, P v) { reinterpret_cast<float4*>(b)[pk] = v; }
     static __device__ __forceinline__ P zero() { return make_float4(0, 0, 0, 0); }
@@ -247,8 +245,8 @@ __device__ __forceinline__ void flush_partials(double2 (*sm)[NWARP], int nslot, 
 // partial[j] = sum_e conj(V_j[e]) w[e], j < J; slot J: ||w||^2 if with_norm.
 // FP32 storage (FP64: gs_f64.cu).
 template <int PKT>
-__global__ void __launch_bounds__(NT) k_mdot(Basis<float2> V, int J, const float2* __restrict__ w, int64_t wsr, int64_t npk,
-                                             Reduce rd, int with_norm, const int* __restrict__ skip) {
+__global__ void __launch_bounds__(NT) k_mdot(Basis<float2> V, int J, const float2* w, int64_t wsr, int64_t npk,
+                                             Reduce rd, int with_norm, const int* skip) {
     pdl_begin();
     using T = float2;
     using O = Ops<T>;
@@ -358,10 +356,10 @@ __global__ void __launch_bounds__(NT) k_maxpy_mdot(Basis<T> V, int J, const doub
 
 // out = (w - sum_j c_j V_j) * scale[col]   (out may alias w)
 template <class T, int PKT>
-__global__ void __launch_bounds__(NT) k_maxpy_scale(Basis<T> V, int J, const double2* __restrict__ coef, int cstride,
+__global__ void __launch_bounds__(NT) k_maxpy_scale(Basis<T> V, int J, const double2* coef, int cstride,
                                                     const T* w, int64_t wsr, T* out, int64_t osr,
-                                                    const double* __restrict__ scale, int64_t npk,
-                                                    const int* __restrict__ skip) {
+                                                    const double* scale, int64_t npk,
+                                                    const int* skip) {
     pdl_begin();
     using O = Ops<T>;
     const int col = blockIdx.y;
@@ -407,9 +405,9 @@ __global__ void __launch_bounds__(NT) k_maxpy_scale(Basis<T> V, int J, const dou
 
 // x += sum_j c_j V_j in FP64 (x complex128), j < min(J, kk[col]).
 template <class T, int PKT>
-__global__ void __launch_bounds__(NT) k_update_x(Basis<T> V, int J, const double2* __restrict__ coef, int cstride,
-                                                 double2* __restrict__ x, int64_t xsr, int64_t npk,
-                                                 const int* __restrict__ skip, const int* __restrict__ kk) {
+__global__ void __launch_bounds__(NT) k_update_x(Basis<T> V, int J, const double2* coef, int cstride,
+                                                 double2* x, int64_t xsr, int64_t npk,
+                                                 const int* skip, const int* kk) {
     pdl_begin();
     using O = Ops<T>;
     const int col = blockIdx.y;
@@ -464,10 +462,10 @@ __global__ void __launch_bounds__(NT) k_update_x(Basis<T> V, int J, const double
 // registers and ran at half the speed.  Products and the sum over j in the
 // storage precision; the add to xs in FP64.
 template <class T, int SG>
-__global__ void __launch_bounds__(NT) k_update_shifts(Basis<T> V, int J, const double2* __restrict__ y, int s,
-                                                      int kmax, double2* __restrict__ xs, int64_t xs_shift,
-                                                      int64_t xs_col, int64_t npk, const int* __restrict__ skip,
-                                                      const int* __restrict__ kk) {
+__global__ void __launch_bounds__(NT) k_update_shifts(Basis<T> V, int J, const double2* y, int s,
+                                                      int kmax, double2* xs, int64_t xs_shift,
+                                                      int64_t xs_col, int64_t npk, const int* skip,
+                                                      const int* kk) {
     pdl_begin();
     using O = Ops<T>;
     const int col = blockIdx.y;
@@ -515,9 +513,9 @@ __global__ void __launch_bounds__(NT) k_update_shifts(Basis<T> V, int J, const d
 // (the closing pass of a cycle) only s and u^dag u (slot J).
 // FP32 storage (FP64: gs_f64.cu).
 template <int PKT>
-__global__ void __launch_bounds__(NT) k_dcgs_dots(Basis<float2> V, int J, const float2* __restrict__ u,
-                                                  const float2* __restrict__ z, int64_t wsr, int64_t npk, Reduce rd,
-                                                  const int* __restrict__ skip) {
+__global__ void __launch_bounds__(NT) k_dcgs_dots(Basis<float2> V, int J, const float2* u,
+                                                  const float2* z, int64_t wsr, int64_t npk, Reduce rd,
+                                                  const int* skip) {
     pdl_begin();
     using T = float2;
     using O = Ops<T>;
@@ -640,10 +638,10 @@ __global__ void __launch_bounds__(NT) k_dcgs_dots(Basis<float2> V, int J, const 
 // Coefficients per column: [0,J) s, [J,2J) c, 2J: (1/rho, 0), 2J+1: d.
 // FP32 storage (FP64: gs_f64.cu).
 template <int PKT>
-__global__ void __launch_bounds__(NT) k_dcgs_update(Basis<float2> V, int J, const double2* __restrict__ coef,
-                                                    int cstride, float2* u, const float2* __restrict__ z, float2* next,
+__global__ void __launch_bounds__(NT) k_dcgs_update(Basis<float2> V, int J, const double2* coef,
+                                                    int cstride, float2* u, const float2* z, float2* next,
                                                     int64_t wsr, int64_t npk, double2* H, int km,
-                                                    const int* __restrict__ skip) {
+                                                    const int* skip) {
     pdl_begin();
     using T = float2;
     using O = Ops<T>;
@@ -752,7 +750,7 @@ __device__ __forceinline__ double2 slot_sum(const Reduce& rd, int col, int slot,
 // RM_STORE and RM_SIGNED: every slot on its own.  Grid (column, NT / LPS slots).
 template <int LPS>
 __global__ void __launch_bounds__(NT) k_reduce_store(Reduce rd, int nslot, int mode, DevState S,
-                                                     const double2* __restrict__ lambda) {
+                                                     const double2* lambda) {
     pdl_begin();
     const int col = blockIdx.x;
     if (S.skip[col]) return;

@@ -73,7 +73,7 @@ __device__ __forceinline__ double reduce_few(double (&a)[N], int lane) {
 // with the step's coefficients s = red[0, j), c = red[j, 2j), 1 / rho = red[2j], d = red[2j + 1].
 // Four lanes per row.  Not inlined: in the FP32 update it would take that kernel from 80 to 107
 // registers, a third of its resident warps (74 -> 87 us on 120 columns of 10^4).
-__device__ __noinline__ static void hess_column(double2* __restrict__ H, const double2* __restrict__ red, int j, int km) {
+__device__ __noinline__ static void hess_column(double2* H, const double2* red, int j, int km) {
     const int q = threadIdx.x & 3;
     const double ir = red[2 * j].x;
     for (int i0 = 0; i0 <= j; i0 += blockDim.x / 4) {

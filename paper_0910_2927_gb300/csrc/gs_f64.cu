@@ -40,8 +40,8 @@ __device__ __forceinline__ void dot_acc(double& re, double& im, double2 v, doubl
 // E elements per thread and chunk of the CTA's elements.
 template <int NF, int E>
 __global__ void __launch_bounds__(32 * MAXW, 3)
-    k_dots_f64(Basis<double2> V, int J, const double2* __restrict__ u, const double2* __restrict__ z, int64_t wsr,
-               int64_t n, int64_t per, Reduce rd, int norm, const int* __restrict__ skip) {
+    k_dots_f64(Basis<double2> V, int J, const double2* u, const double2* z, int64_t wsr,
+               int64_t n, int64_t per, Reduce rd, int norm, const int* skip) {
     pdl_begin();
     constexpr int VG = 16 / NF;
     const int col = blockIdx.y;
@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(32 * MAXW, 3)
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             const int64_t i = c0 + threadIdx.x + e * (int)blockDim.x;
-            q[e] = i < b1 ? __ldg(f + i) : make_double2(0, 0);
+            q[e] = i < b1 ? f[i] : make_double2(0, 0);
         }
     };
     auto cta_sum = [&](double r, int buf) {  // valid in warp 0
@@ -167,9 +167,9 @@ cudaError_t launch(Basis<double2> V, int J, const double2* u, const double2* z, 
 // 32 elements: warp w takes the basis vectors w, w + S, ..., and warp 0 adds their sums.
 template <int S>
 __global__ void __launch_bounds__(S == 1 ? 64 : 32 * S)
-    k_dcgs_update_f64(Basis<double2> V, int J, const double2* __restrict__ coef, int cstride, double2* u,
-                      const double2* __restrict__ z, double2* next, int64_t wsr, int64_t n, double2* H, int km,
-                      const int* __restrict__ skip) {
+    k_dcgs_update_f64(Basis<double2> V, int J, const double2* coef, int cstride, double2* u,
+                      const double2* z, double2* next, int64_t wsr, int64_t n, double2* H, int km,
+                      const int* skip) {
     pdl_begin();
     const int col = blockIdx.y;
     if (skip && skip[col]) return;
@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(S == 1 ? 64 : 32 * S)
     for (int l0 = w0; l0 < J; l0 += UNR * S) {
         double2 q[UNR];
 #pragma unroll
-        for (int g = 0; g < UNR; ++g) q[g] = l0 + g * S < J ? __ldg(vb + (l0 + g * S) * V.sj) : make_double2(0, 0);
+        for (int g = 0; g < UNR; ++g) q[g] = l0 + g * S < J ? vb[(l0 + g * S) * V.sj] : make_double2(0, 0);
 #pragma unroll
         for (int g = 0; g < UNR; ++g) {
             const int l = l0 + g * S;

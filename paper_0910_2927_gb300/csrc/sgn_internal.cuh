@@ -39,8 +39,10 @@ inline void count_launch(long long k = 1) { g_launches += k; }
 // The kernels of an Arnoldi step follow one another on one stream and most run for a few
 // microseconds, of which a full launch takes one to two.  Launched by launch_pdl, a kernel is
 // set up while its predecessor runs and waits in pdl_begin() until that one has completed and its
-// writes are visible.  Every kernel launched so calls pdl_begin() before anything else, on every
-// path: that a kernel has completed then means that all before it have.
+// writes are visible.  Every kernel launched so calls pdl_begin() on every path, before it touches
+// anything that a kernel of the stream writes: that a kernel has completed then means that all
+// before it have.  Such data are read by plain loads: a const __restrict__ pointer or __ldg would say
+// that they do not change while the kernel runs, and let the load move ahead of the wait.
 template <class... KA, class... A>
 inline void launch_pdl(void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
     cudaLaunchAttribute at{};

@@ -1225,7 +1225,7 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
         return SGN_OK;
     };
 
-    // A system once corrected is done below rtol * accept, six times its correction's aim: the first
+    // A system once corrected is done below rtol * accept, twelve times its correction's aim: the first
     // correction of a solution from 16-bit links may leave it anywhere below rtol.
     std::vector<double> accept(nall, 1.0);
     // Correction solves by BiCGStab, each system to its own residual; the systems it gave up on are
@@ -1269,7 +1269,7 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
                 if (G->h_done[j] != BI_DONE)
                     failed.push_back(todo[t0 + j]);
                 else
-                    accept[todo[t0 + j].at] = std::min(1.0, 6.0 / margin[todo[t0 + j].at / ncol]);
+                    accept[todo[t0 + j].at] = std::min(1.0, 12.0 / margin[todo[t0 + j].at / ncol]);
             if (debug_log())
                 fprintf(stderr, "[sgn mixed]   batch at %zu (%d systems): %d iterations, %zu failed so far\n", t0, nb,
                         iters, failed.size());

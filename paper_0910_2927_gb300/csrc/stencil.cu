@@ -56,12 +56,12 @@ struct Field<float> {
     using T = float2;
     // NAT: natural order, entries 0..11 of a site contiguous (96 bytes)
     template <bool NAT>
-    static __device__ __forceinline__ void load(const float2* __restrict__ f, int64_t site, int64_t vol2,
+    static __device__ __forceinline__ void load(const float2* f, int64_t site, int64_t vol2,
                                                 Cx<float> p[12]) {
         const float2* s = f + (NAT ? 12 : 2) * site;
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-            const float4 v = __ldg(reinterpret_cast<const float4*>(s + (NAT ? 2 * k : k * vol2)));
+            const float4 v = *reinterpret_cast<const float4*>(s + (NAT ? 2 * k : k * vol2));
             p[2 * k] = {v.x, v.y};
             p[2 * k + 1] = {v.z, v.w};
         }
@@ -194,7 +194,7 @@ __device__ __forceinline__ void hop_links(Cx<R> (&acc)[NR][12], const Cx<R> (&h0
 
 
 template <class R, class LinkT, int NU, int S, int NR, bool NAT>
-__device__ __forceinline__ void hop(Cx<R> (&acc)[NR][12], const typename Field<R>::T* __restrict__ in,
+__device__ __forceinline__ void hop(Cx<R> (&acc)[NR][12], const typename Field<R>::T* in,
                                     int64_t stride_rhs, const bool (&act)[NR], const LinkT* __restrict__ U,
                                     int64_t link_site, int64_t nb, R coef, int64_t vol) {
     Cx<R> h0[NR][3], h1[NR][3];
@@ -213,7 +213,7 @@ __device__ __forceinline__ void hop(Cx<R> (&acc)[NR][12], const typename Field<R
 }
 
 template <class R, class LinkT, int NU, int NR, bool NAT>
-__device__ __forceinline__ void both_hops(Cx<R> (&acc)[NR][12], const typename Field<R>::T* __restrict__ in,
+__device__ __forceinline__ void both_hops(Cx<R> (&acc)[NR][12], const typename Field<R>::T* in,
                                           const bool (&act)[NR], const LinkT* __restrict__ U, int64_t site,
                                           const int co[4], const StencilParams& P) {
     int64_t stride = 1;
@@ -247,8 +247,8 @@ __device__ __forceinline__ void both_hops(Cx<R> (&acc)[NR][12], const typename F
 // result would otherwise push it out of L2 first.
 template <class R, class LinkT, int NR, bool CS, bool NAT>
 __global__ void __launch_bounds__(NR == 1 ? 384 : 256)
-    k_hw(typename Field<R>::T* __restrict__ out, const typename Field<R>::T* __restrict__ in,
-         const LinkT* __restrict__ U, int nrhs, StencilParams P, const int* __restrict__ skip, int ngrp) {
+    k_hw(typename Field<R>::T* __restrict__ out, const typename Field<R>::T* in,
+         const LinkT* __restrict__ U, int nrhs, StencilParams P, const int* skip, int ngrp) {
     pdl_begin();
     const int64_t tile = blockIdx.x / (unsigned)ngrp;
     const int grp = (int)(blockIdx.x - tile * ngrp);
@@ -315,7 +315,7 @@ __device__ __forceinline__ float2 f2s(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
 template <class LinkT, int NU, int S, bool NAT>
-__device__ __forceinline__ void hop_x2(float2 (&ar)[12], float2 (&ai)[12], const float2* __restrict__ in,
+__device__ __forceinline__ void hop_x2(float2 (&ar)[12], float2 (&ai)[12], const float2* in,
                                        int64_t stride_rhs, const bool (&act)[2], const LinkT* __restrict__ U,
                                        int64_t link_site, int64_t nb, float coef, int64_t vol) {
     float2 hr0[3], hi0[3], hr1[3], hi1[3];  // the two projected colour vectors, paired over fields
@@ -409,7 +409,7 @@ __device__ __forceinline__ void hop_x2(float2 (&ar)[12], float2 (&ai)[12], const
 }
 
 template <class LinkT, int NU, bool NAT>
-__device__ __forceinline__ void both_hops_x2(float2 (&ar)[12], float2 (&ai)[12], const float2* __restrict__ in,
+__device__ __forceinline__ void both_hops_x2(float2 (&ar)[12], float2 (&ai)[12], const float2* in,
                                              const bool (&act)[2], const LinkT* __restrict__ U, int64_t site,
                                              const int co[4], const StencilParams& P) {
     int64_t stride = 1;
@@ -434,9 +434,9 @@ __device__ __forceinline__ void both_hops_x2(float2 (&ar)[12], float2 (&ai)[12],
 
 // One site, fields rhs0 and rhs0 + 1.
 template <class LinkT, bool CS, bool NAT>
-__device__ __forceinline__ void x2_site(float2* __restrict__ out, const float2* __restrict__ in,
+__device__ __forceinline__ void x2_site(float2* __restrict__ out, const float2* in,
                                         const LinkT* __restrict__ U, int nrhs, const StencilParams& P,
-                                        const int* __restrict__ skip, int64_t site, int rhs0) {
+                                        const int* skip, int64_t site, int rhs0) {
     if (site >= P.vol || rhs0 >= nrhs) return;
     bool act[2];
 #pragma unroll
@@ -495,9 +495,9 @@ __device__ __forceinline__ void x2_site(float2* __restrict__ out, const float2* 
 
 // Grid and thread layout as k_hw with NR = 2.
 template <class LinkT, bool CS, bool NAT>
-__device__ __forceinline__ void hw_x2_body(float2* __restrict__ out, const float2* __restrict__ in,
+__device__ __forceinline__ void hw_x2_body(float2* __restrict__ out, const float2* in,
                                            const LinkT* __restrict__ U, int nrhs, const StencilParams& P,
-                                           const int* __restrict__ skip, int ngrp) {
+                                           const int* skip, int ngrp) {
     const int64_t tile = blockIdx.x / (unsigned)ngrp;
     const int grp = (int)(blockIdx.x - tile * ngrp);
     x2_site<LinkT, CS, NAT>(out, in, U, nrhs, P, skip, tile * blockDim.x + threadIdx.x,
@@ -508,15 +508,15 @@ __device__ __forceinline__ void hw_x2_body(float2* __restrict__ out, const float
 // registers (16 warps per SM, a few values spilled to local memory).
 template <class LinkT, bool CS, bool NAT>
 __global__ void __launch_bounds__(256)
-    k_hw_x2(float2* __restrict__ out, const float2* __restrict__ in, const LinkT* __restrict__ U, int nrhs,
-            StencilParams P, const int* __restrict__ skip, int ngrp) {
+    k_hw_x2(float2* __restrict__ out, const float2* in, const LinkT* __restrict__ U, int nrhs,
+            StencilParams P, const int* skip, int ngrp) {
     pdl_begin();
     hw_x2_body<LinkT, CS, NAT>(out, in, U, nrhs, P, skip, ngrp);
 }
 template <class LinkT, bool CS, bool NAT>
 __global__ void __launch_bounds__(256, 2)
-    k_hw_x2_r128(float2* __restrict__ out, const float2* __restrict__ in, const LinkT* __restrict__ U, int nrhs,
-                 StencilParams P, const int* __restrict__ skip, int ngrp) {
+    k_hw_x2_r128(float2* __restrict__ out, const float2* in, const LinkT* __restrict__ U, int nrhs,
+                 StencilParams P, const int* skip, int ngrp) {
     pdl_begin();
     hw_x2_body<LinkT, CS, NAT>(out, in, U, nrhs, P, skip, ngrp);
 }
@@ -638,8 +638,8 @@ __device__ __forceinline__ void pipe_stage(Cx<float> (&acc)[NR][12], const PipeC
 
 template <class LinkT, int NR, bool CS, bool NAT>
 __global__ void __launch_bounds__(256)
-    k_hw_pipe(float2* __restrict__ out, const float2* __restrict__ in, const LinkT* __restrict__ U, int nrhs,
-              StencilParams P, const int* __restrict__ skip, int ngrp) {
+    k_hw_pipe(float2* __restrict__ out, const float2* in, const LinkT* __restrict__ U, int nrhs,
+              StencilParams P, const int* skip, int ngrp) {
     pdl_begin();
     extern __shared__ float4 sbuf[];
     const int64_t tile = blockIdx.x / (unsigned)ngrp;
@@ -720,8 +720,8 @@ __global__ void __launch_bounds__(256)
 // takes site group tile * (warps / fw) + w / fw (10 sites) and field group * fw + w % fw.
 constexpr int kCsSites = 10;  // sites per warp
 
-__device__ __forceinline__ Cx<float> ldc(const float2* __restrict__ p) {
-    const float2 v = __ldg(p);
+__device__ __forceinline__ Cx<float> ldc(const float2* p) {
+    const float2 v = *p;
     return {v.x, v.y};
 }
 __device__ __forceinline__ Cx<float> shfl_cx(Cx<float> v, int src) {
@@ -740,7 +740,7 @@ __device__ __forceinline__ int64_t entry_cs(int64_t site, int k, int64_t vol2) {
 }
 
 template <class LinkT, int NU, int S, bool NAT>
-__device__ __forceinline__ void hop_cs(Cx<float> (&acc)[4], const float2* __restrict__ fin, int64_t vol2,
+__device__ __forceinline__ void hop_cs(Cx<float> (&acc)[4], const float2* fin, int64_t vol2,
                                        bool act, const LinkT* __restrict__ U, int64_t link_site, int64_t nb,
                                        float coef, int64_t vol, int a, int a1, int a2, int src1, int src2) {
     // spins 0..3 of colour a at the neighbour
@@ -803,7 +803,7 @@ __device__ __forceinline__ void hop_cs(Cx<float> (&acc)[4], const float2* __rest
 }
 
 template <class LinkT, int NU, bool NAT>
-__device__ __forceinline__ void both_hops_cs(Cx<float> (&acc)[4], const float2* __restrict__ fin, bool act,
+__device__ __forceinline__ void both_hops_cs(Cx<float> (&acc)[4], const float2* fin, bool act,
                                              const LinkT* __restrict__ U, int64_t site, const int co[4],
                                              const StencilParams& P, int a, int a1, int a2, int src1, int src2) {
     int64_t stride = 1;
@@ -828,8 +828,8 @@ __device__ __forceinline__ void both_hops_cs(Cx<float> (&acc)[4], const float2* 
 
 template <class LinkT, bool CS, bool NAT>
 __global__ void __launch_bounds__(256, 4)
-    k_hw_cs(float2* __restrict__ out, const float2* __restrict__ in, const LinkT* __restrict__ U, int nrhs,
-            StencilParams P, const int* __restrict__ skip, int ngrp, int fw) {
+    k_hw_cs(float2* __restrict__ out, const float2* in, const LinkT* __restrict__ U, int nrhs,
+            StencilParams P, const int* skip, int ngrp, int fw) {
     pdl_begin();
     const int warp = threadIdx.y, lane = threadIdx.x;
     const int64_t tile = blockIdx.x / (unsigned)ngrp;

@@ -53,8 +53,8 @@ __device__ __forceinline__ int64_t entry(int64_t site, int k, int64_t vol) {
 // every hop is scaled by its own coefficient (dH_W/dmu, whose space hops are zero).
 template <bool NAT, bool RATIO>
 __global__ void __launch_bounds__(kMaxThreads, 4)
-    k_hw_hops(double2* __restrict__ out, const double2* __restrict__ in, const double2* __restrict__ U, int nrhs,
-              StencilParams P, HopRatios Q, const int* __restrict__ skip) {
+    k_hw_hops(double2* out, const double2* in, const double2* __restrict__ U, int nrhs,
+              StencilParams P, HopRatios Q, const int* skip) {
     pdl_begin();
     const int64_t tile = blockIdx.x / (unsigned)nrhs;
     const int rhs = (int)(blockIdx.x - tile * nrhs);
@@ -96,10 +96,10 @@ __global__ void __launch_bounds__(kMaxThreads, 4)
     double2 h0[3], h1[3], qa[3], qb[3], u[9];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        h0[c] = __ldg(f + entry<NAT>(nb, c, P.vol));
-        h1[c] = __ldg(f + entry<NAT>(nb, 3 + c, P.vol));
-        qa[c] = __ldg(f + entry<NAT>(nb, ka + c, P.vol));
-        qb[c] = __ldg(f + entry<NAT>(nb, kb + c, P.vol));
+        h0[c] = *(f + entry<NAT>(nb, c, P.vol));
+        h1[c] = *(f + entry<NAT>(nb, 3 + c, P.vol));
+        qa[c] = *(f + entry<NAT>(nb, ka + c, P.vol));
+        qb[c] = *(f + entry<NAT>(nb, kb + c, P.vol));
     }
     const double2* lb = U + (int64_t)nu * 9 * P.vol + (fwd ? site : nb);
     const int ra = fwd ? 3 : 1, rb = fwd ? 1 : 3;
@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(kMaxThreads, 4)
     for (int i = 0; i < 3; ++i) {
         const int r = 3 * l + i;
         at[i] = 2 * entry<NAT>(site, r >> 1, P.vol) + (r & 1);
-        psi[i] = __ldg(own + at[i]);
+        psi[i] = own[at[i]];
     }
     // spin projection h = psi_up + S B psi_dn, S = -1 forward, +1 backward (see stencil.cu)
     const unsigned sS = fwd ? NEG : 0u;

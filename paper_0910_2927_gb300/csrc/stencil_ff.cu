@@ -88,8 +88,8 @@ __device__ __forceinline__ ffc phase(ffc v, bool imag, unsigned c) {
     const ff a = imag ? v.im : v.re, b = imag ? v.re : v.im;
     return {flip(a, imag ? c ^ 0x80000000u : c), flip(b, c)};
 }
-__device__ __forceinline__ ffc ld(const float4* __restrict__ p) {
-    const float4 v = __ldg(p);
+__device__ __forceinline__ ffc ld(const float4* p) {
+    const float4 v = *p;
     return {{v.x, v.z}, {v.y, v.w}};
 }
 __device__ __forceinline__ ff shfl_xor(ff a, int o) {
@@ -120,7 +120,7 @@ struct FfResidual {
 // CTA b: site tile b / nrhs (blockDim.x / 8 sites) of field b % nrhs.
 template <bool NAT, FfOut OUT>
 __global__ void __launch_bounds__(kMaxThreads, 4)
-    k_hw_ff(void* __restrict__ out, const float4* __restrict__ in, const float4* __restrict__ Uf, int nrhs,
+    k_hw_ff(void* out, const float4* in, const float4* Uf, int nrhs,
             StencilParams P, FfResidual R) {
     pdl_begin();
     const int64_t tile = blockIdx.x / (unsigned)nrhs;
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(kMaxThreads, 4)
     for (int i = 0; i < 3; ++i) {
         const int r = 3 * l + i, im = r & 1;
         const int64_t e = entry<NAT>(site, r >> 1, P.vol);
-        const ff psi = {__ldg(own + 4 * e + im), __ldg(own + 4 * e + 2 + im)};
+        const ff psi = {own[4 * e + im], own[4 * e + 2 + im]};
         ff z = ff_add_u(ff_mul(psi, d), y[i]);
         z = flip(two_sum(z.hi, z.lo), g5);
         const int64_t o = rhs * P.stride_rhs + e;
@@ -253,16 +253,16 @@ __global__ void __launch_bounds__(kMaxThreads, 4)
                 *q = zd;
             } else {
                 const int sh = rhs / R.ncol, col = rhs - sh * R.ncol;
-                const double bv = __ldg(reinterpret_cast<const double*>(R.b + col * P.stride_rhs + e) + im);
-                const double xv = __ldg(reinterpret_cast<const double*>(R.x + o) + im);
-                *q = fma(__ldg(R.sigma + sh), xv, bv - zd);
+                const double bv = reinterpret_cast<const double*>(R.b + col * P.stride_rhs + e)[im];
+                const double xv = reinterpret_cast<const double*>(R.x + o)[im];
+                *q = fma(R.sigma[sh], xv, bv - zd);
             }
         }
     }
 }
 
 // complex128 -> float-float, elementwise
-__global__ void k_split_ff(const double2* __restrict__ in, float4* __restrict__ out, int64_t count) {
+__global__ void k_split_ff(const double2* in, float4* out, int64_t count) {
     pdl_begin();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
         const double2 v = in[i];
