@@ -501,9 +501,9 @@ SGN_API int sgn_hw_apply(sgn_ctx* c, const void* in, void* out, int nrhs, int pr
     if (precision == SGN_PREC_FP64) {
         const double2* pi = reinterpret_cast<const double2*>(in);
         double2* po = reinterpret_cast<double2*>(out);
-        if (ffa) {  // the float-float copy of the input; both stencils read and write either order
+        if (ffa) {  // the float-float copy of the input; the result goes out in the caller's order
             SGN_CHECK(dev_alloc(c, c->stage, nn * sizeof(float4)));
-            SGN_CUDA(split_ff(pi, as<float4>(c->stage), (int64_t)nn, c->work));
+            SGN_CUDA(split_fields_ff(pi, as<float4>(c->stage), c->vol, nrhs, !packed, c->work));
             SGN_CUDA(hw_ff_doubles(po, as<float4>(c->stage), as<float4>(c->Uff), nrhs, stencil_params(c, adjoint),
                                    !packed, c->work));
         } else {

@@ -153,17 +153,19 @@ cudaError_t launch_hw_f32_bf16links(float2* out, const float2* in, const __nv_bf
                                     StencilShape sh = {}, bool nat = false);
 cudaError_t launch_hw_f32_f16links(float2* out, const float2* in, const __half2* U, int nrhs,
                                    const StencilParams& p, const int* skip, cudaStream_t st, StencilShape sh = {}, bool nat = false);
-// Float-float stencil (stencil_ff.cu): fields and links as a float4 (Re hi, Im hi, Re lo, Im lo) per
-// complex number, in the place the complex128 number has (packed, or natural with nat); about
-// 1e-13 of the FP64 result.  The result as float-float, as complex128, or as the true residuals
-// r_f = b_c - H in_f + sigma_i x_f of fields f = i ncol + c (sigma: device, one per shift).
+// Float-float stencil (stencil_ff.cu): a float4 (Re hi, Im hi, Re lo, Im lo) per complex number,
+// fields in entry planes (entry k of site s at k vol + s), links in the packed order; about 1e-13 of
+// the FP64 result.  The result as float-float planes, as complex128 (natural order with nat, else
+// packed), or as the true residuals r_f = b_c - H in_f + sigma_i x_f (packed complex128) of fields
+// f = i ncol + c (sigma: device, one per shift).
 cudaError_t hw_ff(float4* out, const float4* in, const float4* Uf, int nrhs, const StencilParams& p, cudaStream_t st);
 cudaError_t hw_ff_doubles(double2* out, const float4* in, const float4* Uf, int nrhs, const StencilParams& p, bool nat,
                           cudaStream_t st);
 cudaError_t hw_ff_residual(double2* r, const float4* in, const float4* Uf, int nrhs, const StencilParams& p,
                            const double2* b, int ncol, const double2* x, const double* sigma, cudaStream_t st);
-// complex128 -> float-float, elementwise (fields and links)
+// complex128 -> float-float: elementwise (links), and fields (natural with nat, else packed) to planes.
 cudaError_t split_ff(const double2* in, float4* out, int64_t count, cudaStream_t st);
+cudaError_t split_fields_ff(const double2* in, float4* out, int64_t vol, int nfield, bool nat, cudaStream_t st);
 
 // ------------------------------------------------------------ vector ops --
 // A "basis" is J fields per column: element e of vector j of column r lives at

@@ -1297,7 +1297,7 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
             for (int i = 0; i < s; i += fsh) {
                 const int g = std::min(fsh, s - i), nc = g * ncol;
                 const double2* xi = xs + (size_t)i * nf;
-                SGN_CUDA(split_ff(xi, xf, (int64_t)(g * nf), st));
+                SGN_CUDA(split_fields_ff(xi, xf, c->vol, nc, false, st));
                 SGN_CUDA(hw_ff(tf, xf, Uf, nc, pf, st));
                 SGN_CUDA(hw_ff_residual(rsd + (size_t)i * nf, tf, Uf, nc, pf, bt, ncol, xi, sig_dev + i, st));
             }

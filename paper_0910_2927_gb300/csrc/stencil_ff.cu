@@ -9,14 +9,20 @@
 // rate: the FP64 stencil is bound by the FP64 pipe.  The float-float stencil reaches ~1e-13 of the
 // FP64 result with FP32 instructions only.
 //
-// Layout: a float4 (Re hi, Im hi, Re lo, Im lo) per complex number, in the place the complex128
-// number has in the natural or the packed order, so that conversion is elementwise; links too.
-// Eight lanes per site and field, one per hop, as in stencil_f64.cu (see there for the hop-dependent
-// selects): about 1,500 instructions per lane.  One thread per site (11,000) needed 128 registers
-// for its accumulators and waited for loads most of the time (FMA pipe 32 % busy).  Measured per
-// launch: 16^4 x 4 fields 201 -> 179 us, 10^4 x 12 85 -> 76; 6^4 x 1 27.5 us per shift, now 20 us for
-// twenty shifts together.  The conversions were bound by FP64 conversion instructions (cvt.cuh): split
-// 47 -> 31 us on 16^4 x 4; the join (36 us) and the residual assembly are part of the stencil.
+// Layout: fields as twelve planes, one per spin-colour entry k = 3 spin + colour, of a float4
+// (Re hi, Im hi, Re lo, Im lo) per site (entry k of site s at k vol + s), links as [dir][3][3][site]
+// of the same float4: every load of a warp is 512 contiguous bytes.
+// A CTA takes 32 sites of one field with a warp per hop (direction, forward or backward): a warp
+// projects its neighbours, multiplies by its links and leaves the two colour vectors in shared
+// memory (24 KB), then six warps add the eight hops, a colour and a spin half each, and write the
+// result.  No thread holds a site's 48 accumulators: 80 registers, 24 warps per SM.
+// What bounds it: about 3,000 warp instructions per 32 sites and field, nearly all of them FP32.
+// Measured us per launch at 10^4 x 12 fields, thread per site (128 registers, waiting for loads: FMA
+// pipe 32 % busy) / eight lanes per site, one per hop (L1 79 % busy with up to 32 lines per load) /
+// now: 85 / 76 / 65; 6^4 x 1 27.5 per shift / 20 / 19 for twenty shifts together; a whole call on
+// 16^4 x 4 fields 357 / 213 / 172.  The conversions were bound by FP64 conversion instructions
+// (cvt.cuh): splitting 10^4 x 12 fields 23 -> 10 us; the join and the residual assembly (29 us) are
+// part of the stencil.
 #include "cvt.cuh"
 #include "sgn_internal.cuh"
 
@@ -83,27 +89,17 @@ __device__ __forceinline__ ffc cadd(ffc a, ffc b) { return {ff_add_u(a.re, b.re)
 // x with its sign flipped where mask is 0x80000000 (0: unchanged)
 __device__ __forceinline__ float flip(float x, unsigned mask) { return __uint_as_float(__float_as_uint(x) ^ mask); }
 __device__ __forceinline__ ff flip(ff a, unsigned mask) { return {flip(a.hi, mask), flip(a.lo, mask)}; }
-// c v (imag = false) or c i v (imag = true), c = +-1 given by its sign mask
-__device__ __forceinline__ ffc phase(ffc v, bool imag, unsigned c) {
-    const ff a = imag ? v.im : v.re, b = imag ? v.re : v.im;
-    return {flip(a, imag ? c ^ 0x80000000u : c), flip(b, c)};
+// c v, or c i v with IMAG, c = +-1 given by its sign mask
+template <bool IMAG>
+__device__ __forceinline__ ffc phase(ffc v, unsigned c) {
+    if constexpr (IMAG) return {flip(v.im, c ^ 0x80000000u), flip(v.re, c)};
+    return {flip(v.re, c), flip(v.im, c)};
 }
-__device__ __forceinline__ ffc ld(const float4* p) {
-    const float4 v = *p;
-    return {{v.x, v.z}, {v.y, v.w}};
-}
-__device__ __forceinline__ ff shfl_xor(ff a, int o) {
-    return {__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
-}
-__device__ __forceinline__ ff sel(bool c, ff a, ff b) { return {c ? a.hi : b.hi, c ? a.lo : b.lo}; }
+__device__ __forceinline__ ffc ffc_of(float4 v) { return {{v.x, v.z}, {v.y, v.w}}; }
+__device__ __forceinline__ ffc ld(const float4* p) { return ffc_of(*p); }
 
-// Offset of entry k of a site: natural order, or plane k/2 of the packed order.
-template <bool NAT>
-__device__ __forceinline__ int64_t entry(int64_t site, int k, int64_t vol) {
-    return NAT ? site * 12 + k : (int64_t)(k >> 1) * 2 * vol + 2 * site + (k & 1);
-}
-
-constexpr int kMaxThreads = 128;
+constexpr int kSites = 32;
+constexpr int kThreads = 8 * kSites;  // a warp per hop
 
 // What becomes of H psi.
 enum FfOut {
@@ -117,157 +113,185 @@ struct FfResidual {
     int ncol;
 };
 
-// CTA b: site tile b / nrhs (blockDim.x / 8 sites) of field b % nrhs.
-template <bool NAT, FfOut OUT>
-__global__ void __launch_bounds__(kMaxThreads, 4)
-    k_hw_ff(void* out, const float4* in, const float4* Uf, int nrhs,
-            StencilParams P, FfResidual R) {
-    pdl_begin();
-    const int64_t tile = blockIdx.x / (unsigned)nrhs;
-    const int rhs = (int)(blockIdx.x - tile * nrhs);
-    const int64_t s0 = tile * (blockDim.x >> 3) + (threadIdx.x >> 3);
-    const bool act = s0 < P.vol;
-    const int64_t site = act ? s0 : P.vol - 1;  // idle lanes take part in the shuffles
-    const int l = threadIdx.x & 7, nu = l >> 1;
-    const bool fwd = !(l & 1);
-    const float4* f = in + rhs * P.stride_rhs;
-
-    int co, L;
-    int64_t stride;
-    {
-        const uint32_t q0 = P.div[0].div((uint32_t)site);
-        const uint32_t q1 = P.div[1].div(q0);
-        const uint32_t q2 = P.div[2].div(q1);
-        const int c0 = (int)((uint32_t)site - q0 * (uint32_t)P.L[0]), c1 = (int)(q0 - q1 * (uint32_t)P.L[1]),
-                  c2 = (int)(q1 - q2 * (uint32_t)P.L[2]), c3 = (int)q2;
-        co = nu < 2 ? (nu == 0 ? c0 : c1) : (nu == 2 ? c2 : c3);
-        L = nu < 2 ? (nu == 0 ? P.L[0] : P.L[1]) : (nu == 2 ? P.L[2] : P.L[3]);
-        const int64_t s1 = P.L[0], s2 = s1 * P.L[1], s3 = s2 * P.L[2];
-        stride = nu < 2 ? (nu == 0 ? 1 : s1) : (nu == 2 ? s2 : s3);
-    }
-    const bool wrap = fwd ? co == L - 1 : co == 0;
-    const int64_t nb = fwd ? (wrap ? site - (int64_t)(L - 1) * stride : site + stride)
-                           : (wrap ? site + (int64_t)(L - 1) * stride : site - stride);
-    const int apf = nu < 2 ? (nu == 0 ? P.ap[0] : P.ap[1]) : (nu == 2 ? P.ap[2] : P.ap[3]);
-
-    const unsigned NEG = 0x80000000u;
-    const unsigned bs = wrap && apf ? NEG : 0u;  // sign of a hop across an antiperiodic boundary
-    const bool imag = !(nu & 1);
-    const int ka = nu < 2 ? 9 : 6, kb = nu < 2 ? 6 : 9;
-    // spin projection h = psi_up + S B psi_dn, S = -1 forward, +1 backward
-    const unsigned sS = fwd ? NEG : 0u;
-    const unsigned c0 = nu == 3 ? sS : sS ^ NEG;  // factors of the paired spins: -S, -S, -S, S (times i for nu even)
-    const unsigned c1 = nu == 0 ? sS ^ NEG : sS;  // -S, S, S, S
-    ffc h0[3], h1[3], u[9];
-    const float4* lb = Uf + (int64_t)nu * 9 * P.vol + (fwd ? site : nb);
-    const int ra = fwd ? 3 : 1, rb = fwd ? 1 : 3;
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b) u[3 * a + b] = ld(lb + (int64_t)(ra * a + rb * b) * P.vol);
+// One hop of a warp's 32 sites: g = W (1 + S gamma_nu) psi(nb), boundary sign included, in units of
+// -1/2; sm[4 a + {0..3}] = Re, Im of the two colour vectors' entry a.  IMAG: the projector pairs the
+// spins with +-i (nu = 0, 2).  All other arguments are uniform over the warp: signs as masks, ka
+// and kb the entries of the lower spins that pair with spins 0 and 1.
+template <bool IMAG>
+__device__ __forceinline__ void hop(float2 (*sm)[kSites], const float4* f,
+                                    const float4* __restrict__ lb, int64_t vol, int ka, int kb, unsigned c0,
+                                    unsigned c1, unsigned bs, unsigned cj, int ra, int rb, bool time, ff tc) {
+    const int lane = threadIdx.x & 31;
+    ffc h0[3], h1[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const ffc p0 = ld(f + entry<NAT>(nb, c, P.vol)), p1 = ld(f + entry<NAT>(nb, 3 + c, P.vol));
-        const ffc qa = ld(f + entry<NAT>(nb, ka + c, P.vol)), qb = ld(f + entry<NAT>(nb, kb + c, P.vol));
-        h0[c] = cadd(p0, phase(qa, imag, c0));
-        h1[c] = cadd(p1, phase(qb, imag, c1));
+        const ffc p = cadd(ld(f + c * vol), phase<IMAG>(ld(f + (ka + c) * vol), c0));
+        const ffc q = cadd(ld(f + (3 + c) * vol), phase<IMAG>(ld(f + (kb + c) * vol), c1));
+        h0[c] = {flip(p.re, bs), flip(p.im, bs)};
+        h1[c] = {flip(q.re, bs), flip(q.im, bs)};
     }
-    const unsigned cj = fwd ? 0u : NEG;
-    const ff tc = fwd ? ff{P.cf32[3], P.cf_lo[3]} : ff{P.cb32[3], P.cb_lo[3]};
-    const float sc = fwd ? (nu == 0 ? P.cf32[0] : nu == 1 ? P.cf32[1] : P.cf32[2])
-                         : (nu == 0 ? P.cb32[0] : nu == 1 ? P.cb32[1] : P.cb32[2]);  // -1/2: exact
-    ff v[24];  // the hop's contribution: spins 0, 1 from g0, g1, spins 2, 3 by reconstruction
-    const unsigned c3 = (nu == 1 || nu == 2) ? sS ^ NEG : sS;  // spin 3: S, -S, -S, S (times i for nu even)
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         Dot g0r, g0i, g1r, g1i;
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
-            const ff ur = u[3 * a + b].re, ui = flip(u[3 * a + b].im, cj), nui = flip(ui, NEG);
-            g0r.add(ur, h0[b].re);
+            const ffc u = ffc_of(__ldg(lb + (int64_t)(ra * a + rb * b) * vol));
+            const ff ui = flip(u.im, cj), nui = {-ui.hi, -ui.lo};
+            g0r.add(u.re, h0[b].re);
             g0r.add(nui, h0[b].im);
-            g0i.add(ur, h0[b].im);
+            g0i.add(u.re, h0[b].im);
             g0i.add(ui, h0[b].re);
-            g1r.add(ur, h1[b].re);
+            g1r.add(u.re, h1[b].re);
             g1r.add(nui, h1[b].im);
-            g1i.add(ur, h1[b].im);
+            g1i.add(u.re, h1[b].im);
             g1i.add(ui, h1[b].re);
         }
         ff g[4] = {g0r.value(), g0i.value(), g1r.value(), g1i.value()};
+        if (time)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) g[k] = ff_mul(g[k], tc);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) sm[4 * a + k][lane] = make_float2(g[k].hi, g[k].lo);
+    }
+}
+
+// CTA b: 32 sites from 32 (b / nrhs) of field b % nrhs (the fields of a site tile run together and
+// share its links in L2).  NAT: complex128 output in natural order, else packed.
+template <FfOut OUT, bool NAT>
+__global__ void __launch_bounds__(kThreads, 3)
+    k_hw_ff(void* out, const float4* in, const float4* __restrict__ Uf, int nrhs,
+            StencilParams P, FfResidual R) {
+    pdl_begin();
+    __shared__ float2 sm[8][12][kSites];  // [hop][colour a: g0 re, g0 im, g1 re, g1 im][site]
+    const int64_t tile = blockIdx.x / (unsigned)nrhs;
+    const int rhs = (int)(blockIdx.x - tile * nrhs);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t s0 = tile * kSites + lane;
+    const int64_t site = s0 < P.vol ? s0 : P.vol - 1;  // the last tile's idle lanes repeat a site
+    const float4* f = in + rhs * P.stride_rhs;
+    {
+        const int nu = warp >> 1;
+        const bool fwd = !(warp & 1);
+        const uint32_t q0 = P.div[0].div((uint32_t)site);
+        const uint32_t q1 = P.div[1].div(q0);
+        const uint32_t q2 = P.div[2].div(q1);
+        const int co = nu == 0   ? (int)((uint32_t)site - q0 * (uint32_t)P.L[0])
+                       : nu == 1 ? (int)(q0 - q1 * (uint32_t)P.L[1])
+                       : nu == 2 ? (int)(q1 - q2 * (uint32_t)P.L[2])
+                                 : (int)q2;
+        const int L = P.L[nu];
+        const int64_t s1 = P.L[0], s2 = s1 * P.L[1], s3 = s2 * P.L[2];
+        const int64_t stride = nu == 0 ? 1 : nu == 1 ? s1 : nu == 2 ? s2 : s3;
+        const bool wrap = fwd ? co == L - 1 : co == 0;
+        const int64_t nb = fwd ? (wrap ? site - (int64_t)(L - 1) * stride : site + stride)
+                               : (wrap ? site + (int64_t)(L - 1) * stride : site - stride);
+        const unsigned NEG = 0x80000000u;
+        const unsigned bs = wrap && P.ap[nu] ? NEG : 0u;  // a hop across an antiperiodic boundary
+        // spin projection h = psi_up + S B psi_dn, S = -1 forward, +1 backward (see stencil.cu)
+        const unsigned sS = fwd ? NEG : 0u;
+        const unsigned c0 = nu == 3 ? sS : sS ^ NEG;  // factors of the paired spins: -S, -S, -S, S
+        const unsigned c1 = nu == 0 ? sS ^ NEG : sS;  // -S, S, S, S (times i for nu even)
+        const int ka = nu < 2 ? 9 : 6, kb = nu < 2 ? 6 : 9;
+        const float4* lb = Uf + (int64_t)nu * 9 * P.vol + (fwd ? site : nb);
+        const unsigned cj = fwd ? 0u : NEG;
+        const int ra = fwd ? 3 : 1, rb = fwd ? 1 : 3;  // U(site), or the transpose of U(nb), conjugated
+        // the time hops' coefficient -1/2 e^{+-mu} over the space hops' -1/2
+        const ff tc = fwd ? ff{-2.f * P.cf32[3], -2.f * P.cf_lo[3]} : ff{-2.f * P.cb32[3], -2.f * P.cb_lo[3]};
+        if (nu & 1)
+            hop<false>(sm[warp], f + nb, lb, P.vol, ka, kb, c0, c1, bs, cj, ra, rb, nu == 3, tc);
+        else
+            hop<true>(sm[warp], f + nb, lb, P.vol, ka, kb, c0, c1, bs, cj, ra, rb, false, tc);
+    }
+    __syncthreads();
+    if (warp >= 6 || s0 >= P.vol) return;
+    // warp: colour a, upper (spins 0, 1) or lower (2, 3) half
+    const bool lower = warp >= 3;
+    const int a = lower ? warp - 3 : warp, k0 = lower ? 6 + a : a;  // entries k0 and k0 + 3
+    const ffc p0 = ld(f + k0 * P.vol + site), p1 = ld(f + (k0 + 3) * P.vol + site);
+    ff z[4];  // Re, Im of the two entries: the sum over the hops
+#pragma unroll
+    for (int h = 0; h < 8; ++h) {
+        ff g[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            g[k] = nu == 3 ? ff_mul(g[k], tc) : ff{g[k].hi * sc, g[k].lo * sc};
-            g[k] = flip(g[k], bs);
+            const float2 v = sm[h][4 * a + k][lane];
+            g[k] = {v.x, v.y};
         }
-        const ffc g0 = {g[0], g[1]}, g1 = {g[2], g[3]};
-        const ffc e2 = {sel(nu < 2, g1.re, g0.re), sel(nu < 2, g1.im, g0.im)},
-                  e3 = {sel(nu < 2, g0.re, g1.re), sel(nu < 2, g0.im, g1.im)};
-        const ffc l2 = phase(e2, imag, sS), l3 = phase(e3, imag, c3);
-        v[2 * a] = g0.re;
-        v[2 * a + 1] = g0.im;
-        v[6 + 2 * a] = g1.re;
-        v[6 + 2 * a + 1] = g1.im;
-        v[12 + 2 * a] = l2.re;
-        v[12 + 2 * a + 1] = l2.im;
-        v[18 + 2 * a] = l3.re;
-        v[18 + 2 * a + 1] = l3.im;
-    }
-    // sum over the eight hops: at each level a lane keeps one half of its numbers and adds the
-    // partner's same half; lane l ends with numbers 3 l .. 3 l + 2
-    ff w[12], x[6], y[3];
+        ff e[4] = {g[0], g[1], g[2], g[3]};
+        if (lower) {  // S B^dag g: (i g1, i g0), (g1, -g0), (i g0, -i g1), (g0, g1) for nu = 0..3
+            const int nu = h >> 1;
+            const int src0 = nu < 2 ? 2 : 0, src1 = nu < 2 ? 0 : 2;
+            const bool im = !(nu & 1);
+            const unsigned S = h & 1 ? 0u : 0x80000000u;                      // backward +, forward -
+            const unsigned T = (nu == 1 || nu == 2) ? S ^ 0x80000000u : S;  // of the second entry
+            e[0] = im ? flip(g[src0 + 1], S ^ 0x80000000u) : flip(g[src0], S);
+            e[1] = im ? flip(g[src0], S) : flip(g[src0 + 1], S);
+            e[2] = im ? flip(g[src1 + 1], T ^ 0x80000000u) : flip(g[src1], T);
+            e[3] = im ? flip(g[src1], T) : flip(g[src1 + 1], T);
+        }
 #pragma unroll
-    for (int i = 0; i < 12; ++i) {
-        const bool up = l & 4;
-        w[i] = ff_add_u(sel(up, v[12 + i], v[i]), shfl_xor(sel(up, v[i], v[12 + i]), 4));
+        for (int k = 0; k < 4; ++k) z[k] = h == 0 ? e[k] : ff_add_u(z[k], e[k]);
     }
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        const bool up = l & 2;
-        x[i] = ff_add_u(sel(up, w[6 + i], w[i]), shfl_xor(sel(up, w[i], w[6 + i]), 2));
-    }
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        const bool up = l & 1;
-        y[i] = ff_add_u(sel(up, x[3 + i], x[i]), shfl_xor(sel(up, x[i], x[3 + i]), 1));
-    }
-    if (!act) return;
-    const unsigned g5 = l & 4 ? NEG : 0u;  // gamma5 = diag(1, 1, -1, -1): numbers 12.. are spins 2, 3
-    const float* own = reinterpret_cast<const float*>(f);
+    const unsigned g5 = lower ? 0x80000000u : 0u;  // gamma5 = diag(1, 1, -1, -1)
     const ff d = {P.diag32, P.diag_lo};
+    const ff psi[4] = {p0.re, p0.im, p1.re, p1.im};
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        const int r = 3 * l + i, im = r & 1;
-        const int64_t e = entry<NAT>(site, r >> 1, P.vol);
-        const ff psi = {own[4 * e + im], own[4 * e + 2 + im]};
-        ff z = ff_add_u(ff_mul(psi, d), y[i]);
-        z = flip(two_sum(z.hi, z.lo), g5);
-        const int64_t o = rhs * P.stride_rhs + e;
+    for (int k = 0; k < 4; ++k) {
+        const ff v = ff_add_u(ff_mul(psi[k], d), {-0.5f * z[k].hi, -0.5f * z[k].lo});
+        z[k] = flip(two_sum(v.hi, v.lo), g5);
+    }
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const int k = k0 + 3 * e;
+        const ff re = z[2 * e], im = z[2 * e + 1];
+        const int64_t base = rhs * P.stride_rhs;
         if constexpr (OUT == FF_PAIRS) {
-            float* q = reinterpret_cast<float*>(out) + 4 * o;
-            q[im] = z.hi;
-            q[2 + im] = z.lo;
+            reinterpret_cast<float4*>(out)[base + k * P.vol + site] = make_float4(re.hi, im.hi, re.lo, im.lo);
         } else {
-            const double zd = f2d(z.hi) + f2d(z.lo);
-            double* q = reinterpret_cast<double*>(out) + 2 * o + im;
-            if constexpr (OUT == FF_DOUBLES) {
-                *q = zd;
-            } else {
+            const int64_t o = NAT ? site * 12 + k : (int64_t)(k >> 1) * 2 * P.vol + 2 * site + (k & 1);
+            double2 v = make_double2(f2d(re.hi) + f2d(re.lo), f2d(im.hi) + f2d(im.lo));
+            if constexpr (OUT == FF_RESIDUAL) {
                 const int sh = rhs / R.ncol, col = rhs - sh * R.ncol;
-                const double bv = reinterpret_cast<const double*>(R.b + col * P.stride_rhs + e)[im];
-                const double xv = reinterpret_cast<const double*>(R.x + o)[im];
-                *q = fma(R.sigma[sh], xv, bv - zd);
+                const double2 b = R.b[col * P.stride_rhs + o], x = R.x[base + o];
+                const double sg = R.sigma[sh];
+                v = make_double2(fma(sg, x.x, b.x - v.x), fma(sg, x.y, b.y - v.y));
             }
+            reinterpret_cast<double2*>(out)[base + o] = v;
         }
     }
 }
 
+__device__ __forceinline__ float4 split1(double2 v) {
+    const float2 re = d2ff(v.x), im = d2ff(v.y);
+    return make_float4(re.x, im.x, re.y, im.y);
+}
 // complex128 -> float-float, elementwise
-__global__ void k_split_ff(const double2* in, float4* out, int64_t count) {
-    pdl_begin();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
-        const double2 v = in[i];
-        const float2 re = d2ff(v.x), im = d2ff(v.y);
-        out[i] = make_float4(re.x, im.x, re.y, im.y);
+__global__ void k_split_ff(const double2* __restrict__ in, float4* __restrict__ out, int64_t count) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x)
+        out[i] = split1(in[i]);
+}
+// complex128 fields (NAT: natural order, else packed) -> entry planes.  CTA: 32 sites of field blockIdx.y;
+// natural-order entries turn through shared memory.
+template <bool NAT>
+__global__ void __launch_bounds__(128) k_split_fields_ff(const double2* __restrict__ in, float4* __restrict__ out,
+                                                         int64_t vol) {
+    const int64_t s0 = (int64_t)blockIdx.x * kSites;
+    const int ns = (int)(vol - s0 < kSites ? vol - s0 : kSites);
+    const double2* f = in + (int64_t)blockIdx.y * 12 * vol;
+    float4* o = out + (int64_t)blockIdx.y * 12 * vol;
+    __shared__ float4 sm[NAT ? 12 * (kSites + 1) : 1];
+    if constexpr (NAT) {
+        for (int i = threadIdx.x; i < 12 * ns; i += 128) sm[(i % 12) * (kSites + 1) + i / 12] = split1(f[s0 * 12 + i]);
+        __syncthreads();
+        for (int i = threadIdx.x; i < 12 * kSites; i += 128) {
+            const int k = i / kSites, s = i % kSites;
+            if (s < ns) o[k * vol + s0 + s] = sm[k * (kSites + 1) + s];
+        }
+    } else {
+        for (int i = threadIdx.x; i < 12 * kSites; i += 128) {  // entries 2 p + j of site s: 2 p vol + 2 s + j
+            const int p = i / (2 * kSites), r = i % (2 * kSites), s = r >> 1, k = 2 * p + (r & 1);
+            if (s < ns) o[k * vol + s0 + s] = split1(f[(int64_t)p * 2 * vol + 2 * s0 + r]);
+        }
     }
 }
 
@@ -276,18 +300,13 @@ unsigned grid_of(int64_t count) {
     return (unsigned)(b < 152 * 16 ? (b > 0 ? b : 1) : 152 * 16);
 }
 
-template <FfOut OUT>
-cudaError_t launch_ff(void* out, const float4* in, const float4* Uf, int nrhs, const StencilParams& p, bool nat,
+template <FfOut OUT, bool NAT>
+cudaError_t launch_ff(void* out, const float4* in, const float4* Uf, int nrhs, const StencilParams& p,
                       const FfResidual& r, cudaStream_t st) {
     if (nrhs <= 0 || p.vol <= 0) return cudaSuccess;
-    // one-warp CTAs (4 sites) while they fit in a few per SM, as in stencil_f64.cu
-    const int threads = p.vol * nrhs < 4 * 16 * 152 ? 32 : kMaxThreads, sites = threads / 8;
-    const int64_t blocks = (p.vol + sites - 1) / sites * nrhs;
+    const int64_t blocks = (p.vol + kSites - 1) / kSites * nrhs;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    if (nat)
-        launch_pdl(k_hw_ff<true, OUT>, (unsigned)blocks, threads, 0, st, out, in, Uf, nrhs, p, r);
-    else
-        launch_pdl(k_hw_ff<false, OUT>, (unsigned)blocks, threads, 0, st, out, in, Uf, nrhs, p, r);
+    launch_pdl(k_hw_ff<OUT, NAT>, (unsigned)blocks, kThreads, 0, st, out, in, Uf, nrhs, p, r);
     count_launch();
     return cudaGetLastError();
 }
@@ -295,21 +314,36 @@ cudaError_t launch_ff(void* out, const float4* in, const float4* Uf, int nrhs, c
 }  // namespace
 
 cudaError_t hw_ff(float4* out, const float4* in, const float4* Uf, int nrhs, const StencilParams& p, cudaStream_t st) {
-    return launch_ff<FF_PAIRS>(out, in, Uf, nrhs, p, false, {}, st);
+    return launch_ff<FF_PAIRS, false>(out, in, Uf, nrhs, p, {}, st);
 }
 cudaError_t hw_ff_doubles(double2* out, const float4* in, const float4* Uf, int nrhs, const StencilParams& p, bool nat,
                           cudaStream_t st) {
-    return launch_ff<FF_DOUBLES>(out, in, Uf, nrhs, p, nat, {}, st);
+    if (nat) return launch_ff<FF_DOUBLES, true>(out, in, Uf, nrhs, p, {}, st);
+    return launch_ff<FF_DOUBLES, false>(out, in, Uf, nrhs, p, {}, st);
 }
 cudaError_t hw_ff_residual(double2* r, const float4* in, const float4* Uf, int nrhs, const StencilParams& p,
                            const double2* b, int ncol, const double2* x, const double* sigma, cudaStream_t st) {
-    return launch_ff<FF_RESIDUAL>(r, in, Uf, nrhs, p, false, {b, x, sigma, ncol}, st);
+    return launch_ff<FF_RESIDUAL, false>(r, in, Uf, nrhs, p, {b, x, sigma, ncol}, st);
 }
 
 cudaError_t split_ff(const double2* in, float4* out, int64_t count, cudaStream_t st) {
     if (count <= 0) return cudaSuccess;
-    launch_pdl(k_split_ff, grid_of(count), 256, 0, st, in, out, count);
+    k_split_ff<<<grid_of(count), 256, 0, st>>>(in, out, count);
     count_launch();
+    return cudaGetLastError();
+}
+cudaError_t split_fields_ff(const double2* in, float4* out, int64_t vol, int nfield, bool nat, cudaStream_t st) {
+    if (nfield <= 0 || vol <= 0) return cudaSuccess;
+    for (int f0 = 0; f0 < nfield; f0 += 65535) {
+        const dim3 grid((unsigned)((vol + kSites - 1) / kSites), nfield - f0 < 65535 ? nfield - f0 : 65535);
+        const double2* i = in + (int64_t)f0 * 12 * vol;
+        float4* o = out + (int64_t)f0 * 12 * vol;
+        if (nat)
+            k_split_fields_ff<true><<<grid, 128, 0, st>>>(i, o, vol);
+        else
+            k_split_fields_ff<false><<<grid, 128, 0, st>>>(i, o, vol);
+        count_launch();
+    }
     return cudaGetLastError();
 }
 
