@@ -137,7 +137,8 @@ cudaError_t pack_links(const double2* natural, double2* packed, int64_t vol, cud
 // pipe = 1 selects the FP32 kernel that stages neighbour spinors through shared
 // memory with cp.async (a stage ahead of the computation; nr <= 2); pipe = 2 the
 // FP32 kernel with paired (FFMA2) arithmetic over two fields (nr = 2), pipe = 3 the
-// same kernel capped at 128 registers.
+// same kernel capped at 128 registers; pipe = 4 the colour-split kernel; pipe = 5 a lane per hop
+// (hops.cuh; rb = 3: and a warp per row of the link).
 struct StencilShape {
     int sx = 0;
     int rb = 0;

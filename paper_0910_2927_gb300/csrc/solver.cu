@@ -149,6 +149,12 @@ int tune_stencil(sgn_ctx* c, int prec, int ncol, void* in, void* out, bool nat) 
     for (int fw : {1, 2, 3, 4, 6, 8})
         for (int sg : {1, 2, 4, 8})
             if (fw <= ncol && sg * fw <= 8 && sg * fw >= 2) cands.push_back({sg, fw, 1, 4});
+    // a lane per hop: an eighth of the chain per thread where threads are few (at most four CTAs of the
+    // other kernels per SM), too many instructions elsewhere
+    if (c->vol * ncol <= 152 * 512) {
+        cands.push_back({32, 1, 1, 5});
+        cands.push_back({32, 3, 1, 5});
+    }
     if (cands.empty()) cands.push_back({});
     auto run = [&](StencilShape sh) -> cudaError_t {
         if (prec == 2)

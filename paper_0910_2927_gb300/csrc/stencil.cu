@@ -11,6 +11,7 @@
 // Each hop uses the rank-2 spin projector (1 -/+ gamma_nu): two colour
 // vectors are multiplied by the link instead of four, and gamma5 is folded
 // into the write (spins 2, 3 negated).
+#include "hops.cuh"
 #include "sgn_internal.cuh"
 
 namespace sgn {
@@ -1014,6 +1015,11 @@ template <class R, class LinkT, bool NAT>
 cudaError_t launch(typename Field<R>::T* out, const typename Field<R>::T* in, const LinkT* U, int nrhs,
                    const StencilParams& p, const int* skip, cudaStream_t st, StencilShape sh) {
     if (nrhs <= 0 || p.vol <= 0) return cudaSuccess;
+    if (sh.pipe == 5) {  // eight lanes per site, one per hop
+        if (sh.nr != 1 || (sh.rb != 1 && sh.rb != 3)) return cudaErrorInvalidValue;
+        if (sh.rb == 3) return hops::launch<R, LinkT, true>(out, in, U, nrhs, p, skip, st, NAT);
+        return hops::launch<R, LinkT, false>(out, in, U, nrhs, p, skip, st, NAT);
+    }
     if (sh.pipe == 4) {  // the colour-split kernel: sx site groups of 10 sites, rb fields per CTA
         if (sh.nr != 1) return cudaErrorInvalidValue;
         return launch_cs<LinkT, NAT>(out, in, U, nrhs, p, skip, st, sh.sx, sh.rb);
