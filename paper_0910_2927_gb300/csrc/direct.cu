@@ -6,8 +6,14 @@
 // Arnoldi steps use the FP64 stencil and two classical Gram-Schmidt passes, in blocks of at
 // most 128 basis vectors per kernel (the reduction's slot limit).  The Newton iterations run
 // on the GPU for all columns at once: X^{-1} by Gauss-Jordan elimination with partial
-// pivoting on [X | I], one launch pair per pivot (captured once as a CUDA graph), with the
+// pivoting on [X | I], one launch per pivot (captured once as a CUDA graph), with the
 // matrices of shorter Krylov dimension padded by the identity (sign(I) = I).
+//
+// What bounds it: the Gram-Schmidt passes' FP64 products (16 multiply-adds per basis entry and step),
+// so nothing else may hold them up: the Hessenberg matrix, the norms and the breakdown flags stay on
+// the device, and the host only looks every 32 steps whether a column is still growing.  With four
+// host round trips per step, a pair of launches per pivot and one CTA for the Newton update,
+// k = 100 on 8^4 x 2 took 43 ms; now 28.
 #include "ctx.cuh"
 #include "dense_eig.h"
 
@@ -24,99 +30,100 @@ __device__ __forceinline__ double2 cdiv_d(double2 a, double2 b) {
     return make_double2((a.x * b.x + a.y * b.y) / den, (a.y * b.x - a.x * b.y) / den);
 }
 
-// Gauss-Jordan step p on the augmented matrices A[col] = [X | I] (q rows, 2q columns,
-// row-major): pivot row = the first row i >= p of largest |A[i][p]|, swapped with row p,
-// row p scaled by 1 / pivot, and the column of elimination factors A[i][p] saved to fac.
-// One CTA per matrix.  A zero pivot (singular X: an eigenvalue of H_k on the imaginary
-// axis) sets bad[col].
-__global__ void __launch_bounds__(256) k_gj_pivot(double2* __restrict__ A, int q, int p, double2* __restrict__ fac,
-                                                  int* __restrict__ bad) {
-    const int col = blockIdx.x;
-    double2* M = A + (size_t)col * q * 2 * q;
-    const int ld = 2 * q;
-    __shared__ double sv[256];
-    __shared__ int si[256];
-    double best = -1.0;
-    int bi = p;
-    for (int i = p + threadIdx.x; i < q; i += blockDim.x) {
-        const double2 v = M[(size_t)i * ld + p];
-        const double a = v.x * v.x + v.y * v.y;
-        if (a > best) {
-            best = a;
-            bi = i;
-        }
-    }
-    sv[threadIdx.x] = best;
-    si[threadIdx.x] = bi;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {  // ties keep the lower row (first maximal pivot)
-        if (threadIdx.x < s) {
-            const double o = sv[threadIdx.x + s];
-            const int oi = si[threadIdx.x + s];
-            if (o > sv[threadIdx.x] || (o == sv[threadIdx.x] && oi < si[threadIdx.x])) {
-                sv[threadIdx.x] = o;
-                si[threadIdx.x] = oi;
-            }
-        }
-        __syncthreads();
-    }
-    const int r = si[0];
-    if (!(sv[0] > 0.0)) {
-        if (threadIdx.x == 0) bad[col] = 1;
-        return;
-    }
-    if (r != p)
-        for (int j = threadIdx.x; j < ld; j += blockDim.x) {
-            const double2 t = M[(size_t)p * ld + j];
-            M[(size_t)p * ld + j] = M[(size_t)r * ld + j];
-            M[(size_t)r * ld + j] = t;
-        }
-    __syncthreads();
-    const double2 piv = M[(size_t)p * ld + p];
-    __syncthreads();
-    for (int j = threadIdx.x; j < ld; j += blockDim.x) M[(size_t)p * ld + j] = cdiv_d(M[(size_t)p * ld + j], piv);
-    __syncthreads();
-    for (int i = threadIdx.x; i < q; i += blockDim.x) fac[(size_t)col * q + i] = M[(size_t)i * ld + p];
-}
+constexpr int GJ_COLS = 4;  // columns per CTA of an elimination step
 
-// A[i][j] -= fac[i] A[p][j] for every row i != p (columns j >= p on the left half carry
-// the reduction; the right half is the inverse being formed).
-__global__ void __launch_bounds__(256) k_gj_eliminate(double2* __restrict__ A, int q, int p,
-                                                      const double2* __restrict__ fac, const int* __restrict__ bad) {
+// Gauss-Jordan step p on the augmented matrices A[col] = [X | I] (q rows, 2q columns, row-major).
+// fac: column p before the step.  Every CTA finds the pivot row r (the first row i >= p of largest
+// |fac[i]|) for itself, and on its columns j > p exchanges rows r and p, scales row p by 1 / pivot and
+// subtracts fac[i] times it from the others; the CTA of column p + 1 leaves that column in next.  A zero
+// pivot (singular X: an eigenvalue of H_k on the imaginary axis), or no finite one, sets bad[col].
+// A latency chain: moduli are compared as bit patterns and one warp forms the reciprocal, as FP64
+// instructions take 64 cycles.
+__global__ void __launch_bounds__(256) k_gj_step(double2* A, int q, int p, const double2* fac, double2* next,
+                                                 int* bad) {
+    pdl_begin();
     const int col = blockIdx.y;
     if (bad[col]) return;
     double2* M = A + (size_t)col * q * 2 * q;
-    const int ld = 2 * q;
-    const int w = ld - p;  // columns p .. 2q-1
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (int64_t)q * w) return;
-    const int i = (int)(e / w);
-    const int j = p + (int)(e - (int64_t)i * w);
-    if (i == p) return;
-    const double2 f = fac[(size_t)col * q + i];
-    const double2 pr = M[(size_t)p * ld + j];
-    double2 v = M[(size_t)i * ld + j];
-    v.x -= f.x * pr.x - f.y * pr.y;
-    v.y -= f.x * pr.y + f.y * pr.x;
-    M[(size_t)i * ld + j] = v;
+    const double2* f = fac + (size_t)col * q;
+    const int ld = 2 * q, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ long long sv[8];
+    __shared__ int si[8];
+    __shared__ double2 pinv_sh;
+    long long best = -1;
+    int r = p;
+    for (int i = p + tid; i < q; i += 256) {
+        const double2 v = f[i];
+        const double a2 = v.x * v.x + v.y * v.y;
+        long long a = __double_as_longlong(a2);
+        if (a >= 0x7ff0000000000000LL) a = -1;  // not finite
+        if (a > best) {
+            best = a;
+            r = i;
+        }
+    }
+    auto take = [&](long long o, int oi) {  // ties keep the lower row (first maximal pivot)
+        if (o > best || (o == best && oi < r)) {
+            best = o;
+            r = oi;
+        }
+    };
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) take(__shfl_xor_sync(0xffffffffu, best, o), __shfl_xor_sync(0xffffffffu, r, o));
+    if (lane == 0) {
+        sv[warp] = best;
+        si[warp] = r;
+    }
+    __syncthreads();
+    for (int w = 0; w < 8; ++w) take(sv[w], si[w]);
+    if (!(best > 0)) {
+        if (blockIdx.x == 0 && tid == 0) bad[col] = 1;
+        return;
+    }
+    if (warp == 0) {
+        const double2 pinv = cdiv_d(make_double2(1.0, 0.0), f[r]);
+        if (lane == 0) pinv_sh = pinv;
+    }
+    const int j = p + 1 + blockIdx.x * GJ_COLS + tid % GJ_COLS;
+    const bool act = j < ld;
+    double2 ar = make_double2(0, 0), ap = ar;
+    if (act) {
+        ar = M[(size_t)r * ld + j];
+        ap = M[(size_t)p * ld + j];
+    }
+    __syncthreads();  // rows r and p are read by all before any of them is written
+    if (!act) return;
+    const double2 prow = cmul(ar, pinv_sh);
+    for (int i = tid / GJ_COLS; i < q; i += 256 / GJ_COLS) {
+        double2 v = prow;
+        if (i != p) {
+            const double2 g = f[i == r ? p : i], o = i == r ? ap : M[(size_t)i * ld + j];
+            v = make_double2(o.x - (g.x * prow.x - g.y * prow.y), o.y - (g.x * prow.y + g.y * prow.x));
+        }
+        M[(size_t)i * ld + j] = v;
+        if (j == p + 1) next[(size_t)col * q + i] = v;
+    }
 }
 
-// [X | I] from X (q x q per column), and after the inversion the Newton update
-// X <- (X + X^{-1}) / 2 with the per-column sums ||X_new - X||^2 and ||X_new||^2.
-__global__ void k_gj_load(const double2* __restrict__ X, double2* __restrict__ A, int q) {
+// [X | I] and its first column from X (q x q per column), and after the inversion the Newton update
+// X <- (X + X^{-1}) / 2 with the sums ||X_new - X||^2 and ||X_new||^2 of each CTA (gridDim.x per column).
+__global__ void k_gj_load(const double2* X, double2* A, double2* fac, int q) {
+    pdl_begin();
     const int col = blockIdx.y;
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (int64_t)q * 2 * q) return;
     const int i = (int)(e / (2 * q)), j = (int)(e - (int64_t)i * 2 * q);
     A[(size_t)col * q * 2 * q + e] =
         j < q ? X[(size_t)col * q * q + (size_t)i * q + j] : make_double2(j - q == i ? 1.0 : 0.0, 0.0);
+    if (j == 0) fac[(size_t)col * q + i] = X[(size_t)col * q * q + (size_t)i * q];
 }
-__global__ void __launch_bounds__(256) k_newton_update(double2* __restrict__ X, const double2* __restrict__ A, int q,
-                                                       double* __restrict__ sums) {
-    const int col = blockIdx.x;
+__global__ void __launch_bounds__(256) k_newton_update(double2* X, const double2* A, int q, double* sums) {
+    pdl_begin();
+    const int col = blockIdx.y;
     __shared__ double sd[256], sx[256];
     double dn = 0, xn = 0;
-    for (int64_t e = threadIdx.x; e < (int64_t)q * q; e += blockDim.x) {
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < (int64_t)q * q;
+         e += (int64_t)gridDim.x * blockDim.x) {
         const int i = (int)(e / q), j = (int)(e - (int64_t)i * q);
         const double2 xo = X[(size_t)col * q * q + e];
         const double2 xi = A[(size_t)col * q * 2 * q + (size_t)i * 2 * q + q + j];
@@ -136,9 +143,74 @@ __global__ void __launch_bounds__(256) k_newton_update(double2* __restrict__ X, 
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        sums[2 * col] = sd[0];
-        sums[2 * col + 1] = sx[0];
+        sums[2 * (col * gridDim.x + blockIdx.x)] = sd[0];
+        sums[2 * (col * gridDim.x + blockIdx.x) + 1] = sx[0];
     }
+}
+
+// Second stage of a Gram-Schmidt pass over J basis vectors from i0: the coefficients go to red and are
+// added to column j of H (k + 1 rows of k per column).  Eight lanes per coefficient.
+__global__ void __launch_bounds__(256) k_direct_coef(Reduce rd, int J, int i0, int j, int k, double2* red, int rs,
+                                                     double2* H) {
+    pdl_begin();
+    const int col = blockIdx.x, slot = blockIdx.y * 32 + threadIdx.x / 8, seg = threadIdx.x & 7;
+    double2 a = make_double2(0, 0);
+    if (slot < J) {
+        const double2* p = rd.partial + ((int64_t)col * rd.stride + slot) * rd.nblk;
+#pragma unroll 8
+        for (int b = seg; b < rd.nblk; b += 8) a = cadd(a, p[b]);
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+        a.x += __shfl_xor_sync(0xffffffffu, a.x, o);
+        a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
+    }
+    if (slot >= J || seg) return;
+    red[(int64_t)col * rs + slot] = a;
+    double2* h = H + ((int64_t)col * (k + 1) + i0 + slot) * k + j;
+    *h = cadd(*h, a);
+}
+
+// The norm of step j (j = -1: of the start vector, to beta): H[j+1][j] = ||w||, scale = 1 / ||w||; a column
+// with ||w|| <= 1e-14 ||A v_j|| has an invariant subspace of dimension kk = j + 1, where the projection
+// is exact: its further basis vectors are zero.
+__global__ void __launch_bounds__(256) k_direct_norm(Reduce rd, int j, int k, double2* H, double* scale, double* beta,
+                                                     int* kk, int* live) {
+    pdl_begin();
+    const int col = blockIdx.x, tid = threadIdx.x;
+    __shared__ double s2[256], sh[256];
+    double a = 0, h2 = 0;
+    const double2* p = rd.partial + (int64_t)col * rd.stride * rd.nblk;
+    for (int b = tid; b < rd.nblk; b += 256) a += p[b].x;
+    for (int i = tid; i <= j; i += 256) h2 += cabs2(H[((int64_t)col * (k + 1) + i) * k + j]);
+    s2[tid] = a;
+    sh[tid] = h2;
+    __syncthreads();
+    for (int s = 128; s > 0; s >>= 1) {
+        if (tid < s) {
+            s2[tid] += s2[tid + s];
+            sh[tid] += sh[tid + s];
+        }
+        __syncthreads();
+    }
+    if (tid != 0) return;
+    const double n2 = s2[0] < 0 ? 0.0 : s2[0], nr = sqrt(n2);  // not finite stays so: the Newton iteration fails
+    double sc = 0.0;
+    if (j < 0) {
+        beta[col] = nr;
+        live[col] = nr > 0;
+        kk[col] = nr > 0 ? k : 0;
+        sc = nr > 0 ? 1.0 / nr : 0.0;
+    } else if (live[col]) {
+        if (nr <= 1e-14 * sqrt(n2 + sh[0])) {
+            live[col] = 0;
+            kk[col] = j + 1;
+        } else {
+            H[((int64_t)col * (k + 1) + j + 1) * k + j] = make_double2(nr, 0);
+            sc = 1.0 / nr;
+        }
+    }
+    scale[col] = sc;
 }
 
 // sign(X_col) for ncol matrices of size q (row-major, device) by Roberts' Newton iteration,
@@ -148,9 +220,10 @@ int newton_sign_gpu(sgn_ctx* c, double2* X, int q, int ncol, int* failed) {
     cudaStream_t st = c->work;
     const size_t aug = (size_t)ncol * q * 2 * q;
     DevBuf buf;
-    const size_t oA = 0, of = align256(sizeof(double2) * aug), ob = of + align256(sizeof(double2) * ncol * q),
+    const int nu = (int)std::min<int64_t>(16, ((int64_t)q * q + 255) / 256);  // CTAs per matrix of the Newton update
+    const size_t oA = 0, of = align256(sizeof(double2) * aug), ob = of + align256(sizeof(double2) * 2 * ncol * q),
                  os = ob + align256(sizeof(int) * ncol);
-    SGN_CHECK(dev_alloc(c, buf, os + align256(sizeof(double) * 2 * ncol)));
+    SGN_CHECK(dev_alloc(c, buf, os + align256(sizeof(double) * 2 * ncol * nu)));
     char* base = reinterpret_cast<char*>(buf.p);
     double2* A = reinterpret_cast<double2*>(base + oA);
     double2* fac = reinterpret_cast<double2*>(base + of);
@@ -160,20 +233,20 @@ int newton_sign_gpu(sgn_ctx* c, double2* X, int q, int ncol, int* failed) {
         dev_free(c, buf);
         return rc;
     };
-    // one inversion = 2q launches: captured once, replayed every Newton step
+    // one inversion = q + 1 launches: captured once, replayed every Newton step
     cudaGraph_t g = nullptr;
     cudaGraphExec_t ge = nullptr;
     cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
         const int64_t cells = (int64_t)q * 2 * q;
-        k_gj_load<<<dim3((unsigned)((cells + 255) / 256), ncol), 256, 0, st>>>(X, A, q);
+        launch_pdl(k_gj_load, dim3((unsigned)((cells + 255) / 256), ncol), 256, 0, st, X, A, fac, q);
+        double2* two[2] = {fac, fac + (size_t)ncol * q};  // column p and column p + 1
         for (int p = 0; p < q && e == cudaSuccess; ++p) {
-            k_gj_pivot<<<ncol, 256, 0, st>>>(A, q, p, fac, bad);
-            const int64_t work = (int64_t)q * (2 * q - p);
-            k_gj_eliminate<<<dim3((unsigned)((work + 255) / 256), ncol), 256, 0, st>>>(A, q, p, fac, bad);
+            launch_pdl(k_gj_step, dim3((2 * q - p - 1 + GJ_COLS - 1) / GJ_COLS, ncol), 256, 0, st, A, q, p, two[p & 1],
+                       two[(p + 1) & 1], bad);
             e = cudaGetLastError();
         }
-        k_newton_update<<<ncol, 256, 0, st>>>(X, A, q, sums);
+        launch_pdl(k_newton_update, dim3(nu, ncol), 256, 0, st, X, A, q, sums);
         cudaError_t ee = cudaStreamEndCapture(st, &g);
         if (e == cudaSuccess) e = ee;
     }
@@ -185,18 +258,18 @@ int newton_sign_gpu(sgn_ctx* c, double2* X, int q, int ncol, int* failed) {
     }
     // per column: 0 iterating, 1 update below 1e-12 of the iterate (one more step to take),
     // 2 finished; every column steps with the others (a converged X is a fixed point)
-    std::vector<double> hs(2 * ncol);
+    std::vector<double> hs(2 * (size_t)ncol * nu);
     std::vector<int> hb(ncol), state(ncol, 0);
     bool launch_ok = cudaMemsetAsync(bad, 0, sizeof(int) * ncol, st) == cudaSuccess;
     for (int it = 0; it < 100 && launch_ok; ++it) {
         if (cudaGraphLaunch(ge, st) != cudaSuccess ||
-            cudaMemcpyAsync(hs.data(), sums, sizeof(double) * 2 * ncol, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+            cudaMemcpyAsync(hs.data(), sums, sizeof(double) * hs.size(), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
             cudaMemcpyAsync(hb.data(), bad, sizeof(int) * ncol, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess) {
             launch_ok = false;
             break;
         }
-        count_launch(2 + 2LL * q);
+        count_launch(2 + q);
         bool all = true;
         for (int col = 0; col < ncol; ++col) {
             if (hb[col] || state[col] == 2) continue;
@@ -204,7 +277,12 @@ int newton_sign_gpu(sgn_ctx* c, double2* X, int q, int ncol, int* failed) {
                 state[col] = 2;
                 continue;
             }
-            if (std::sqrt(hs[2 * col]) <= 1e-12 * std::sqrt(hs[2 * col + 1])) state[col] = 1;
+            double dn = 0, xn = 0;
+            for (int u = 0; u < nu; ++u) {
+                dn += hs[2 * (col * (size_t)nu + u)];
+                xn += hs[2 * (col * (size_t)nu + u) + 1];
+            }
+            if (std::sqrt(dn) <= 1e-12 * std::sqrt(xn)) state[col] = 1;
             all = false;
         }
         if (all) break;
@@ -234,7 +312,9 @@ int direct_projection(sgn_ctx* c, const double2* b, double2* x, int ncol, int k,
     const size_t ored = op + align256(sizeof(double2) * (size_t)ncol * rs * nblk);
     const size_t ocoef = ored + align256(sizeof(double2) * (size_t)ncol * rs);
     const size_t oflag = ocoef + align256(sizeof(double2) * (size_t)ncol * rs);
-    const size_t total = oflag + align256(sizeof(int) * 2 * (size_t)ncol);
+    const size_t hcount = (size_t)ncol * (k + 1) * k;
+    const size_t oH = oflag + align256(sizeof(int) * 4 * (size_t)ncol), osc = oH + align256(sizeof(double2) * hcount);
+    const size_t total = osc + align256(sizeof(double) * 2 * (size_t)ncol);
     DevBuf buf;
     SGN_CHECK(dev_alloc(c, buf, total));
     char* base = reinterpret_cast<char*>(buf.p);
@@ -248,7 +328,10 @@ int direct_projection(sgn_ctx* c, const double2* b, double2* x, int ncol, int k,
     S.done = S.skip + ncol;
     S.rstride = rs;
     const int64_t sj = (int64_t)ncol * n;
-    std::vector<double2> hbuf((size_t)ncol * rs);
+    int *kk_dev = S.skip + 2 * ncol, *live_dev = kk_dev + ncol;
+    double2* Hd = reinterpret_cast<double2*>(base + oH);
+    double* scale = reinterpret_cast<double*>(base + osc);
+    double* beta_dev = scale + ncol;
     auto bail = [&](int e) {
         dev_free(c, buf);
         return e;
@@ -261,10 +344,6 @@ int direct_projection(sgn_ctx* c, const double2* b, double2* x, int ncol, int k,
             return bail(SGN_ERR_CUDA);                                               \
         }                                                                            \
     } while (0)
-    auto fetch = [&]() -> cudaError_t {
-        cudaError_t e = cudaMemcpyAsync(hbuf.data(), S.red, sizeof(double2) * hbuf.size(), cudaMemcpyDeviceToHost, st);
-        return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
-    };
     auto upload = [&](const std::vector<cd>& C, int J, int j0) -> cudaError_t {  // C[col][j0 .. j0+J) -> coef
         std::vector<double2> h((size_t)ncol * rs, make_double2(0, 0));
         const int ld = (int)(C.size() / ncol);
@@ -296,33 +375,20 @@ int direct_projection(sgn_ctx* c, const double2* b, double2* x, int ncol, int k,
     } else {
         DC(cudaMemcpyAsync(w, b, field * ncol, cudaMemcpyDeviceToDevice, st));
     }
-    auto norms = [&](std::vector<double>& out) -> cudaError_t {  // ||w|| per column
+    // Arnoldi on A (eq. (2.4)) with two classical Gram-Schmidt passes; a column stops growing at its
+    // first breakdown
+    DC(cudaMemsetAsync(Hd, 0, sizeof(double2) * hcount, st));
+    auto next_vector = [&](int j) -> cudaError_t {  // v_{j+1} = w / ||w||
         cudaError_t e = mdot<double2>(Basis<double2>{w, 0, n}, 0, w, n, n, ncol, rd, 1, nullptr, st);
-        if (e == cudaSuccess) e = reduce(rd, 1, ncol, RM_STORE, 0, S, nullptr, st);
-        if (e == cudaSuccess) e = fetch();
-        for (int col = 0; col < ncol && e == cudaSuccess; ++col) out[col] = std::sqrt(std::max(hbuf[(size_t)col * rs].x, 0.0));
-        return e;
+        if (e != cudaSuccess) return e;
+        launch_pdl(k_direct_norm, ncol, 256, 0, st, rd, j, k, Hd, scale, beta_dev, kk_dev, live_dev);
+        count_launch();
+        return maxpy_scale<double2>(Basis<double2>{w, 0, n}, 0, coef, rs, w, n, V + (size_t)(j + 1) * sj, n, scale, n,
+                                    ncol, nullptr, st);
     };
-    auto normalize_into = [&](double2* dst, const std::vector<double>& nr) -> cudaError_t {  // dst = w / nr
-        std::vector<cd> D(ncol);
-        for (int col = 0; col < ncol; ++col) D[col] = nr[col] > 0 ? 1.0 / nr[col] : 0.0;
-        cudaError_t e = upload(D, 1, 0);
-        if (e == cudaSuccess) e = cudaMemsetAsync(dst, 0, field * ncol, st);
-        if (e == cudaSuccess)
-            e = update_x<double2>(Basis<double2>{w, 0, n}, 1, coef, rs, dst, n, n, ncol, nullptr, nullptr, st);
-        return e;
-    };
-    std::vector<double> beta(ncol), hn(ncol);
-    DC(norms(beta));
-    DC(normalize_into(V, beta));
-    // Arnoldi on A (eq. (2.4)); column col stops growing at its first breakdown
-    std::vector<cd> H((size_t)ncol * (k + 1) * k, 0.0);
-    std::vector<int> kk(ncol, k);
-    std::vector<char> live(ncol);
-    for (int col = 0; col < ncol; ++col) {
-        live[col] = beta[col] > 0;
-        if (!live[col]) kk[col] = 0;
-    }
+    std::vector<double> beta(ncol);
+    std::vector<int> flags(2 * (size_t)ncol);  // kk, live
+    DC(next_vector(-1));
     for (int j = 0; j < k; ++j) {
         DC(apply_hw64(c, w, V + (size_t)j * sj, ncol, adjoint, nullptr, st));
         for (int pass = 0; pass < 2; ++pass)
@@ -330,34 +396,22 @@ int direct_projection(sgn_ctx* c, const double2* b, double2* x, int ncol, int k,
                 const int J = std::min(GS_BLOCK, j + 1 - i0);
                 const Basis<double2> VB{V + (size_t)i0 * sj, sj, n};
                 DC(mdot<double2>(VB, J, w, n, n, ncol, rd, 0, nullptr, st));
-                DC(reduce(rd, J, ncol, RM_STORE, 0, S, nullptr, st));
-                DC(fetch());
-                for (int col = 0; col < ncol; ++col)
-                    for (int i = 0; i < J; ++i) {
-                        const double2 h = hbuf[(size_t)col * rs + i];
-                        H[((size_t)col * (k + 1) + i0 + i) * k + j] += cd(h.x, h.y);
-                    }
+                launch_pdl(k_direct_coef, dim3(ncol, (J + 31) / 32), 256, 0, st, rd, J, i0, j, k, S.red, rs, Hd);
+                count_launch();
                 DC(maxpy_scale<double2>(VB, J, S.red, rs, w, n, w, n, nullptr, n, ncol, nullptr, st));
             }
-        DC(norms(hn));
-        for (int col = 0; col < ncol; ++col) {
-            if (!live[col]) {
-                hn[col] = 0;
-                continue;
-            }
-            double cn = hn[col] * hn[col];
-            for (int i = 0; i <= j; ++i) cn += std::norm(H[((size_t)col * (k + 1) + i) * k + j]);
-            if (hn[col] <= 1e-14 * std::sqrt(cn)) {  // invariant subspace: the projection is exact
-                live[col] = 0;
-                kk[col] = j + 1;
-                hn[col] = 0;
-            } else {
-                H[((size_t)col * (k + 1) + j + 1) * k + j] = hn[col];
-            }
+        DC(next_vector(j));
+        if ((j + 1) % 32 == 0 || j + 1 == k) {
+            DC(cudaMemcpyAsync(flags.data(), kk_dev, sizeof(int) * flags.size(), cudaMemcpyDeviceToHost, st));
+            DC(cudaStreamSynchronize(st));
+            if (std::none_of(flags.begin() + ncol, flags.end(), [](int v) { return v != 0; })) break;
         }
-        DC(normalize_into(V + (size_t)(j + 1) * sj, hn));
-        if (std::none_of(live.begin(), live.end(), [](char v) { return v != 0; })) break;
     }
+    std::vector<cd> H(hcount);
+    DC(cudaMemcpyAsync(beta.data(), beta_dev, sizeof(double) * ncol, cudaMemcpyDeviceToHost, st));
+    DC(cudaMemcpyAsync(H.data(), Hd, sizeof(double2) * hcount, cudaMemcpyDeviceToHost, st));
+    DC(cudaStreamSynchronize(st));
+    const std::vector<int> kk(flags.begin(), flags.begin() + ncol);
     // y_col = beta sign(H_kk) e_1: Roberts' Newton iteration for all columns on the GPU,
     // each H_kk padded to the largest Krylov dimension with the identity
     const int kmaxu = *std::max_element(kk.begin(), kk.end());
