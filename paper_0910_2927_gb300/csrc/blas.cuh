@@ -28,11 +28,6 @@ struct DevState {
     int* done;         // [col] converged (column work is skipped)
     int* skip;         // [col] done or broken down in this cycle
     int* err;          // [1] device error word (bit 0: singular shifted system; bit 1: non-finite)
-    // Optional (both or neither): per-slot sums and per-column arrival counters for the
-    // split second-stage reduction (several CTAs per column, the last one does the
-    // column's scalar work).  Null: one CTA per column.
-    double2* sums = nullptr;  // [col][rstride]
-    int* rcount = nullptr;    // [col], zero between launches
     int kmax;
     int s;
     int rstride;

@@ -44,6 +44,22 @@ inline void count_launch(long long k = 1) { g_launches += k; }
 // before it have.  Such data are read by plain loads: a const __restrict__ pointer or __ldg would say
 // that they do not change while the kernel runs, and let the load move ahead of the wait.
 template <class... KA, class... A>
+inline void launch_pdl_cluster(void (*kernel)(KA...), dim3 grid, dim3 block, dim3 cluster, cudaStream_t st,
+                               A&&... args) {
+    cudaLaunchAttribute at[2]{};
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim = {cluster.x, cluster.y, cluster.z};
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = cluster.x * cluster.y * cluster.z > 1 ? 2 : 1;
+    cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);  // an error stays for cudaGetLastError
+}
+template <class... KA, class... A>
 inline void launch_pdl(void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -522,8 +522,6 @@ int get_engine(sgn_ctx* c, int ncol, int k, int s, int prec, Engine** out) {
     size_t oi[3];
     for (int i = 0; i < 3; ++i) oi[i] = take(nc * sizeof(int));
     size_t oerr = take(sizeof(int));
-    size_t osums = take(nc * E->rstride * sizeof(double2));
-    size_t ocnt = take(nc * sizeof(int));
     size_t ogres = take(nc * (size_t)(k + 1) * sizeof(double2));
     size_t oneg = take(nc * sizeof(double));
     size_t ocyc = take(sizeof(int));
@@ -555,8 +553,6 @@ int get_engine(sgn_ctx* c, int ncol, int k, int s, int prec, Engine** out) {
     S.done = reinterpret_cast<int*>(base + oi[1]);
     S.skip = reinterpret_cast<int*>(base + oi[2]);
     S.err = reinterpret_cast<int*>(base + oerr);
-    S.sums = reinterpret_cast<double2*>(base + osums);
-    S.rcount = reinterpret_cast<int*>(base + ocnt);
     S.gres = reinterpret_cast<double2*>(base + ogres);
     S.kmax = k;
     S.s = s;
