@@ -390,8 +390,10 @@ cudaError_t cycle_dcgs(const sgn_ctx* c, Engine& E, const CycleArgs& a, cudaStre
     } else {
         CU(shifted_solves(S, ncol, st));
     }
-    CU(combine_shifts(S, ncol, st));
-    if (a.xacc) CU(update_x<T>(VB, k, S.coef, S.rstride, a.xacc, a.xsr, n, ncol, S.done, S.kk, st));
+    if (a.xacc) {
+        CU(combine_shifts(S, ncol, st));
+        CU(update_x<T>(VB, k, S.coef, S.rstride, a.xacc, a.xsr, n, ncol, S.done, S.kk, st));
+    }
     if (a.xs) {
         // the basis once (the shift groups of a tile share it through L2), every per-shift
         // iterate read and written (FP64)
