@@ -8,8 +8,8 @@
 // orthogonalisation) and loses convergence at every restart.  BiCGStab moves 9 fields per
 // application besides the two stencils' 4.5 and never restarts.  Every kernel below is bound by
 // HBM (FP32, two complex numbers per 16-byte load), on small lattices by launch latency.
-// Measured: the refinement of the 10^4 x 12 solve (240 systems, tol 1e-10) 75 ms with FOM(16), 33 ms
-// now; the whole solve 133 -> 86 ms; the 6^4 x 1 solve 15.0 -> 11.2 ms.
+// Measured: the refinement of the 10^4 x 12 solve (240 systems, tol 1e-10) 75 ms with FOM(16), 34 to 38 ms
+// now; the whole solve 133 -> 86 to 90 ms; the 6^4 x 1 solve 15.0 -> 11.2 ms.
 //
 // One iteration: w = A^2 p, k_bi_v, k_bi_s, t = A^2 s, k_bi_t, k_bi_x.  The shift enters as
 // w - sigma p and t - sigma s where these are used.  Sums: FP32 within a CTA, FP64 over the CTAs of a

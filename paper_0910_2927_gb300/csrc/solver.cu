@@ -1229,13 +1229,15 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
         return SGN_OK;
     };
 
-    // A system once corrected is done below rtol * accept, twelve times its correction's aim: the first
-    // correction of a solution from 16-bit links may leave it anywhere below rtol.
+    // A system once corrected is done below rtol * accept: twelve times its correction's aim, or three
+    // times where one correction cannot get near the aim (a solution from 16-bit links starts at
+    // 1e-3, and FP32 fields gain kBiFloor: accepted below rtol it gave an error of 2e-8 for BF16 links
+    // at tol 1e-8).
     std::vector<double> accept(nall, 1.0);
     // Correction solves by BiCGStab, each system to its own residual; the systems it gave up on are
     // left as they were and returned in `failed`.  What a residual r_i leaves in x is about
     // omega_i r_i / (spectrum - sigma_i), largest for the smallest shifts, which are also the slow
-    // ones: the systems aim at tol / margin_i, margin_i from 36 for the largest omega / |sigma| down
+    // ones: the systems aim at tol / margin_i, margin_i from 54 for the largest omega / |sigma| down
     // with its fourth root (at a margin of 9 for all, the error of x on the 10^4 workload was 2.3
     // times that of FOM corrections).
     std::vector<double> margin(s);
@@ -1246,7 +1248,7 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
             if (std::isfinite(margin[i])) wmax = std::max(wmax, margin[i]);
         }
         for (double& w : margin)
-            w = wmax > 0 && std::isfinite(w) ? std::max(4.0, 36.0 * std::sqrt(std::sqrt(w / wmax))) : 36.0;
+            w = wmax > 0 && std::isfinite(w) ? std::max(6.0, 54.0 * std::sqrt(std::sqrt(w / wmax))) : 54.0;
     }
     auto bicg_corrections = [&](const std::vector<System>& todo, std::vector<System>& failed) -> int {
         const int nc = G->ncol;
@@ -1256,8 +1258,10 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
             const int nb = (int)std::min<size_t>(nc, todo.size() - t0);
             for (int j = 0; j < nb; ++j) {
                 const System& y = todo[t0 + j];
+                const double mg = margin[y.at / ncol], aim = rtol / (mg * y.rel);
                 sg[j] = c->sigma[y.at / ncol];
-                tl[j] = std::min(0.1, std::max(kBiFloor, rtol / (margin[y.at / ncol] * y.rel)));
+                tl[j] = std::min(0.1, std::max(kBiFloor, aim));
+                accept[y.at] = std::min(1.0, (aim < kBiFloor / 2 ? 3.0 : 12.0) / mg);
                 off_h[j] = (long long)y.at * n;
             }
             SGN_CUDA(cudaMemcpyAsync(G->sigma, sg.data(), sizeof(double) * nc, cudaMemcpyHostToDevice, st));
@@ -1270,10 +1274,10 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
             SGN_CHECK(run_bicg(c, *G, adjoint, cap, &iters));
             ref_cycles += iters;
             for (int j = 0; j < nb; ++j)
-                if (G->h_done[j] != BI_DONE)
+                if (G->h_done[j] != BI_DONE) {
                     failed.push_back(todo[t0 + j]);
-                else
-                    accept[todo[t0 + j].at] = std::min(1.0, 12.0 / margin[todo[t0 + j].at / ncol]);
+                    accept[todo[t0 + j].at] = 1.0;
+                }
             if (debug_log())
                 fprintf(stderr, "[sgn mixed]   batch at %zu (%d systems): %d iterations, %zu failed so far\n", t0, nb,
                         iters, failed.size());
@@ -1291,7 +1295,7 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
         // the corrections (r_i -= R c_i with x_i += R (Lambda^2 - sigma_i)^{-1} c_i,
         // r_i -= (A^2 - sigma_i) d_i with x_i += d_i), where FP32 products of the small d_i are
         // exact to ~1e-6 ||r_i||: from scratch again where that is not far below the tolerance
-        // (solutions from 16-bit links, whose first residuals are about 1e-3).
+        // (solutions from 16-bit links, whose first residuals are 1e-4 to 1e-3).
         // From scratch means A^2 x_i in float-float arithmetic on the FP32 units (stencil_ff.cu; ~1e-13
         // of the FP64 stencil, which GB300 runs at 1/64 of the FP32 rate), fsh shifts at a time.
         if (round == 0 || 1e-6 * worst > 0.02 * rtol) {
