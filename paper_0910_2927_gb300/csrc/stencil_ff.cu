@@ -46,7 +46,6 @@ __device__ __forceinline__ ff fast_two_sum(float a, float b) {
     const float s = __fadd_rn(a, b);
     return {s, __fsub_rn(b, __fsub_rn(s, a))};
 }
-__device__ __forceinline__ ff ff_neg(ff a) { return {-a.hi, -a.lo}; }
 // Sum of two float-float numbers, left unnormalised: hi is the rounded sum of the high parts, lo
 // collects its error and the low parts (|lo| stays within a few units of 2^-24 |hi| unless the sum
 // cancels, and hi + lo is the sum to about 2^-46 of the operands either way).  The stencil's
