@@ -652,8 +652,8 @@ def solve_roofline(kt, steps, t_step, hbm, peak_src):
     """The whole solve against HBM: the algorithmic bytes the library counts for its timed
     kernel classes (stencil, Gram-Schmidt reduction and update, second-stage reductions,
     per-shift update) per step, divided by the headline (uninstrumented) step time.  The
-    kernels it does not count (the refinement's FP64 true residuals and projections, format
-    conversions) add time but no bytes, so this is a lower bound of the solve's fraction."""
+    kernels it does not count (the refinement's correction solves, true residuals and projections,
+    format conversions) add time but no bytes, so this is a lower bound of the solve's fraction."""
     if not steps or not t_step > 0:
         return None
     per_step = sum(v["bytes"] for v in kt.values()) / steps
