@@ -270,23 +270,20 @@ __global__ void __launch_bounds__(NT) k_bi_x(BiState S) {
     }
 }
 
-// x_j += d_j and r_j += sigma_j d_j - w_j (w_j = A^2 d_j in FP32) for the converged systems:
-// x_j at x + off[j], r_j at r + off[j], d_j and w_j FP32 at j n.
-__global__ void __launch_bounds__(NT) k_apply_corrections(double2* __restrict__ x, double2* __restrict__ r,
-                                                          const long long* __restrict__ off,
-                                                          const double* __restrict__ sig, const int* __restrict__ done,
-                                                          const float2* __restrict__ w, const float2* __restrict__ d,
-                                                          int64_t n) {
+__device__ __forceinline__ double2 to_d(float2 v) { return make_double2(f2d(v.x), f2d(v.y)); }
+__device__ __forceinline__ double2 to_d(double2 v) { return v; }
+// x_j += d_j, x_j at x + off[j], d_j at j n; with done, for the converged systems.
+template <class T>
+__global__ void __launch_bounds__(NT) k_add_corrections(double2* __restrict__ x, const long long* __restrict__ off,
+                                                        const int* __restrict__ done, const T* __restrict__ d,
+                                                        int64_t n) {
     const int j = blockIdx.y;
     if (done && done[j] != BI_DONE) return;
-    double2 *xj = x + off[j], *rj = r + off[j];
-    const double sg = sig[j];
-    const float2 *wj = w + (int64_t)j * n, *dj = d + (int64_t)j * n;
+    double2* xj = x + off[j];
+    const T* dj = d + (int64_t)j * n;
     for (int64_t e = (int64_t)blockIdx.x * NT + threadIdx.x; e < n; e += (int64_t)gridDim.x * NT) {
-        const float2 wv = wj[e], df = dj[e];
-        const double2 dv = make_double2(f2d(df.x), f2d(df.y)), xv = xj[e], rv = rj[e];
+        const double2 dv = to_d(dj[e]), xv = xj[e];
         xj[e] = make_double2(xv.x + dv.x, xv.y + dv.y);
-        rj[e] = make_double2(fma(sg, dv.x, rv.x - f2d(wv.x)), fma(sg, dv.y, rv.y - f2d(wv.y)));
     }
 }
 
@@ -331,14 +328,19 @@ cudaError_t bi_x(const BiState& S, int ncol, cudaStream_t st) {
     return launch(S, ncol, st, k_bi_x<1>, k_bi_x<2>, k_bi_x<4>);
 }
 
-cudaError_t apply_corrections(double2* x, double2* r, const long long* off, const double* sig, const int* done,
-                              const float2* w, const float2* d, int64_t n, int nb, cudaStream_t st) {
+template <class T>
+cudaError_t add_corrections(double2* x, const long long* off, const int* done, const T* d, int64_t n, int nb,
+                            cudaStream_t st) {
     if (nb < 1) return cudaSuccess;
     if (nb > 65535) return cudaErrorInvalidValue;
     const int64_t gx = (n + NT - 1) / NT;
-    k_apply_corrections<<<dim3((unsigned)(gx < 1024 ? gx : 1024), nb), NT, 0, st>>>(x, r, off, sig, done, w, d, n);
+    k_add_corrections<T><<<dim3((unsigned)(gx < 1024 ? gx : 1024), nb), NT, 0, st>>>(x, off, done, d, n);
     count_launch();
     return cudaGetLastError();
 }
+template cudaError_t add_corrections<float2>(double2*, const long long*, const int*, const float2*, int64_t, int,
+                                             cudaStream_t);
+template cudaError_t add_corrections<double2>(double2*, const long long*, const int*, const double2*, int64_t, int,
+                                              cudaStream_t);
 
 }  // namespace sgn

@@ -210,10 +210,11 @@ cudaError_t bi_s(const BiState& S, int ncol, cudaStream_t st);
 cudaError_t bi_t(const BiState& S, int ncol, cudaStream_t st);
 cudaError_t bi_x(const BiState& S, int ncol, cudaStream_t st);
 
-// x_j += d_j and r_j += sigma_j d_j - w_j (w_j = A^2 d_j) for nb systems: x_j, r_j at off[j], d_j
-// and w_j (FP32) at j n; with done, only systems marked BI_DONE.
-cudaError_t apply_corrections(double2* x, double2* r, const long long* off, const double* sig, const int* done,
-                              const float2* w, const float2* d, int64_t n, int nb, cudaStream_t st);
+// x_j += d_j for nb systems: x_j at off[j], d_j (float2 or double2) at j n; with done, only systems
+// marked BI_DONE.
+template <class T>
+cudaError_t add_corrections(double2* x, const long long* off, const int* done, const T* d, int64_t n, int nb,
+                            cudaStream_t st);
 
 // Tall-skinny products of a basis V (J <= 64 fields, stride sv) with N columns W
 // (complex128, stride sw): tsmm_tn writes the partials of V^dag W into rd (then

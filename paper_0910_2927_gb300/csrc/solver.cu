@@ -1049,7 +1049,7 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
     size_t o_red = take(sizeof(double2) * ncmax * rs64);
     size_t o_part = take(sizeof(double2) * (size_t)ncmax * rs64 * nblk64);
     size_t o_flags = take(sizeof(int) * 2 * ncmax);
-    size_t o_roff = take(sizeof(long long) * B), o_rsig = take(sizeof(double) * B);
+    size_t o_roff = take(sizeof(long long) * B);
     SGN_CHECK(ensure_io(c, off));
     char* io = reinterpret_cast<char*>(c->io.p);
     double2* xs = reinterpret_cast<double2*>(io + o_xs);
@@ -1062,7 +1062,6 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
     double2* rsd = reinterpret_cast<double2*>(io + o_rs);  // true residuals r_i, [i][col][n]
     double2* omtab = reinterpret_cast<double2*>(io + o_om);
     long long* roff_dev = reinterpret_cast<long long*>(io + o_roff);
-    double* rsig_dev = reinterpret_cast<double*>(io + o_rsig);
     // FP64 reductions use their own partials and state (the FP32 engines size theirs for float packs)
     DevState S64{};
     S64.red = reinterpret_cast<double2*>(io + o_red);
@@ -1177,7 +1176,7 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
         a1.xs = d;
         a1.xs_shift = (int64_t)B * n;
         a1.xs_col = n;
-        std::vector<double> sig1(B), om1(B, 1.0), rsig(B);
+        std::vector<double> sig1(B), om1(B, 1.0);
         std::vector<long long> roff(B);
         for (size_t t0 = 0; t0 < todo.size(); t0 += B) {
             const int nb = (int)std::min<size_t>(B, todo.size() - t0);
@@ -1211,20 +1210,9 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
                 SGN_CUDA(cudaMemsetAsync(E1->S.err, 0, sizeof(int), st));
             }
             if (st1 != SGN_OK) return st1;
-            // x_i += d_i, r_i -= (A^2 - sigma_i) d_i: A^2 d in FP32 on the engine's fields.  FP32 links
-            // even when the solves run on 16-bit ones: the carried residual must see the true
-            // operator, not the one the corrections were solved with
-            float2 *d32 = reinterpret_cast<float2*>(E1->w), *t32 = reinterpret_cast<float2*>(E1->t);
-            SGN_CUDA(convert_f64_to_f32(d, d32, (int64_t)nb * n, st));
-            SGN_CUDA(apply_hw32(c, t32, d32, nb, adjoint, nullptr, st, true));
-            SGN_CUDA(apply_hw32(c, V0, t32, nb, adjoint, nullptr, st, true));
-            for (int j = 0; j < nb; ++j) {
-                roff[j] = (long long)todo[t0 + j].at * n;
-                rsig[j] = c->sigma[todo[t0 + j].at / ncol];
-            }
+            for (int j = 0; j < nb; ++j) roff[j] = (long long)todo[t0 + j].at * n;
             SGN_CUDA(cudaMemcpyAsync(roff_dev, roff.data(), sizeof(long long) * nb, cudaMemcpyHostToDevice, st));
-            SGN_CUDA(cudaMemcpyAsync(rsig_dev, rsig.data(), sizeof(double) * nb, cudaMemcpyHostToDevice, st));
-            SGN_CUDA(apply_corrections(xs, rsd, roff_dev, rsig_dev, nullptr, V0, d32, n, nb, st));
+            SGN_CUDA(add_corrections<double2>(xs, roff_dev, nullptr, d, n, nb, st));
         }
         return SGN_OK;
     };
@@ -1282,23 +1270,19 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
                 fprintf(stderr, "[sgn mixed]   batch at %zu (%d systems): %d iterations, %zu failed so far\n", t0, nb,
                         iters, failed.size());
             const BiState& S = G->S;
-            SGN_CUDA(apply_hw32(c, S.t, S.d, nc, adjoint, nullptr, st, true));
-            SGN_CUDA(apply_hw32(c, S.w, S.t, nc, adjoint, nullptr, st, true));
-            SGN_CUDA(apply_corrections(xs, rsd, G->off, G->sigma, S.done, S.w, S.d, n, nb, st));
+            SGN_CUDA(add_corrections<float2>(xs, G->off, S.done, S.d, n, nb, st));
             SGN_CUDA(cudaStreamSynchronize(st));  // the host tables are filled again
         }
         return SGN_OK;
     };
     for (int round = 0; round <= max_rounds; ++round) {
-        // true residuals r_i = b~ - (A^2 - sigma_i) x_i of every shifted system: from
-        // scratch in refinement round 0, assembled in FP64; later rounds carry them along with
-        // the corrections (r_i -= R c_i with x_i += R (Lambda^2 - sigma_i)^{-1} c_i,
-        // r_i -= (A^2 - sigma_i) d_i with x_i += d_i), where FP32 products of the small d_i are
-        // exact to ~1e-6 ||r_i||: from scratch again where that is not far below the tolerance
-        // (solutions from 16-bit links, whose first residuals are 1e-4 to 1e-3).
-        // From scratch means A^2 x_i in float-float arithmetic on the FP32 units (stencil_ff.cu; ~1e-13
-        // of the FP64 stencil, which GB300 runs at 1/64 of the FP32 rate), fsh shifts at a time.
-        if (round == 0 || 1e-6 * worst > 0.02 * rtol) {
+        // true residuals r_i = b~ - (A^2 - sigma_i) x_i of every shifted system, assembled in FP64: A^2 x_i
+        // in float-float arithmetic on the FP32 units (stencil_ff.cu; ~1e-13 of the FP64 stencil, which
+        // GB300 runs at 1/64 of the FP32 rate), fsh shifts at a time.  In every round: carried along with
+        // the corrections (r_i -= (A^2 - sigma_i) d_i with FP32 products) they are off by the rounding
+        // of A^2 d_i, and ||A^2|| ||d_i|| / ||r_i|| reaches ||A^2|| / |lambda^2 - sigma_i|: on an operator
+        // with |lambda| = 0.003 a system reported below 1e-11 was at 2.4e-10.
+        {
             const size_t nf = (size_t)ncol * n;
             const StencilParams pf = stencil_params(c, adjoint);
             const float4* Uf = reinterpret_cast<const float4*>(c->Uff.p);
