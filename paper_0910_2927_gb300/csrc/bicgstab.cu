@@ -96,20 +96,31 @@ __device__ __forceinline__ bool column_sum(float (&v)[NV], const BiState& S, int
     return true;
 }
 
-// r = rt = p = fl32(src at off[col]), d = 0, rho = ||r||^2.  Columns from nb on are idle.
+// 2^e, |e| <= 1022
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+// fl32(2^-e v), two complex numbers
+__device__ __forceinline__ float4 scaled_f32(const double2* f, int64_t i, double q) {
+    const double2 a = f[2 * i], b = f[2 * i + 1];
+    return make_float4(d2f(a.x * q), d2f(a.y * q), d2f(b.x * q), d2f(b.y * q));
+}
+
+// r = rt = p = fl32(2^-ex[col] src at off[col]), d = 0, rho = ||r||^2.  Columns from nb on are idle.
+// The caller's 2^ex is the residual's size: the sums square FP32 numbers that go down to 1e-6 of it, so
+// that unscaled residuals of right-hand sides of norm 1e-12 underflowed (three times the iterations,
+// and at 1e-14 no convergence).
 __global__ void __launch_bounds__(NT) k_bi_init(const double2* __restrict__ src, const long long* __restrict__ off,
-                                                int nb, BiState S) {
+                                                const int* __restrict__ ex, int nb, BiState S) {
     const int col = blockIdx.y;
     if (col >= nb) {
         if (blockIdx.x == 0 && threadIdx.x == 0) S.done[col] = BI_IDLE;
         return;
     }
     const double2* f = src + off[col];
+    const double q = pow2(-ex[col]);
     const int64_t c = (int64_t)col * 2 * S.npk;
     float v[1] = {0.f};
     for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < S.npk; i += (int64_t)gridDim.x * NT) {
-        const double2 a = f[2 * i], b = f[2 * i + 1];
-        const float4 r = make_float4(d2f(a.x), d2f(a.y), d2f(b.x), d2f(b.y));
+        const float4 r = scaled_f32(f, i, q);
         st(S.r + c, i, r);
         st(S.rt + c, i, r);
         st(S.p + c, i, r);
@@ -272,19 +283,34 @@ __global__ void __launch_bounds__(NT) k_bi_x(BiState S) {
 
 __device__ __forceinline__ double2 to_d(float2 v) { return make_double2(f2d(v.x), f2d(v.y)); }
 __device__ __forceinline__ double2 to_d(double2 v) { return v; }
-// x_j += d_j, x_j at x + off[j], d_j at j n; with done, for the converged systems.
+// x_j += 2^ex[j] d_j, x_j at x + off[j], d_j at j n; with done, for the converged systems.
 template <class T>
 __global__ void __launch_bounds__(NT) k_add_corrections(double2* __restrict__ x, const long long* __restrict__ off,
-                                                        const int* __restrict__ done, const T* __restrict__ d,
-                                                        int64_t n) {
+                                                        const int* __restrict__ ex, const int* __restrict__ done,
+                                                        const T* __restrict__ d, int64_t n) {
     const int j = blockIdx.y;
     if (done && done[j] != BI_DONE) return;
     double2* xj = x + off[j];
     const T* dj = d + (int64_t)j * n;
+    const double q = pow2(ex[j]);
     for (int64_t e = (int64_t)blockIdx.x * NT + threadIdx.x; e < n; e += (int64_t)gridDim.x * NT) {
         const double2 dv = to_d(dj[e]), xv = xj[e];
-        xj[e] = make_double2(xv.x + dv.x, xv.y + dv.y);
+        xj[e] = make_double2(fma(q, dv.x, xv.x), fma(q, dv.y, xv.y));
     }
+}
+// out_j = fl32(2^-ex[j] src at off[j])
+__global__ void __launch_bounds__(NT) k_scaled_residuals(const double2* __restrict__ src,
+                                                         const long long* __restrict__ off,
+                                                         const int* __restrict__ ex, float2* __restrict__ out,
+                                                         int64_t npk) {
+    const int j = blockIdx.y;
+    const double q = pow2(-ex[j]);
+    for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < npk; i += (int64_t)gridDim.x * NT)
+        st(out + (int64_t)j * 2 * npk, i, scaled_f32(src + off[j], i, q));
+}
+dim3 field_grid(int64_t count, int nb) {
+    const int64_t gx = (count + NT - 1) / NT;
+    return dim3((unsigned)(gx < 1024 ? gx : 1024), nb);
 }
 
 template <class K1, class K2, class K4>
@@ -310,8 +336,9 @@ void bi_shape(BiState& S, int64_t n, int ncol) {
 }
 size_t bi_partial_bytes(const BiState& S, int ncol) { return sizeof(float) * MAXV * (size_t)S.nblk * ncol; }
 
-cudaError_t bi_init(const BiState& S, int ncol, const double2* src, const long long* off, int nb, cudaStream_t st) {
-    k_bi_init<<<dim3(S.nblk, ncol), NT, 0, st>>>(src, off, nb, S);
+cudaError_t bi_init(const BiState& S, int ncol, const double2* src, const long long* off, const int* ex, int nb,
+                    cudaStream_t st) {
+    k_bi_init<<<dim3(S.nblk, ncol), NT, 0, st>>>(src, off, ex, nb, S);
     count_launch();
     return cudaGetLastError();
 }
@@ -329,18 +356,25 @@ cudaError_t bi_x(const BiState& S, int ncol, cudaStream_t st) {
 }
 
 template <class T>
-cudaError_t add_corrections(double2* x, const long long* off, const int* done, const T* d, int64_t n, int nb,
-                            cudaStream_t st) {
+cudaError_t add_corrections(double2* x, const long long* off, const int* ex, const int* done, const T* d, int64_t n,
+                            int nb, cudaStream_t st) {
     if (nb < 1) return cudaSuccess;
     if (nb > 65535) return cudaErrorInvalidValue;
-    const int64_t gx = (n + NT - 1) / NT;
-    k_add_corrections<T><<<dim3((unsigned)(gx < 1024 ? gx : 1024), nb), NT, 0, st>>>(x, off, done, d, n);
+    k_add_corrections<T><<<field_grid(n, nb), NT, 0, st>>>(x, off, ex, done, d, n);
     count_launch();
     return cudaGetLastError();
 }
-template cudaError_t add_corrections<float2>(double2*, const long long*, const int*, const float2*, int64_t, int,
-                                             cudaStream_t);
-template cudaError_t add_corrections<double2>(double2*, const long long*, const int*, const double2*, int64_t, int,
-                                              cudaStream_t);
+template cudaError_t add_corrections<float2>(double2*, const long long*, const int*, const int*, const float2*,
+                                             int64_t, int, cudaStream_t);
+template cudaError_t add_corrections<double2>(double2*, const long long*, const int*, const int*, const double2*,
+                                              int64_t, int, cudaStream_t);
+cudaError_t scaled_residuals(const double2* src, const long long* off, const int* ex, float2* out, int64_t n, int nb,
+                             cudaStream_t st) {
+    if (nb < 1) return cudaSuccess;
+    if (nb > 65535) return cudaErrorInvalidValue;
+    k_scaled_residuals<<<field_grid(n / 2, nb), NT, 0, st>>>(src, off, ex, out, n / 2);
+    count_launch();
+    return cudaGetLastError();
+}
 
 }  // namespace sgn

@@ -204,17 +204,21 @@ struct BiState {
 };
 void bi_shape(BiState& S, int64_t n, int ncol);
 size_t bi_partial_bytes(const BiState& S, int ncol);
-cudaError_t bi_init(const BiState& S, int ncol, const double2* src, const long long* off, int nb, cudaStream_t st);
+cudaError_t bi_init(const BiState& S, int ncol, const double2* src, const long long* off, const int* ex, int nb,
+                    cudaStream_t st);
 cudaError_t bi_v(const BiState& S, int ncol, cudaStream_t st);
 cudaError_t bi_s(const BiState& S, int ncol, cudaStream_t st);
 cudaError_t bi_t(const BiState& S, int ncol, cudaStream_t st);
 cudaError_t bi_x(const BiState& S, int ncol, cudaStream_t st);
 
-// x_j += d_j for nb systems: x_j at off[j], d_j (float2 or double2) at j n; with done, only systems
-// marked BI_DONE.
+// Corrections are solved for residuals scaled to about norm one, by an exact power of two: fl32(2^-ex[j] r_j)
+// for nb systems, r_j at off[j] of src (bi_init takes the same), and x_j += 2^ex[j] d_j, x_j at
+// off[j], d_j (float2 or double2) at j n; with done, only systems marked BI_DONE.  |ex| <= 1022.
+cudaError_t scaled_residuals(const double2* src, const long long* off, const int* ex, float2* out, int64_t n, int nb,
+                             cudaStream_t st);
 template <class T>
-cudaError_t add_corrections(double2* x, const long long* off, const int* done, const T* d, int64_t n, int nb,
-                            cudaStream_t st);
+cudaError_t add_corrections(double2* x, const long long* off, const int* ex, const int* done, const T* d, int64_t n,
+                            int nb, cudaStream_t st);
 
 // Tall-skinny products of a basis V (J <= 64 fields, stride sv) with N columns W
 // (complex128, stride sw): tsmm_tn writes the partials of V^dag W into rd (then

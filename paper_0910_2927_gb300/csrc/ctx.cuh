@@ -72,6 +72,7 @@ struct BiCg {
     BiState S{};
     double *tol = nullptr, *sigma = nullptr;
     long long* off = nullptr;  // [ncol] offset of each system's x and r
+    int* ex = nullptr;         // [ncol] binary exponent of each residual's norm
     int *err = nullptr, *cyc = nullptr;
     int* h_done = nullptr;  // pinned: done[ncol], err, cyc
     cudaGraphExec_t one = nullptr, loop = nullptr;

@@ -901,7 +901,7 @@ int get_bicg(sgn_ctx* c, int ncol, BiCg** out) {
         off += align256(bytes);
         return o;
     };
-    size_t of[7], oc[4], od[4], oi[2];
+    size_t of[7], oc[4], od[4], oi[3];
     for (size_t& o : of) o = take(field);
     for (size_t& o : oc) o = take(nc * sizeof(double2));
     for (size_t& o : od) o = take(nc * sizeof(double));
@@ -921,6 +921,7 @@ int get_bicg(sgn_ctx* c, int ncol, BiCg** out) {
     G->off = reinterpret_cast<long long*>(b + ooff);
     S.done = reinterpret_cast<int*>(b + oi[0]);
     S.count = reinterpret_cast<int*>(b + oi[1]);
+    G->ex = reinterpret_cast<int*>(b + oi[2]);
     G->err = reinterpret_cast<int*>(b + oe);
     G->cyc = G->err + 1;
     S.partial = reinterpret_cast<float*>(b + op);
@@ -1049,7 +1050,7 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
     size_t o_red = take(sizeof(double2) * ncmax * rs64);
     size_t o_part = take(sizeof(double2) * (size_t)ncmax * rs64 * nblk64);
     size_t o_flags = take(sizeof(int) * 2 * ncmax);
-    size_t o_roff = take(sizeof(long long) * B);
+    size_t o_roff = take(sizeof(long long) * B), o_rex = take(sizeof(int) * B);
     SGN_CHECK(ensure_io(c, off));
     char* io = reinterpret_cast<char*>(c->io.p);
     double2* xs = reinterpret_cast<double2*>(io + o_xs);
@@ -1062,6 +1063,7 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
     double2* rsd = reinterpret_cast<double2*>(io + o_rs);  // true residuals r_i, [i][col][n]
     double2* omtab = reinterpret_cast<double2*>(io + o_om);
     long long* roff_dev = reinterpret_cast<long long*>(io + o_roff);
+    int* rex_dev = reinterpret_cast<int*>(io + o_rex);
     // FP64 reductions use their own partials and state (the FP32 engines size theirs for float packs)
     DevState S64{};
     S64.red = reinterpret_cast<double2*>(io + o_red);
@@ -1150,6 +1152,10 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
         int at;
         double rel;
     };
+    // binary exponent of a residual's norm: the corrections are solved for residuals scaled by it
+    auto exponent = [&](const System& y) {
+        return std::clamp(std::ilogb(y.rel * bnorm[y.at % ncol]), -1000, 1000);
+    };
 
     // Correction solves by restarted FOM (Galerkin, like the multishift phase); a batch whose
     // FOM does not converge within kFomCap cycles, or meets a non-finite value, is solved again
@@ -1178,6 +1184,7 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
         a1.xs_col = n;
         std::vector<double> sig1(B), om1(B, 1.0);
         std::vector<long long> roff(B);
+        std::vector<int> rex(B);
         for (size_t t0 = 0; t0 < todo.size(); t0 += B) {
             const int nb = (int)std::min<size_t>(B, todo.size() - t0);
             float2* V0 = reinterpret_cast<float2*>(E1->V);
@@ -1186,14 +1193,20 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
             // the correction needs to reduce the worst residual of the batch to a third
             // of the tolerance, not further (FP32 bases reach about 1e-6 at best)
             double brel = 0;
-            for (int j = 0; j < nb; ++j) brel = std::max(brel, todo[t0 + j].rel);
+            for (int j = 0; j < nb; ++j) {
+                const System& y = todo[t0 + j];
+                brel = std::max(brel, y.rel);
+                roff[j] = (long long)y.at * n;
+                rex[j] = exponent(y);
+            }
+            SGN_CUDA(cudaMemcpyAsync(roff_dev, roff.data(), sizeof(long long) * nb, cudaMemcpyHostToDevice, st));
+            SGN_CUDA(cudaMemcpyAsync(rex_dev, rex.data(), sizeof(int) * nb, cudaMemcpyHostToDevice, st));
             int st1 = SGN_OK;
             RunResult r1;
             for (int attempt = 0; attempt < 2; ++attempt) {
                 a1.gmres = attempt == 1;
                 SGN_CUDA(cudaMemsetAsync(V0, 0, sizeof(float2) * (size_t)B * n, st));
-                for (int j = 0; j < nb; ++j)
-                    SGN_CUDA(convert_f64_to_f32(rsd + (size_t)todo[t0 + j].at * n, V0 + (size_t)j * n, n, st));
+                SGN_CUDA(scaled_residuals(rsd, roff_dev, rex_dev, V0, n, nb, st));
                 SGN_CUDA(cudaMemsetAsync(d, 0, field * B, st));
                 const double inner = std::min(0.1, std::max(1e-5, rtol / ((a1.gmres ? 9.0 : 3.0) * brel)));
                 st1 = run_engine<float2>(c, *E1, a1, inner, a1.gmres ? c->max_cycles : std::min(c->max_cycles, kFomCap),
@@ -1210,9 +1223,7 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
                 SGN_CUDA(cudaMemsetAsync(E1->S.err, 0, sizeof(int), st));
             }
             if (st1 != SGN_OK) return st1;
-            for (int j = 0; j < nb; ++j) roff[j] = (long long)todo[t0 + j].at * n;
-            SGN_CUDA(cudaMemcpyAsync(roff_dev, roff.data(), sizeof(long long) * nb, cudaMemcpyHostToDevice, st));
-            SGN_CUDA(add_corrections<double2>(xs, roff_dev, nullptr, d, n, nb, st));
+            SGN_CUDA(add_corrections<double2>(xs, roff_dev, rex_dev, nullptr, d, n, nb, st));
         }
         return SGN_OK;
     };
@@ -1242,6 +1253,7 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
         const int nc = G->ncol;
         std::vector<double> sg(nc, -1.0), tl(nc, 1.0);
         std::vector<long long> off_h(nc, 0);
+        std::vector<int> ex_h(nc, 0);
         for (size_t t0 = 0; t0 < todo.size(); t0 += nc) {
             const int nb = (int)std::min<size_t>(nc, todo.size() - t0);
             for (int j = 0; j < nb; ++j) {
@@ -1251,11 +1263,13 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
                 tl[j] = std::min(0.1, std::max(kBiFloor, aim));
                 accept[y.at] = std::min(1.0, (aim < kBiFloor / 2 ? 3.0 : 12.0) / mg);
                 off_h[j] = (long long)y.at * n;
+                ex_h[j] = exponent(y);
             }
             SGN_CUDA(cudaMemcpyAsync(G->sigma, sg.data(), sizeof(double) * nc, cudaMemcpyHostToDevice, st));
             SGN_CUDA(cudaMemcpyAsync(G->tol, tl.data(), sizeof(double) * nc, cudaMemcpyHostToDevice, st));
             SGN_CUDA(cudaMemcpyAsync(G->off, off_h.data(), sizeof(long long) * nc, cudaMemcpyHostToDevice, st));
-            SGN_CUDA(bi_init(G->S, nc, rsd, G->off, nb, st));
+            SGN_CUDA(cudaMemcpyAsync(G->ex, ex_h.data(), sizeof(int) * nc, cudaMemcpyHostToDevice, st));
+            SGN_CUDA(bi_init(G->S, nc, rsd, G->off, G->ex, nb, st));
             int iters = 0;
             // as many applications of A^2 as FOM's cycle cap allows
             const int cap = (int)std::min<long long>(kBiCap, std::max<long long>(2, (long long)c->max_cycles * k1 / 2));
@@ -1270,7 +1284,7 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
                 fprintf(stderr, "[sgn mixed]   batch at %zu (%d systems): %d iterations, %zu failed so far\n", t0, nb,
                         iters, failed.size());
             const BiState& S = G->S;
-            SGN_CUDA(add_corrections<float2>(xs, G->off, S.done, S.d, n, nb, st));
+            SGN_CUDA(add_corrections<float2>(xs, G->off, G->ex, S.done, S.d, n, nb, st));
             SGN_CUDA(cudaStreamSynchronize(st));  // the host tables are filled again
         }
         return SGN_OK;
