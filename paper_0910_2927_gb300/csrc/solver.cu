@@ -17,6 +17,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <limits>
 #include <string>
 
 namespace sgn {
@@ -1233,6 +1234,11 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
     // 1e-3, and FP32 fields gain kBiFloor: accepted below rtol it gave an error of 2e-8 for BF16 links
     // at tol 1e-8).
     std::vector<double> accept(nall, 1.0);
+    // What a BiCGStab column reports is its recursive FP32 residual, which parts from the true one where the
+    // iterates grew on the way.  The true residual of the next round decides: a system that a correction
+    // did not bring to half of before is done if it is below rtol, and goes to FOM from then on if not.
+    std::vector<double> before(nall, std::numeric_limits<double>::infinity());  // of the last correction
+    std::vector<char> to_fom(nall, 0);
     // Correction solves by BiCGStab, each system to its own residual; the systems it gave up on are
     // left as they were and returned in `failed`.  What a residual r_i leaves in x is about
     // omega_i r_i / (spectrum - sigma_i), largest for the smallest shifts, which are also the slow
@@ -1262,6 +1268,7 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
                 sg[j] = c->sigma[y.at / ncol];
                 tl[j] = std::min(0.1, std::max(kBiFloor, aim));
                 accept[y.at] = std::min(1.0, (aim < kBiFloor / 2 ? 3.0 : 12.0) / mg);
+                before[y.at] = y.rel;
                 off_h[j] = (long long)y.at * n;
                 ex_h[j] = exponent(y);
             }
@@ -1279,9 +1286,10 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
                 if (G->h_done[j] != BI_DONE) {
                     failed.push_back(todo[t0 + j]);
                     accept[todo[t0 + j].at] = 1.0;
+                    before[todo[t0 + j].at] = std::numeric_limits<double>::infinity();
                 }
             if (debug_log())
-                fprintf(stderr, "[sgn mixed]   batch at %zu (%d systems): %d iterations, %zu failed so far\n", t0, nb,
+                fprintf(stderr, "[sgn mixed]   batch at %zu (%d systems): %d iterations, %zu to FOM so far\n", t0, nb,
                         iters, failed.size());
             const BiState& S = G->S;
             SGN_CUDA(add_corrections<float2>(xs, G->off, G->ex, S.done, S.d, n, nb, st));
@@ -1312,7 +1320,7 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
         SGN_CUDA(reduce(rd64, 1, nall, RM_STORE, 0, S64, nullptr, st));
         SGN_CUDA(cudaMemcpyAsync(hall.data(), S64.red, sizeof(double2) * hall.size(), cudaMemcpyDeviceToHost, st));
         SGN_CUDA(cudaStreamSynchronize(st));
-        std::vector<System> todo;
+        std::vector<System> todo, rest;  // rest: to FOM
         worst = 0;
         for (int i = 0; i < s; ++i)
             for (int col = 0; col < ncol; ++col) {
@@ -1323,12 +1331,18 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
                     return SGN_ERR_NONFINITE;
                 }
                 worst = std::max(worst, rel);
-                if (rel > rtol * accept[i * ncol + col]) todo.push_back({i * ncol + col, rel});
+                const int at = i * ncol + col;
+                if (rel > 0.5 * before[at]) {
+                    accept[at] = 1.0;
+                    to_fom[at] = rel > rtol;
+                }
+                if (rel > rtol * accept[at]) (shortrec && !to_fom[at] ? todo : rest).push_back({at, rel});
             }
         if (debug_log())
-            fprintf(stderr, "[sgn mixed] round %d: worst true residual %.3e, %zu of %d systems above tol\n", round,
-                    worst, todo.size(), nall);
-        if (todo.empty() || round == max_rounds) break;
+            fprintf(stderr, "[sgn mixed] round %d: worst true residual %.3e, %zu of %d systems above tol, %d stuck\n",
+                    round, worst, todo.size() + rest.size(), nall,
+                    (int)std::count(to_fom.begin(), to_fom.end(), 1));
+        if ((todo.empty() && rest.empty()) || round == max_rounds) break;
         ++ref_rounds;
         if (m > 0) {
             // the range(P) part of each residual is solved exactly in the eigenbasis,
@@ -1352,11 +1366,7 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
             SGN_CUDA(tsmm_nn<float2>(Rb32, n, m, S64.red, rs64, xs, n, nall, n, 1.0, st));
             SGN_CUDA(cudaStreamSynchronize(st));
         }
-        std::vector<System> rest;
-        if (shortrec)
-            SGN_CHECK(bicg_corrections(todo, rest));
-        else
-            rest = todo;
+        if (!todo.empty()) SGN_CHECK(bicg_corrections(todo, rest));
         if (!rest.empty()) SGN_CHECK(fom_corrections(rest));
     }
     // x = x_P + sum_i omega_i x_i
