@@ -12,8 +12,8 @@
 // now; the whole solve 133 -> 86 to 90 ms; the 6^4 x 1 solve 15.0 -> 11.2 ms.
 //
 // One iteration: w = A^2 p, k_bi_v, k_bi_s, t = A^2 s, k_bi_t, k_bi_x.  The shift enters as
-// w - sigma p and t - sigma s where these are used.  Sums: FP32 within a CTA, FP64 over the CTAs of a
-// column, done by the column's last CTA to arrive (same sums whatever the order), which then forms
+// w - sigma p and t - sigma s where these are used.  Sums: FP32 within a thread (up to eight complex
+// products), pairs of floats over a CTA, FP64 over the CTAs of a column, done by the column's last CTA to arrive (same sums whatever the order), which then forms
 // the column's next coefficients: no kernel waits for another.
 #include "blas.cuh"
 #include "cvt.cuh"
@@ -22,7 +22,6 @@ namespace sgn {
 namespace {
 
 constexpr int NT = 256;
-constexpr int NW = NT / 32;
 constexpr int MAXV = 7;  // real sums per kernel
 
 __device__ __forceinline__ float4 ld(const float2* f, int64_t i) { return reinterpret_cast<const float4*>(f)[i]; }
@@ -57,24 +56,21 @@ __device__ __forceinline__ double2 divc(double2 a, double2 b) {
 // Adds v over the column's CTAs.  True in thread 0 of the last CTA to arrive, with the sums in tot.
 template <int NV>
 __device__ __forceinline__ bool column_sum(float (&v)[NV], const BiState& S, int col, double (&tot)[NV]) {
-    __shared__ float sm[NV][NW];
+    __shared__ float sm[NV][NT];
     __shared__ double sd[NV];
     __shared__ int last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    static_assert(NV <= NT / 32, "a warp per sum");
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-        if (lane == 0) sm[k][warp] = v[k];
-    }
+    for (int k = 0; k < NV; ++k) sm[k][threadIdx.x] = v[k];
     __syncthreads();
-    float* part = S.partial + (int64_t)col * MAXV * S.nblk;
-    if (threadIdx.x < NV) {
-        float a = 0.f;
-#pragma unroll
-        for (int w = 0; w < NW; ++w) a += sm[threadIdx.x][w];
-        part[threadIdx.x * S.nblk + blockIdx.x] = a;
-        __threadfence();  // visible device-wide before this CTA is counted
+    double* part = S.partial + (int64_t)col * MAXV * S.nblk;
+    if (warp < NV) {
+        const double a = cta_sum_df<NT>(sm[warp], lane);
+        if (lane == 0) {
+            part[warp * S.nblk + blockIdx.x] = a;
+            __threadfence();  // visible device-wide before this CTA is counted
+        }
     }
     __syncthreads();
     if (threadIdx.x == 0) last = atomicAdd(&S.count[col], 1) == (int)gridDim.x - 1;
@@ -83,7 +79,7 @@ __device__ __forceinline__ bool column_sum(float (&v)[NV], const BiState& S, int
     __threadfence();
     if (warp < NV) {
         double a = 0.0;
-        for (int b = lane; b < (int)gridDim.x; b += 32) a += (double)__ldcg(part + warp * S.nblk + b);
+        for (int b = lane; b < (int)gridDim.x; b += 32) a += __ldcg(part + warp * S.nblk + b);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
         if (lane == 0) sd[warp] = a;
@@ -222,10 +218,10 @@ __global__ void __launch_bounds__(NT) k_bi_t(BiState S) {
     double tot[7];
     if (column_sum(v, S, col, tot)) {
         // q = 0 (with s = 0): r = s is the exact solution's residual, omega = 0 ends the column
-        const double iq = tot[6] > 0 ? 1.0 / tot[6] : 0.0;
+        const double iq = tot[6] == 0 ? 0.0 : 1.0 / tot[6];
         const double2 om = make_double2(tot[0] * iq, tot[1] * iq);
         const double2 rho = csub(make_double2(tot[2], tot[3]), cmul(om, make_double2(tot[4], tot[5])));
-        const double2 be = tot[6] > 0 ? divc(cmul(rho, S.alpha[col]), cmul(S.rho[col], om)) : make_double2(0, 0);
+        const double2 be = tot[6] == 0 ? make_double2(0, 0) : divc(cmul(rho, S.alpha[col]), cmul(S.rho[col], om));
         S.omega[col] = om;
         S.beta[col] = be;
         S.rho[col] = rho;
@@ -334,7 +330,7 @@ void bi_shape(BiState& S, int64_t n, int ncol) {
     S.pkt = 1;
     while (S.pkt < 4 && (int64_t)NT * S.pkt * S.nblk < S.npk) S.pkt *= 2;
 }
-size_t bi_partial_bytes(const BiState& S, int ncol) { return sizeof(float) * MAXV * (size_t)S.nblk * ncol; }
+size_t bi_partial_bytes(const BiState& S, int ncol) { return sizeof(double) * MAXV * (size_t)S.nblk * ncol; }
 
 cudaError_t bi_init(const BiState& S, int ncol, const double2* src, const long long* off, const int* ex, int nb,
                     cudaStream_t st) {

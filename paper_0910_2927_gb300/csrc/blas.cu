@@ -194,35 +194,6 @@ __device__ __forceinline__ float2 warp_sum_pair(float v) {
     }
     return make_float2(hi, lo);
 }
-// Double-float sum of the 256 FP32 values st[0..255] (one per thread of the CTA)
-// by one warp: 8 values per lane with TwoSum, then the lane butterfly.
-__device__ __forceinline__ double cta_sum_df(const float* st, int lane) {
-    float hi = 0.f, lo = 0.f;
-#pragma unroll
-    for (int q = 0; q < NT / 32; ++q) {
-        const float v = st[lane + 32 * q];
-        const float s = __fadd_rn(hi, v);
-        const float bp = __fsub_rn(s, hi);
-        const float ap = __fsub_rn(s, bp);
-        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, ap), __fsub_rn(v, bp)));
-        hi = s;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float ohi = __shfl_xor_sync(0xffffffffu, hi, o);
-        const float olo = __shfl_xor_sync(0xffffffffu, lo, o);
-        const float s = __fadd_rn(hi, ohi);
-        const float bp = __fsub_rn(s, hi);
-        const float ap = __fsub_rn(s, bp);
-        const float e = __fadd_rn(__fsub_rn(hi, ap), __fsub_rn(ohi, bp));
-        const float t = __fadd_rn(e, __fadd_rn(lo, olo));
-        const float nh = __fadd_rn(s, t);
-        lo = __fsub_rn(t, __fsub_rn(nh, s));
-        hi = nh;
-    }
-    return (double)hi + (double)lo;
-}
-
 // Warp sums of a per-thread FP32 complex partial (re, im); lane 0 stores the
 // FP64 result in sm[slot][warp].
 __device__ __forceinline__ void warp_store_f(double2 (*sm)[NWARP], int slot, float re, float im, int lane, int warp) {
@@ -618,7 +589,7 @@ __global__ void __launch_bounds__(NT) k_dcgs_dots(Basis<float2> V, int J, const 
     __syncthreads();
     const int bs = zc ? 2 * J : J;
     if (warp < (zc ? 4 : 1)) {
-        const double r = cta_sum_df(st[warp], lane);
+        const double r = cta_sum_df<NT>(st[warp], lane);
         if (lane == 0) {
             if (warp == 0) {
                 put(bs, 0, r);

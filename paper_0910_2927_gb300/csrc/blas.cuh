@@ -63,6 +63,36 @@ __device__ __forceinline__ double reduce_few(double (&a)[N], int lane) {
     return reduce_scatter<N>(a, lane);
 }
 
+// Sum of the N FP32 values st[0..N) (one per thread of a CTA) by one warp as an unevaluated pair (hi,
+// lo): N / 32 values per lane with TwoSum, then the lane butterfly.
+template <int N>
+__device__ __forceinline__ double cta_sum_df(const float* st, int lane) {
+    float hi = 0.f, lo = 0.f;
+#pragma unroll
+    for (int q = 0; q < N / 32; ++q) {
+        const float v = st[lane + 32 * q];
+        const float s = __fadd_rn(hi, v);
+        const float bp = __fsub_rn(s, hi);
+        const float ap = __fsub_rn(s, bp);
+        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, ap), __fsub_rn(v, bp)));
+        hi = s;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float ohi = __shfl_xor_sync(0xffffffffu, hi, o);
+        const float olo = __shfl_xor_sync(0xffffffffu, lo, o);
+        const float s = __fadd_rn(hi, ohi);
+        const float bp = __fsub_rn(s, hi);
+        const float ap = __fsub_rn(s, bp);
+        const float e = __fadd_rn(__fsub_rn(hi, ap), __fsub_rn(ohi, bp));
+        const float t = __fadd_rn(e, __fadd_rn(lo, olo));
+        const float nh = __fadd_rn(s, t);
+        lo = __fsub_rn(t, __fsub_rn(nh, s));
+        hi = nh;
+    }
+    return (double)hi + (double)lo;
+}
+
 // Tentative column j of the Hessenberg matrix in a delayed-CGS2 step, by one CTA:
 //   H[i][j] = c_i - g_i / rho (i < j),  H[j][j] = d - g_j / rho,  g = H[0:j+1, 0:j] s,
 // with the step's coefficients s = red[0, j), c = red[j, 2j), 1 / rho = red[2j], d = red[2j + 1].
@@ -198,7 +228,7 @@ struct BiState {
     const double* sigma;
     int* done;            // BiStatus (non-zero: skip)
     int* count;           // arrival counters of the sums
-    float* partial;
+    double* partial;
     int64_t npk;          // packs of two complex numbers per column
     int nblk, pkt;        // CTAs per column, packs per thread
 };

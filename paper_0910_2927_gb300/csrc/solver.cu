@@ -925,7 +925,7 @@ int get_bicg(sgn_ctx* c, int ncol, BiCg** out) {
     G->ex = reinterpret_cast<int*>(b + oi[2]);
     G->err = reinterpret_cast<int*>(b + oe);
     G->cyc = G->err + 1;
-    S.partial = reinterpret_cast<float*>(b + op);
+    S.partial = reinterpret_cast<double*>(b + op);
     // zero the whole arena once so no kernel ever reads uninitialised memory
     SGN_CUDA(cudaMemsetAsync(G->arena.p, 0, off, c->work));
     SGN_CUDA(cudaHostAlloc(&G->h_done, (nc + 1) * sizeof(int), cudaHostAllocDefault));
