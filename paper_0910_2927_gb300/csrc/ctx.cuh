@@ -63,6 +63,13 @@ struct Engine {
     // kernel timing: event pairs recorded inside the cycle (class, algorithmic bytes)
     std::vector<cudaEvent_t> tev;
     std::vector<std::pair<int, double>> tmarks;
+
+    Engine() = default;
+    Engine(const Engine&) = delete;
+    ~Engine() {
+        for (void* p : {(void*)h_done, (void*)h_resest, (void*)h_err, (void*)h_kk})
+            if (p) cudaFreeHost(p);
+    }
 };
 
 // Workspace and captured iterations of the refinement's BiCGStab corrections for ncol columns.
@@ -79,6 +86,12 @@ struct BiCg {
     uint64_t one_key = 0, loop_key = 0;
     long long kernels = 0;
     bool loop_unavailable = false;
+
+    BiCg() = default;
+    BiCg(const BiCg&) = delete;
+    ~BiCg() {
+        if (h_done) cudaFreeHost(h_done);
+    }
 };
 
 }  // namespace sgn

@@ -528,6 +528,11 @@ int get_engine(sgn_ctx* c, int ncol, int k, int s, int prec, Engine** out) {
     size_t ogres = take(nc * (size_t)(k + 1) * sizeof(double2));
     size_t oneg = take(nc * sizeof(double));
     size_t ocyc = take(sizeof(int));
+    // pinned memory first: it goes with the engine if the workspace cannot be had
+    SGN_CUDA(cudaHostAlloc(&E->h_done, nc * sizeof(int), cudaHostAllocDefault));
+    SGN_CUDA(cudaHostAlloc(&E->h_resest, nc * sizeof(double), cudaHostAllocDefault));
+    SGN_CUDA(cudaHostAlloc(&E->h_err, sizeof(int), cudaHostAllocDefault));
+    SGN_CUDA(cudaHostAlloc(&E->h_kk, nc * sizeof(int), cudaHostAllocDefault));
     SGN_CHECK(dev_alloc(c, E->arena, off));
     char* base = reinterpret_cast<char*>(E->arena.p);
     E->V = base + oV;
@@ -570,10 +575,6 @@ int get_engine(sgn_ctx* c, int ncol, int k, int s, int prec, Engine** out) {
         SGN_CUDA(cudaMemcpyAsync(E->neg1, m1.data(), nc * sizeof(double), cudaMemcpyHostToDevice, c->work));
         SGN_CUDA(cudaStreamSynchronize(c->work));  // m1 is released on return
     }
-    SGN_CUDA(cudaHostAlloc(&E->h_done, nc * sizeof(int), cudaHostAllocDefault));
-    SGN_CUDA(cudaHostAlloc(&E->h_resest, nc * sizeof(double), cudaHostAllocDefault));
-    SGN_CUDA(cudaHostAlloc(&E->h_err, sizeof(int), cudaHostAllocDefault));
-    SGN_CUDA(cudaHostAlloc(&E->h_kk, nc * sizeof(int), cudaHostAllocDefault));
     *out = E.get();
     c->engines[key] = std::move(E);
     return SGN_OK;
@@ -588,10 +589,6 @@ void release_engines(sgn_ctx* c) {
         if (E.loop) cudaGraphExecDestroy(E.loop);
         for (cudaEvent_t ev : E.tev) cudaEventDestroy(ev);
         dev_free(c, E.arena);
-        if (E.h_done) cudaFreeHost(E.h_done);
-        if (E.h_resest) cudaFreeHost(E.h_resest);
-        if (E.h_err) cudaFreeHost(E.h_err);
-        if (E.h_kk) cudaFreeHost(E.h_kk);
     }
     c->engines.clear();
     for (auto& kv : c->bicg) {
@@ -599,7 +596,6 @@ void release_engines(sgn_ctx* c) {
         if (G.one) cudaGraphExecDestroy(G.one);
         if (G.loop) cudaGraphExecDestroy(G.loop);
         dev_free(c, G.arena);
-        if (G.h_done) cudaFreeHost(G.h_done);
     }
     c->bicg.clear();
     dev_free(c, c->fom_d);
@@ -909,6 +905,7 @@ int get_bicg(sgn_ctx* c, int ncol, BiCg** out) {
     const size_t ooff = take(nc * sizeof(long long));
     for (size_t& o : oi) o = take(nc * sizeof(int));
     const size_t oe = take(2 * sizeof(int)), op = take(bi_partial_bytes(S, ncol));
+    SGN_CUDA(cudaHostAlloc(&G->h_done, (nc + 1) * sizeof(int), cudaHostAllocDefault));
     SGN_CHECK(dev_alloc(c, G->arena, off));
     char* b = reinterpret_cast<char*>(G->arena.p);
     float2** fields[7] = {&S.r, &S.rt, &S.p, &S.w, &S.s, &S.t, &S.d};
@@ -928,7 +925,6 @@ int get_bicg(sgn_ctx* c, int ncol, BiCg** out) {
     S.partial = reinterpret_cast<double*>(b + op);
     // zero the whole arena once so no kernel ever reads uninitialised memory
     SGN_CUDA(cudaMemsetAsync(G->arena.p, 0, off, c->work));
-    SGN_CUDA(cudaHostAlloc(&G->h_done, (nc + 1) * sizeof(int), cudaHostAllocDefault));
     *out = G.get();
     c->bicg[ncol] = std::move(G);
     return SGN_OK;
