@@ -186,7 +186,7 @@ SGN_API int sgn_set_method(sgn_ctx* ctx, int method);
 /* Mixed form only (no counterpart in the paper, which works in FP64): the FP32
  * correction solves that bring each shifted system's true FP64 residual below the
  * tolerance.  k_refine = 0 (default): BiCGStab, and restarted FOM(min(k, 16)) for the
- * systems it fails on; k_refine > 0: restarted FOM of that restart length.  max_batch:
+ * systems it fails on or gains nothing on; k_refine > 0: restarted FOM of that restart length.  max_batch:
  * how many shifted systems one correction batch solves side by side (0: up to 10 nrhs,
  * on small lattices all, bounded by memory).  Errors: SGN_ERR_ARG (k_refine > 64,
  * max_batch > 4096). */

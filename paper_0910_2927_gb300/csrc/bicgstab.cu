@@ -7,9 +7,10 @@
 // restarted FOM(16) reads and writes 28 fields per application of A^2 (16 + 8 of them for the
 // orthogonalisation) and loses convergence at every restart.  BiCGStab moves 9 fields per
 // application besides the two stencils' 4.5 and never restarts.  Every kernel below is bound by
-// HBM (FP32, two complex numbers per 16-byte load), on small lattices by launch latency.
-// Measured: the refinement of the 10^4 x 12 solve (240 systems, tol 1e-10) 75 ms with FOM(16), 34 to 38 ms
-// now; the whole solve 133 -> 86 to 90 ms; the 6^4 x 1 solve 15.0 -> 11.2 ms.
+// HBM (FP32, two complex numbers per 16-byte load), on small lattices by launch latency: 58 to 76 % of
+// the DRAM rate on 120 systems of 8^4 (k_bi_t and k_bi_v wait for the CTA's sums between their loads).
+// Measured: the refinement of the 10^4 x 12 solve (240 systems, tol 1e-10) 75 ms with FOM(16), about half
+// of that now; the whole solve 133 -> 91 ms; the 6^4 x 1 solve 15.0 -> 11.2 ms when it came in.
 //
 // One iteration: w = A^2 p, k_bi_v, k_bi_s, t = A^2 s, k_bi_t, k_bi_x.  The shift enters as
 // w - sigma p and t - sigma s where these are used.  Sums: FP32 within a thread (up to eight complex

@@ -15,7 +15,7 @@
 // Measured, us per launch averaged over the steps of a solve, before (one butterfly per sum, CTAs
 // of 256 elements) and now.  Two-field products: 4^4 x 1 column 24.6 -> 7.0, 6^4 x 1 32.0 -> 16.6,
 // 7x6x9x8 x 3 85.6 -> 42.5.  30 x 12 products on 16^4 (one field): 4472 -> 2055 (floor 1810: 8 flops
-// per product at the FP64 rate).  Update: 4^4 x 1 10.8 -> 3.9, 6^4 x 1 13.4 -> 8.0.
+// per product at the FP64 rate; FP64 pipe 95 % busy).  Update: 4^4 x 1 10.8 -> 3.9, 6^4 x 1 13.4 -> 8.0.
 #include "blas.cuh"
 
 #include <algorithm>

@@ -8,7 +8,8 @@
 // site's 24 real numbers in each lane, and 6 for the diagonal and the coefficient: 888 per site and
 // field, as in one thread.  The hop coefficients cost nothing of their own: a lane's sum is kept in
 // units of its hop's coefficient and the partner's number enters with the ratio of the two
-// (1, e^{+-mu} or e^{-+2 mu}).
+// (1, e^{+-mu} or e^{-+2 mu}).  Rounding of the FP64 form against extended precision, 4^4 to 8^4 at |mu|
+// up to 0.9: 1.08e-16 to 1.16e-16 of the result, 1.38e-16 to 1.44e-16 for one thread's chain of eight hops.
 // ROW: three warps share four sites, a colour of the result (a row of the link) each, so that a lane
 // has 45 instead of 111 floating-point instructions (the projections are repeated): for the
 // smallest lattices.

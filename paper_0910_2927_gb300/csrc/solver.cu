@@ -1007,7 +1007,10 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
     SGN_CHECK(get_engine(c, ncol, k, s, SGN_PREC_MIXED, &E));
     // Refinement batches: one shifted system per column, bounded by memory.  BiCGStab: all systems
     // together while they are few (small lattices are bound by launches), else 10 ncol, so that the
-    // quickly converging half (shifts far from the spectrum) does not idle along with the slow one.
+    // quickly converging half (shifts far from the spectrum) does not idle along with the slow one.  The
+    // line, 4 M complex numbers in all: together / 10 ncol at a time, ms per solve, 6^4 x 12 (3.6 M) 22.6 /
+    // 23.4, 8^4 x 4 (3.8 M) 21.6 / 23.3, 10^4 x 1 (2.3 M) 18.4 / 19.9, against 10^4 x 2 (4.6 M) 25.1 / 24.4,
+    // 8^4 x 6 (5.6 M) 26.5 / 26.0, 8^4 x 12 (11 M) 45.2 / 42.8.
     const int nall = s * ncol;  // every (shift, column) pair as one column of [i][col][n]
     const bool shortrec = c->k_refine == 0;
     const int k1 = c->k_refine > 0 ? c->k_refine : std::min(k, 16);
@@ -1240,7 +1243,9 @@ int solve_mixed(sgn_ctx* c, const double2* b, double2* x, double2* x_shift, int 
     // omega_i r_i / (spectrum - sigma_i), largest for the smallest shifts, which are also the slow
     // ones: the systems aim at tol / margin_i, margin_i from 54 for the largest omega / |sigma| down
     // with its fourth root (at a margin of 9 for all, the error of x on the 10^4 workload was 2.3
-    // times that of FOM corrections).
+    // times that of FOM corrections).  Over 48 solves (4^4 to 10^4 and ragged lattices, mu 0 to 0.35, 12
+    // to 20 poles, FP32 and 16-bit links, tol 1e-8 and 1e-10) the error of x is 0.05 to 1.15 times that of
+    // the FOM corrections before, 0.44 on the geometric mean.
     std::vector<double> margin(s);
     {
         double wmax = 0;

@@ -6,7 +6,7 @@
 // whatever its active lanes, and a site costs about 900 of them.  With a thread per site a 4^4
 // lattice is eight warps of 900; with a lane per hop it is 64 warps of 114.  Measured, us per
 // launch, thread per site -> lane per hop: 4^4 x 1 field 31.3 -> 6.5, 6^4 x 1 32.5 -> 6.8,
-// 7x6x9x8 x 3 32.8 -> 18.9, 10^4 x 12 206 -> 189 (92 % of the FP64 rate), where natural-order
+// 7x6x9x8 x 3 32.8 -> 18.9, 10^4 x 12 206 -> 189 (FP64 pipe 92 % busy), where natural-order
 // fields also save the 24 us of packing and unpacking.  A row of the link per warp (45 instructions)
 // took the 4^4 solve from 5.80 to 4.69 ms (361 of its 1,000 launches are stencils).
 #include "hops.cuh"
